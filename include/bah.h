@@ -68,7 +68,8 @@ extern "C" {
  * BAH_MIXED mode, the operator w = H z and the update x += Z y on the FP32
  * flexible basis); the Hessenberg least-squares update, the true residual and
  * x are FP64 always */
-#define BAH_KRYLOV_FP64 0  /* IEEE FP64 */
+#define BAH_KRYLOV_FP64 0  /* FP64 vectors; the basis and the sums of the dots and updates in 60-bit block
+                              fixed point (256 entries share an exponent), no less accurate than FP64 sums */
 #define BAH_KRYLOV_DF   1  /* double-FP32: each real is an FP32 pair hi + lo (48-bit significand),
                               products and sums by error-free FP32 transformations */
 

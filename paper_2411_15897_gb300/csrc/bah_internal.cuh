@@ -289,8 +289,10 @@ void launch_convert(const Vin* x, Vout* y, size_t n, cudaStream_t st);
 
 // Krylov (k_krylov.cu), batched over right-hand sides
 constexpr int RED_CTAS = 296;   // partial sums per reduction (2 per SM on 148+ SMs)
+constexpr int GS_CTAS = 608;    // most partial sums of a Gram-Schmidt kernel (4 CTAs on each of 152 SMs)
 struct KS {                     // per-right-hand-side element strides and active flags
     size_t sv = 0;              // basis V (m+1 vectors)
+    size_t se = 0;              // tile exponents of the basis
     size_t sw = 0;              // work vector w
     size_t sp = 0;              // dot partials
     size_t so = 0;              // small per-rhs arrays (h1, h2, cs, sn, g, y)
@@ -299,14 +301,22 @@ struct KS {                     // per-right-hand-side element strides and activ
     size_t sx = 0;              // solution x
     const int* active = nullptr;
 };
-void launch_dot_norm(const double2* V, int k, const double2* w, size_t n, double2* partial, double2* out,
+// The FP64 basis in block fixed point (k_gs.cu): vector i's limbs at
+// VL + i * tiles * 256, its tile exponents at VE + i * tiles.
+int gs_prepare();   // once per context, before the first launch
+void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, size_t n, double2* partial, double2* out,
                      const int* flag, int nrhs, const KS& ks, cudaStream_t st);
-void launch_axpy_norm(const double2* V, int k, const double2* coef, double2* w, size_t n, double* npart,
-                      const int* flag, int nrhs, const KS& ks, cudaStream_t st);
+// returns the number of partial sums of |w_new|^2 in npart
+int launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
+                     const int* flag, int nrhs, const KS& ks, cudaStream_t st);
+// v = w / sc[slot] as FP64 (vc, stride ks.sw) and as a basis vector (vl, ve)
+void launch_basis_store(const double2* w, const double* sc, int slot, double2* vc, int4* vl, int* ve, size_t n,
+                        size_t sw, int nrhs, const KS& ks, cudaStream_t st);
 // flag = 1 (second pass) when ||w'||^2 < eta2 ||w||^2 (DGKS criterion; eta2 = 1/2 classically)
-void launch_dgks_decide(const double* npart, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
+void launch_dgks_decide(const double* npart, int np, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
                         const KS& ks, cudaStream_t st, double eta2 = 0.5);
-void launch_pass2_norm(const double* npart, const int* flag, double* sc, int nrhs, const KS& ks, cudaStream_t st);
+void launch_pass2_norm(const double* npart, int np, const int* flag, double* sc, int nrhs, const KS& ks,
+                       cudaStream_t st);
 void launch_norm2(const double2* w, size_t n, double* partial, double* sc, int slot, int nrhs, const KS& ks,
                   cudaStream_t st);
 template <class Vz>
@@ -325,7 +335,7 @@ void launch_init_arnoldi(const double* sc, double2* g, int m, double* status, in
 // double-float Krylov kernels (k_krylov_df.cu)
 void launch_dot_norm_df(const float4* V, int k, const float4* w, size_t n, double2* partial, double2* out,
                         const int* flag, int nrhs, const KS& ks, cudaStream_t st);
-void launch_axpy_norm_df(const float4* V, int k, const double2* coef, float4* w, size_t n, double* npart,
+int launch_axpy_norm_df(const float4* V, int k, const double2* coef, float4* w, size_t n, double* npart,
                          const int* flag, int nrhs, const KS& ks, cudaStream_t st);
 void launch_scale_copy_df(const void* w, bool from64, const double* sc, int slot, float4* v, size_t n, size_t sw,
                           size_t sv, int nrhs, const KS& ks, cudaStream_t st);

@@ -38,149 +38,10 @@ __device__ __forceinline__ bool inactive(const KS& ks, int r) { return ks.active
 
 // ---------------------------------------------------------------------------
 // Gram-Schmidt with selective reorthogonalisation (Daniel-Gragg-Kaufman-Stewart
-// criterion): pass 1 forms h1 = V^H w together with ||w||^2 and then
-// w' = w - V h1 together with ||w'||^2; a second pass runs only if
-// ||w'|| < ||w|| / sqrt(2).  The pass-2 kernels read the per-right-hand-side
-// flag and return at once when it is clear.
+// criterion): a second pass runs only if ||w'|| < ||w|| / sqrt(2).  The
+// projections and updates themselves are in k_gs.cu (FP64 basis) and
+// k_krylov_df.cu; npart holds np partial sums of ||w'||^2 per right-hand side.
 // ---------------------------------------------------------------------------
-// The FP64 pipe (2 FMA/clk/SM on GB300, 1/64 of FP32) bounds these kernels,
-// so every complex multiply-add is written as four explicit fused
-// multiply-adds into the accumulator (a plain "acc += a*b + c*d" compiles to a
-// multiply, an FMA and an add: six FP64 instructions per complex MAC).
-__device__ __forceinline__ void cmac_conj(double2& acc, const double2& a, const double2& b) {   // acc += conj(a) b
-    acc.x = fma(a.x, b.x, acc.x);
-    acc.x = fma(a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y);
-    acc.y = fma(-a.y, b.x, acc.y);
-}
-__device__ __forceinline__ void cmsub(double2& acc, const double2& c, const double2& v) {       // acc -= c v
-    acc.x = fma(-c.x, v.x, acc.x);
-    acc.x = fma(c.y, v.y, acc.x);
-    acc.y = fma(-c.x, v.y, acc.y);
-    acc.y = fma(-c.y, v.x, acc.y);
-}
-
-// Partial sums of rows y0 .. y0+kG-1 (blockIdx.y = row group): row y < k is
-// conj(V_y) w, row k is |w|^2 (imaginary part 0).  Each thread loads w once per
-// element for the kG rows of its group.  The kG complex partials of the CTA are
-// reduced through shared memory: thread t sums quantity t / 16 over a slice of
-// 16 threads, then 16-lane shuffles finish it (few FP64 adds per thread).
-constexpr int kDotG = 8;
-__global__ void __launch_bounds__(256) k_dot_norm_partial(const double2* __restrict__ V, int k,
-                                                          const double2* __restrict__ w, size_t n,
-                                                          double2* __restrict__ partial, const int* flag, KS ks) {
-    pdl_prologue();
-    const int r = blockIdx.z;
-    if (inactive(ks, r) || (flag && flag[r] == 0)) return;
-    V += r * ks.sv;
-    w += r * ks.sw;
-    partial += r * ks.sp;
-    const int y0 = blockIdx.y * kDotG;
-    const int ny = min(kDotG, k + 1 - y0);          // rows of this group (the norm row is row k)
-    double2 acc[kDotG];
-#pragma unroll
-    for (int q = 0; q < kDotG; ++q) acc[q] = make_double2(0.0, 0.0);
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += stride) {
-        const double2 b = __ldg(w + e);
-        double2 a[kDotG];
-#pragma unroll
-        for (int q = 0; q < kDotG; ++q)
-            if (q < ny && y0 + q < k) a[q] = __ldg(V + (size_t)(y0 + q) * n + e);
-#pragma unroll
-        for (int q = 0; q < kDotG; ++q) {
-            if (q >= ny) break;
-            if (y0 + q < k) {
-                cmac_conj(acc[q], a[q], b);
-            } else {
-                acc[q].x = fma(b.x, b.x, acc[q].x);
-                acc[q].x = fma(b.y, b.y, acc[q].x);
-            }
-        }
-    }
-    __shared__ double sh[2 * kDotG][256];
-#pragma unroll
-    for (int q = 0; q < kDotG; ++q) {
-        sh[2 * q][threadIdx.x] = acc[q].x;
-        sh[2 * q + 1][threadIdx.x] = acc[q].y;
-    }
-    __syncthreads();
-    const int qv = threadIdx.x >> 4, sl = threadIdx.x & 15;     // quantity, slice
-    double s = 0.0;
-#pragma unroll
-    for (int u = 0; u < 16; ++u) s += sh[qv][sl * 16 + u];
-    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (sl == 0 && (qv >> 1) < ny) {
-        double* dst = reinterpret_cast<double*>(partial + (size_t)(y0 + (qv >> 1)) * gridDim.x + blockIdx.x);
-        dst[qv & 1] = s;
-    }
-}
-__global__ void __launch_bounds__(256) k_reduce_rows(const double2* __restrict__ partial, int np, double2* out,
-                                                     const int* flag, KS ks) {
-    pdl_prologue();
-    const int r = blockIdx.z;
-    if (inactive(ks, r)) return;
-    partial += r * ks.sp;
-    out += r * ks.so;
-    if (flag && flag[r] == 0) {
-        if (threadIdx.x == 0) out[blockIdx.y] = make_double2(0.0, 0.0);
-        return;
-    }
-    double2 acc = make_double2(0.0, 0.0);
-    for (int e = threadIdx.x; e < np; e += blockDim.x) {
-        const double2 a = partial[(size_t)blockIdx.y * np + e];
-        acc.x += a.x;
-        acc.y += a.y;
-    }
-    acc = block_sum2(acc);
-    if (threadIdx.x == 0) out[blockIdx.y] = acc;
-}
-void launch_dot_norm(const double2* V, int k, const double2* w, size_t n, double2* partial, double2* out,
-                     const int* flag, int nrhs, const KS& ks, cudaStream_t st) {
-    const int groups = (k + 1 + kDotG - 1) / kDotG;
-    launch_pdl(k_dot_norm_partial, dim3(dim3(RED_CTAS, groups, nrhs)), dim3(256), 0, st, V, k, w, n, partial, flag, ks);
-    launch_pdl(k_reduce_rows, dim3(dim3(1, k + 1, nrhs)), dim3(256), 0, st, partial, RED_CTAS, out, flag, ks);
-}
-
-// w -= sum_i coef[i] V_i, and per-CTA partial sums of |w_new|^2
-__global__ void __launch_bounds__(512) k_axpy_norm(const double2* __restrict__ V, int k,
-                                                   const double2* __restrict__ coef, double2* __restrict__ w, size_t n,
-                                                   double* __restrict__ npart, const int* flag, KS ks) {
-    pdl_prologue();
-    const int r = blockIdx.z;
-    if (inactive(ks, r) || (flag && flag[r] == 0)) return;
-    V += r * ks.sv;
-    w += r * ks.sw;
-    coef += r * ks.so;
-    npart += r * RED_CTAS;
-    __shared__ double2 c[64];
-    if (threadIdx.x < k) c[threadIdx.x] = coef[threadIdx.x];
-    __syncthreads();
-    double nn = 0.0;
-    constexpr int kU = 8;   // rows whose loads go out together
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        double2 acc = w[e];
-        int i = 0;
-        for (; i + kU <= k; i += kU) {
-            double2 v[kU];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) v[u] = __ldg(V + (size_t)(i + u) * n + e);
-#pragma unroll
-            for (int u = 0; u < kU; ++u) cmsub(acc, c[i + u], v[u]);
-        }
-        for (; i < k; ++i) cmsub(acc, c[i], __ldg(V + (size_t)i * n + e));
-        w[e] = acc;
-        nn = fma(acc.x, acc.x, nn);
-        nn = fma(acc.y, acc.y, nn);
-    }
-    double2 rs = block_sum2(make_double2(nn, 0.0));
-    if (threadIdx.x == 0) npart[blockIdx.x] = rs.x;
-}
-void launch_axpy_norm(const double2* V, int k, const double2* coef, double2* w, size_t n, double* npart,
-                      const int* flag, int nrhs, const KS& ks, cudaStream_t st) {
-    launch_pdl(k_axpy_norm, dim3(dim3(RED_CTAS, 1, nrhs)), dim3(512), 0, st, V, k, coef, w, n, npart, flag, ks);
-}
-
 // reduce the pass-1 norm, decide on the second pass, set ||w|| for the Givens
 // step: sc[2] = ||w_final||, sc[3] counts second passes; flag = 1 when
 // ||w'||^2 < ||w||^2 / 2
@@ -189,7 +50,7 @@ __global__ void __launch_bounds__(256) k_dgks_decide(const double* npart, int np
     pdl_prologue();
     const int r = blockIdx.x;
     if (inactive(ks, r)) return;
-    npart += r * RED_CTAS;
+    npart += r * GS_CTAS;
     double acc = 0.0;
     for (int e = threadIdx.x; e < np; e += blockDim.x) acc += npart[e];
     double2 s = block_sum2(make_double2(acc, 0.0));
@@ -201,23 +62,24 @@ __global__ void __launch_bounds__(256) k_dgks_decide(const double* npart, int np
         sc[r * 8 + 3] += (double)f;
     }
 }
-void launch_dgks_decide(const double* npart, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
+void launch_dgks_decide(const double* npart, int np, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
                         const KS& ks, cudaStream_t st, double eta2) {
-    launch_pdl(k_dgks_decide, dim3(nrhs), dim3(256), 0, st, npart, RED_CTAS, h1norm, k, flag, sc, eta2, ks);
+    launch_pdl(k_dgks_decide, dim3(nrhs), dim3(256), 0, st, npart, np, h1norm, k, flag, sc, eta2, ks);
 }
 // after pass 2: ||w''|| replaces ||w'||
 __global__ void __launch_bounds__(256) k_pass2_norm(const double* npart, int np, const int* flag, double* sc, KS ks) {
     pdl_prologue();
     const int r = blockIdx.x;
     if (inactive(ks, r) || flag[r] == 0) return;
-    npart += r * RED_CTAS;
+    npart += r * GS_CTAS;
     double acc = 0.0;
     for (int e = threadIdx.x; e < np; e += blockDim.x) acc += npart[e];
     double2 s = block_sum2(make_double2(acc, 0.0));
     if (threadIdx.x == 0) sc[r * 8 + 2] = sqrt(s.x);
 }
-void launch_pass2_norm(const double* npart, const int* flag, double* sc, int nrhs, const KS& ks, cudaStream_t st) {
-    launch_pdl(k_pass2_norm, dim3(nrhs), dim3(256), 0, st, npart, RED_CTAS, flag, sc, ks);
+void launch_pass2_norm(const double* npart, int np, const int* flag, double* sc, int nrhs, const KS& ks,
+                       cudaStream_t st) {
+    launch_pdl(k_pass2_norm, dim3(nrhs), dim3(256), 0, st, npart, np, flag, sc, ks);
 }
 
 // ---------------------------------------------------------------------------

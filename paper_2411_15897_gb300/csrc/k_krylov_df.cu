@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(512) k_axpy_norm_df(const float4* __restrict__
     V += r * ks.sv;
     w += r * ks.sw;
     coef += r * ks.so;
-    npart += r * RED_CTAS;
+    npart += r * GS_CTAS;
     __shared__ float4 c[64];
     if (threadIdx.x < k) c[threadIdx.x] = cdf_from_double2(coef[threadIdx.x]);
     __syncthreads();
@@ -158,9 +158,10 @@ __global__ void __launch_bounds__(512) k_axpy_norm_df(const float4* __restrict__
     double2 rs = block_sum2_df(make_double2(nn.value(), 0.0));
     if (threadIdx.x == 0) npart[blockIdx.x] = rs.x;
 }
-void launch_axpy_norm_df(const float4* V, int k, const double2* coef, float4* w, size_t n, double* npart,
+int launch_axpy_norm_df(const float4* V, int k, const double2* coef, float4* w, size_t n, double* npart,
                          const int* flag, int nrhs, const KS& ks, cudaStream_t st) {
     launch_pdl(k_axpy_norm_df, dim3(dim3(RED_CTAS, 1, nrhs)), dim3(512), 0, st, V, k, coef, w, n, npart, flag, ks);
+    return RED_CTAS;
 }
 
 // v = w / sc[slot]: from a double-float w, or (from64) from an FP64 vector

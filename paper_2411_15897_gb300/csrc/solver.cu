@@ -7,6 +7,7 @@
 // and FGMRES (right preconditioned, two-pass classical Gram-Schmidt, Givens
 // rotations on the device) wraps it with the FP64 operator H of Eq. 2.6.
 #include "bah_internal.cuh"
+#include "fix60.cuh"
 
 #include <algorithm>
 #include <array>
@@ -65,6 +66,11 @@ struct Ctx {
     // Krylov workspace
     int m = 20;
     double2 *V = nullptr, *W = nullptr, *R = nullptr, *Bs = nullptr, *X = nullptr;
+    // the FP64 basis of the lockstep solve: limbs and tile exponents (fix60.cuh), and the newest
+    // vector in FP64, the preconditioner's input (V itself holds the other two kinds of basis)
+    int4* VL = nullptr;
+    int* VE = nullptr;
+    double2* Vc = nullptr;
     double2 *Hm = nullptr, *h1v = nullptr, *h2v = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr;
     double2* partial = nullptr;
     double *nrm = nullptr, *dpart = nullptr, *status = nullptr;
@@ -115,7 +121,9 @@ struct Ctx {
     bool exact = false;
     Fine5<double, double2> f5x{};       // FP64 block operators, diagonals shifted by block_alpha
     int mi = 60;                        // inner restart length
-    double2 *iV = nullptr, *iZ = nullptr, *iW = nullptr, *iR = nullptr, *iH = nullptr;
+    int4* iVL = nullptr;
+    int* iVE = nullptr;
+    double2 *iVc = nullptr, *iZ = nullptr, *iW = nullptr, *iR = nullptr, *iH = nullptr;
     double2 *ih1 = nullptr, *ih2 = nullptr, *ics = nullptr, *isn = nullptr, *igv = nullptr, *iy = nullptr;
     double2* ipart = nullptr;
     double *inrm = nullptr, *idpart = nullptr, *istatus = nullptr;
@@ -649,11 +657,11 @@ static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t
     int total = 0;
     while (beta > rtol * bn) {
         if (total >= c.o.block_maxit) { ++c.block_failures; break; }
-        launch_scale_copy(c.iR, c.inrm, 0, c.iV, np, 0, 0, 1, ks, st);
+        launch_basis_store(c.iR, c.inrm, 0, c.iVc, c.iVL, c.iVE, np, 0, 1, ks, st);
         launch_init_arnoldi(c.inrm, c.igv, m, c.istatus, 1, ks, st);
         int jd = 0;
         for (int j = 0; j < m && total < c.o.block_maxit; ++j) {
-            const double2* vj = c.iV + (size_t)j * np;
+            const double2* vj = c.iVc;
             double2* zj = c.iZ + (size_t)j * np;
             // z_j = (one multigrid cycle of the block) v_j
             if constexpr (MODE == BAH_MIXED) {
@@ -668,14 +676,15 @@ static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t
             }
             // w = M z_j, Gram-Schmidt with selective reorthogonalisation, Givens, v_{j+1}
             launch_block_apply64(c.f5x, b, zj, c.iW, nullptr, st);
-            launch_dot_norm(c.iV, j + 1, c.iW, np, c.ipart, c.ih1, nullptr, 1, ks, st);
-            launch_axpy_norm(c.iV, j + 1, c.ih1, c.iW, np, c.idpart, nullptr, 1, ks, st);
-            launch_dgks_decide(c.idpart, c.ih1, j + 1, c.iflag, c.inrm, 1, ks, st);
-            launch_dot_norm(c.iV, j + 1, c.iW, np, c.ipart, c.ih2, c.iflag, 1, ks, st);
-            launch_axpy_norm(c.iV, j + 1, c.ih2, c.iW, np, c.idpart, c.iflag, 1, ks, st);
-            launch_pass2_norm(c.idpart, c.iflag, c.inrm, 1, ks, st);
+            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih1, nullptr, 1, ks, st);
+            const int npt = launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih1, c.iW, np, c.idpart, nullptr, 1, ks, st);
+            launch_dgks_decide(c.idpart, npt, c.ih1, j + 1, c.iflag, c.inrm, 1, ks, st);
+            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih2, c.iflag, 1, ks, st);
+            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih2, c.iW, np, c.idpart, c.iflag, 1, ks, st);
+            launch_pass2_norm(c.idpart, npt, c.iflag, c.inrm, 1, ks, st);
             launch_arnoldi_givens(c.iH, m + 1, c.ih1, c.ih2, c.inrm, j, c.ics, c.isn, c.igv, c.istatus, 1, ks, st);
-            launch_scale_copy(c.iW, c.inrm, 2, c.iV + (size_t)(j + 1) * np, np, 0, 0, 1, ks, st);
+            launch_basis_store(c.iW, c.inrm, 2, c.iVc, c.iVL + (j + 1) * tiles_of(np) * kTile,
+                               c.iVE + (j + 1) * tiles_of(np), np, 0, 1, ks, st);
             BAH_CUDA_TRY(cudaMemcpyAsync(c.histat, c.istatus, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
             BAH_CUDA_TRY(cudaStreamSynchronize(st));
             ++total;
@@ -800,7 +809,15 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     const int m = c.m;
     const size_t nbt = c.nbatch;
     const size_t so = m + 2;
-    TRY(c.alloc_t(&c.V, n * (m + 1) * nbt));
+    const size_t nt = tiles_of(n);
+    if (c.kdf || c.o.block_krylov) {
+        TRY(c.alloc_t(&c.V, n * (m + 1) * nbt));
+    } else {
+        TRY(gs_prepare());
+        TRY(c.alloc_t(&c.VL, nt * kTile * (m + 1) * nbt));
+        TRY(c.alloc_t(&c.VE, nt * (m + 1) * nbt));
+        TRY(c.alloc_t(&c.Vc, n * nbt));
+    }
     TRY(c.alloc(&c.Z, n * m * c.vsz * nbt));
     TRY(c.alloc_t(&c.W, n * nbt)); TRY(c.alloc_t(&c.R, n * nbt)); TRY(c.alloc_t(&c.Bs, n * nbt));
     TRY(c.alloc_t(&c.X, n * nbt));
@@ -810,8 +827,8 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     TRY(c.alloc_t(&c.gsflag, nbt));
     TRY(c.alloc_t(&c.cs, so * nbt)); TRY(c.alloc_t(&c.sn, so * nbt)); TRY(c.alloc_t(&c.g, so * nbt));
     TRY(c.alloc_t(&c.y, so * nbt));
-    TRY(c.alloc_t(&c.partial, so * RED_CTAS * nbt));
-    TRY(c.alloc_t(&c.dpart, (size_t)RED_CTAS * nbt));
+    TRY(c.alloc_t(&c.partial, so * GS_CTAS * nbt));
+    TRY(c.alloc_t(&c.dpart, (size_t)GS_CTAS * nbt));
     TRY(c.alloc_t(&c.nrm, 8 * nbt));
     TRY(c.alloc_t(&c.status, 4 * nbt));
     TRY(c.alloc_t(&c.active, nbt));
@@ -819,7 +836,8 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     BAH_CUDA_TRY(cudaMemsetAsync(c.nrm, 0, 8 * nbt * sizeof(double), st));
     BAH_CUDA_TRY(cudaMallocHost((void**)&c.hstatus, (4 * (size_t)(m + 1) * nbt + 8 * nbt) * sizeof(double)));
     BAH_CUDA_TRY(cudaMallocHost((void**)&c.hint, kIntSlots * nbt * sizeof(int)));
-    c.ks.sv = (size_t)(m + 1) * n; c.ks.sw = n; c.ks.sp = so * RED_CTAS; c.ks.so = so;
+    c.ks.sv = (size_t)(m + 1) * (c.VL ? nt * kTile : n); c.ks.se = (size_t)(m + 1) * nt;
+    c.ks.sw = n; c.ks.sp = so * GS_CTAS; c.ks.so = so;
     c.ks.sh = (size_t)(m + 1) * m; c.ks.sz = (size_t)m * n; c.ks.sx = n; c.ks.active = c.active;
     BAH_CUDA_TRY(cudaStreamCreateWithFlags(&c.cap_stream, cudaStreamNonBlocking));
     c.ig.assign(m, Ctx::IterGraph());
@@ -1029,12 +1047,14 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
         }
         c.f5x = Fine5<double, double2>{c.n1, c.n2, c.cx, c.cz, c.nx, c.nz, c.wx, c.wz, dgb[0], dgb[1], dgb[2], c.dAp};
         const size_t so = c.mi + 2;
-        TRY(c.alloc_t(&c.iV, (size_t)(c.mi + 1) * np)); TRY(c.alloc_t(&c.iZ, (size_t)c.mi * np));
+        TRY(gs_prepare());
+        TRY(c.alloc_t(&c.iVL, (c.mi + 1) * tiles_of(np) * kTile)); TRY(c.alloc_t(&c.iVE, (c.mi + 1) * tiles_of(np)));
+        TRY(c.alloc_t(&c.iVc, np)); TRY(c.alloc_t(&c.iZ, (size_t)c.mi * np));
         TRY(c.alloc_t(&c.iW, np)); TRY(c.alloc_t(&c.iR, np));
         TRY(c.alloc_t(&c.iH, (size_t)(c.mi + 1) * c.mi));
         TRY(c.alloc_t(&c.ih1, so)); TRY(c.alloc_t(&c.ih2, so)); TRY(c.alloc_t(&c.ics, so)); TRY(c.alloc_t(&c.isn, so));
         TRY(c.alloc_t(&c.igv, so)); TRY(c.alloc_t(&c.iy, so));
-        TRY(c.alloc_t(&c.ipart, so * RED_CTAS)); TRY(c.alloc_t(&c.idpart, (size_t)RED_CTAS));
+        TRY(c.alloc_t(&c.ipart, so * GS_CTAS)); TRY(c.alloc_t(&c.idpart, (size_t)GS_CTAS));
         TRY(c.alloc_t(&c.inrm, 8)); TRY(c.alloc_t(&c.istatus, 4)); TRY(c.alloc_t(&c.iflag, 1)); TRY(c.alloc_t(&c.ijk, 1));
         TRY(c.alloc_t(&c.ez, 3 * (size_t)np)); TRY(c.alloc_t(&c.etp, np)); TRY(c.alloc_t(&c.esu, 2 * (size_t)np));
         BAH_CUDA_TRY(cudaMemsetAsync(c.inrm, 0, 8 * sizeof(double), st));
@@ -1175,39 +1195,41 @@ static void iter_body(Ctx& c, int j, cudaStream_t st) {
     float4* Vd = (float4*)c.V;
     float4* Wd = (float4*)c.W;
     if (c.kdf) precond_any(c, Vd + (size_t)j * n, ks.sv, zj, ks.sz, bt, st);
-    else precond_any(c, c.V + (size_t)j * n, ks.sv, zj, ks.sz, bt, st);
+    else precond_any(c, (const double2*)c.Vc, n, zj, ks.sz, bt, st);
     op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
     const double k1 = j + 1;
+    int npt = 0;                 // partial sums of ||w'||^2
     {
         Prof pr(c, BAH_K_DOT, st, nb * (k1 + 1) * n * 16.0, 2);
         if (c.kdf) launch_dot_norm_df(Vd, j + 1, Wd, n, c.partial, c.h1v, nullptr, nb, ks, st);
-        else launch_dot_norm(c.V, j + 1, c.W, n, c.partial, c.h1v, nullptr, nb, ks, st);
+        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h1v, nullptr, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_AXPY, st, nb * (k1 + 2) * n * 16.0);
-        if (c.kdf) launch_axpy_norm_df(Vd, j + 1, c.h1v, Wd, n, c.dpart, nullptr, nb, ks, st);
-        else launch_axpy_norm(c.V, j + 1, c.h1v, c.W, n, c.dpart, nullptr, nb, ks, st);
+        if (c.kdf) npt = launch_axpy_norm_df(Vd, j + 1, c.h1v, Wd, n, c.dpart, nullptr, nb, ks, st);
+        else npt = launch_axpy_norm(c.VL, c.VE, j + 1, c.h1v, c.W, n, c.dpart, nullptr, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_NORM, st, 0.0);
-        launch_dgks_decide(c.dpart, c.h1v, j + 1, c.gsflag, c.nrm, nb, ks, st, c.dgks_eta2);
+        launch_dgks_decide(c.dpart, npt, c.h1v, j + 1, c.gsflag, c.nrm, nb, ks, st, c.dgks_eta2);
     }
     {
         Prof pr(c, BAH_K_DOT, st, 0.0, 2);      // runs only where the flag is set (bytes counted as zero)
         if (c.kdf) launch_dot_norm_df(Vd, j + 1, Wd, n, c.partial, c.h2v, c.gsflag, nb, ks, st);
-        else launch_dot_norm(c.V, j + 1, c.W, n, c.partial, c.h2v, c.gsflag, nb, ks, st);
+        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h2v, c.gsflag, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_AXPY, st, 0.0);
         if (c.kdf) launch_axpy_norm_df(Vd, j + 1, c.h2v, Wd, n, c.dpart, c.gsflag, nb, ks, st);
-        else launch_axpy_norm(c.V, j + 1, c.h2v, c.W, n, c.dpart, c.gsflag, nb, ks, st);
+        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h2v, c.W, n, c.dpart, c.gsflag, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_SMALL, st, nb * n * 32.0, 3);
-        launch_pass2_norm(c.dpart, c.gsflag, c.nrm, nb, ks, st);
+        launch_pass2_norm(c.dpart, npt, c.gsflag, c.nrm, nb, ks, st);
         launch_arnoldi_givens(c.Hm, m + 1, c.h1v, c.h2v, c.nrm, j, c.cs, c.sn, c.g, c.status, nb, ks, st);
         if (c.kdf) launch_scale_copy_df(c.W, false, c.nrm, 2, Vd + (size_t)(j + 1) * n, n, n, ks.sv, nb, ks, st);
-        else launch_scale_copy(c.W, c.nrm, 2, c.V + (size_t)(j + 1) * n, n, n, ks.sv, nb, ks, st);
+        else launch_basis_store(c.W, c.nrm, 2, c.Vc, c.VL + (j + 1) * tiles_of(n) * kTile, c.VE + (j + 1) * tiles_of(n), n,
+                                n, nb, ks, st);
     }
     cudaMemcpyAsync(status_slot(c, j), c.status, 4 * (size_t)nb * sizeof(double), cudaMemcpyDeviceToHost, st);
 }
@@ -1309,7 +1331,7 @@ static int fgmres_batch(Ctx& c, const double2* b, double2* x, int nr, double rto
         {
             Prof pr(c, BAH_K_SMALL, st, (double)nr * n * 32.0, 2);
             if (c.kdf) launch_scale_copy_df(c.R, true, c.nrm, 0, (float4*)c.V, n, n, ks.sv, nb, ks, st);
-            else launch_scale_copy(c.R, c.nrm, 0, c.V, n, n, ks.sv, nb, ks, st);
+            else launch_basis_store(c.R, c.nrm, 0, c.Vc, c.VL, c.VE, n, n, nb, ks, st);
             launch_init_arnoldi(c.nrm, c.g, m, c.status, nb, ks, st);
         }
         const int mm = std::min(m, c.o.maxit - total);
