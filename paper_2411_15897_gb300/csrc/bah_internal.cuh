@@ -196,8 +196,9 @@ struct SmArgs {
     const __nv_bfloat162* S[2][kMaxLevels];   // global stencils (levels below the coarsest)
     const float2* gb[2];      // level-l0 right-hand sides (right-hand side r at r * points)
     float2* gx[2];            // level-l0 iterates / results
-    const double2* inv[2];    // coarsest FP64 inverses (global memory; the product is formed in FP64)
-    unsigned off_g;           // gathered coarsest right-hand side
+    const int4* inv[2];       // coarsest inverses in block fixed point (global memory), exponent per row
+    const int* inve[2];
+    unsigned off_g, off_r;    // gathered coarsest right-hand side, reduction scratch
     const int* active;
 };
 // fills the shared-memory layout of a (n1, n2, slot counts per level from l0);
@@ -268,9 +269,12 @@ void launch_restrict(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::C
 template <int MODE>
 void launch_prolong_add(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fine,
                         const typename Prec<MODE>::V* const* coarse_x, cudaStream_t st, size_t coarse_stride = 0);
+int coarse_prepare();   // once per context, before the first launch
+// x = A_c^{-1} b, the inverse as limbs and row exponents (launch_inverse_limbs)
 template <int MODE>
-void launch_coarse_apply(int nb, int npts, const double2* const* inv, const typename Prec<MODE>::V* const* b,
-                         typename Prec<MODE>::V* const* x, cudaStream_t st, int nrhs = 1, RhsStride rs = RhsStride());
+void launch_coarse_apply(int nb, int npts, const int4* const* inv, const int* const* inve,
+                         const typename Prec<MODE>::V* const* b, typename Prec<MODE>::V* const* x, cudaStream_t st,
+                         int nrhs = 1, RhsStride rs = RhsStride());
 template <int MODE, class RIN = double2>
 void launch_distributor(int n1, int n2, double ihx, double ihz,
                         const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f5,
@@ -396,6 +400,8 @@ template <class V>
 void launch_prolong3(int type0, int nq, const int* nf, const V* const* ec, V* const* x, cudaStream_t st);
 void launch_galerkin3(int type, const int* nf, int nsf, const double2* Sf, double2* Sc, int* err, cudaStream_t st);
 int coarse_invert3(int type, const int* n, const double2* S, double2* inv, double2* work, int* flag, cudaStream_t st);
+// an n x n FP64 matrix in place to block fixed point (fix60.cuh), one exponent per row
+void launch_inverse_limbs(int n, double2* X, int* e, cudaStream_t st);
 // dense FP64 inverse X = A^{-1} of an n x n matrix by Gauss-Jordan elimination
 // (A is overwritten; X enters as the identity; f holds n scratch entries)
 int gauss_jordan(int n, double2* A, double2* X, double2* f, int* flag, cudaStream_t st);

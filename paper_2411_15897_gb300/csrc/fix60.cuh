@@ -52,8 +52,25 @@ __device__ __forceinline__ void limbs(long long v, int& h, int& l) {
     h = (int)((v + (1 << 29)) >> 30);
     l = (int)(v - ((long long)h << 30));
 }
+// the same for an FP32 number (24 bits: exact down to 2^-36 of the largest)
+__device__ __forceinline__ long long fix60(float x, int eb) {
+    const unsigned b = (unsigned)__float_as_int(x);
+    const int e = (int)((b >> 23) & 0xffu);
+    const unsigned long long m = (unsigned long long)((b << 8) | 0x80000000u) << 32;
+    const int sh = eb - (e - 127 + 1023) + 3;
+    const long long v = sh > 63 || e == 0 ? 0 : (long long)(((m >> sh) + 1) >> 1);
+    const long long sg = (long long)((int)b >> 31);
+    return (v ^ sg) - sg;
+}
+__device__ __forceinline__ int abs_hi(float x) { return __float_as_int(x) & 0x7fffffff; }
+// biased tile exponent from the largest abs_hi of FP64 (double) or FP32 (float) numbers
+template <class R> __device__ __forceinline__ int tile_exp_of(int max_hi) {
+    if (sizeof(R) == 8) return tile_exp(max_hi);
+    const int f = max_hi >> 23;
+    return f >= 0xff ? kExpBad : f - 127 + 1023 + 1;
+}
 // re.h, re.l, im.h, im.l
-__device__ __forceinline__ int4 limbs2(double2 z, int eb) {
+template <class V> __device__ __forceinline__ int4 limbs2(V z, int eb) {
     int4 r;
     limbs(fix60(z.x, eb), r.x, r.y);
     limbs(fix60(z.y, eb), r.z, r.w);
@@ -67,6 +84,14 @@ __device__ __forceinline__ void mad(long long& acc, int a, int b) {
 // 2^p (0 below the normal range, infinity above it)
 __device__ __forceinline__ double pow2(int p) {
     return p < -1022 ? 0.0 : __hiloint2double((p > 1023 ? 0x7ff : p + 1023) << 20, 0);
+}
+
+// A lane's exact sum hh 2^60 + cr 2^30 (|hh| <= 2^62, |cr| <= 2^63) as
+// hi 2^65 + lo 2^39, lo < 2^26: the sums of 32 lanes' parts fit 64 and 32 bits
+__device__ __forceinline__ void split65(long long hh, long long cr, long long& hi, unsigned& lo) {
+    const long long t = hh + (cr >> 30);
+    hi = t >> 5;
+    lo = ((unsigned)t & 31u) << 21 | (((unsigned)cr >> 9) & 0x1fffffu);
 }
 
 // Sum over the warp's lanes of NV values at once: each step adds half of the
@@ -86,6 +111,94 @@ __device__ __forceinline__ T warp_sum_values(T* v, int lane) {
     }
     for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     return v[0];
+}
+
+// ---------------------------------------------------------------------------
+// Dense product x = A g with A's rows in block fixed point (one exponent per
+// row) and g converted once per CTA: the coarsest solve with the FP64 inverse.
+// dense_head(np): bits that g gives up so that a lane's np / 32 products of
+// 2 x 2^58 fit 2^62 (none up to 256 points, 4 at 4096).
+// Bound: reading the inverse from L2.  With FP64 multiply-adds the solve was
+// bound by the FP64 pipe, on 16 SMs inside the cluster kernel: W(1,2) on
+// 400 x 128 (800 points, 4 or 8 solves per launch) 215 -> 89 us per launch,
+// 64 x 64 (256 points) 27.6 -> 21.5 us, 48 x 40 x 28 (840 points, three blocks,
+// all SMs) 32 -> 14 us per launch.
+// ---------------------------------------------------------------------------
+__host__ __device__ inline int dense_head(int np) {
+    int h = 0;
+    while ((256 << h) < np) ++h;
+    return h;
+}
+// one warp: sum over c < np of arow[c] g[c], valid in lane 0
+__device__ __forceinline__ double2 dense_row(const int4* __restrict__ arow, int ea, const int4* g, int eg, int np,
+                                             int lane) {
+    long long hr = 0, cr = 0, hi = 0, ci = 0;
+    auto mac = [&](const int4& a, const int4& b) {
+        // a b = (ax bx - ay by) + i (ax by + ay bx)
+        const int nz = -b.z, nw = -b.w;
+        mad(hr, a.x, b.x); mad(hr, a.z, nz);
+        mad(cr, a.x, b.y); mad(cr, a.y, b.x);
+        mad(cr, a.z, nw); mad(cr, a.w, nz);
+        mad(hi, a.x, b.z); mad(hi, a.z, b.x);
+        mad(ci, a.x, b.w); mad(ci, a.y, b.z);
+        mad(ci, a.z, b.y); mad(ci, a.w, b.x);
+    };
+    auto carry = [&]() {                       // the cross sums hold 8 products
+        hr += cr >> 30; cr &= 0x3fffffff;
+        hi += ci >> 30; ci &= 0x3fffffff;
+    };
+    constexpr int kU = 8;
+    int c = lane;
+    for (; c + 32 * (kU - 1) < np; c += 32 * kU) {
+        int4 a[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) a[u] = __ldg(arow + c + 32 * u);
+#pragma unroll
+        for (int u = 0; u < kU; ++u) mac(a[u], g[c + 32 * u]);
+        carry();
+    }
+    if (c < np) {
+        int4 a[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) a[u] = c + 32 * u < np ? __ldg(arow + c + 32 * u) : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (c + 32 * u < np) mac(a[u], g[c + 32 * u]);
+    }
+    long long v[2];
+    unsigned lo[2];
+    split65(hr, cr, v[0], lo[0]);
+    split65(hi, ci, v[1], lo[1]);
+    const long long sv = warp_sum_values<2>(v, lane);            // lanes 0-15 the real part, 16-31 the imaginary
+    const unsigned sl = warp_sum_values<2>(lo, lane);
+    const int p = (ea - 1023) + (eg - 1023) - 118;
+    double s = fma((double)sv, pow2(p + 65), (double)sl * pow2(p + 39));
+    if (ea == kExpBad || eg >= kExpBad) s = __longlong_as_double(0x7ff8000000000000ll);
+    return make_double2(s, __shfl_down_sync(0xffffffffu, s, 16));
+}
+// one CTA: g[0 .. np) = limbs of the entries get(c), their exponent returned
+// (blockDim.x a multiple of 32, at most 1024; red: 32 ints of shared memory;
+// ends with a barrier)
+template <class V, class R, class F>
+__device__ __forceinline__ int dense_load(int4* g, int np, int* red, F get) {
+    int mx = 0;
+    for (int c = threadIdx.x; c < np; c += blockDim.x) {
+        const V v = get(c);
+        *reinterpret_cast<V*>(g + c) = v;
+        mx = max(mx, max(abs_hi(v.x), abs_hi(v.y)));
+    }
+    mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    mx = (int)__reduce_max_sync(0xffffffffu, lane < nw ? (unsigned)red[lane] : 0u);
+    const int eg = tile_exp_of<R>(mx) + dense_head(np);
+    for (int c = threadIdx.x; c < np; c += blockDim.x) {
+        const V v = *reinterpret_cast<const V*>(g + c);
+        g[c] = limbs2(v, eg);
+    }
+    __syncthreads();
+    return eg;
 }
 
 }  // namespace bah

@@ -6,8 +6,9 @@
 // slabs, one per CTA; a CTA stores, for the points of its slab, the level's
 // Galerkin stencil (bfloat16 complex, slot-major), the iterate, a work
 // vector and the right-hand side.  The coarsest level is solved with the
-// dense FP64 inverse, read from global memory (it stays in L2) and applied in
-// FP64 arithmetic to the gathered FP32 right-hand side.  A stencil, restriction or prolongation tap
+// dense FP64 inverse, held in block fixed point (fix60.cuh), read from global
+// memory (it stays in L2) and applied to the gathered FP32 right-hand side with
+// exact integer sums.  A stencil, restriction or prolongation tap
 // that falls into another CTA's slab is read from that CTA's shared memory
 // through the cluster's distributed shared memory (mapa + ld.shared::cluster).
 //
@@ -26,6 +27,7 @@
 // whole cluster at once), and a final barrier keeps every CTA's shared
 // memory alive until no CTA of the cluster can still read it.
 #include "bah_internal.cuh"
+#include "fix60.cuh"
 #include "intergrid.cuh"
 
 #include <algorithm>
@@ -262,39 +264,19 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
             x[lt] = acc;
         }
     };
-    auto coarse = [&]() {                                   // x_c = A_c^{-1} b_c on own rows, in FP64
+    auto coarse = [&]() {                                   // x_c = A_c^{-1} b_c on own rows, exact integer sums
         const SmLevel& L = a.lv[kc];
         const int npc = L.n1 * L.n2, own = nown(L), g0 = p0(L);
-        V* gath = vec(a.off_g);
-        for (int g = tid; g < npc; g += nth) gath[g] = ld_cluster_at(row_addr(L, L.off_b, g / L.n1) + (uint32_t)(g % L.n1) * 8u);
-        __syncthreads();
+        int4* gath = reinterpret_cast<int4*>(sm + a.off_g);
+        const int eg = dense_load<V, float>(gath, npc, reinterpret_cast<int*>(sm + a.off_r), [&](int g) {
+            return ld_cluster_at(row_addr(L, L.off_b, g / L.n1) + (uint32_t)(g % L.n1) * 8u);
+        });
         V* x = vec(L.off_x);
         const int lane = tid & 31;
         for (int row = tid >> 5; row < own; row += nth >> 5) {
-            // the FP64 inverse row from global memory (L2-resident), eight loads in flight per lane
-            const double2* arow = a.inv[z] + (size_t)(g0 + row) * npc;
-            double re = 0.0, im = 0.0;
-            auto mac = [&](const double2& m, const V& v) {
-                const double vx = (double)v.x, vy = (double)v.y;
-                re = fma(m.x, vx, re);
-                re = fma(-m.y, vy, re);
-                im = fma(m.x, vy, im);
-                im = fma(m.y, vx, im);
-            };
-            int c = lane;
-            for (; c + 32 * 7 < npc; c += 32 * 8) {
-                double2 m[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) m[u] = __ldg(arow + c + 32 * u);
-#pragma unroll
-                for (int u = 0; u < 8; ++u) mac(m[u], gath[c + 32 * u]);
-            }
-            for (; c < npc; c += 32) mac(__ldg(arow + c), gath[c]);
-            for (int o = 16; o > 0; o >>= 1) {
-                re += __shfl_xor_sync(0xffffffffu, re, o);
-                im += __shfl_xor_sync(0xffffffffu, im, o);
-            }
-            if (lane == 0) x[row] = cmk<V>((float)re, (float)im);
+            // the inverse's row from global memory (L2-resident)
+            const double2 s = dense_row(a.inv[z] + (size_t)(g0 + row) * npc, a.inve[z][g0 + row], gath, eg, npc, lane);
+            if (lane == 0) x[row] = cconv<V>(s);
         }
     };
     auto zero_vec = [&](int k, unsigned off) {
@@ -478,7 +460,8 @@ size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max
     }
     const SmLevel& Lc = a.lv[nlev - 1];
     const size_t npc = (size_t)Lc.n1 * Lc.n2;
-    a.off_g = take(npc * 8);
+    a.off_g = take(npc * 16);
+    a.off_r = take(32 * 4);
     return off;
 }
 

@@ -39,14 +39,6 @@ __device__ __forceinline__ int load_tile(const double2* __restrict__ w, size_t e
     return tile_exp((int)__reduce_max_sync(0xffffffffu, (unsigned)mx));
 }
 
-// A lane's exact sum hh 2^60 + cr 2^30 (|hh| <= 2^62, |cr| <= 2^63) as
-// hi 2^65 + lo 2^39, lo < 2^26: the sums of 32 lanes' parts fit 64 and 32 bits
-__device__ __forceinline__ void split65(long long hh, long long cr, long long& hi, unsigned& lo) {
-    const long long t = hh + (cr >> 30);
-    hi = t >> 5;
-    lo = ((unsigned)t & 31u) << 21 | (((unsigned)cr >> 9) & 0x1fffffu);
-}
-
 // ---------------------------------------------------------------------------
 // Partial sums of rows 0 .. k of one CTA's tiles: row y < k is conj(V_y) w,
 // row k is |w|^2.  One warp per tile: w is converted to limbs once; for each

@@ -7,6 +7,7 @@
 // Level 0 reads the 5-point operator from per-point coefficient arrays
 // (Fine5); coarser levels read explicit Galerkin stencils of radius (rx, rz).
 #include "bah_internal.cuh"
+#include "fix60.cuh"
 #include "intergrid.cuh"
 #include "mg_device.cuh"
 
@@ -316,74 +317,61 @@ void launch_prolong_add(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>
 
 // ---------------------------------------------------------------------------
 // coarsest level: x = A_c^{-1} b with the stored FP64 inverse (one warp per
-// row).  The product is formed in FP64 in both modes -- the coarsest-grid
-// solve is one of the steps kept in FP64 -- from the right-hand side in the
-// cycle's precision; the result is rounded once to the cycle's precision.
-// Each lane issues its eight row loads before the first multiply-add.
+// row).  The inverse and the right-hand side are in block fixed point and the
+// products are exact integers (fix60.cuh): no less accurate than FP64 sums, at
+// the integer pipe's rate instead of 2 FP64 multiply-adds per clock and SM.
+// Each CTA converts the right-hand side once; the result is rounded once to
+// the cycle's precision.
 // ---------------------------------------------------------------------------
-constexpr int kCoarseSmem = 3072;   // points staged in shared memory
-
 template <class V>
-__global__ void __launch_bounds__(256) k_coarse_apply(int npts, PtrSet<const double2> inv, PtrSet<const V> b,
-                                                      PtrSet<V> x, const int* active) {
+__global__ void __launch_bounds__(256) k_coarse_apply(int npts, int rows, PtrSet<const int4> inv, PtrSet<const int> inve,
+                                                      PtrSet<const V> b, PtrSet<V> x, const int* active) {
     pdl_prologue();
     const int z = blockIdx.y;
     const int rr = blockIdx.z;
     if (active && !active[rr]) return;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    extern __shared__ __align__(16) unsigned char coarse_raw[];
-    V* bsh = reinterpret_cast<V*>(coarse_raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    extern __shared__ int4 g[];
+    __shared__ int red[32];
     const V* bb = pick(b, z) + rr * b.s;
-    const bool staged = npts <= kCoarseSmem;
-    if (staged) {
-        for (int c = threadIdx.x; c < npts; c += blockDim.x) bsh[c] = bb[c];
-        __syncthreads();
+    const int eg = dense_load<V, typename VecTraits<V>::R>(g, npts, red, [&](int c) { return bb[c]; });
+    const int r1 = min(npts, (int)(blockIdx.x + 1) * rows);
+    for (int row = blockIdx.x * rows + warp; row < r1; row += 8) {
+        const double2 s = dense_row(pick(inv, z) + (size_t)row * npts, pick(inve, z)[row], g, eg, npts, lane);
+        if (lane == 0) pick(x, z)[rr * x.s + row] = cconv<V>(s);
     }
-    if (warp >= npts) return;
-    const double2* row = pick(inv, z) + (size_t)warp * npts;
-    double re = 0.0, im = 0.0;
-    auto mac = [&](const double2& a, const V& v) {
-        const double vx = (double)v.x, vy = (double)v.y;
-        re = fma(a.x, vx, re);
-        re = fma(-a.y, vy, re);
-        im = fma(a.x, vy, im);
-        im = fma(a.y, vx, im);
-    };
-    constexpr int kU = 8;
-    int c = lane;
-    for (; c + 32 * (kU - 1) < npts; c += 32 * kU) {
-        double2 a[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) a[u] = __ldg(row + c + 32 * u);
-#pragma unroll
-        for (int u = 0; u < kU; ++u) mac(a[u], staged ? bsh[c + 32 * u] : bb[c + 32 * u]);
-    }
-    for (; c < npts; c += 32) mac(__ldg(row + c), staged ? bsh[c] : bb[c]);
-    for (int o = 16; o > 0; o >>= 1) {
-        re += __shfl_xor_sync(0xffffffffu, re, o);
-        im += __shfl_xor_sync(0xffffffffu, im, o);
-    }
-    if (lane == 0) pick(x, z)[rr * x.s + warp] = cmk<V>((typename VecTraits<V>::R)re, (typename VecTraits<V>::R)im);
+}
+int coarse_prepare() {
+    BAH_CUDA_TRY(cudaFuncSetAttribute((const void*)k_coarse_apply<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      4096 * (int)sizeof(int4)));
+    BAH_CUDA_TRY(cudaFuncSetAttribute((const void*)k_coarse_apply<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      4096 * (int)sizeof(int4)));
+    return BAH_OK;
 }
 
 template <int MODE>
-void launch_coarse_apply(int nb, int npts, const double2* const* inv, const typename Prec<MODE>::V* const* b,
-                         typename Prec<MODE>::V* const* x, cudaStream_t st, int nrhs, RhsStride rs) {
+void launch_coarse_apply(int nb, int npts, const int4* const* inv, const int* const* inve,
+                         const typename Prec<MODE>::V* const* b, typename Prec<MODE>::V* const* x, cudaStream_t st,
+                         int nrhs, RhsStride rs) {
     using V = typename Prec<MODE>::V;
-    PtrSet<const double2> pi;
+    PtrSet<const int4> pi;
+    PtrSet<const int> pe;
     PtrSet<const V> pb;
     PtrSet<V> px;
     for (int z = 0; z < 3; ++z) {
         pi.p[z] = z < nb ? inv[z] : nullptr;
+        pe.p[z] = z < nb ? inve[z] : nullptr;
         pb.p[z] = z < nb ? b[z] : nullptr;
         px.p[z] = z < nb ? x[z] : nullptr;
     }
     pb.s = rs.s0;
     px.s = rs.s1;
-    dim3 g((npts * 32 + 255) / 256, nb, nrhs);
-    const size_t smem = npts <= kCoarseSmem ? (size_t)npts * sizeof(V) : 0;
-    launch_pdl(k_coarse_apply<V>, dim3(g), dim3(256), smem, st, npts, pi, pb, px, rs.active);
+    // rows per CTA: eight (one per warp) while all CTAs are resident at once, more for a batch
+    int rows = 8;
+    while (rows < 64 && (npts + rows - 1) / rows * nb * nrhs > 1216) rows *= 2;
+    dim3 g((npts + rows - 1) / rows, nb, nrhs);
+    launch_pdl(k_coarse_apply<V>, dim3(g), dim3(256), (size_t)npts * sizeof(int4), st, npts, rows, pi, pe, pb, px,
+               rs.active);
 }
 
 // ---------------------------------------------------------------------------
@@ -418,8 +406,9 @@ void launch_block_apply64(const Fine5<double, double2>& f5, int type, const doub
                                         cudaStream_t, size_t);                                                     \
     template void launch_prolong_add<MODE>(const LvlSet<Prec<MODE>::V, Prec<MODE>::CC>&,                           \
                                            const Prec<MODE>::V* const*, cudaStream_t, size_t);                     \
-    template void launch_coarse_apply<MODE>(int, int, const double2* const*, const Prec<MODE>::V* const*,   \
-                                            Prec<MODE>::V* const*, cudaStream_t, int, RhsStride);
+    template void launch_coarse_apply<MODE>(int, int, const int4* const*, const int* const*,                       \
+                                            const Prec<MODE>::V* const*, Prec<MODE>::V* const*, cudaStream_t, int, \
+                                            RhsStride);
 INST(BAH_FP64)
 INST(BAH_MIXED)
 

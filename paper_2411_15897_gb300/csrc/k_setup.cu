@@ -3,6 +3,7 @@
 // stencils of Eq. 4.1, 4.2, 4.4, and the FP64 inverse of the coarsest level
 // (the direct coarse solve of Sec. 4.4.1).  All FP64; run once per context.
 #include "bah_internal.cuh"
+#include "fix60.cuh"
 #include "intergrid.cuh"
 
 #include <cmath>
@@ -366,6 +367,26 @@ int coarse_invert(int type, const StencilF64& S, double2* inv, double2* work, in
     k_dense_assemble<<<g, 128, 0, st>>>(type, S.S, S.rx, S.rz, S.n1, S.n2, A, inv);
     return gauss_jordan(n, A, inv, f, flag, st);
 }
+
+// one row per CTA; each thread converts the entries that it read itself
+__global__ void __launch_bounds__(256) k_inverse_limbs(int n, double2* X, int* e) {
+    double2* row = X + (size_t)blockIdx.x * n;
+    int mx = 0;
+    for (int c = threadIdx.x; c < n; c += 256) mx = max(mx, max(abs_hi(row[c].x), abs_hi(row[c].y)));
+    __shared__ int red[8];
+    mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    mx = red[0];
+    for (int q = 1; q < 8; ++q) mx = max(mx, red[q]);
+    const int eb = tile_exp(mx);
+    for (int c = threadIdx.x; c < n; c += 256) {
+        const int4 v = limbs2(row[c], eb);
+        *reinterpret_cast<int4*>(row + c) = v;
+    }
+    if (threadIdx.x == 0) e[blockIdx.x] = eb;
+}
+void launch_inverse_limbs(int n, double2* X, int* e, cudaStream_t st) { k_inverse_limbs<<<n, 256, 0, st>>>(n, X, e); }
 
 // CTAs per cluster for the Gauss-Jordan kernel: 16 where the device allows
 // non-portable clusters, else 8

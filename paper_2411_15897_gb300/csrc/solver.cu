@@ -61,7 +61,8 @@ struct Ctx {
     std::vector<int> ln1, ln2;
     std::vector<std::array<StencilF64, 3>> s64;   // FP64 stencils per level (level 0: 3x3 fine operator)
     std::vector<std::array<void*, 3>> sst;        // storage-precision stencils, levels >= 1
-    double2* inv[3] = {nullptr, nullptr, nullptr};
+    int4* inv[3] = {nullptr, nullptr, nullptr};   // coarsest inverses in block fixed point
+    int* inve[3] = {nullptr, nullptr, nullptr};
     std::vector<std::array<void*, 3>> vX, vB, vT; // multigrid vectors per level and block
     // Krylov workspace
     int m = 20;
@@ -146,7 +147,8 @@ struct Ctx {
     std::vector<std::array<double2*, 4>> s3;       // FP64 stencils (level 0: 7-point, coarser: 27-point)
     std::vector<std::array<void*, 4>> s3s;         // the same in storage precision, bf16 in mixed mode (levels below the coarsest)
     std::vector<std::array<void*, 4>> v3B, v3X, v3T;
-    double2* inv3[4] = {nullptr, nullptr, nullptr, nullptr};
+    int4* inv3[4] = {nullptr, nullptr, nullptr, nullptr};
+    int* inv3e[4] = {nullptr, nullptr, nullptr, nullptr};
 
     static void clear_graph(IterGraph& G) {
         if (G.exec) cudaGraphExecDestroy(G.exec);
@@ -361,6 +363,7 @@ struct MG {
                 a.gb[z] = (const float2*)c.vB[l0][b];
                 a.gx[z] = (float2*)c.vX[l0][b];
                 a.inv[z] = c.inv[b];
+                a.inve[z] = c.inve[b];
             }
             double bytes = 0;
             for (int k = 0; k < nlev - 1; ++k) bytes += coef_bytes(c, l0 + k, b0, nb) * bt.nr;
@@ -383,14 +386,15 @@ struct MG {
         const double vs = sizeof(V), ccs = sizeof(CC);
         const double nr = bt.nr;
         if (l == c.L - 1) {
-            const double2* inv[3];
+            const int4* inv[3];
+            const int* inve[3];
             const V* bb[3];
             V* xx[3];
-            for (int z = 0; z < nb; ++z) { inv[z] = c.inv[b0 + z]; bb[z] = (const V*)c.vB[l][b0 + z]; xx[z] = out[z]; }
+            for (int z = 0; z < nb; ++z) { inv[z] = c.inv[b0 + z]; inve[z] = c.inve[b0 + z]; bb[z] = (const V*)c.vB[l][b0 + z]; xx[z] = out[z]; }
             RhsStride rs;
             rs.s0 = npl; rs.s1 = ostride; rs.active = bt.active;
             Prof pr(c, BAH_K_COARSE, st, nb * (double)npl * npl * 16.0 + nr * nb * 2.0 * npl * vs);
-            launch_coarse_apply<MODE>(nb, (int)npl, inv, bb, xx, st, bt.nr, rs);
+            launch_coarse_apply<MODE>(nb, (int)npl, inv, inve, bb, xx, st, bt.nr, rs);
             return;
         }
         Fine5<C, CC> f5 = fine5(c);
@@ -541,13 +545,15 @@ struct MG3 {
         if (l == c.L - 1) {
             const double vb = sizeof(V);
             Prof pr(c, BAH_K_COARSE, st, nq * ((double)np * np * 16.0 + 2.0 * np * vb));
-            const double2* inv[3];
+            const int4* inv[3];
+            const int* inve[3];
             const V* bb[3];
             for (int y = 0; y < nq; ++y) {
                 inv[y] = c.inv3[q0 + y];
+                inve[y] = c.inv3e[q0 + y];
                 bb[y] = (const V*)c.v3B[l][q0 + y];
             }
-            launch_coarse_apply<MODE>(nq, (int)np, inv, bb, x, st);
+            launch_coarse_apply<MODE>(nq, (int)np, inv, inve, bb, x, st);
             return;
         }
         // the two buffers of each block's ping-pong; the current iterate is in A[y] when inA
@@ -957,6 +963,7 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     }
     BAH_CUDA_TRY(cudaGetLastError());
     // coarsest-level inverses
+    TRY(coarse_prepare());
     {
         NvtxRange nvi("coarsest inverses");
         const int nc = c.ln1[c.L - 1] * c.ln2[c.L - 1];
@@ -966,7 +973,9 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
         TRY(c.alloc_t(&flag, 1));
         for (int b = 0; b < 3; ++b) {
             TRY(c.alloc_t(&c.inv[b], (size_t)nc * nc));
-            TRY(coarse_invert(b, c.s64[c.L - 1][b], c.inv[b], (double2*)work, flag, st));
+            TRY(c.alloc_t(&c.inve[b], nc));
+            TRY(coarse_invert(b, c.s64[c.L - 1][b], (double2*)c.inv[b], (double2*)work, flag, st));
+            launch_inverse_limbs(nc, (double2*)c.inv[b], c.inve[b], st);
         }
     }
     // multigrid vectors
@@ -1127,13 +1136,16 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
         return BAH_ERR_CUDA;
     }
     // coarsest inverses
+    TRY(coarse_prepare());
     {
         const size_t nc = pts(c.L - 1);
         void* work;
         TRY(c.alloc(&work, (nc * nc + nc) * sizeof(double2)));
         for (int q = 0; q < 4; ++q) {
             TRY(c.alloc_t(&c.inv3[q], nc * nc));
-            TRY(coarse_invert3(q, c.d3[c.L - 1].data(), c.s3[c.L - 1][q], c.inv3[q], (double2*)work, err + 1, st));
+            TRY(c.alloc_t(&c.inv3e[q], nc));
+            TRY(coarse_invert3(q, c.d3[c.L - 1].data(), c.s3[c.L - 1][q], (double2*)c.inv3[q], (double2*)work, err + 1, st));
+            launch_inverse_limbs((int)nc, (double2*)c.inv3[q], c.inv3e[q], st);
         }
     }
     // multigrid vectors
