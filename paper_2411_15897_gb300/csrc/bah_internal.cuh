@@ -344,19 +344,20 @@ int launch_axpy_norm_df(const float4* V, int k, const double2* coef, float4* w, 
 void launch_scale_copy_df(const void* w, bool from64, const double* sc, int slot, float4* v, size_t n, size_t sw,
                           size_t sv, int nrhs, const KS& ks, cudaStream_t st);
 
-// block FGMRES kernels (k_block.cu); s <= 16 columns; rows of A (and Z) for
-// block i, column a at A + a * sa + i * n
-void launch_block_dot(const double2* A, size_t sa, int k, int s, const double2* W, size_t n, double2* partial,
-                      double2* C, cudaStream_t st);
-void launch_block_update(const double2* A, size_t sa, int k, int s, const double2* C, double2* W, size_t n,
-                         int subtract, cudaStream_t st);
-void launch_block_scale(const double2* W, int s, const double2* T, double2* V, size_t sv, size_t n, cudaStream_t st);
+// block FGMRES kernels (k_block.cu); s <= 16 columns; the basis in block fixed
+// point: block i, column a at VL + a * sv + i * tiles * 256 and VE + a * se + i * tiles
+int block_prepare();   // once per context, before the first launch
+void launch_block_dot(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
+                      double2* partial, double2* C, cudaStream_t st);
+void launch_block_gram(int s, const double2* W, size_t n, double2* partial, double2* C, cudaStream_t st);
+void launch_block_update(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* C, double2* W,
+                         size_t n, cudaStream_t st);
+void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStream_t st);
+void launch_block_scale(const double2* W, int s, const double2* T, double2* dst, int4* vl, int* ve, size_t sv, size_t se,
+                        size_t n, cudaStream_t st);
 template <class Vz>
 void launch_block_xupdate(const Vz* Z, size_t sz, int k, int s, const double2* Y, double2* X, size_t n,
                           cudaStream_t st);
-// allow the block update kernels the given dynamic shared memory
-void block_kernels_smem(size_t bytes);
-
 // adjoint gradient (k_grad.cu)
 void launch_conj(double2* v, size_t n, cudaStream_t st);
 void launch_misfit(const double2* x, const double2* d, const int* rec, int nrec, int nrhs, size_t vlen, double2* adj,

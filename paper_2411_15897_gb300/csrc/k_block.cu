@@ -1,175 +1,435 @@
 // Kernels of block FGMRES: one Krylov space for a block of s right-hand sides
 // (the batched form of the outer solve; FGMRES of Sec. 2.2 and Sec. 4 applied
-// to a block).  The block basis uses the batched layout of the lockstep
-// solver: column a of basis block i is V + a * sv + i * n (sv = the per-
-// right-hand-side basis stride), W and X hold column b at b * n.
+// to a block).  The basis is stored in block fixed point (fix60.cuh): column a
+// of basis block i has its limbs at VL + a * sv + i * tiles * 256 and its tile
+// exponents at VE + a * se + i * tiles; the newest block is also kept in FP64
+// (Vc, column b at b * n).  W and X hold column b at b * n.
 //
 //   block dot    C[(i, a), b] = sum_e conj(V_i[a][e]) W[b][e]      ((k s) x s, k blocks)
+//   block Gram   C[a, b] = sum_e conj(W[a][e]) W[b][e]
 //   block update W[b][e] -= sum_(i, a) V_i[a][e] C[(i, a), b]
-//   block scale  V[b][e] = sum_(b' <= b) W[b'][e] T[b', b]          (W R^{-1}, CholQR)
-//   solution     X[b][e] += sum_(i, a) Z_i[a][e] Y[(i, a), b]       (Z in the multigrid's precision)
+//   Cholesky     G = L L^H, R = L^H, T = R^{-1}                    (CholQR, one warp)
+//   block scale  V[b][e] = sum_(b' <= b) W[b'][e] T[b', b]         (W R^{-1})
+//   solution     X[b][e] += sum_(i, a) Z_i[a][e] Y[(i, a), b]      (Z in the multigrid's precision)
 //
-// FP64 arithmetic with explicit fused multiply-adds; the dot partial sums are
-// reduced in a fixed order.
+// The dots, the Gram matrix, the updates and the scaling sum exact integer
+// products; with FP64 multiply-adds (4 per entry, row and column, 2 per clock
+// and SM) they were bound by the FP64 pipe.
 #include "bah_internal.cuh"
+#include "fix60.cuh"
+
+#include <algorithm>
 
 namespace bah {
 
-constexpr int kBlockMaxS = 16;     // right-hand sides per block (columns)
+constexpr int kBlkRows = 32;       // rows of a dot CTA
 
-__device__ __forceinline__ void bmac_conj(double2& acc, const double2& a, const double2& b) {   // acc += conj(a) b
-    acc.x = fma(a.x, b.x, acc.x);
-    acc.x = fma(a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y);
-    acc.y = fma(-a.y, b.x, acc.y);
-}
 __device__ __forceinline__ void bmac(double2& acc, const double2& a, const double2& b) {        // acc += a b
     acc.x = fma(a.x, b.x, acc.x);
     acc.x = fma(-a.y, b.y, acc.x);
     acc.y = fma(a.x, b.y, acc.y);
     acc.y = fma(a.y, b.x, acc.y);
 }
-__device__ __forceinline__ void bmsub(double2& acc, const double2& a, const double2& b) {       // acc -= a b
-    acc.x = fma(-a.x, b.x, acc.x);
-    acc.x = fma(a.y, b.y, acc.x);
-    acc.y = fma(-a.x, b.y, acc.y);
-    acc.y = fma(-a.y, b.x, acc.y);
+
+// one warp: column b's entries of tile t as limbs in g[0 .. kTile); the exponent
+__device__ __forceinline__ int stage_tile(const double2* __restrict__ w, size_t t, size_t n, int4* g, int lane) {
+    const size_t e0 = t * kTile + lane;
+    double2 x[kTileU];
+    int mx = 0;
+#pragma unroll
+    for (int u = 0; u < kTileU; ++u) x[u] = e0 + 32 * u < n ? w[e0 + 32 * u] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int u = 0; u < kTileU; ++u) mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
+    const int eb = tile_exp((int)__reduce_max_sync(0xffffffffu, (unsigned)mx));
+#pragma unroll
+    for (int u = 0; u < kTileU; ++u) g[32 * u + lane] = limbs2(x[u], eb);
+    return eb;
 }
 
-// partial[row][b][cta] for row = i * s + a (i < k), one row per blockIdx.y;
-// rows of A are at A + a * sa + i * n
-template <int S>
-__global__ void __launch_bounds__(256) k_bdot_partial(const double2* __restrict__ A, size_t sa, int s,
-                                                      const double2* __restrict__ W, size_t n,
-                                                      double2* __restrict__ partial) {
+// ---------------------------------------------------------------------------
+// partial[(row * s + b) * gridDim.x + cta] for the CTA's 32 rows (blockIdx.y)
+// and tiles.  The s columns of W are converted to limbs in shared memory once
+// per tile and CTA; each warp takes every eighth row, holds its tile in
+// registers and meets all columns, so a basis row is read once for s columns.
+// SELF: the rows are the columns of W themselves (the l l products, which add
+// up where both factors are the same number, are kept).
+// ---------------------------------------------------------------------------
+template <int S, bool SELF>
+__global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, const int* __restrict__ VE, size_t sv,
+                                                 size_t se, int k, int s, const double2* __restrict__ W, size_t n,
+                                                 double2* __restrict__ partial) {
     pdl_prologue();
-    const int row = blockIdx.y;
-    const int i = row / s, a = row % s;
-    const double2* v = A + (size_t)a * sa + (size_t)i * n;
-    double2 acc[S];
-#pragma unroll
-    for (int b = 0; b < S; ++b) acc[b] = make_double2(0.0, 0.0);
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const double2 x = __ldg(v + e);
-#pragma unroll
-        for (int b = 0; b < S; ++b)
-            if (b < s) bmac_conj(acc[b], x, __ldg(W + (size_t)b * n + e));
-    }
-    __shared__ double2 sh[256 / 32][S];
+    extern __shared__ int4 g[];                                   // S x kTile
+    constexpr int CG = S < 8 ? S : 8, NV = 2 * CG;                // columns and values of one lane reduction
+    __shared__ int ew[S];
+    __shared__ double sum[kBlkRows][2 * S];
+    const size_t nt = tiles_of(n), npad = nt * kTile;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-#pragma unroll
-    for (int b = 0; b < S; ++b) {
-        double2 t = acc[b];
-        for (int o = 16; o > 0; o >>= 1) {
-            t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
-            t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+    const int nrow = SELF ? s : k * s, row0 = blockIdx.y * kBlkRows;
+    for (int q = threadIdx.x; q < kBlkRows * 2 * S; q += 256) (&sum[0][0])[q] = 0.0;
+    const int myval = lane / (32 / NV);
+    for (size_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        __syncthreads();
+        for (int b = wp; b < s; b += 8) {
+            const int e = stage_tile(W + (size_t)b * n, t, n, g + b * kTile, lane);
+            if (lane == 0) ew[b] = e;
         }
-        if (lane == 0) sh[wp][b] = t;
+        __syncthreads();
+        for (int rl = wp; rl < kBlkRows && row0 + rl < nrow; rl += 8) {
+            const int row = row0 + rl, i = row / s, a = row % s;
+            int4 v[kTileU];
+            int ev;
+            if (SELF) {
+                ev = ew[row];
+#pragma unroll
+                for (int u = 0; u < kTileU; ++u) v[u] = g[row * kTile + 32 * u + lane];
+            } else {
+                ev = VE[(size_t)a * se + (size_t)i * nt + t];
+                const int4* src = VL + (size_t)a * sv + (size_t)i * npad + t * kTile + lane;
+#pragma unroll
+                for (int u = 0; u < kTileU; ++u) v[u] = __ldg(src + 32 * u);
+            }
+#pragma unroll 1
+            for (int c0 = 0; c0 < s; c0 += CG) {
+                long long vh[NV];
+                unsigned vl[NV];
+#pragma unroll
+                for (int q = 0; q < NV; ++q) { vh[q] = 0; vl[q] = 0; }
+#pragma unroll
+                for (int c = 0; c < CG; ++c) {
+                    if (c0 + c >= s) break;
+                    const int4* col = g + (c0 + c) * kTile + lane;
+                    long long hr = 0, cr = 0, hi = 0, ci = 0, hn = 0, cn = 0, ll = 0, ln = 0;
+#pragma unroll
+                    for (int u = 0; u < kTileU; ++u) {
+                        const int4 w = col[32 * u];
+                        // conj(v) w = (vx wx + vy wy) + i (vx wy - vy wx)
+                        mad(hr, v[u].x, w.x); mad(hr, v[u].z, w.z);
+                        mad(cr, v[u].x, w.y); mad(cr, v[u].y, w.x);
+                        mad(cr, v[u].z, w.w); mad(cr, v[u].w, w.z);
+                        mad(hi, v[u].x, w.z); mad(hn, v[u].z, w.x);
+                        mad(ci, v[u].x, w.w); mad(ci, v[u].y, w.z);
+                        mad(cn, v[u].z, w.y); mad(cn, v[u].w, w.x);
+                        if (SELF) {
+                            mad(ll, v[u].y, w.y); mad(ll, v[u].w, w.w);
+                            mad(ln, v[u].y, w.w); mad(ln, -v[u].w, w.y);
+                        }
+                    }
+                    split65(hr + (cr >> 30), (cr & 0x3fffffff) + (ll >> 30), vh[2 * c], vl[2 * c]);
+                    split65(hi - hn + (ci >> 30) - (cn >> 30), (ci & 0x3fffffff) - (cn & 0x3fffffff) + (ln >> 30),
+                            vh[2 * c + 1], vl[2 * c + 1]);
+                }
+                const long long th = warp_sum_values<NV>(vh, lane);
+                const unsigned tl = warp_sum_values<NV>(vl, lane);
+                const int b = c0 + (myval >> 1);
+                if (lane % (32 / NV) == 0 && b < s) {
+                    const int p = (ev - 1023) + (ew[b] - 1023) - 118;
+                    double x = fma((double)th, pow2(p + 65), (double)tl * pow2(p + 39));
+                    if (ev == kExpBad || ew[b] == kExpBad) x = __longlong_as_double(0x7ff8000000000000ll);
+                    sum[rl][2 * b + (myval & 1)] += x;
+                }
+            }
+        }
     }
     __syncthreads();
-    if (threadIdx.x < s) {
-        double2 t = make_double2(0.0, 0.0);
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            t.x += sh[w][threadIdx.x].x;
-            t.y += sh[w][threadIdx.x].y;
-        }
-        partial[((size_t)row * s + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+    for (int q = threadIdx.x; q < kBlkRows * s; q += 256) {
+        const int rl = q / s, b = q % s;
+        if (row0 + rl < nrow)
+            partial[((size_t)(row0 + rl) * s + b) * gridDim.x + blockIdx.x] = make_double2(sum[rl][2 * b], sum[rl][2 * b + 1]);
     }
 }
-// C[row * s + b] = sum over the CTAs' partials (fixed order)
-__global__ void __launch_bounds__(256) k_bdot_reduce(const double2* __restrict__ partial, int np, double2* C) {
+// C[row * s + b] = sum over the CTAs' partials (fixed order), one warp each
+__global__ void __launch_bounds__(128) k_bdot_reduce(const double2* __restrict__ partial, int np, int count, double2* C) {
     pdl_prologue();
-    const int q = blockIdx.x;                       // row * s + b
+    const int q = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;      // row * s + b
+    if (q >= count) return;
     double2 t = make_double2(0.0, 0.0);
-    for (int e = threadIdx.x; e < np; e += blockDim.x) {
+    for (int e = lane; e < np; e += 32) {
         const double2 v = partial[(size_t)q * np + e];
         t.x += v.x;
         t.y += v.y;
     }
-    __shared__ double2 sh[256];
-    sh[threadIdx.x] = t;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) { sh[threadIdx.x].x += sh[threadIdx.x + o].x; sh[threadIdx.x].y += sh[threadIdx.x + o].y; }
-        __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+        t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+        t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
     }
-    if (threadIdx.x == 0) C[q] = sh[0];
+    if (lane == 0) C[q] = t;
 }
-template <int S>
-static void bdot_t(const double2* A, size_t sa, int k, int s, const double2* W, size_t n, double2* partial, double2* C,
-                   cudaStream_t st) {
-    launch_pdl(k_bdot_partial<S>, dim3(RED_CTAS, k * s), dim3(256), 0, st, A, sa, s, W, n, partial);
-    launch_pdl(k_bdot_reduce, dim3(k * s * s), dim3(256), 0, st, (const double2*)partial, RED_CTAS, C);
+template <int S, bool SELF>
+static void bdot_t(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
+                   double2* partial, double2* C, cudaStream_t st) {
+    const int rows = SELF ? s : k * s, chunks = (rows + kBlkRows - 1) / kBlkRows;
+    // two CTAs per SM in all, whole rounds of tiles
+    const size_t nt = tiles_of(n), most = std::max(1, RED_CTAS / chunks), per = (nt + most - 1) / most;
+    const int nc = (int)((nt + per - 1) / per);
+    launch_pdl(k_bdot<S, SELF>, dim3(nc, chunks), dim3(256), (size_t)s * kTile * sizeof(int4), st, VL, VE, sv, se, k, s, W,
+               n, partial);
+    launch_pdl(k_bdot_reduce, dim3((rows * s + 3) / 4), dim3(128), 0, st, (const double2*)partial, nc, rows * s, C);
 }
-void launch_block_dot(const double2* A, size_t sa, int k, int s, const double2* W, size_t n, double2* partial,
-                      double2* C, cudaStream_t st) {
-    if (s <= 4) bdot_t<4>(A, sa, k, s, W, n, partial, C, st);
-    else if (s <= 8) bdot_t<8>(A, sa, k, s, W, n, partial, C, st);
-    else bdot_t<16>(A, sa, k, s, W, n, partial, C, st);
+void launch_block_dot(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
+                      double2* partial, double2* C, cudaStream_t st) {
+    if (s <= 4) bdot_t<4, false>(VL, VE, sv, se, k, s, W, n, partial, C, st);
+    else if (s <= 8) bdot_t<8, false>(VL, VE, sv, se, k, s, W, n, partial, C, st);
+    else bdot_t<16, false>(VL, VE, sv, se, k, s, W, n, partial, C, st);
+}
+void launch_block_gram(int s, const double2* W, size_t n, double2* partial, double2* C, cudaStream_t st) {
+    if (s <= 4) bdot_t<4, true>(nullptr, nullptr, 0, 0, 1, s, W, n, partial, C, st);
+    else if (s <= 8) bdot_t<8, true>(nullptr, nullptr, 0, 0, 1, s, W, n, partial, C, st);
+    else bdot_t<16, true>(nullptr, nullptr, 0, 0, 1, s, W, n, partial, C, st);
 }
 
-// W[b][e] -= sum over rows (i, a) < k s of V_i[a][e] C[row, b]; coefficients in shared memory
+// ---------------------------------------------------------------------------
+// Sums of one column over rows: a warp's accumulators for the eight entries per
+// lane of a tile, sum_row V_row[e] c[row], every row's products sharing the
+// exponent eo (biased twice); the coefficients keep 60 - head bits so that the
+// rows' products fit 62 bits.
+// ---------------------------------------------------------------------------
+__host__ __device__ inline int rows_head(int rows) {
+    int h = 2;
+    while ((8 << h) < rows) ++h;
+    return h;
+}
+struct ColSum {
+    long long hr[kTileU], cr[kTileU], hi[kTileU], ci[kTileU];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int u = 0; u < kTileU; ++u) hr[u] = cr[u] = hi[u] = ci[u] = 0;
+    }
+    __device__ __forceinline__ void add(const int4* row, const int4& c) {      // row: this lane's entries at 32 u
+        const int nz = -c.z, nw = -c.w;
+#pragma unroll
+        for (int u = 0; u < kTileU; ++u) {
+            const int4 b = row[32 * u];
+            mad(hr[u], c.x, b.x); mad(hr[u], nz, b.z);
+            mad(cr[u], c.x, b.y); mad(cr[u], c.y, b.x);
+            mad(cr[u], nz, b.w); mad(cr[u], nw, b.z);
+            mad(hi[u], c.x, b.z); mad(hi[u], c.z, b.x);
+            mad(ci[u], c.x, b.w); mad(ci[u], c.y, b.z);
+            mad(ci[u], c.z, b.y); mad(ci[u], c.w, b.x);
+        }
+    }
+    __device__ __forceinline__ void carry() {                                  // at least every 4 rows
+#pragma unroll
+        for (int u = 0; u < kTileU; ++u) {
+            hr[u] += cr[u] >> 30; cr[u] &= 0x3fffffff;
+            hi[u] += ci[u] >> 30; ci[u] &= 0x3fffffff;
+        }
+    }
+    // x - sum, with s1 = 2^60 and s2 = 2^30 times the scale of the integers
+    __device__ __forceinline__ double2 minus(const double2& x, int u, double s1, double s2) const {
+        return make_double2(fma(-(double)hr[u], s1, fma(-(double)cr[u], s2, x.x)),
+                            fma(-(double)hi[u], s1, fma(-(double)ci[u], s2, x.y)));
+    }
+};
+__device__ __forceinline__ int coef_exp(const double2& c) { return max(abs_hi(c.x), abs_hi(c.y)) >> 20; }
+
+// W[b][e] -= sum over rows (i, a) < k s of V_i[a][e] C[row, b].  One CTA of S
+// warps per tile, warp b on column b; the basis rows pass through a ring of
+// shared-memory slots (cp.async, groups of four rows, one barrier per group),
+// so a row is read once for all columns.
+constexpr int kUpG = 4, kUpSlots = 3;
 template <int S>
-__global__ void __launch_bounds__(256) k_bupdate(const double2* __restrict__ A, size_t sa, int k, int s,
-                                                 const double2* __restrict__ C, double2* __restrict__ W, size_t n,
-                                                 int subtract) {
+__global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL, const int* __restrict__ VE, size_t sv,
+                                                    size_t se, int k, int s, const double2* __restrict__ C,
+                                                    double2* __restrict__ W, size_t n) {
     pdl_prologue();
-    extern __shared__ double2 cs[];                  // (k s) x s
-    for (int q = threadIdx.x; q < k * s * s; q += blockDim.x) cs[q] = C[q];
-    __syncthreads();
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        double2 acc[S];
-#pragma unroll
-        for (int b = 0; b < S; ++b) acc[b] = b < s ? W[(size_t)b * n + e] : make_double2(0.0, 0.0);
-        for (int row = 0; row < k * s; ++row) {
-            const int i = row / s, a = row % s;
-            const double2 v = __ldg(A + (size_t)a * sa + (size_t)i * n + e);
-#pragma unroll
-            for (int b = 0; b < S; ++b)
-                if (b < s) {
-                    if (subtract) bmsub(acc[b], v, cs[row * s + b]);
-                    else bmac(acc[b], v, cs[row * s + b]);
+    extern __shared__ int4 ring[];                                // kUpSlots x kUpG x kTile
+    __shared__ int4 csh[S][32];
+    const size_t nt = tiles_of(n), npad = nt * kTile;
+    const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
+    const int rows = k * s, head = rows_head(rows), ngrp = (rows + kUpG - 1) / kUpG;
+    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+    for (size_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        auto fetch = [&](int gq) {                                // group gq's rows into its slot
+            if (gq < ngrp)
+                for (int e = threadIdx.x; e < kUpG * kTile; e += 32 * S) {
+                    const int row = gq * kUpG + e / kTile;
+                    if (row < rows) {
+                        const int4* src = VL + (size_t)(row % s) * sv + (size_t)(row / s) * npad + t * kTile + e % kTile;
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                         ring_s + (uint32_t)((gq % kUpSlots) * kUpG * kTile + e) * 16u),
+                                     "l"(src)
+                                     : "memory");
+                    }
                 }
-        }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        __syncthreads();                                          // the last tile's slots are free
 #pragma unroll
-        for (int b = 0; b < S; ++b)
-            if (b < s) W[(size_t)b * n + e] = acc[b];
+        for (int q = 0; q < kUpSlots - 1; ++q) fetch(q);
+        // the common exponent of the column
+        int eo = 0;
+        bool bad = false;
+        if (b < s)
+            for (int row = lane; row < rows; row += 32) {
+                const int ec = coef_exp(C[(size_t)row * s + b]);
+                const int ev = VE[(size_t)(row % s) * se + (size_t)(row / s) * nt + t];
+                if (ec > 0) eo = max(eo, ev + ec + 1 + head);
+                bad |= ec == 0x7ff || ev == kExpBad;
+            }
+        eo = (int)__reduce_max_sync(0xffffffffu, (unsigned)eo);
+        bad = __any_sync(0xffffffffu, bad);
+        ColSum acc;
+        acc.clear();
+        for (int gq = 0; gq < ngrp; ++gq) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kUpSlots - 2) : "memory");
+            __syncthreads();                                      // group gq arrived; every warp is done with gq - 1
+            fetch(gq + kUpSlots - 1);
+            if (b >= s) continue;
+            if ((gq * kUpG) % 32 == 0) {                          // limbs of the next 32 coefficients
+                __syncwarp();
+                const int row = gq * kUpG + lane;
+                if (row < rows) {
+                    const double2 c = C[(size_t)row * s + b];
+                    const int eb = eo - VE[(size_t)(row % s) * se + (size_t)(row / s) * nt + t];
+                    csh[b][lane] = coef_exp(c) > 0 && eb >= kExpMin ? limbs2(c, eb) : make_int4(0, 0, 0, 0);
+                }
+                __syncwarp();
+            }
+            const int4* slot = ring + (gq % kUpSlots) * kUpG * kTile + lane;
+            for (int q = 0; q < kUpG && gq * kUpG + q < rows; ++q) acc.add(slot + q * kTile, csh[b][(gq * kUpG + q) & 31]);
+            acc.carry();
+        }
+        if (b < s) {
+            // integers scaled by 2^(59 - Ev) 2^(59 - Ec)
+            const int p = (eo - 2 * 1023) - 118;
+            double s1 = pow2(p + 60), s2 = pow2(p + 30);
+            if (bad) s1 = __longlong_as_double(0x7ff8000000000000ll);
+            double2* w = W + (size_t)b * n;
+            const size_t e0 = t * kTile + lane;
+#pragma unroll
+            for (int u = 0; u < kTileU; ++u)
+                if (e0 + 32 * u < n) w[e0 + 32 * u] = acc.minus(w[e0 + 32 * u], u, s1, s2);
+        }
     }
 }
-void launch_block_update(const double2* A, size_t sa, int k, int s, const double2* C, double2* W, size_t n,
-                         int subtract, cudaStream_t st) {
-    const size_t smem = (size_t)k * s * s * sizeof(double2);
-    if (s <= 4) launch_pdl(k_bupdate<4>, dim3(RED_CTAS * 2), dim3(256), smem, st, A, sa, k, s, C, W, n, subtract);
-    else if (s <= 8) launch_pdl(k_bupdate<8>, dim3(RED_CTAS * 2), dim3(256), smem, st, A, sa, k, s, C, W, n, subtract);
-    else launch_pdl(k_bupdate<16>, dim3(RED_CTAS * 2), dim3(256), smem, st, A, sa, k, s, C, W, n, subtract);
+void launch_block_update(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* C, double2* W,
+                         size_t n, cudaStream_t st) {
+    const size_t smem = (size_t)kUpSlots * kUpG * kTile * sizeof(int4);
+    const unsigned nt = (unsigned)tiles_of(n);
+    if (s <= 4) launch_pdl(k_bupdate<4>, dim3(std::min(nt, 608u)), dim3(128), smem, st, VL, VE, sv, se, k, s, C, W, n);
+    else if (s <= 8) launch_pdl(k_bupdate<8>, dim3(std::min(nt, 304u)), dim3(256), smem, st, VL, VE, sv, se, k, s, C, W, n);
+    else launch_pdl(k_bupdate<16>, dim3(std::min(nt, 152u)), dim3(512), smem, st, VL, VE, sv, se, k, s, C, W, n);
 }
 
-// V[b] (at V + b * sv) = sum_(b' <= b) W[b'] T[b', b] (T upper triangular, s x s, row-major)
-template <int S>
-__global__ void __launch_bounds__(256) k_bscale(const double2* W, int s, const double2* __restrict__ T, double2* V,
-                                                size_t sv, size_t n) {
+// ---------------------------------------------------------------------------
+// Cholesky factor of the s x s Hermitian G (row-major) and the inverse of
+// R = L^H, one warp.  A pivot that is not positive and finite makes R and T NaN
+// (the host reads R).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(32) k_bchol(const double2* __restrict__ G, int s, double2* R, double2* T) {
     pdl_prologue();
-    __shared__ double2 ts[S * S];
-    for (int q = threadIdx.x; q < s * s; q += blockDim.x) ts[q] = T[q];
-    __syncthreads();
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        double2 w[S];
+    __shared__ double2 A[16][17], X[16][17];
+    const int lane = threadIdx.x;
+    for (int q = lane; q < s * s; q += 32) {
+        A[q / s][q % s] = G[q];
+        X[q / s][q % s] = make_double2(0.0, 0.0);
+    }
+    __syncwarp();
+    for (int j = 0; j < s; ++j) {
+        const double d = A[j][j].x;
+        const double l = d > 0.0 && isfinite(d) ? sqrt(d) : __longlong_as_double(0x7ff8000000000000ll);
+        const double il = 1.0 / l;
+        __syncwarp();
+        if (lane == j) A[j][j] = make_double2(l, 0.0);
+        else if (lane > j && lane < s) A[lane][j] = cscale(A[lane][j], il);
+        __syncwarp();
+        // trailing lower triangle: A[i][k] -= L[i][j] conj(L[k][j])
+        const int m = s - j - 1;
+        for (int q = lane; q < m * m; q += 32) {
+            const int i = j + 1 + q / m, k = j + 1 + q % m;
+            if (k <= i) bmac(A[i][k], cscale(A[i][j], -1.0), cconj(A[k][j]));
+        }
+        __syncwarp();
+    }
+    // X = R^{-1} column by column (lane = column), R[q][k] = conj(L[k][q])
+    if (lane < s)
+        for (int q = lane; q >= 0; --q) {
+            double2 acc = make_double2(q == lane ? 1.0 : 0.0, 0.0);
+            for (int k = q + 1; k <= lane; ++k) bmac(acc, cscale(cconj(A[k][q]), -1.0), X[k][lane]);
+            X[q][lane] = cscale(acc, 1.0 / A[q][q].x);
+        }
+    __syncwarp();
+    for (int q = lane; q < s * s; q += 32) {
+        const int i = q / s, j = q % s;
+        R[q] = j >= i ? cconj(A[j][i]) : make_double2(0.0, 0.0);
+        T[q] = j >= i ? X[i][j] : make_double2(0.0, 0.0);
+    }
+}
+void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStream_t st) {
+    launch_pdl(k_bchol, dim3(1), dim3(32), 0, st, G, s, R, T);
+}
+
+// V[b] = sum_(b' <= b) W[b'] T[b', b] (T upper triangular, s x s, row-major),
+// written to dst (column b at b * n; may be W itself) and, with vl, as basis
+// columns.  One CTA of S warps per tile: warp b converts column b to limbs in
+// shared memory, then sums column b of the product.
+template <int S>
+__global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, const double2* __restrict__ T, double2* dst,
+                                                   int4* __restrict__ vl, int* __restrict__ ve, size_t sv, size_t se,
+                                                   size_t n) {
+    pdl_prologue();
+    extern __shared__ int4 g[];                                   // S x kTile
+    __shared__ int ew[S];
+    __shared__ int4 csh[S][16];
+    const size_t nt = tiles_of(n);
+    const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
+    const double2 c = lane <= b && b < s ? T[lane * s + b] : make_double2(0.0, 0.0);
+    const int ec = coef_exp(c), head = 2;
+    for (size_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        __syncthreads();
+        if (b < s) {
+            const int e = stage_tile(W + (size_t)b * n, t, n, g + b * kTile, lane);
+            if (lane == 0) ew[b] = e;
+        }
+        __syncthreads();                                          // all of the tile is in shared memory: dst may be W
+        if (b >= s) continue;
+        const int ev = lane <= b ? ew[lane] : kExpMin;
+        const int eo = (int)__reduce_max_sync(0xffffffffu, ec > 0 ? (unsigned)(ev + ec + 1 + head) : 0u);
+        const bool bad = __any_sync(0xffffffffu, ec == 0x7ff || ev == kExpBad);
+        __syncwarp();
+        if (lane <= b) {
+            const int eb = eo - ev;
+            csh[b][lane] = ec > 0 && eb >= kExpMin ? limbs2(c, eb) : make_int4(0, 0, 0, 0);
+        }
+        __syncwarp();
+        ColSum acc;
+        acc.clear();
+        for (int q = 0; q <= b; ++q) {
+            acc.add(g + q * kTile + lane, csh[b][q]);
+            if ((q & 3) == 3) acc.carry();
+        }
+        const int p = (eo - 2 * 1023) - 118;
+        double s1 = -pow2(p + 60);
+        const double s2 = -pow2(p + 30);
+        if (bad) s1 = __longlong_as_double(0x7ff8000000000000ll);
+        const size_t e0 = t * kTile + lane;
+        double2 x[kTileU];
+        int mx = 0;
 #pragma unroll
-        for (int b = 0; b < S; ++b) w[b] = b < s ? W[(size_t)b * n + e] : make_double2(0.0, 0.0);
+        for (int u = 0; u < kTileU; ++u) {
+            x[u] = make_double2(0.0, 0.0);
+            if (e0 + 32 * u < n) {
+                x[u] = acc.minus(x[u], u, s1, s2);
+                dst[(size_t)b * n + e0 + 32 * u] = x[u];
+            }
+            mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
+        }
+        if (vl) {
+            const int eb = tile_exp((int)__reduce_max_sync(0xffffffffu, (unsigned)mx));
+            if (lane == 0) ve[(size_t)b * se + t] = eb;
 #pragma unroll
-        for (int b = 0; b < S; ++b) {
-            if (b >= s) break;
-            double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-            for (int q = 0; q <= b; ++q) bmac(acc, w[q], ts[q * s + b]);
-            V[(size_t)b * sv + e] = acc;
+            for (int u = 0; u < kTileU; ++u) vl[(size_t)b * sv + e0 + 32 * u] = limbs2(x[u], eb);
         }
     }
 }
-void launch_block_scale(const double2* W, int s, const double2* T, double2* V, size_t sv, size_t n, cudaStream_t st) {
-    if (s <= 4) launch_pdl(k_bscale<4>, dim3(RED_CTAS * 2), dim3(256), 0, st, W, s, T, V, sv, n);
-    else if (s <= 8) launch_pdl(k_bscale<8>, dim3(RED_CTAS * 2), dim3(256), 0, st, W, s, T, V, sv, n);
-    else launch_pdl(k_bscale<16>, dim3(RED_CTAS * 2), dim3(256), 0, st, W, s, T, V, sv, n);
+void launch_block_scale(const double2* W, int s, const double2* T, double2* dst, int4* vl, int* ve, size_t sv, size_t se,
+                        size_t n, cudaStream_t st) {
+    const size_t smem = (size_t)s * kTile * sizeof(int4);
+    const unsigned nt = (unsigned)tiles_of(n);
+    if (s <= 4) launch_pdl(k_bscale<4>, dim3(std::min(nt, 608u)), dim3(128), smem, st, W, s, T, dst, vl, ve, sv, se, n);
+    else if (s <= 8) launch_pdl(k_bscale<8>, dim3(std::min(nt, 304u)), dim3(256), smem, st, W, s, T, dst, vl, ve, sv, se, n);
+    else launch_pdl(k_bscale<16>, dim3(std::min(nt, 152u)), dim3(512), smem, st, W, s, T, dst, vl, ve, sv, se, n);
 }
 
 // X[b][e] += sum over rows (i, a) < k s of Z_i[a][e] Y[row, b]  (Z FP32 or FP64 complex)
@@ -200,19 +460,25 @@ __global__ void __launch_bounds__(256) k_bxupdate(const Vz* __restrict__ Z, size
 template <class Vz>
 void launch_block_xupdate(const Vz* Z, size_t sz, int k, int s, const double2* Y, double2* X, size_t n,
                           cudaStream_t st) {
-    const size_t smem = (size_t)k * s * s * sizeof(double2);
-    if (s <= 4) launch_pdl(k_bxupdate<4, Vz>, dim3(RED_CTAS * 2), dim3(256), smem, st, Z, sz, k, s, Y, X, n);
-    else if (s <= 8) launch_pdl(k_bxupdate<8, Vz>, dim3(RED_CTAS * 2), dim3(256), smem, st, Z, sz, k, s, Y, X, n);
-    else launch_pdl(k_bxupdate<16, Vz>, dim3(RED_CTAS * 2), dim3(256), smem, st, Z, sz, k, s, Y, X, n);
+    const int most = std::max(1, 49152 / (s * s * (int)sizeof(double2)));      // blocks whose coefficients fit 48 KiB
+    for (int i = 0; i < k; i += most) {
+        const int kk = std::min(most, k - i);
+        const size_t smem = (size_t)kk * s * s * sizeof(double2);
+        const Vz* z = Z + (size_t)i * n;
+        const double2* y = Y + (size_t)i * s * s;
+        const dim3 g(RED_CTAS * 2), b(256);
+        if (s <= 4) launch_pdl(k_bxupdate<4, Vz>, g, b, smem, st, z, sz, kk, s, y, X, n);
+        else if (s <= 8) launch_pdl(k_bxupdate<8, Vz>, g, b, smem, st, z, sz, kk, s, y, X, n);
+        else launch_pdl(k_bxupdate<16, Vz>, g, b, smem, st, z, sz, kk, s, y, X, n);
+    }
 }
-void block_kernels_smem(size_t bytes) {
-    if (bytes <= 48 * 1024) return;
-    const void* fns[] = {(const void*)k_bupdate<4>, (const void*)k_bupdate<8>, (const void*)k_bupdate<16>,
-                         (const void*)k_bxupdate<4, float2>, (const void*)k_bxupdate<8, float2>,
-                         (const void*)k_bxupdate<16, float2>, (const void*)k_bxupdate<4, double2>,
-                         (const void*)k_bxupdate<8, double2>, (const void*)k_bxupdate<16, double2>};
-    for (const void* f : fns) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    cudaGetLastError();
+int block_prepare() {
+    const int ring = (int)(kUpSlots * kUpG * kTile * sizeof(int4)), cols = (int)(16 * kTile * sizeof(int4));
+    const struct { const void* f; int b; } fns[] = {
+        {(const void*)k_bdot<16, false>, cols}, {(const void*)k_bdot<16, true>, cols}, {(const void*)k_bscale<16>, cols},
+        {(const void*)k_bupdate<4>, ring},      {(const void*)k_bupdate<8>, ring},     {(const void*)k_bupdate<16>, ring}};
+    for (const auto& q : fns) BAH_CUDA_TRY(cudaFuncSetAttribute(q.f, cudaFuncAttributeMaxDynamicSharedMemorySize, q.b));
+    return BAH_OK;
 }
 template void launch_block_xupdate<float2>(const float2*, size_t, int, int, const double2*, double2*, size_t,
                                            cudaStream_t);

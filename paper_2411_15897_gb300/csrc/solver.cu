@@ -136,8 +136,9 @@ struct Ctx {
     int exact_status = BAH_OK;          // first failure of a block solve inside a preconditioner call
 
     // block FGMRES workspace (block_krylov = 1)
-    double2 *bC = nullptr, *bT = nullptr, *bpart = nullptr;
-    double2* bhost = nullptr;           // pinned
+    double2 *bC = nullptr, *bG = nullptr, *bT = nullptr, *bpart = nullptr;
+    double2* bhost = nullptr;           // pinned, two slots of bslot entries
+    size_t bslot = 0;
 
     // three-dimensional grids (dim == 3): n1 x n2 x n3 cells
     int n3 = 1;
@@ -816,7 +817,7 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     const size_t nbt = c.nbatch;
     const size_t so = m + 2;
     const size_t nt = tiles_of(n);
-    if (c.kdf || c.o.block_krylov) {
+    if (c.kdf) {
         TRY(c.alloc_t(&c.V, n * (m + 1) * nbt));
     } else {
         TRY(gs_prepare());
@@ -1030,11 +1031,13 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     }
     TRY(alloc_krylov(c, st));
     if (c.o.block_krylov) {
-        const size_t sq = (size_t)(c.m + 1) * c.nbatch * c.nbatch;
-        TRY(c.alloc_t(&c.bC, sq)); TRY(c.alloc_t(&c.bT, (size_t)c.nbatch * c.nbatch));
-        TRY(c.alloc_t(&c.bpart, sq * RED_CTAS));
-        BAH_CUDA_TRY(cudaMallocHost((void**)&c.bhost, sq * sizeof(double2)));
-        block_kernels_smem((size_t)(c.m + 1) * c.nbatch * c.nbatch * sizeof(double2));
+        // a step's R_1, R_2 (CholQR2) and the two passes' coefficients, copied to the host together
+        const size_t s2 = (size_t)c.nbatch * c.nbatch;
+        c.bslot = 2 * s2 + 2 * (size_t)c.m * s2;
+        TRY(block_prepare());
+        TRY(c.alloc_t(&c.bC, c.bslot)); TRY(c.alloc_t(&c.bG, s2)); TRY(c.alloc_t(&c.bT, s2));
+        TRY(c.alloc_t(&c.bpart, (size_t)(c.m + 1) * s2 * RED_CTAS));
+        BAH_CUDA_TRY(cudaMallocHost((void**)&c.bhost, 2 * c.bslot * sizeof(double2)));
     }
     if (c.exact) {
         // the blocks solved exactly: the fine operators of Eq. 2.6 / 3.4 with their
@@ -1429,88 +1432,41 @@ static int fgmres_batch(Ctx& c, const double2* b, double2* x, int nr, double rto
 // right-hand sides.  Per step j: Z_j = M(V_j) and W = H Z_j for the s columns
 // (the batched preconditioner and operator), two passes of block classical
 // Gram-Schmidt C = [V_0..V_j]^H W, W -= [V_0..V_j] C on the device, the new
-// block's QR by CholQR2 (the s x s Gram matrices on the device, their
-// Cholesky factors on the host), and the block Hessenberg least squares
+// block's QR by CholQR2 on the device, and the block Hessenberg least squares
 // min ||E_1 S_0 - Hbar Y||_F on the host by Householder reflections added
-// block column by block column.  FP64 basis and arithmetic; the flexible
+// block column by block column while the next step runs.  The basis and its
+// sums in block fixed point (k_block.cu); the flexible
 // basis Z in the multigrid's precision.  The oracle's block_fgmres follows the
 // same steps.
 // ---------------------------------------------------------------------------
 using cdx = std::complex<double>;
 
-// Cholesky G = L L^H of an s x s Hermitian matrix (row-major); false if not
-// positive definite
-static bool host_cholesky(int s, const std::vector<cdx>& G, std::vector<cdx>& L) {
-    L.assign((size_t)s * s, 0.0);
-    for (int j = 0; j < s; ++j) {
-        double d = G[(size_t)j * s + j].real();
-        for (int k = 0; k < j; ++k) d -= std::norm(L[(size_t)j * s + k]);
-        if (!(d > 0.0) || !std::isfinite(d)) return false;
-        const double ljj = std::sqrt(d);
-        L[(size_t)j * s + j] = ljj;
-        for (int i = j + 1; i < s; ++i) {
-            cdx v = G[(size_t)i * s + j];
-            for (int k = 0; k < j; ++k) v -= L[(size_t)i * s + k] * std::conj(L[(size_t)j * s + k]);
-            L[(size_t)i * s + j] = v / ljj;
-        }
-    }
-    return true;
+// CholQR2 of the s columns of W, enqueued: dst (and the basis columns vl, ve)
+// = Q with W = Q R, R = R_2 R_1, both written to R12 (2 s x s, row-major; NaN
+// where a Gram matrix is not positive definite).  W is overwritten.
+static void enqueue_cholqr2(Ctx& c, int s, double2* W, size_t n, double2* dst, int4* vl, int* ve, double2* R12,
+                            cudaStream_t st) {
+    launch_block_gram(s, W, n, c.bpart, c.bG, st);
+    launch_block_chol(c.bG, s, R12, c.bT, st);
+    launch_block_scale(W, s, c.bT, W, nullptr, nullptr, 0, 0, n, st);
+    launch_block_gram(s, W, n, c.bpart, c.bG, st);
+    launch_block_chol(c.bG, s, R12 + s * s, c.bT, st);
+    launch_block_scale(W, s, c.bT, dst, vl, ve, c.ks.sv, c.ks.se, n, st);
 }
-
-struct BlockWork {
-    int s = 0, m = 0;
-    double2* C = nullptr;        // device (m+1) s x s coefficients / Gram matrices / Y
-    double2* T = nullptr;        // device s x s triangular factor
-    double2* part = nullptr;     // device dot partials
-    double2* hbuf = nullptr;     // pinned host staging ((m+1) s x s)
-};
-
-// One CholQR pass: G = W^H W (W: s columns at stride n), G = L L^H, and the
-// columns W R^{-1} (R = L^H) written to dst (stride sd; may be W itself).
-// R returned (row-major, upper triangular).
-static int cholqr_pass(Ctx& c, BlockWork& bw, const double2* W, size_t n, double2* dst, size_t sd,
-                       std::vector<cdx>& R, cudaStream_t st) {
-    const int s = bw.s;
-    launch_block_dot(W, n, 1, s, W, n, bw.part, bw.C, st);
-    BAH_CUDA_TRY(cudaMemcpyAsync(bw.hbuf, bw.C, (size_t)s * s * sizeof(double2), cudaMemcpyDeviceToHost, st));
-    BAH_CUDA_TRY(cudaStreamSynchronize(st));
-    std::vector<cdx> G((size_t)s * s), L;
-    for (int q = 0; q < s * s; ++q) G[q] = cdx(bw.hbuf[q].x, bw.hbuf[q].y);     // G[a][b] = conj(w_a) . w_b
-    if (!host_cholesky(s, G, L)) {
-        set_error("block FGMRES: the new block is numerically rank deficient (Cholesky QR failed)");
-        return BAH_ERR_NONFINITE;
-    }
-    // R = L^H (upper); T = R^{-1} by back substitution, row-major T[q][b]
-    R.assign((size_t)s * s, 0.0);
-    for (int i = 0; i < s; ++i)
-        for (int j = i; j < s; ++j) R[(size_t)i * s + j] = std::conj(L[(size_t)j * s + i]);
-    std::vector<cdx> T((size_t)s * s, 0.0);
-    for (int b = 0; b < s; ++b) {
-        T[(size_t)b * s + b] = 1.0 / R[(size_t)b * s + b];
-        for (int q = b - 1; q >= 0; --q) {
-            cdx acc = 0.0;
-            for (int k = q + 1; k <= b; ++k) acc += R[(size_t)q * s + k] * T[(size_t)k * s + b];
-            T[(size_t)q * s + b] = -acc / R[(size_t)q * s + q];
-        }
-    }
-    for (int q = 0; q < s * s; ++q) bw.hbuf[q] = make_double2(T[q].real(), T[q].imag());
-    BAH_CUDA_TRY(cudaMemcpyAsync(bw.T, bw.hbuf, (size_t)s * s * sizeof(double2), cudaMemcpyHostToDevice, st));
-    launch_block_scale(W, s, bw.T, dst, sd, n, st);
-    BAH_CUDA_TRY(cudaStreamSynchronize(st));         // the staging buffer is reused next
-    return BAH_OK;
-}
-// CholQR2: dst = Q with W = Q R (W is overwritten by the first pass)
-static int cholqr2(Ctx& c, BlockWork& bw, double2* W, size_t n, double2* dst, size_t sd, std::vector<cdx>& R,
-                   cudaStream_t st) {
-    const int s = bw.s;
-    std::vector<cdx> R1, R2;
-    TRY(cholqr_pass(c, bw, W, n, W, n, R1, st));
-    TRY(cholqr_pass(c, bw, W, n, dst, sd, R2, st));
+// R = R_2 R_1 from the host copy of R12
+static int host_r(int s, const double2* R12, std::vector<cdx>& R) {
     R.assign((size_t)s * s, 0.0);
     for (int i = 0; i < s; ++i)
         for (int j = i; j < s; ++j) {
             cdx acc = 0.0;
-            for (int k = i; k <= j; ++k) acc += R2[(size_t)i * s + k] * R1[(size_t)k * s + j];
+            for (int k = i; k <= j; ++k) {
+                const double2 r1 = R12[k * s + j], r2 = R12[s * s + i * s + k];
+                acc += cdx(r2.x, r2.y) * cdx(r1.x, r1.y);
+            }
+            if (!std::isfinite(acc.real()) || !std::isfinite(acc.imag())) {
+                set_error("block FGMRES: the new block is numerically rank deficient (Cholesky QR failed)");
+                return BAH_ERR_NONFINITE;
+            }
             R[(size_t)i * s + j] = acc;
         }
     return BAH_OK;
@@ -1595,16 +1551,32 @@ struct BlockLS {
 };
 
 static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol, bah_stats* out, cudaStream_t st) {
-    const size_t n = c.vec_len(), sv = c.ks.sv;
+    const size_t n = c.vec_len(), nt = tiles_of(n);
     const int m = c.m;
     KS ks = c.ks;
     ks.active = nullptr;
     Batch bt;
     bt.nr = s;
     bt.active = nullptr;
-    BlockWork bw;
-    bw.s = s; bw.m = m;
-    bw.C = c.bC; bw.T = c.bT; bw.part = c.bpart; bw.hbuf = c.bhost;
+    const size_t s2 = (size_t)s * s;
+    // step j up to and including its copy to host slot j & 1: [R_1 | R_2 | C_1 | C_2]
+    auto enqueue = [&](int j) {
+        NvtxRange nvs("block fgmres step");
+        void* zj = (char*)c.Z + (size_t)j * n * c.vsz;
+        precond_any(c, (const double2*)c.Vc, n, zj, ks.sz, bt, st);
+        op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
+        const size_t cnt = (size_t)(j + 1) * s2;
+        for (int pass = 0; pass < 2; ++pass) {            // block CGS2
+            double2* C = c.bC + 2 * s2 + pass * cnt;
+            launch_block_dot(c.VL, c.VE, ks.sv, ks.se, j + 1, s, c.W, n, c.bpart, C, st);
+            launch_block_update(c.VL, c.VE, ks.sv, ks.se, j + 1, s, C, c.W, n, st);
+        }
+        enqueue_cholqr2(c, s, c.W, n, c.Vc, c.VL + (j + 1) * nt * kTile, c.VE + (j + 1) * nt, c.bC, st);
+        BAH_CUDA_TRY(cudaMemcpyAsync(c.bhost + (j & 1) * c.bslot, c.bC, (2 * s2 + 2 * cnt) * sizeof(double2),
+                                     cudaMemcpyDeviceToHost, st));
+        BAH_CUDA_TRY(cudaEventRecord(c.itev[j], st));
+        return BAH_OK;
+    };
     std::vector<double> bn(s), beta(s), est(s, 1.0);
     launch_norm2(b, n, c.dpart, c.nrm, 1, s, ks, st);
     {
@@ -1630,26 +1602,27 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
     while (!done() && total < c.o.maxit) {
         NvtxRange nvc("block fgmres restart cycle");
         // R_0 = V_0 S_0
-        TRY(cholqr2(c, bw, c.R, n, c.V, sv, S0, st));
+        enqueue_cholqr2(c, s, c.R, n, c.Vc, c.VL, c.VE, c.bC, st);
+        BAH_CUDA_TRY(cudaMemcpyAsync(c.bhost, c.bC, 2 * s2 * sizeof(double2), cudaMemcpyDeviceToHost, st));
+        BAH_CUDA_TRY(cudaStreamSynchronize(st));
+        TRY(host_r(s, c.bhost, S0));
         BlockLS ls;
         ls.init(s, m, S0);
         const int mm = std::min(m, c.o.maxit - total);
         int jd = 0;
+        TRY(enqueue(0));
         for (int j = 0; j < mm; ++j) {
-            void* zj = (char*)c.Z + (size_t)j * n * c.vsz;
-            precond_any(c, c.V + (size_t)j * n, sv, zj, ks.sz, bt, st);
-            op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
-            for (int pass = 0; pass < 2; ++pass) {            // block CGS2
-                launch_block_dot(c.V, sv, j + 1, s, c.W, n, bw.part, bw.C, st);
-                const size_t cnt = (size_t)(j + 1) * s * s;
-                BAH_CUDA_TRY(cudaMemcpyAsync(bw.hbuf, bw.C, cnt * sizeof(double2), cudaMemcpyDeviceToHost, st));
-                launch_block_update(c.V, sv, j + 1, s, bw.C, c.W, n, 1, st);
-                BAH_CUDA_TRY(cudaStreamSynchronize(st));
-                for (int row = 0; row < (j + 1) * s; ++row)
-                    for (int q = 0; q < s; ++q)
-                        ls.h(row, j * s + q) += cdx(bw.hbuf[(size_t)row * s + q].x, bw.hbuf[(size_t)row * s + q].y);
-            }
-            TRY(cholqr2(c, bw, c.W, n, c.V + (size_t)(j + 1) * n, sv, R, st));
+            // step j + 1 runs while the host extends the least-squares problem by step j
+            if (j + 1 < mm) TRY(enqueue(j + 1));
+            BAH_CUDA_TRY(cudaEventSynchronize(c.itev[j]));
+            const double2* hb = c.bhost + (j & 1) * c.bslot;
+            const size_t cnt = (size_t)(j + 1) * s2;
+            TRY(host_r(s, hb, R));
+            for (int row = 0; row < (j + 1) * s; ++row)
+                for (int q = 0; q < s; ++q) {
+                    const double2 c1 = hb[2 * s2 + (size_t)row * s + q], c2 = hb[2 * s2 + cnt + (size_t)row * s + q];
+                    ls.h(row, j * s + q) = cdx(c1.x + c2.x, c1.y + c2.y);
+                }
             for (int i = 0; i < s; ++i)
                 for (int q = 0; q < s; ++q) ls.h((j + 1) * s + i, j * s + q) = R[(size_t)i * s + q];
             ls.add_block(j, res);
@@ -1665,10 +1638,11 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
         }
         // X += [Z_0 .. Z_{jd-1}] Y
         ls.solve(jd, Y);
-        for (size_t q = 0; q < Y.size(); ++q) bw.hbuf[q] = make_double2(Y[q].real(), Y[q].imag());
-        BAH_CUDA_TRY(cudaMemcpyAsync(bw.C, bw.hbuf, Y.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
-        if (c.mode == BAH_MIXED) launch_block_xupdate<float2>((const float2*)c.Z, ks.sz, jd, s, bw.C, x, n, st);
-        else launch_block_xupdate<double2>((const double2*)c.Z, ks.sz, jd, s, bw.C, x, n, st);
+        BAH_CUDA_TRY(cudaStreamSynchronize(st));         // a step queued beyond the last one still writes its slot
+        for (size_t q = 0; q < Y.size(); ++q) c.bhost[q] = make_double2(Y[q].real(), Y[q].imag());
+        BAH_CUDA_TRY(cudaMemcpyAsync(c.bC, c.bhost, Y.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
+        if (c.mode == BAH_MIXED) launch_block_xupdate<float2>((const float2*)c.Z, ks.sz, jd, s, c.bC, x, n, st);
+        else launch_block_xupdate<double2>((const double2*)c.Z, ks.sz, jd, s, c.bC, x, n, st);
         apply_h(c, x, n, c.R, n, b, n, 0, s, st);
         launch_norm2(c.R, n, c.dpart, c.nrm, 0, s, ks, st);
         std::vector<double> tmp(c.nbatch);
