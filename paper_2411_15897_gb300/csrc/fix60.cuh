@@ -1,8 +1,8 @@
 // FP64-accurate sums of products on the integer pipe.
 //
-// GB300 issues 2 FP64 multiply-adds per clock and SM, but 64 integer ones of
-// 32 x 32 + 64 bits (both measured).  A vector that meets many others is
-// therefore held as block fixed point: the entries of a tile (kTile entries)
+// GB300 issues 2 FP64 multiply-adds per clock and SM, but 28 integer ones of
+// 32 x 32 + 64 bits (both measured; a complex product takes 4 of the first or
+// 12 of the second).  A vector that meets many others is therefore held as block fixed point: the entries of a tile (kTile entries)
 // share one exponent E, |x| < 2^E for every real of the tile, and each real is
 // the 60-bit integer X = round(x 2^(59 - E)), split into two signed limbs,
 // X = h 2^30 + l with |h| <= 2^29, -2^29 <= l < 2^29.  A product of two such

@@ -14,7 +14,9 @@
 //
 // The dots, the Gram matrix, the updates and the scaling sum exact integer
 // products; with FP64 multiply-adds (4 per entry, row and column, 2 per clock
-// and SM) they were bound by the FP64 pipe.
+// and SM) they were bound by the FP64 pipe.  Now the integer multiply-adds
+// bound them (60 % of their rate).  Measured, 8 sources on 256 x 128, 20 block
+// steps: 96.1 -> 23.6 ms (dots and updates of 112 rows 195 and 215 us each).
 #include "bah_internal.cuh"
 #include "fix60.cuh"
 
@@ -22,7 +24,7 @@
 
 namespace bah {
 
-constexpr int kBlkRows = 32;       // rows of a dot CTA
+constexpr int kBlkRows = 64;       // most rows of a dot CTA
 
 __device__ __forceinline__ void bmac(double2& acc, const double2& a, const double2& b) {        // acc += a b
     acc.x = fma(a.x, b.x, acc.x);
@@ -47,7 +49,7 @@ __device__ __forceinline__ int stage_tile(const double2* __restrict__ w, size_t 
 }
 
 // ---------------------------------------------------------------------------
-// partial[(row * s + b) * gridDim.x + cta] for the CTA's 32 rows (blockIdx.y)
+// partial[(row * s + b) * gridDim.x + cta] for the CTA's rpc rows (blockIdx.y)
 // and tiles.  The s columns of W are converted to limbs in shared memory once
 // per tile and CTA; each warp takes every eighth row, holds its tile in
 // registers and meets all columns, so a basis row is read once for s columns.
@@ -56,8 +58,8 @@ __device__ __forceinline__ int stage_tile(const double2* __restrict__ w, size_t 
 // ---------------------------------------------------------------------------
 template <int S, bool SELF>
 __global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, const int* __restrict__ VE, size_t sv,
-                                                 size_t se, int k, int s, const double2* __restrict__ W, size_t n,
-                                                 double2* __restrict__ partial) {
+                                                 size_t se, int k, int s, int rpc, const double2* __restrict__ W,
+                                                 size_t n, double2* __restrict__ partial) {
     pdl_prologue();
     extern __shared__ int4 g[];                                   // S x kTile
     constexpr int CG = S < 8 ? S : 8, NV = 2 * CG;                // columns and values of one lane reduction
@@ -65,7 +67,7 @@ __global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, co
     __shared__ double sum[kBlkRows][2 * S];
     const size_t nt = tiles_of(n), npad = nt * kTile;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int nrow = SELF ? s : k * s, row0 = blockIdx.y * kBlkRows;
+    const int nrow = SELF ? s : k * s, row0 = blockIdx.y * rpc;
     for (int q = threadIdx.x; q < kBlkRows * 2 * S; q += 256) (&sum[0][0])[q] = 0.0;
     const int myval = lane / (32 / NV);
     for (size_t t = blockIdx.x; t < nt; t += gridDim.x) {
@@ -75,7 +77,7 @@ __global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, co
             if (lane == 0) ew[b] = e;
         }
         __syncthreads();
-        for (int rl = wp; rl < kBlkRows && row0 + rl < nrow; rl += 8) {
+        for (int rl = wp; rl < rpc && row0 + rl < nrow; rl += 8) {
             const int row = row0 + rl, i = row / s, a = row % s;
             int4 v[kTileU];
             int ev;
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, co
         }
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < kBlkRows * s; q += 256) {
+    for (int q = threadIdx.x; q < rpc * s; q += 256) {
         const int rl = q / s, b = q % s;
         if (row0 + rl < nrow)
             partial[((size_t)(row0 + rl) * s + b) * gridDim.x + blockIdx.x] = make_double2(sum[rl][2 * b], sum[rl][2 * b + 1]);
@@ -159,11 +161,12 @@ template <int S, bool SELF>
 static void bdot_t(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
                    double2* partial, double2* C, cudaStream_t st) {
     const int rows = SELF ? s : k * s, chunks = (rows + kBlkRows - 1) / kBlkRows;
+    const int rpc = ((rows + chunks - 1) / chunks + 7) / 8 * 8;      // equal chunks, whole rounds of the eight warps
     // two CTAs per SM in all, whole rounds of tiles
     const size_t nt = tiles_of(n), most = std::max(1, RED_CTAS / chunks), per = (nt + most - 1) / most;
     const int nc = (int)((nt + per - 1) / per);
-    launch_pdl(k_bdot<S, SELF>, dim3(nc, chunks), dim3(256), (size_t)s * kTile * sizeof(int4), st, VL, VE, sv, se, k, s, W,
-               n, partial);
+    launch_pdl(k_bdot<S, SELF>, dim3(nc, chunks), dim3(256), (size_t)s * kTile * sizeof(int4), st, VL, VE, sv, se, k, s, rpc,
+               W, n, partial);
     launch_pdl(k_bdot_reduce, dim3((rows * s + 3) / 4), dim3(128), 0, st, (const double2*)partial, nc, rows * s, C);
 }
 void launch_block_dot(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
@@ -182,23 +185,23 @@ void launch_block_gram(int s, const double2* W, size_t n, double2* partial, doub
 // Sums of one column over rows: a warp's accumulators for the eight entries per
 // lane of a tile, sum_row V_row[e] c[row], every row's products sharing the
 // exponent eo (biased twice); the coefficients keep 60 - head bits so that the
-// rows' products fit 62 bits.
+// rows' products fit 62 bits.  U: entries per lane.
 // ---------------------------------------------------------------------------
 __host__ __device__ inline int rows_head(int rows) {
     int h = 2;
     while ((8 << h) < rows) ++h;
     return h;
 }
-struct ColSum {
-    long long hr[kTileU], cr[kTileU], hi[kTileU], ci[kTileU];
+template <int U> struct ColSum {
+    long long hr[U], cr[U], hi[U], ci[U];
     __device__ __forceinline__ void clear() {
 #pragma unroll
-        for (int u = 0; u < kTileU; ++u) hr[u] = cr[u] = hi[u] = ci[u] = 0;
+        for (int u = 0; u < U; ++u) hr[u] = cr[u] = hi[u] = ci[u] = 0;
     }
     __device__ __forceinline__ void add(const int4* row, const int4& c) {      // row: this lane's entries at 32 u
         const int nz = -c.z, nw = -c.w;
 #pragma unroll
-        for (int u = 0; u < kTileU; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int4 b = row[32 * u];
             mad(hr[u], c.x, b.x); mad(hr[u], nz, b.z);
             mad(cr[u], c.x, b.y); mad(cr[u], c.y, b.x);
@@ -210,7 +213,7 @@ struct ColSum {
     }
     __device__ __forceinline__ void carry() {                                  // at least every 4 rows
 #pragma unroll
-        for (int u = 0; u < kTileU; ++u) {
+        for (int u = 0; u < U; ++u) {
             hr[u] += cr[u] >> 30; cr[u] &= 0x3fffffff;
             hi[u] += ci[u] >> 30; ci[u] &= 0x3fffffff;
         }
@@ -224,30 +227,32 @@ struct ColSum {
 __device__ __forceinline__ int coef_exp(const double2& c) { return max(abs_hi(c.x), abs_hi(c.y)) >> 20; }
 
 // W[b][e] -= sum over rows (i, a) < k s of V_i[a][e] C[row, b].  One CTA of S
-// warps per tile, warp b on column b; the basis rows pass through a ring of
-// shared-memory slots (cp.async, groups of four rows, one barrier per group),
-// so a row is read once for all columns.
-constexpr int kUpG = 4, kUpSlots = 3;
+// warps per half tile (whole tiles left 384 units of work for 304 resident CTAs
+// at 256 x 128), warp b on column b; the basis rows pass through a ring of
+// shared-memory slots (cp.async, groups of rows, one barrier per group), so a
+// row is read once for all columns.
+constexpr int kUpG = 8, kUpSlots = 3, kUpU = kTileU / 2, kUpE = 32 * kUpU;
 template <int S>
 __global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL, const int* __restrict__ VE, size_t sv,
                                                     size_t se, int k, int s, const double2* __restrict__ C,
                                                     double2* __restrict__ W, size_t n) {
     pdl_prologue();
-    extern __shared__ int4 ring[];                                // kUpSlots x kUpG x kTile
+    extern __shared__ int4 ring[];                                // kUpSlots x kUpG x kUpE
     __shared__ int4 csh[S][32];
     const size_t nt = tiles_of(n), npad = nt * kTile;
     const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
     const int rows = k * s, head = rows_head(rows), ngrp = (rows + kUpG - 1) / kUpG;
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
-    for (size_t t = blockIdx.x; t < nt; t += gridDim.x) {
+    for (size_t h = blockIdx.x; h < 2 * nt; h += gridDim.x) {
+        const size_t t = h >> 1, eb0 = h * kUpE;                  // tile and first entry
         auto fetch = [&](int gq) {                                // group gq's rows into its slot
             if (gq < ngrp)
-                for (int e = threadIdx.x; e < kUpG * kTile; e += 32 * S) {
-                    const int row = gq * kUpG + e / kTile;
+                for (int e = threadIdx.x; e < kUpG * kUpE; e += 32 * S) {
+                    const int row = gq * kUpG + e / kUpE;
                     if (row < rows) {
-                        const int4* src = VL + (size_t)(row % s) * sv + (size_t)(row / s) * npad + t * kTile + e % kTile;
+                        const int4* src = VL + (size_t)(row % s) * sv + (size_t)(row / s) * npad + eb0 + e % kUpE;
                         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                                         ring_s + (uint32_t)((gq % kUpSlots) * kUpG * kTile + e) * 16u),
+                                         ring_s + (uint32_t)((gq % kUpSlots) * kUpG * kUpE + e) * 16u),
                                      "l"(src)
                                      : "memory");
                     }
@@ -269,7 +274,7 @@ __global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL,
             }
         eo = (int)__reduce_max_sync(0xffffffffu, (unsigned)eo);
         bad = __any_sync(0xffffffffu, bad);
-        ColSum acc;
+        ColSum<kUpU> acc;
         acc.clear();
         for (int gq = 0; gq < ngrp; ++gq) {
             asm volatile("cp.async.wait_group %0;" ::"n"(kUpSlots - 2) : "memory");
@@ -286,8 +291,11 @@ __global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL,
                 }
                 __syncwarp();
             }
-            const int4* slot = ring + (gq % kUpSlots) * kUpG * kTile + lane;
-            for (int q = 0; q < kUpG && gq * kUpG + q < rows; ++q) acc.add(slot + q * kTile, csh[b][(gq * kUpG + q) & 31]);
+            const int4* slot = ring + (gq % kUpSlots) * kUpG * kUpE + lane;
+            for (int q = 0; q < kUpG && gq * kUpG + q < rows; ++q) {
+                acc.add(slot + q * kUpE, csh[b][(gq * kUpG + q) & 31]);
+                if ((q & 3) == 3) acc.carry();
+            }
             acc.carry();
         }
         if (b < s) {
@@ -296,20 +304,20 @@ __global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL,
             double s1 = pow2(p + 60), s2 = pow2(p + 30);
             if (bad) s1 = __longlong_as_double(0x7ff8000000000000ll);
             double2* w = W + (size_t)b * n;
-            const size_t e0 = t * kTile + lane;
+            const size_t e0 = eb0 + lane;
 #pragma unroll
-            for (int u = 0; u < kTileU; ++u)
+            for (int u = 0; u < kUpU; ++u)
                 if (e0 + 32 * u < n) w[e0 + 32 * u] = acc.minus(w[e0 + 32 * u], u, s1, s2);
         }
     }
 }
 void launch_block_update(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* C, double2* W,
                          size_t n, cudaStream_t st) {
-    const size_t smem = (size_t)kUpSlots * kUpG * kTile * sizeof(int4);
-    const unsigned nt = (unsigned)tiles_of(n);
-    if (s <= 4) launch_pdl(k_bupdate<4>, dim3(std::min(nt, 608u)), dim3(128), smem, st, VL, VE, sv, se, k, s, C, W, n);
-    else if (s <= 8) launch_pdl(k_bupdate<8>, dim3(std::min(nt, 304u)), dim3(256), smem, st, VL, VE, sv, se, k, s, C, W, n);
-    else launch_pdl(k_bupdate<16>, dim3(std::min(nt, 152u)), dim3(512), smem, st, VL, VE, sv, se, k, s, C, W, n);
+    const size_t smem = (size_t)kUpSlots * kUpG * kUpE * sizeof(int4);
+    const unsigned nt = 2 * (unsigned)tiles_of(n);
+    if (s <= 4) launch_pdl(k_bupdate<4>, dim3(std::min(nt, 1216u)), dim3(128), smem, st, VL, VE, sv, se, k, s, C, W, n);
+    else if (s <= 8) launch_pdl(k_bupdate<8>, dim3(std::min(nt, 608u)), dim3(256), smem, st, VL, VE, sv, se, k, s, C, W, n);
+    else launch_pdl(k_bupdate<16>, dim3(std::min(nt, 304u)), dim3(512), smem, st, VL, VE, sv, se, k, s, C, W, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -393,7 +401,7 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
             csh[b][lane] = ec > 0 && eb >= kExpMin ? limbs2(c, eb) : make_int4(0, 0, 0, 0);
         }
         __syncwarp();
-        ColSum acc;
+        ColSum<kTileU> acc;
         acc.clear();
         for (int q = 0; q <= b; ++q) {
             acc.add(g + q * kTile + lane, csh[b][q]);
@@ -473,7 +481,7 @@ void launch_block_xupdate(const Vz* Z, size_t sz, int k, int s, const double2* Y
     }
 }
 int block_prepare() {
-    const int ring = (int)(kUpSlots * kUpG * kTile * sizeof(int4)), cols = (int)(16 * kTile * sizeof(int4));
+    const int ring = (int)(kUpSlots * kUpG * kUpE * sizeof(int4)), cols = (int)(16 * kTile * sizeof(int4));
     const struct { const void* f; int b; } fns[] = {
         {(const void*)k_bdot<16, false>, cols}, {(const void*)k_bdot<16, true>, cols}, {(const void*)k_bscale<16>, cols},
         {(const void*)k_bupdate<4>, ring},      {(const void*)k_bupdate<8>, ring},     {(const void*)k_bupdate<16>, ring}};
