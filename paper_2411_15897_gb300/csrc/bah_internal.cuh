@@ -115,8 +115,51 @@ template <class V> __host__ __device__ __forceinline__ V cdiv(V b, V a) {
     typename VecTraits<V>::R d = a.x * a.x + a.y * a.y;
     return cmk<V>((b.x * a.x + b.y * a.y) / d, (b.y * a.x - b.x * a.y) / d);
 }
+// FP32 to FP64 with integer instructions: a conversion instruction runs at the
+// FP64 pipe's 2 per clock and SM, these at 64.  A subnormal is scaled by 2^64
+// first (exact in FP32); there is no branch, because the compiler would turn one
+// into a predicated conversion that still takes its slot.
+__host__ __device__ __forceinline__ double f2d(float f) {
+#ifdef __CUDA_ARCH__
+    const bool sub = fabsf(f) < 1.17549435e-38f;
+    const float g = sub ? f * 18446744073709551616.f : f;
+    const unsigned b = __float_as_uint(g), m = b & 0x7fffffffu;
+    unsigned hi = (m >> 3) + (sub ? 0x34000000u : 0x38000000u);        // exponent - 127 + 1023 (- 64)
+    if (m >= 0x7f800000u) hi = (m >> 3) + 0x70000000u;                 // infinity, NaN: exponent 2047
+    if (m == 0) hi = 0;
+    return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(b << 29));
+#else
+    return (double)f;
+#endif
+}
 template <class To, class From> __host__ __device__ __forceinline__ To cconv(From a) {
     return cmk<To>((typename VecTraits<To>::R)a.x, (typename VecTraits<To>::R)a.y);
+}
+// -x if neg is 1, x if it is 0 (the compiler negates a selected FP64 value on the FP64 pipe)
+__device__ __forceinline__ double flip_sign(double x, int neg) {
+    return __hiloint2double(__double2hiint(x) ^ (neg << 31), __double2loint(x));
+}
+// FP64 to FP32, round to nearest even, the same way (the conversion instruction
+// runs at 5.5 per clock and SM; results outside the FP32 normal range take it)
+__device__ __noinline__ inline float d2f_slow(double x) { return (float)x; }   // a call: a branch, not a predicate
+__host__ __device__ __forceinline__ float d2f(double x) {
+#ifdef __CUDA_ARCH__
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if ((hi << 1) == 0 && lo == 0) return __uint_as_float(hi);
+    if (e - 897u >= 253u) return d2f_slow(x);                  // below 2^-126 or from 2^127 on
+    const unsigned long long r = (((unsigned long long)hi << 32) | lo) + 0x0fffffffull + ((lo >> 29) & 1u);
+    const unsigned rh = (unsigned)(r >> 32), rl = (unsigned)r;
+    return __uint_as_float((hi & 0x80000000u) | (((rh & 0x7fffffffu) - 0x38000000u) << 3 | rl >> 29));
+#else
+    return (float)x;
+#endif
+}
+template <> __host__ __device__ __forceinline__ float2 cconv<float2, double2>(double2 a) {
+    return cmk<float2>(d2f(a.x), d2f(a.y));
+}
+template <> __host__ __device__ __forceinline__ double2 cconv<double2, float2>(float2 a) {
+    return cmk<double2>(f2d(a.x), f2d(a.y));
 }
 
 __host__ __device__ __forceinline__ bool valid_pt(int type, int i, int j) {
@@ -275,6 +318,7 @@ template <int MODE>
 void launch_coarse_apply(int nb, int npts, const int4* const* inv, const int* const* inve,
                          const typename Prec<MODE>::V* const* b, typename Prec<MODE>::V* const* x, cudaStream_t st,
                          int nrhs = 1, RhsStride rs = RhsStride());
+// RIN: the input vector's entries, FP64, double-float or (mixed mode) already rounded to FP32
 template <int MODE, class RIN = double2>
 void launch_distributor(int n1, int n2, double ihx, double ihz,
                         const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f5,
@@ -313,8 +357,10 @@ void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, siz
 // returns the number of partial sums of |w_new|^2 in npart
 int launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
                      const int* flag, int nrhs, const KS& ks, cudaStream_t st);
-// v = w / sc[slot] as FP64 (vc, stride ks.sw) and as a basis vector (vl, ve)
-void launch_basis_store(const double2* w, const double* sc, int slot, double2* vc, int4* vl, int* ve, size_t n,
+// v = w / sc[slot] as the preconditioner's input (vc, FP64 or rounded to FP32,
+// stride ks.sw) and as a basis vector (vl, ve)
+template <class Vc>
+void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, size_t n,
                         size_t sw, int nrhs, const KS& ks, cudaStream_t st);
 // flag = 1 (second pass) when ||w'||^2 < eta2 ||w||^2 (DGKS criterion; eta2 = 1/2 classically)
 void launch_dgks_decide(const double* npart, int np, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
@@ -353,7 +399,9 @@ void launch_block_gram(int s, const double2* W, size_t n, double2* partial, doub
 void launch_block_update(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* C, double2* W,
                          size_t n, cudaStream_t st);
 void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStream_t st);
-void launch_block_scale(const double2* W, int s, const double2* T, double2* dst, int4* vl, int* ve, size_t sv, size_t se,
+// dst: FP64, or (with vl) rounded to FP32
+template <class Vd>
+void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, int4* vl, int* ve, size_t sv, size_t se,
                         size_t n, cudaStream_t st);
 template <class Vz>
 void launch_block_xupdate(const Vz* Z, size_t sz, int k, int s, const double2* Y, double2* X, size_t n,
@@ -367,13 +415,13 @@ void launch_gradient(int n1, int n2, double h1, double h2, double omega, const d
                      cudaStream_t st);
 
 // three-dimensional grids (k_3d.cu).  FP64 operator coefficients of H on
-// n[0] x n[1] x n[2] cells; mue[e] is the edge mean of mu for the pair of axes
-// other than e, zero on boundary edges.
+// n[0] x n[1] x n[2] cells; the edge mean mue[e] of mu belongs to the pair of
+// axes other than e and is zero on boundary edges.
 struct Op3 {
     int n[3];
     double ih[3], ih2[3];     // 1/h_a, 1/h_a^2
-    const double* muc;        // mu at cells
-    const double* mue[3];
+    const double* cmu[3];     // mu / h_a^2 at cells (one array where the spacings are equal)
+    const double* cme[3][3];  // [e][b]: the edge mean mue[e] / h_b^2 (one array per e where they are equal)
     const double2* dg[3];     // diagonal of A_a (unshifted, with -omega^2 A_f(rho~))
     const double* cinv;       // 1/(lambda+mu)
     const double2* mrt;       // omega^2 rho~ at cells
@@ -381,6 +429,7 @@ struct Op3 {
 void launch_prep3(const Op3& op, double omega, double alpha, const double* lam, const double* mu, const double* rho,
                   const double* gam, double* cinv, double2* mrt, double* const* mue, double2* const* dg,
                   double2* const* S, cudaStream_t st);
+void launch_scale_real(const double* src, double f, double* dst, size_t n, cudaStream_t st);   // dst = f src
 template <class Vin>
 void launch_apply3(const Op3& op, const Vin* x, double2* y, const double2* b, int conj, int nrhs, size_t sx, size_t sy,
                    size_t sb, cudaStream_t st);

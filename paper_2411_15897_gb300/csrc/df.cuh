@@ -11,8 +11,7 @@
 // hi + lo equals the double to 2^-47 relative.  Values below the FP32 normal
 // range (|x| < 1.2e-38) are flushed to zero.
 #pragma once
-#include <cuda_runtime.h>
-#include <stdint.h>
+#include "bah_internal.cuh"
 
 namespace bah {
 
@@ -38,7 +37,7 @@ __device__ __forceinline__ dfl df_from_double(double x) {
     return r;
 }
 
-__device__ __forceinline__ double df_to_double(dfl a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double df_to_double(dfl a) { return f2d(a.hi) + f2d(a.lo); }
 
 // exact sum of two floats: s + e = a + b
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -103,7 +102,7 @@ struct dfacc {
         hi = s + e;
         lo = e - (hi - s);
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ double value() const { return f2d(hi) + f2d(lo); }
 };
 
 // complex double-float stored as float4 (re.hi, re.lo, im.hi, im.lo)
@@ -112,7 +111,7 @@ __device__ __forceinline__ dfl im_of(const float4& v) { dfl r; r.hi = v.z; r.lo 
 __device__ __forceinline__ float4 cdf_make(dfl re, dfl im) { return make_float4(re.hi, re.lo, im.hi, im.lo); }
 __device__ __forceinline__ float4 cdf_from_double2(double2 z) { return cdf_make(df_from_double(z.x), df_from_double(z.y)); }
 __device__ __forceinline__ double2 cdf_to_double2(const float4& v) {
-    return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+    return make_double2(f2d(v.x) + f2d(v.y), f2d(v.z) + f2d(v.w));
 }
 
 }  // namespace bah

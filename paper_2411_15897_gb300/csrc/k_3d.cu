@@ -15,6 +15,7 @@
 // with pdl_prologue() and are launched with programmatic dependent launch; the
 // level kernels run the three displacement blocks of a level in one launch.
 #include "bah_internal.cuh"
+#include "op_rows.cuh"
 
 #include <type_traits>
 
@@ -86,7 +87,8 @@ __global__ void k_prep3_cells(int n1, int n2, int n3, double omega, const double
 // (Eq. 3.4: B B^T diag((lambda+2mu)/(lambda+mu)) - omega^2 diag(rho~/(lambda+mu)),
 // shifted by i alpha omega^2 rho/(lambda+mu))
 __global__ void k_prep3_blocks(Op3 op, double alpha, double omega, const double* __restrict__ rho,
-                               const double* __restrict__ mu, double2* dg0, double2* dg1, double2* dg2,
+                               const double* __restrict__ mu, const double* mue0, const double* mue1,
+                               const double* mue2, double2* dg0, double2* dg1, double2* dg2,
                                double2* S0, double2* S1, double2* S2, double2* S3) {
     const int n1 = op.n[0], n2 = op.n[1], n3 = op.n[2];
     const int np = n1 * n2 * n3;
@@ -95,6 +97,7 @@ __global__ void k_prep3_blocks(Op3 op, double alpha, double omega, const double*
     int c[3];
     coords3(p, n1, n2, c);
     const int st[3] = {1, n1, n1 * n2};
+    const double* mue[3] = {mue0, mue1, mue2};
     double2* dg[3] = {dg0, dg1, dg2};
     double2* S[4] = {S0, S1, S2, S3};
     const double aw2 = alpha * omega * omega;
@@ -109,7 +112,7 @@ __global__ void k_prep3_blocks(Op3 op, double alpha, double omega, const double*
             if (c[a] + 1 <= op.n[a] - 1) e[2 + 2 * a].x = -op.ih2[a] * mu[p];
             for (int b = 0; b < 3; ++b) {
                 if (b == a) continue;
-                const double* me = op.mue[3 - a - b];
+                const double* me = mue[3 - a - b];
                 const double lo = c[b] >= 1 ? me[p] : 0.0;
                 const double hi = c[b] + 1 <= op.n[b] - 1 ? me[p + st[b]] : 0.0;
                 dr += op.ih2[b] * (lo + hi);
@@ -153,7 +156,15 @@ void launch_prep3(const Op3& op, double omega, double alpha, const double* lam, 
     const int nb = (np + 255) / 256;
     k_prep3_cells<<<nb, 256, 0, st>>>(op.n[0], op.n[1], op.n[2], omega, lam, mu, rho, gam, cinv, mrt, mue[0], mue[1],
                                       mue[2]);
-    k_prep3_blocks<<<nb, 256, 0, st>>>(op, alpha, omega, rho, mu, dg[0], dg[1], dg[2], S[0], S[1], S[2], S[3]);
+    k_prep3_blocks<<<nb, 256, 0, st>>>(op, alpha, omega, rho, mu, mue[0], mue[1], mue[2], dg[0], dg[1], dg[2], S[0], S[1], S[2], S[3]);
+}
+
+__global__ void k_scale_real(const double* __restrict__ src, double f, double* __restrict__ dst, size_t n) {
+    const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (e < n) dst[e] = f * src[e];
+}
+void launch_scale_real(const double* src, double f, double* dst, size_t n, cudaStream_t st) {
+    k_scale_real<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, f, dst, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -177,33 +188,49 @@ __global__ void __launch_bounds__(256) k_apply3(Op3 op, const Vin* __restrict__ 
     coords3(p, n1, n2, c);
     const int st[3] = {1, n1, n1 * n2};
     auto ld = [&](int comp, int q) { return cconv<double2>(x[(size_t)comp * np + q]); };
-    const double2 pc = ld(3, p);
+    // 74 FP64 operations per cell, all fused, from coefficients divided by h^2 at
+    // setup; the FP64 pipe (2 per clock and SM) bounds the kernel.  With FP32 input at
+    // 128^3: 643 us when every load was converted by the FP64 pipe and every
+    // coefficient formed in the kernel, 385 us now
+    auto add = [](double2& acc, double k, const double2& v) {
+        acc.x = fma(k, v.x, acc.x);
+        acc.y = fma(k, v.y, acc.y);
+    };
+    auto sub = [](double2& acc, double k, const double2& v) {         // negated inside the fma: no instruction of its own
+        acc.x = fma(-k, v.x, acc.x);
+        acc.y = fma(-k, v.y, acc.y);
+    };
+    // every neighbour is loaded (at a clamped index) and its coefficient replaced by 0
+    // outside the grid, so that the loads issue together
+    const double2 pc = ld(3, p), zero = make_double2(0.0, 0.0);
     double2 out[4];
+    double2 div = cscale(pc, -op.cinv[p]);
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (c[a] == 0) { out[a] = make_double2(0.0, 0.0); continue; }
-        double2 d = op.dg[a][p];
-        if (conj) d.y = -d.y;
-        double2 acc = cmul(d, ld(a, p));
-        const int pm = p - st[a];
-        if (c[a] >= 2) acc = csub(acc, cscale(ld(a, pm), op.ih2[a] * op.muc[pm]));
-        if (c[a] + 1 <= op.n[a] - 1) acc = csub(acc, cscale(ld(a, p + st[a]), op.ih2[a] * op.muc[p]));
+        const bool lo = c[a] >= 1, hi = c[a] + 1 <= op.n[a] - 1;
+        const int pm = lo ? p - st[a] : p, pe = hi ? p + st[a] : p;
+        const double2 uc = lo ? ld(a, p) : zero, ue = hi ? ld(a, pe) : zero;
+        add(div, op.ih[a], csub(uc, ue));
+        const double2 uw = ld(a, pm);
+        const double kw = op.cmu[a][pm], ke = op.cmu[a][p];
+        double2 acc = cscale(uw, c[a] >= 2 ? kw : 0.0);
+        add(acc, ke, ue);
+#pragma unroll
         for (int bb = 0; bb < 3; ++bb) {
             if (bb == a) continue;
-            const double* me = op.mue[3 - a - bb];
-            if (c[bb] >= 1) acc = csub(acc, cscale(ld(a, p - st[bb]), op.ih2[bb] * me[p]));
-            if (c[bb] + 1 <= op.n[bb] - 1) acc = csub(acc, cscale(ld(a, p + st[bb]), op.ih2[bb] * me[p + st[bb]]));
+            const double* me = op.cme[3 - a - bb][bb];               // zero on boundary edges
+            const bool bl = c[bb] >= 1, bh = c[bb] + 1 <= op.n[bb] - 1;
+            const int qm = bl ? p - st[bb] : p, qe = bh ? p + st[bb] : p;
+            const double km = me[p], kp = me[qe];
+            const double2 um = ld(a, qm), up = ld(a, qe);
+            add(acc, bl ? km : 0.0, um);
+            add(acc, bh ? kp : 0.0, up);
         }
-        acc = cadd(acc, cscale(csub(pc, ld(3, pm)), op.ih[a]));
-        out[a] = acc;
+        sub(acc, op.ih[a], csub(pc, ld(3, pm)));
+        out[a] = lo ? diag_minus(op.dg[a][p], uc, conj, acc) : zero;
     }
-    {
-        double2 acc = cscale(pc, -op.cinv[p]);
-        for (int a = 0; a < 3; ++a) {
-            if (c[a] >= 1) acc = cadd(acc, cscale(ld(a, p), op.ih[a]));
-            if (c[a] + 1 <= op.n[a] - 1) acc = csub(acc, cscale(ld(a, p + st[a]), op.ih[a]));
-        }
-        out[3] = acc;
-    }
+    out[3] = div;
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
         const bool v = k == 3 || c[k] >= 1;
         double2 o = out[k];
@@ -256,21 +283,28 @@ __global__ void __launch_bounds__(256) k_distrib3(Op3 op, const double2* __restr
     coords3(p, n1, n2, c);
     const int st[3] = {1, n1, n1 * n2};
     const double2* rp = r + (size_t)3 * np;
-    const double2 mrp = cscale(rp[p], op.muc[p]);
-    double2 acc = cmul(op.mrt[p], rp[p]);        // + omega^2 rho~ r_p
+    const double2 r0 = rp[p];
+    const double2 m = op.mrt[p];
+    double2 acc = make_double2(fma(m.x, r0.x, -(m.y * r0.y)), fma(m.x, r0.y, m.y * r0.x));   // + omega^2 rho~ r_p
+    double k0 = 0.0;                             // mu_p times the number of neighbours along each axis / h^2
+    auto add = [&](double k, const double2& v) {
+        acc.x = fma(k, v.x, acc.x);
+        acc.y = fma(k, v.y, acc.y);
+    };
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
         const double2* ra = r + (size_t)a * np;
-        if (c[a] >= 1) {
-            const int q = p - st[a];
-            acc = cadd(acc, cscale(ra[p], op.ih[a]));
-            acc = csub(acc, cscale(csub(mrp, cscale(rp[q], op.muc[q])), op.ih2[a]));
-        }
-        if (c[a] + 1 <= op.n[a] - 1) {
-            const int q = p + st[a];
-            acc = csub(acc, cscale(ra[q], op.ih[a]));
-            acc = csub(acc, cscale(csub(mrp, cscale(rp[q], op.muc[q])), op.ih2[a]));
-        }
+        const bool lo = c[a] >= 1, hi = c[a] + 1 <= op.n[a] - 1;
+        const int qm = lo ? p - st[a] : p, qe = hi ? p + st[a] : p;
+        const double2 gl = ra[p], gh = ra[qe], rl = rp[qm], rh = rp[qe];
+        const double kl = op.cmu[a][qm], kh = op.cmu[a][qe], kp = op.cmu[a][p];
+        const double2 zero = make_double2(0.0, 0.0);
+        add(lo ? kl : 0.0, rl);
+        add(hi ? kh : 0.0, rh);
+        add(op.ih[a], csub(lo ? gl : zero, hi ? gh : zero));
+        k0 += lo && hi ? 2.0 * kp : (lo || hi ? kp : 0.0);
     }
+    add(-k0, r0);
     tp[p] = cconv<V>(acc);
 }
 
@@ -288,13 +322,12 @@ __global__ void __launch_bounds__(256) k_urhs3(Op3 op, const double2* __restrict
     const int st[3] = {1, n1, n1 * n2};
     V* s[3] = {s0, s1, s2};
     const double2 e0 = cconv<double2>(ep[p]);
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        double2 v = make_double2(0.0, 0.0);
-        if (c[a] >= 1) {
-            const double2 g = cscale(csub(e0, cconv<double2>(ep[p - st[a]])), op.ih[a]);
-            v = csub(r[(size_t)a * np + p], g);
-        }
-        s[a][p] = cconv<V>(v);
+        const bool lo = c[a] >= 1;
+        const double2 em = cconv<double2>(ep[lo ? p - st[a] : p]), v = r[(size_t)a * np + p];
+        const double2 o = make_double2(fma(-op.ih[a], e0.x - em.x, v.x), fma(-op.ih[a], e0.y - em.y, v.y));
+        s[a][p] = cconv<V>(lo ? o : make_double2(0.0, 0.0));
     }
 }
 

@@ -372,8 +372,8 @@ void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStre
 // written to dst (column b at b * n; may be W itself) and, with vl, as basis
 // columns.  One CTA of S warps per tile: warp b converts column b to limbs in
 // shared memory, then sums column b of the product.
-template <int S>
-__global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, const double2* __restrict__ T, double2* dst,
+template <int S, class Vd>
+__global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, const double2* __restrict__ T, Vd* dst,
                                                    int4* __restrict__ vl, int* __restrict__ ve, size_t sv, size_t se,
                                                    size_t n) {
     pdl_prologue();
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
             x[u] = make_double2(0.0, 0.0);
             if (e0 + 32 * u < n) {
                 x[u] = acc.minus(x[u], u, s1, s2);
-                dst[(size_t)b * n + e0 + 32 * u] = x[u];
+                dst[(size_t)b * n + e0 + 32 * u] = cconv<Vd>(x[u]);
             }
             mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
         }
@@ -431,13 +431,14 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
         }
     }
 }
-void launch_block_scale(const double2* W, int s, const double2* T, double2* dst, int4* vl, int* ve, size_t sv, size_t se,
+template <class Vd>
+void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, int4* vl, int* ve, size_t sv, size_t se,
                         size_t n, cudaStream_t st) {
     const size_t smem = (size_t)s * kTile * sizeof(int4);
     const unsigned nt = (unsigned)tiles_of(n);
-    if (s <= 4) launch_pdl(k_bscale<4>, dim3(std::min(nt, 608u)), dim3(128), smem, st, W, s, T, dst, vl, ve, sv, se, n);
-    else if (s <= 8) launch_pdl(k_bscale<8>, dim3(std::min(nt, 304u)), dim3(256), smem, st, W, s, T, dst, vl, ve, sv, se, n);
-    else launch_pdl(k_bscale<16>, dim3(std::min(nt, 152u)), dim3(512), smem, st, W, s, T, dst, vl, ve, sv, se, n);
+    if (s <= 4) launch_pdl(k_bscale<4, Vd>, dim3(std::min(nt, 608u)), dim3(128), smem, st, W, s, T, dst, vl, ve, sv, se, n);
+    else if (s <= 8) launch_pdl(k_bscale<8, Vd>, dim3(std::min(nt, 304u)), dim3(256), smem, st, W, s, T, dst, vl, ve, sv, se, n);
+    else launch_pdl(k_bscale<16, Vd>, dim3(std::min(nt, 152u)), dim3(512), smem, st, W, s, T, dst, vl, ve, sv, se, n);
 }
 
 // X[b][e] += sum over rows (i, a) < k s of Z_i[a][e] Y[row, b]  (Z FP32 or FP64 complex)
@@ -455,7 +456,7 @@ __global__ void __launch_bounds__(256) k_bxupdate(const Vz* __restrict__ Z, size
         for (int row = 0; row < k * s; ++row) {
             const int i = row / s, a = row % s;
             const Vz zv = Z[(size_t)a * sz + (size_t)i * n + e];
-            const double2 z = make_double2((double)zv.x, (double)zv.y);
+            const double2 z = cconv<double2>(zv);
 #pragma unroll
             for (int b = 0; b < S; ++b)
                 if (b < s) bmac(acc[b], z, ys[row * s + b]);
@@ -483,11 +484,16 @@ void launch_block_xupdate(const Vz* Z, size_t sz, int k, int s, const double2* Y
 int block_prepare() {
     const int ring = (int)(kUpSlots * kUpG * kUpE * sizeof(int4)), cols = (int)(16 * kTile * sizeof(int4));
     const struct { const void* f; int b; } fns[] = {
-        {(const void*)k_bdot<16, false>, cols}, {(const void*)k_bdot<16, true>, cols}, {(const void*)k_bscale<16>, cols},
+        {(const void*)k_bdot<16, false>, cols}, {(const void*)k_bdot<16, true>, cols}, {(const void*)k_bscale<16, double2>, cols},
+        {(const void*)k_bscale<16, float2>, cols},
         {(const void*)k_bupdate<4>, ring},      {(const void*)k_bupdate<8>, ring},     {(const void*)k_bupdate<16>, ring}};
     for (const auto& q : fns) BAH_CUDA_TRY(cudaFuncSetAttribute(q.f, cudaFuncAttributeMaxDynamicSharedMemorySize, q.b));
     return BAH_OK;
 }
+template void launch_block_scale<double2>(const double2*, int, const double2*, double2*, int4*, int*, size_t, size_t,
+                                          size_t, cudaStream_t);
+template void launch_block_scale<float2>(const double2*, int, const double2*, float2*, int4*, int*, size_t, size_t,
+                                         size_t, cudaStream_t);
 template void launch_block_xupdate<float2>(const float2*, size_t, int, int, const double2*, double2*, size_t,
                                            cudaStream_t);
 template void launch_block_xupdate<double2>(const double2*, size_t, int, int, const double2*, double2*, size_t,

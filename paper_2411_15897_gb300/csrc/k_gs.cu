@@ -405,11 +405,13 @@ int gs_prepare() {
 }
 
 // ---------------------------------------------------------------------------
-// v = w / sc[slot]: the FP64 vector (the next preconditioner input) and its
-// limbs and tile exponents in the basis
+// v = w / sc[slot]: the vector as the next preconditioner input (rounded to
+// FP32 for an FP32 preconditioner, which then reads half the bytes and converts
+// nothing: the distributor of 32 sources of 1024 x 512 493 -> 116 us) and its limbs and tile exponents in the basis
 // ---------------------------------------------------------------------------
+template <class Vc>
 __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restrict__ w, const double* sc, int slot,
-                                                         double2* __restrict__ vc, int4* __restrict__ vl,
+                                                         Vc* __restrict__ vc, int4* __restrict__ vl,
                                                          int* __restrict__ ve, size_t n, size_t sw, KS ks) {
     pdl_prologue();
     const int r = blockIdx.y;
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
             if (e0 + 32 * u < n) {
                 x[u].x *= s;
                 x[u].y *= s;
-                vc[e0 + 32 * u] = x[u];
+                vc[e0 + 32 * u] = cconv<Vc>(x[u]);
             }
             mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
         }
@@ -442,11 +444,16 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
         for (int u = 0; u < kTileU; ++u) vl[e0 + 32 * u] = limbs2(x[u], eb);
     }
 }
-void launch_basis_store(const double2* w, const double* sc, int slot, double2* vc, int4* vl, int* ve, size_t n,
+template <class Vc>
+void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, size_t n,
                         size_t sw, int nrhs, const KS& ks, cudaStream_t st) {
     const size_t nt = tiles_of(n);
-    launch_pdl(k_gs_store, dim3((unsigned)((nt + kGsWarps - 1) / kGsWarps), nrhs), dim3(kGsThreads), 0, st, w, sc, slot, vc,
+    launch_pdl(k_gs_store<Vc>, dim3((unsigned)((nt + kGsWarps - 1) / kGsWarps), nrhs), dim3(kGsThreads), 0, st, w, sc, slot, vc,
                vl, ve, n, sw, ks);
 }
+template void launch_basis_store<double2>(const double2*, const double*, int, double2*, int4*, int*, size_t, size_t, int,
+                                          const KS&, cudaStream_t);
+template void launch_basis_store<float2>(const double2*, const double*, int, float2*, int4*, int*, size_t, size_t, int,
+                                         const KS&, cudaStream_t);
 
 }  // namespace bah

@@ -12,8 +12,7 @@ namespace bah {
 
 template <class V>
 __device__ __forceinline__ double2 ld64(const V* p, int idx) {
-    V v = p[idx];
-    return make_double2((double)v.x, (double)v.y);
+    return cconv<double2>(p[idx]);
 }
 __device__ __forceinline__ double2 ld64(const float4* p, int idx) { return cdf_to_double2(p[idx]); }
 // preconditioner input in the preconditioner's real type R
@@ -26,6 +25,7 @@ template <> struct InLoad<double> {
 };
 template <> struct InLoad<float> {
     __device__ static float2 get(const double2* p, size_t i) { const double2 v = p[i]; return make_float2((float)v.x, (float)v.y); }
+    __device__ static float2 get(const float2* p, size_t i) { return p[i]; }
     __device__ static float2 get(const float4* p, size_t i) { const float4 v = p[i]; return make_float2(v.x + v.y, v.z + v.w); }
 };
 __device__ __forceinline__ void st_out(double2* y, size_t i, double2 v) { y[i] = v; }
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256) k_elastic_apply(OpCoef c, const Vin* __re
     auto U2 = [&](int ii, int jj) { return (ii >= 0 && ii < n1 && jj >= 1 && jj < n2) ? ld64(x2, jj * n1 + ii) : z; };
     auto P = [&](int g) { return ld64(xp, g); };
     double2 y1, y2, yp;
-    elastic_rows(c, i, j, t, conj ? -1.0 : 1.0, U1, U2, P, y1, y2, yp);
+    elastic_rows(c, i, j, t, conj, U1, U2, P, y1, y2, yp);
     if (b) {
         if (i >= 1) y1 = csub(b[t], y1);
         if (j >= 1) y2 = csub(b[np + t], y2);
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(256) k_elastic_apply(OpCoef c, const Vin* __re
 // 48-bit significand)
 __device__ __forceinline__ void st_dfa(float4* y, size_t i, const float4& v) { y[i] = v; }
 __device__ __forceinline__ void st_dfa(double2* y, size_t i, const float4& v) {
-    y[i] = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+    y[i] = cdf_to_double2(v);
 }
 template <class Vout>
 __global__ void __launch_bounds__(256) k_elastic_apply_dfa(OpCoefDF c, const float2* __restrict__ x,
@@ -251,6 +251,9 @@ template void launch_distributor<BAH_FP64, double2>(int, int, double, double, co
 template void launch_distributor<BAH_MIXED, double2>(int, int, double, double,
                                                      const Fine5<__nv_bfloat16, __nv_bfloat162>&, const double2*,
                                                      float2*, cudaStream_t, int, RhsStride);
+template void launch_distributor<BAH_MIXED, float2>(int, int, double, double,
+                                                    const Fine5<__nv_bfloat16, __nv_bfloat162>&, const float2*,
+                                                    float2*, cudaStream_t, int, RhsStride);
 template void launch_distributor<BAH_FP64, float4>(int, int, double, double, const Fine5<double, double2>&,
                                                    const float4*, double2*, cudaStream_t, int, RhsStride);
 template void launch_distributor<BAH_MIXED, float4>(int, int, double, double,
@@ -303,6 +306,8 @@ template void launch_u_rhs<BAH_FP64, double2>(int, int, double, double, const do
                                               double2*, cudaStream_t, int, RhsStride);
 template void launch_u_rhs<BAH_MIXED, double2>(int, int, double, double, const double2*, const float2*, float2*,
                                                float2*, cudaStream_t, int, RhsStride);
+template void launch_u_rhs<BAH_MIXED, float2>(int, int, double, double, const float2*, const float2*, float2*,
+                                              float2*, cudaStream_t, int, RhsStride);
 template void launch_u_rhs<BAH_FP64, float4>(int, int, double, double, const float4*, const double2*, double2*,
                                              double2*, cudaStream_t, int, RhsStride);
 template void launch_u_rhs<BAH_MIXED, float4>(int, int, double, double, const float4*, const float2*, float2*,

@@ -67,11 +67,12 @@ struct Ctx {
     // Krylov workspace
     int m = 20;
     double2 *V = nullptr, *W = nullptr, *R = nullptr, *Bs = nullptr, *X = nullptr;
-    // the FP64 basis of the lockstep solve: limbs and tile exponents (fix60.cuh), and the newest
-    // vector in FP64, the preconditioner's input (V itself holds the other two kinds of basis)
+    // the FP64 basis: limbs and tile exponents (fix60.cuh), and the newest vector as the
+    // preconditioner's input, FP64 or (vc32) rounded to FP32; V is the double-float basis
     int4* VL = nullptr;
     int* VE = nullptr;
-    double2* Vc = nullptr;
+    void* Vc = nullptr;
+    bool vc32 = false;
     double2 *Hm = nullptr, *h1v = nullptr, *h2v = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr;
     double2* partial = nullptr;
     double *nrm = nullptr, *dpart = nullptr, *status = nullptr;
@@ -762,6 +763,19 @@ static void precond_any(Ctx& c, const RIN* r, size_t rstride, void* z, size_t zs
     if (c.mode == BAH_MIXED) MG<BAH_MIXED>::template precond<RIN>(c, r, rstride, (float2*)z, zstride, bt, st);
     else MG<BAH_FP64>::template precond<RIN>(c, r, rstride, (double2*)z, zstride, bt, st);
 }
+// z = P^{-1} D v for the newest basis vector(s)
+static void precond_newest(Ctx& c, void* z, const Batch& bt, cudaStream_t st) {
+    if (c.vc32) MG<BAH_MIXED>::template precond<float2>(c, (const float2*)c.Vc, c.ks.sw, (float2*)z, c.ks.sz, bt, st);
+    else precond_any(c, (const double2*)c.Vc, c.ks.sw, z, c.ks.sz, bt, st);
+}
+// w / sc[slot] as basis vector i and as the newest vector
+static void store_basis(Ctx& c, const double2* w, int slot, int i, cudaStream_t st) {
+    const size_t n = c.vec_len(), nt = tiles_of(n);
+    int4* vl = c.VL + i * nt * kTile;
+    int* ve = c.VE + i * nt;
+    if (c.vc32) launch_basis_store(w, c.nrm, slot, (float2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st);
+    else launch_basis_store(w, c.nrm, slot, (double2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st);
+}
 // algorithmic bytes of one operator apply: input (3 components), FP64
 // output, coefficients cx, nx (z-aliases when h1 == h2), d1, d2, 1/(lambda+mu)
 static double op_bytes(const Ctx& c, double in_bytes, bool residual) {
@@ -823,7 +837,9 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
         TRY(gs_prepare());
         TRY(c.alloc_t(&c.VL, nt * kTile * (m + 1) * nbt));
         TRY(c.alloc_t(&c.VE, nt * (m + 1) * nbt));
-        TRY(c.alloc_t(&c.Vc, n * nbt));
+        // the 2-D FP32 cycles read the newest vector in FP32 only
+        c.vc32 = c.mode == BAH_MIXED && c.dim == 2 && !c.exact;
+        TRY(c.alloc(&c.Vc, n * nbt * (c.vc32 ? sizeof(float2) : sizeof(double2))));
     }
     TRY(c.alloc(&c.Z, n * m * c.vsz * nbt));
     TRY(c.alloc_t(&c.W, n * nbt)); TRY(c.alloc_t(&c.R, n * nbt)); TRY(c.alloc_t(&c.Bs, n * nbt));
@@ -1101,8 +1117,8 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
     o.n[0] = c.n1; o.n[1] = c.n2; o.n[2] = c.n3;
     const double h[3] = {c.h1, c.h2, c.h3};
     for (int a = 0; a < 3; ++a) { o.ih[a] = 1.0 / h[a]; o.ih2[a] = 1.0 / (h[a] * h[a]); }
-    o.muc = mu; o.cinv = cinv; o.mrt = mrt;
-    for (int e = 0; e < 3; ++e) { o.mue[e] = mue[e]; o.dg[e] = dg[e]; }
+    o.cinv = cinv; o.mrt = mrt;
+    for (int e = 0; e < 3; ++e) o.dg[e] = dg[e];
     // level grids and FP64 stencils
     c.d3.assign(c.L, {0, 0, 0});
     for (int l = 0; l < c.L; ++l) c.d3[l] = {c.n1 >> l, c.n2 >> l, c.n3 >> l};
@@ -1111,6 +1127,21 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
     c.s3s.assign(c.L, {nullptr, nullptr, nullptr, nullptr});
     for (int q = 0; q < 4; ++q) TRY(c.alloc_t(&c.s3[0][q], 7 * np));
     launch_prep3(o, c.omega, c.alpha, lam, mu, rho, gam, cinv, mrt, mue, dg, c.s3[0].data(), st);
+    // mu and its edge means divided by the squared spacings
+    auto scaled = [&](const double* src, int a, const double* const* earlier, const double** dst) {
+        for (int b = 0; b < a; ++b)
+            if (o.ih2[b] == o.ih2[a] && earlier[b]) { *dst = earlier[b]; return BAH_OK; }
+        double* d = nullptr;
+        TRY(c.alloc_t(&d, np));
+        launch_scale_real(src, o.ih2[a], d, np, st);
+        *dst = d;
+        return BAH_OK;
+    };
+    for (int a = 0; a < 3; ++a) {
+        TRY(scaled(mu, a, o.cmu, &o.cmu[a]));
+        for (int e = 0; e < 3; ++e)
+            if (e != a) TRY(scaled(mue[e], a, o.cme[e], &o.cme[e][a]));
+    }
     int* err;
     TRY(c.alloc_t(&err, 2));
     BAH_CUDA_TRY(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
@@ -1210,7 +1241,7 @@ static void iter_body(Ctx& c, int j, cudaStream_t st) {
     float4* Vd = (float4*)c.V;
     float4* Wd = (float4*)c.W;
     if (c.kdf) precond_any(c, Vd + (size_t)j * n, ks.sv, zj, ks.sz, bt, st);
-    else precond_any(c, (const double2*)c.Vc, n, zj, ks.sz, bt, st);
+    else precond_newest(c, zj, bt, st);
     op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
     const double k1 = j + 1;
     int npt = 0;                 // partial sums of ||w'||^2
@@ -1243,8 +1274,7 @@ static void iter_body(Ctx& c, int j, cudaStream_t st) {
         launch_pass2_norm(c.dpart, npt, c.gsflag, c.nrm, nb, ks, st);
         launch_arnoldi_givens(c.Hm, m + 1, c.h1v, c.h2v, c.nrm, j, c.cs, c.sn, c.g, c.status, nb, ks, st);
         if (c.kdf) launch_scale_copy_df(c.W, false, c.nrm, 2, Vd + (size_t)(j + 1) * n, n, n, ks.sv, nb, ks, st);
-        else launch_basis_store(c.W, c.nrm, 2, c.Vc, c.VL + (j + 1) * tiles_of(n) * kTile, c.VE + (j + 1) * tiles_of(n), n,
-                                n, nb, ks, st);
+        else store_basis(c, c.W, 2, j + 1, st);
     }
     cudaMemcpyAsync(status_slot(c, j), c.status, 4 * (size_t)nb * sizeof(double), cudaMemcpyDeviceToHost, st);
 }
@@ -1346,7 +1376,7 @@ static int fgmres_batch(Ctx& c, const double2* b, double2* x, int nr, double rto
         {
             Prof pr(c, BAH_K_SMALL, st, (double)nr * n * 32.0, 2);
             if (c.kdf) launch_scale_copy_df(c.R, true, c.nrm, 0, (float4*)c.V, n, n, ks.sv, nb, ks, st);
-            else launch_basis_store(c.R, c.nrm, 0, c.Vc, c.VL, c.VE, n, n, nb, ks, st);
+            else store_basis(c, c.R, 0, 0, st);
             launch_init_arnoldi(c.nrm, c.g, m, c.status, nb, ks, st);
         }
         const int mm = std::min(m, c.o.maxit - total);
@@ -1441,17 +1471,19 @@ static int fgmres_batch(Ctx& c, const double2* b, double2* x, int nr, double rto
 // ---------------------------------------------------------------------------
 using cdx = std::complex<double>;
 
-// CholQR2 of the s columns of W, enqueued: dst (and the basis columns vl, ve)
+// CholQR2 of the s columns of W, enqueued: basis block i and the newest block
 // = Q with W = Q R, R = R_2 R_1, both written to R12 (2 s x s, row-major; NaN
 // where a Gram matrix is not positive definite).  W is overwritten.
-static void enqueue_cholqr2(Ctx& c, int s, double2* W, size_t n, double2* dst, int4* vl, int* ve, double2* R12,
-                            cudaStream_t st) {
+static void enqueue_cholqr2(Ctx& c, int s, double2* W, size_t n, int i, double2* R12, cudaStream_t st) {
+    int4* vl = c.VL + i * tiles_of(n) * kTile;
+    int* ve = c.VE + i * tiles_of(n);
     launch_block_gram(s, W, n, c.bpart, c.bG, st);
     launch_block_chol(c.bG, s, R12, c.bT, st);
     launch_block_scale(W, s, c.bT, W, nullptr, nullptr, 0, 0, n, st);
     launch_block_gram(s, W, n, c.bpart, c.bG, st);
     launch_block_chol(c.bG, s, R12 + s * s, c.bT, st);
-    launch_block_scale(W, s, c.bT, dst, vl, ve, c.ks.sv, c.ks.se, n, st);
+    if (c.vc32) launch_block_scale(W, s, c.bT, (float2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, n, st);
+    else launch_block_scale(W, s, c.bT, (double2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, n, st);
 }
 // R = R_2 R_1 from the host copy of R12
 static int host_r(int s, const double2* R12, std::vector<cdx>& R) {
@@ -1551,7 +1583,7 @@ struct BlockLS {
 };
 
 static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol, bah_stats* out, cudaStream_t st) {
-    const size_t n = c.vec_len(), nt = tiles_of(n);
+    const size_t n = c.vec_len();
     const int m = c.m;
     KS ks = c.ks;
     ks.active = nullptr;
@@ -1563,7 +1595,7 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
     auto enqueue = [&](int j) {
         NvtxRange nvs("block fgmres step");
         void* zj = (char*)c.Z + (size_t)j * n * c.vsz;
-        precond_any(c, (const double2*)c.Vc, n, zj, ks.sz, bt, st);
+        precond_newest(c, zj, bt, st);
         op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
         const size_t cnt = (size_t)(j + 1) * s2;
         for (int pass = 0; pass < 2; ++pass) {            // block CGS2
@@ -1571,7 +1603,7 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
             launch_block_dot(c.VL, c.VE, ks.sv, ks.se, j + 1, s, c.W, n, c.bpart, C, st);
             launch_block_update(c.VL, c.VE, ks.sv, ks.se, j + 1, s, C, c.W, n, st);
         }
-        enqueue_cholqr2(c, s, c.W, n, c.Vc, c.VL + (j + 1) * nt * kTile, c.VE + (j + 1) * nt, c.bC, st);
+        enqueue_cholqr2(c, s, c.W, n, j + 1, c.bC, st);
         BAH_CUDA_TRY(cudaMemcpyAsync(c.bhost + (j & 1) * c.bslot, c.bC, (2 * s2 + 2 * cnt) * sizeof(double2),
                                      cudaMemcpyDeviceToHost, st));
         BAH_CUDA_TRY(cudaEventRecord(c.itev[j], st));
@@ -1602,7 +1634,7 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
     while (!done() && total < c.o.maxit) {
         NvtxRange nvc("block fgmres restart cycle");
         // R_0 = V_0 S_0
-        enqueue_cholqr2(c, s, c.R, n, c.Vc, c.VL, c.VE, c.bC, st);
+        enqueue_cholqr2(c, s, c.R, n, 0, c.bC, st);
         BAH_CUDA_TRY(cudaMemcpyAsync(c.bhost, c.bC, 2 * s2 * sizeof(double2), cudaMemcpyDeviceToHost, st));
         BAH_CUDA_TRY(cudaStreamSynchronize(st));
         TRY(host_r(s, c.bhost, S0));

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256) k_static_residual_partial(OpCoef c, const
         auto U2 = [&](int ii, int jj) { return (ii >= 0 && ii < n1 && jj >= 1 && jj < n2) ? x2[jj * n1 + ii] : z; };
         auto P = [&](int g) { return xp[g]; };
         double2 y1, y2, yp;
-        elastic_rows(c, i, j, t, 1.0, U1, U2, P, y1, y2, yp);
+        elastic_rows(c, i, j, t, 0, U1, U2, P, y1, y2, yp);
         if (i >= 1) {
             const double2 r = csub(b[t], y1);
             rr += r.x * r.x + r.y * r.y;
