@@ -132,6 +132,23 @@ __host__ __device__ __forceinline__ double f2d(float f) {
     return (double)f;
 #endif
 }
+// the same with one division (a reciprocal and two products)
+template <class V> __host__ __device__ __forceinline__ V cdiv1(V b, V a) {
+    const typename VecTraits<V>::R d = 1 / (a.x * a.x + a.y * a.y);
+    return cmk<V>((b.x * a.x + b.y * a.y) * d, (b.y * a.x - b.x * a.y) * d);
+}
+__device__ __forceinline__ void cfma(float2& acc, float2 a, float2 b) {      // acc += a b
+    acc.x = fmaf(a.x, b.x, acc.x);
+    acc.x = fmaf(-a.y, b.y, acc.x);
+    acc.y = fmaf(a.x, b.y, acc.y);
+    acc.y = fmaf(a.y, b.x, acc.y);
+}
+__device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
+    acc.x = fma(a.x, b.x, acc.x);
+    acc.x = fma(-a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y);
+    acc.y = fma(a.y, b.x, acc.y);
+}
 template <class To, class From> __host__ __device__ __forceinline__ To cconv(From a) {
     return cmk<To>((typename VecTraits<To>::R)a.x, (typename VecTraits<To>::R)a.y);
 }
@@ -222,23 +239,23 @@ template <class V, class CC> struct LvlSet {
 };
 
 constexpr int kMaxLevels = 16;
-// shared-memory-resident cluster multigrid (mixed mode): levels l0 .. L-1 of
+// shared-memory-resident cluster multigrid: levels l0 .. L-1 of
 // one block set, one cluster per block and right-hand side; lv[k] is level
 // l0 + k, its rows split in slabs of rp rows per CTA, and off_* are byte
 // offsets of its arrays in each CTA's dynamic shared memory
 struct SmLevel {
     int n1, n2, rp;
-    float inv_rp, inv_n1;     // 1/rp and 1/n1 (row and column from a flat or row index)
-    float w;                  // Jacobi damping
+    float inv_rp, inv_n1, inv_p;   // 1/rp, 1/n1 and 1/pitch (row and column from a flat or row index)
+    double w;                 // Jacobi damping
     unsigned off_c, off_x, off_t, off_b;
 };
 struct SmArgs {
     SmLevel lv[kMaxLevels];
     int nlev, b0, nb, nu_pre, nu_post, intergrid, wcycle, warm;
     int rx[2][kMaxLevels], rz[2][kMaxLevels];
-    const __nv_bfloat162* S[2][kMaxLevels];   // global stencils (levels below the coarsest)
-    const float2* gb[2];      // level-l0 right-hand sides (right-hand side r at r * points)
-    float2* gx[2];            // level-l0 iterates / results
+    const void* S[2][kMaxLevels];   // global stencils (levels below the coarsest)
+    const void* gb[2];        // level-l0 right-hand sides (right-hand side r at r * points)
+    void* gx[2];              // level-l0 iterates / results
     const int4* inv[2];       // coarsest inverses in block fixed point (global memory), exponent per row
     const int* inve[2];
     unsigned off_g, off_r;    // gathered coarsest right-hand side, reduction scratch
@@ -246,10 +263,11 @@ struct SmArgs {
 };
 // fills the shared-memory layout of a (n1, n2, slot counts per level from l0);
 // returns the bytes of dynamic shared memory per CTA
-size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs);
+size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs, int mode,
+                   int rm);
 // sets the kernel attributes; returns how many clusters of cs CTAs fit (0: none)
-int smmg_prepare(int rm, int cs, size_t smem);
-int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, cudaStream_t st);
+int smmg_prepare(int rm, int cs, size_t smem, int mode);
+int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, int mode, cudaStream_t st);
 
 // right-hand-side batching: element strides between consecutive right-hand
 // sides for up to three pointers of a launch (blockIdx.y or .z is the

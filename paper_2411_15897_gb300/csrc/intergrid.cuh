@@ -54,6 +54,25 @@ __host__ __device__ __forceinline__ T pw_axis_t(bool nodal, int nfine, int f, in
     nb = nb < 0 ? 0 : (nb > nc - 1 ? nc - 1 : nb);
     return (c == J ? T(0.75) : T(0)) + (c == nb ? T(0.25) : T(0));
 }
+// the same interpolation as the two coarse indices and weights of fine index f (an
+// unused one with weight 0 at an index in range)
+template <class T>
+__host__ __device__ __forceinline__ void pw_pair(bool nodal, int nfine, int f, int* c, T* w) {
+    const int nc = nfine / 2, J = f >> 1;
+    if (nodal) {
+        const int hi = (f & 1) ? J + 1 : J;
+        w[0] = J >= 1 ? ((f & 1) ? T(0.5) : T(1)) : T(0);
+        w[1] = (f & 1) && hi <= nc - 1 ? T(0.5) : T(0);
+        c[0] = J;
+        c[1] = hi <= nc - 1 ? hi : nc - 1;
+        if (J > nc - 1) { c[0] = nc - 1; w[0] = T(0); }
+        return;
+    }
+    int nb = (f & 1) ? J + 1 : J - 1;
+    nb = nb < 0 ? 0 : (nb > nc - 1 ? nc - 1 : nb);
+    c[0] = J; w[0] = T(0.75);
+    c[1] = nb; w[1] = T(0.25);
+}
 template <class T>
 __host__ __device__ __forceinline__ T rw_axis_t(bool nodal, int intergrid, int nfine, int c, int f) {
     if (!nodal && intergrid == BAH_INTERGRID_MIXED) {

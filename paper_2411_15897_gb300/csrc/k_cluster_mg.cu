@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 namespace bah {
 
@@ -44,28 +45,29 @@ __device__ __forceinline__ uint32_t mapa_rank(uint32_t local_addr, unsigned rank
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ float2 ld_cluster_at(uint32_t cluster_addr) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr));
+template <class V> __device__ __forceinline__ V ld_cluster_at(uint32_t cluster_addr) {
+    V v;
+    if constexpr (sizeof(V) == 8)
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr));
+    else
+        asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(cluster_addr));
     return v;
 }
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+template <int BYTES> __device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
 }
 
 }  // namespace
 
-template <int RM>
+template <int MODE, int RM>
 __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
-    pdl_prologue();
-    using V = float2;
-    using CC = __nv_bfloat162;
+    using V = typename Prec<MODE>::V;
+    using CC = typename Prec<MODE>::CC;
+    using R = typename Prec<MODE>::R;
+    constexpr unsigned kV = sizeof(V);
+    constexpr int G = RM;                               // ghost columns on each side of a row
     const unsigned cid = cluster_index();
     const int z = (int)(cid % (unsigned)a.nb), rr = (int)(cid / (unsigned)a.nb);
-    if (a.active && !a.active[rr]) return;              // uniform over the cluster
     const unsigned q = cluster_rank();
     const int tid = threadIdx.x, nth = blockDim.x;
     const int type = a.b0 + z;
@@ -75,115 +77,140 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
     const int nlev = a.nlev, kc = nlev - 1;
 
     auto p0 = [&](const SmLevel& L) { return (int)q * L.rp * L.n1; };
-    auto nown = [&](const SmLevel& L) {
-        const int r0 = (int)q * L.rp, r1 = min(L.n2, r0 + L.rp);
-        return r1 > r0 ? (r1 - r0) * L.n1 : 0;
-    };
+    auto nrow = [&](const SmLevel& L) { return max(0, min(L.n2 - (int)q * L.rp, L.rp)); };   // own rows
+    auto nown = [&](const SmLevel& L) { return nrow(L) * L.n1; };
+    // own points: b unpadded, x and t with G zero columns before and after each row
     auto vec = [&](unsigned off) { return reinterpret_cast<V*>(sm + off); };
-    // cluster address of column 0 of grid row `row` of vector `off` of level L
-    // (one owner lookup and one mapa per row; the columns follow at 8 bytes)
+    auto at = [&](const SmLevel& L, int r, int i) { return r * (L.n1 + 2 * G) + G + i; };
+    // cluster address of column 0 of grid row `row` of x or t of level L (one owner
+    // lookup and one mapa per row; the columns follow at kV bytes), and of b
     auto row_addr = [&](const SmLevel& L, unsigned off, int row) -> uint32_t {
         const int owner = (int)(((float)row + 0.5f) * L.inv_rp);
-        return mapa_rank(sbase + off + (uint32_t)((row - owner * L.rp) * L.n1) * 8u, (unsigned)owner);
+        return mapa_rank(sbase + off + (uint32_t)at(L, row - owner * L.rp, 0) * kV, (unsigned)owner);
     };
-    // row and column of own point lt of level L
-    auto own_rc = [&](const SmLevel& L, int lt, int& row, int& col) {
-        const int r = (int)(((float)lt + 0.5f) * L.inv_n1);
-        row = (int)q * L.rp + r;
+    auto row_addr_b = [&](const SmLevel& L, int row) -> uint32_t {
+        const int owner = (int)(((float)row + 0.5f) * L.inv_rp);
+        return mapa_rank(sbase + L.off_b + (uint32_t)((row - owner * L.rp) * L.n1) * kV, (unsigned)owner);
+    };
+    // own row and column of own point lt of level L
+    auto own_rc = [&](const SmLevel& L, int lt, int& r, int& col) {
+        r = (int)(((float)lt + 0.5f) * L.inv_n1);
         col = lt - r * L.n1;
     };
     auto coef = [&](int k) { return reinterpret_cast<const CC*>(sm + a.lv[k].off_c); };
 
-    // ---- load: stencils, coarsest inverse rows, level-l0 vectors ----
-    // asynchronous copies (cp.async), so that every thread keeps many loads in
-    // flight; one wait for all of them before the first barrier
+    // ---- load ----
+    // The stencils never change after setup, so they are copied (cp.async: many
+    // copies in flight per thread) before this launch waits for the kernel in front
+    // of it; the level-l0 vectors follow after the wait.
     for (int k = 0; k < kc; ++k) {
         const SmLevel& L = a.lv[k];
         const int np = L.n1 * L.n2, own = nown(L), g0 = p0(L), cap = L.rp * L.n1;
         const int nsl = (2 * a.rx[z][k] + 1) * (2 * a.rz[z][k] + 1);
-        const CC* S = a.S[z][k];
-        for (int s = 0; s < nsl; ++s)
-            for (int t = tid; t < own; t += nth)
-                cp_async4(sbase + L.off_c + (uint32_t)(s * cap + t) * 4u, S + (size_t)s * np + g0 + t);
+        const CC* S = (const CC*)a.S[z][k];
+        // 16 bytes per copy where every slot's slab starts and ends on 16 bytes
+        constexpr int E = 16 / (int)sizeof(CC);
+        if (E == 1 || (np % E == 0 && cap % E == 0 && own % E == 0)) {
+            const int own4 = own / E, cnt4 = nsl * own4;
+            const float inv = 1.0f / (float)max(own4, 1);
+            for (int e = tid; e < cnt4; e += nth) {
+                const int s = (int)(((float)e + 0.5f) * inv), t = (e - s * own4) * E;
+                cp_async<16>(sbase + L.off_c + (uint32_t)(s * cap + t) * (uint32_t)sizeof(CC), S + (size_t)s * np + g0 + t);
+            }
+        } else {
+            for (int s = 0; s < nsl; ++s)
+                for (int t = tid; t < own; t += nth)
+                    cp_async<sizeof(CC)>(sbase + L.off_c + (uint32_t)(s * cap + t) * (uint32_t)sizeof(CC),
+                                         S + (size_t)s * np + g0 + t);
+        }
+        // zero iterates, so that the ghost columns are zero
+        const int cnt = L.rp * (L.n1 + 2 * G);
+        for (int t = tid; t < cnt; t += nth) { vec(L.off_x)[t] = czero<V>(); vec(L.off_t)[t] = czero<V>(); }
     }
+    for (int t = tid; t < a.lv[kc].rp * (a.lv[kc].n1 + 2 * G); t += nth) vec(a.lv[kc].off_x)[t] = czero<V>();
+    pdl_prologue();
+    if (a.active && !a.active[rr]) {                    // uniform over the cluster
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return;
+    }
+    __syncthreads();
     {
         const SmLevel& L = a.lv[0];
         const int own = nown(L), g0 = p0(L);
         const size_t roff = (size_t)rr * L.n1 * L.n2 + g0;
         for (int t = tid; t < own; t += nth) {
-            cp_async8(sbase + L.off_b + (uint32_t)t * 8u, a.gb[z] + roff + t);
-            if (a.warm) cp_async8(sbase + L.off_x + (uint32_t)t * 8u, a.gx[z] + roff + t);
+            cp_async<sizeof(V)>(sbase + L.off_b + (uint32_t)t * kV, (const V*)a.gb[z] + roff + t);
+            if (a.warm) {
+                int r, i;
+                own_rc(L, t, r, i);
+                cp_async<sizeof(V)>(sbase + L.off_x + (uint32_t)at(L, r, i) * kV, (const V*)a.gx[z] + roff + t);
+            }
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     cluster_barrier();
 
-    // ---- phases (own points only; neighbours through distributed shared memory) ----
-    auto stencil = [&](int k, unsigned xoff, int lt) -> V {
+    // ---- phases (own points only) ----
+    // Jacobi sweep (res: residual) of level k with stencil radii RX, RZ: the RZ rows
+    // above and below the slab are first copied from the neighbours' shared memory,
+    // zero outside the grid, so that every tap is an unconditional local load (rows
+    // read through the cluster with a test per tap cost 860 instructions per point,
+    // this 250)
+    V* halo = reinterpret_cast<V*>(sm + a.off_g);       // 2 RZ rows of the input's pitch
+    auto sweep = [&](auto rx_, auto rz_, int k, unsigned xin, unsigned xout, bool res) {
+        constexpr int RX = decltype(rx_)::value, RZ = decltype(rz_)::value;
         const SmLevel& L = a.lv[k];
-        const int rx = a.rx[z][k], rz = a.rz[z][k], wx = 2 * rx + 1, cap = L.rp * L.n1;
-        int j, i;
-        own_rc(L, lt, j, i);
-        const CC* cs = coef(k);
-        V sv[(2 * RM + 1) * (2 * RM + 1)], xv[(2 * RM + 1) * (2 * RM + 1)];
-        bool in[(2 * RM + 1) * (2 * RM + 1)];
-#pragma unroll
-        for (int dz = -RM; dz <= RM; ++dz) {
-            const int jj = j + dz;
-            const bool rok = dz >= -rz && dz <= rz && jj >= 0 && jj < L.n2;
-            const uint32_t ra = row_addr(L, xoff, rok ? jj : j);
-#pragma unroll
-            for (int dx = -RM; dx <= RM; ++dx) {
-                const int qq = (dz + RM) * (2 * RM + 1) + (dx + RM);
-                const int ii = i + dx;
-                in[qq] = rok && dx >= -rx && dx <= rx && ii >= 0 && ii < L.n1;
-                const int slot = in[qq] ? (dz + rz) * wx + (dx + rx) : 0;
-                sv[qq] = ldc(cs[slot * cap + lt]);
-                xv[qq] = ld_cluster_at(ra + (uint32_t)(in[qq] ? ii : i) * 8u);
-            }
+        const int rows = nrow(L), r0 = (int)q * L.rp, P = L.n1 + 2 * G, cap = L.rp * L.n1;
+        for (int e = tid; e < 2 * RZ * P; e += nth) {
+            const int h = (int)(((float)e + 0.5f) * L.inv_p), col = e - h * P - G;
+            const int row = h < RZ ? r0 - RZ + h : r0 + rows + h - RZ;
+            const bool in = row >= 0 && row < L.n2 && col >= 0 && col < L.n1;
+            halo[e] = in ? ld_cluster_at<V>(row_addr(L, xin, row) + (uint32_t)col * kV) : czero<V>();
         }
-        V acc = czero<V>();
-#pragma unroll
-        for (int e = 0; e < (2 * RM + 1) * (2 * RM + 1); ++e) {
-            const float m = in[e] ? 1.f : 0.f;
-            acc.x += m * (sv[e].x * xv[e].x - sv[e].y * xv[e].y);
-            acc.y += m * (sv[e].x * xv[e].y + sv[e].y * xv[e].x);
-        }
-        return acc;
-    };
-    auto diag = [&](int k, int lt) -> V {
-        const SmLevel& L = a.lv[k];
-        const int rx = a.rx[z][k], rz = a.rz[z][k];
-        return ldc(coef(k)[(rz * (2 * rx + 1) + rx) * (L.rp * L.n1) + lt]);
-    };
-    auto jacobi = [&](int k, unsigned xin, unsigned xout, bool zero) {
-        const SmLevel& L = a.lv[k];
-        const int own = nown(L);
+        __syncthreads();
         const V* b = vec(L.off_b);
-        const V* xi = vec(xin);
+        const V* x = vec(xin);
         V* xo = vec(xout);
+        const int own = rows * L.n1;
         for (int lt = tid; lt < own; lt += nth) {
-            int j, i;
-            own_rc(L, lt, j, i);
-            if (!valid_pt(type, i, j)) { xo[lt] = czero<V>(); continue; }
-            const V dg = diag(k, lt);
-            if (zero) { xo[lt] = cscale(cdiv(b[lt], dg), L.w); continue; }
-            const V ax = stencil(k, xin, lt);
-            const V corr = cdiv(csub(b[lt], ax), dg);
-            const V xv = xi[lt];
-            xo[lt] = cmk<V>(xv.x + L.w * corr.x, xv.y + L.w * corr.y);
+            int r, i;
+            own_rc(L, lt, r, i);
+            const int o = at(L, r, i);
+            if (!valid_pt(type, i, r0 + r)) { xo[o] = czero<V>(); continue; }
+            const CC* cs = coef(k) + lt;
+            V ax = czero<V>();
+#pragma unroll
+            for (int dz = -RZ; dz <= RZ; ++dz) {
+                const int t = r + dz;
+                const V* xr = (t < 0 ? halo + (RZ + t) * P : (t >= rows ? halo + (RZ + t - rows) * P : x + t * P)) + G + i;
+#pragma unroll
+                for (int dx = -RX; dx <= RX; ++dx) cfma(ax, ldc(cs[((dz + RZ) * (2 * RX + 1) + dx + RX) * cap]), xr[dx]);
+            }
+            const V d = csub(b[lt], ax);
+            if (res) { xo[o] = d; continue; }
+            const V dg = ldc(cs[(RZ * (2 * RX + 1) + RX) * cap]);
+            const V c = cdiv1(d, dg), xv = x[o];
+            xo[o] = cmk<V>(xv.x + (R)L.w * c.x, xv.y + (R)L.w * c.y);
         }
     };
-    auto residual = [&](int k, unsigned xin, unsigned rout) {
+    auto stencil_phase = [&](int k, unsigned xin, unsigned xout, bool res) {
+        std::integral_constant<int, 1> one;
+        std::integral_constant<int, RM> rm;
+        if (a.rx[z][k] == RM && a.rz[z][k] == RM) sweep(rm, rm, k, xin, xout, res);
+        else if (a.rx[z][k] == RM) sweep(rm, one, k, xin, xout, res);
+        else if (a.rz[z][k] == RM) sweep(one, rm, k, xin, xout, res);
+        else sweep(one, one, k, xin, xout, res);
+    };
+    auto jacobi_zero = [&](int k, unsigned xout) {
         const SmLevel& L = a.lv[k];
         const int own = nown(L);
         const V* b = vec(L.off_b);
-        V* r = vec(rout);
+        V* xo = vec(xout);
+        const CC* cs = coef(k) + (size_t)(a.rz[z][k] * (2 * a.rx[z][k] + 1) + a.rx[z][k]) * (L.rp * L.n1);
         for (int lt = tid; lt < own; lt += nth) {
-            int j, i;
-            own_rc(L, lt, j, i);
-            if (!valid_pt(type, i, j)) { r[lt] = czero<V>(); continue; }
-            r[lt] = csub(b[lt], stencil(k, xin, lt));
+            int r, i;
+            own_rc(L, lt, r, i);
+            xo[at(L, r, i)] = valid_pt(type, i, (int)q * L.rp + r) ? cscale(cdiv1(b[lt], ldc(cs[lt])), (R)L.w) : czero<V>();
         }
     };
     auto restrict_ = [&](int k, unsigned rin) {          // b_{k+1} = R r_k on own coarse points
@@ -194,31 +221,32 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
         for (int lt = tid; lt < own; lt += nth) {
             int J, I;
             own_rc(Lc, lt, J, I);
+            J += (int)q * Lc.rp;
             V acc = czero<V>();
             if (valid_pt(type, I, J)) {
                 const int bx = rbase(nodx, a.intergrid, I), bz = rbase(nodz, a.intergrid, J);
-                float wxs[4], wzs[4];
+                R wxs[4], wzs[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    wxs[e] = rw_axis_t<float>(nodx, a.intergrid, L.n1, I, bx + e);
-                    wzs[e] = rw_axis_t<float>(nodz, a.intergrid, L.n2, J, bz + e);
+                    wxs[e] = rw_axis_t<R>(nodx, a.intergrid, L.n1, I, bx + e);
+                    wzs[e] = rw_axis_t<R>(nodz, a.intergrid, L.n2, J, bz + e);
                 }
                 V v[16];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const bool rok = wzs[e] != 0.f;
+                    const bool rok = wzs[e] != R(0);
                     const uint32_t ra = row_addr(L, rin, rok ? bz + e : 0);
 #pragma unroll
                     for (int f = 0; f < 4; ++f) {
-                        const bool ok = rok && wxs[f] != 0.f;
-                        v[e * 4 + f] = ld_cluster_at(ra + (uint32_t)(ok ? bx + f : 0) * 8u);
+                        const bool ok = rok && wxs[f] != R(0);
+                        v[e * 4 + f] = ld_cluster_at<V>(ra + (uint32_t)(ok ? bx + f : 0) * kV);
                     }
                 }
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
 #pragma unroll
                     for (int f = 0; f < 4; ++f) {
-                        const float wgt = wzs[e] * wxs[f];
+                        const R wgt = wzs[e] * wxs[f];
                         acc.x += wgt * v[e * 4 + f].x;
                         acc.y += wgt * v[e * 4 + f].y;
                     }
@@ -232,61 +260,56 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
         const int own = nown(L);
         V* x = vec(xoff);
         for (int lt = tid; lt < own; lt += nth) {
-            int j, i;
-            own_rc(L, lt, j, i);
+            int r, i;
+            own_rc(L, lt, r, i);
+            const int j = (int)q * L.rp + r;
             if (!valid_pt(type, i, j)) continue;
-            float px[3], pz[3];
+            int cx[2], cz[2];
+            R wx[2], wz[2];
+            pw_pair<R>(nodx, L.n1, i, cx, wx);
+            pw_pair<R>(nodz, L.n2, j, cz, wz);
+            V v[4];
 #pragma unroll
-            for (int e = 0; e < 3; ++e) {
-                px[e] = pw_axis_t<float>(nodx, L.n1, i, (i >> 1) - 1 + e);
-                pz[e] = pw_axis_t<float>(nodz, L.n2, j, (j >> 1) - 1 + e);
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t ra = row_addr(Lc, Lc.off_x, cz[e]);
+#pragma unroll
+                for (int f = 0; f < 2; ++f) v[e * 2 + f] = ld_cluster_at<V>(ra + (uint32_t)cx[f] * kV);
             }
-            V v[9];
+            const int o = at(L, r, i);
+            V acc = x[o];
 #pragma unroll
-            for (int e = 0; e < 3; ++e) {
-                const bool rok = pz[e] != 0.f;
-                const uint32_t ra = row_addr(Lc, Lc.off_x, rok ? (j >> 1) - 1 + e : 0);
+            for (int e = 0; e < 2; ++e)
 #pragma unroll
-                for (int f = 0; f < 3; ++f) {
-                    const bool ok = rok && px[f] != 0.f;
-                    v[e * 3 + f] = ld_cluster_at(ra + (uint32_t)(ok ? (i >> 1) - 1 + f : 0) * 8u);
+                for (int f = 0; f < 2; ++f) {
+                    const R wgt = wz[e] * wx[f];
+                    acc.x += wgt * v[e * 2 + f].x;
+                    acc.y += wgt * v[e * 2 + f].y;
                 }
-            }
-            V acc = x[lt];
-#pragma unroll
-            for (int e = 0; e < 3; ++e)
-#pragma unroll
-                for (int f = 0; f < 3; ++f) {
-                    const float wgt = pz[e] * px[f];
-                    acc.x += wgt * v[e * 3 + f].x;
-                    acc.y += wgt * v[e * 3 + f].y;
-                }
-            x[lt] = acc;
+            x[o] = acc;
         }
     };
     auto coarse = [&]() {                                   // x_c = A_c^{-1} b_c on own rows, exact integer sums
         const SmLevel& L = a.lv[kc];
         const int npc = L.n1 * L.n2, own = nown(L), g0 = p0(L);
         int4* gath = reinterpret_cast<int4*>(sm + a.off_g);
-        const int eg = dense_load<V, float>(gath, npc, reinterpret_cast<int*>(sm + a.off_r), [&](int g) {
-            return ld_cluster_at(row_addr(L, L.off_b, g / L.n1) + (uint32_t)(g % L.n1) * 8u);
+        const int eg = dense_load<V, R>(gath, npc, reinterpret_cast<int*>(sm + a.off_r), [&](int g) {
+            return ld_cluster_at<V>(row_addr_b(L, g / L.n1) + (uint32_t)(g % L.n1) * kV);
         });
         V* x = vec(L.off_x);
         const int lane = tid & 31;
         for (int row = tid >> 5; row < own; row += nth >> 5) {
             // the inverse's row from global memory (L2-resident)
             const double2 s = dense_row(a.inv[z] + (size_t)(g0 + row) * npc, a.inve[z][g0 + row], gath, eg, npc, lane);
-            if (lane == 0) x[row] = cconv<V>(s);
+            if (lane == 0) x[at(L, row / L.n1, row % L.n1)] = cconv<V>(s);
         }
     };
     auto zero_vec = [&](int k, unsigned off) {
-        V* x = vec(off);
-        for (int lt = tid; lt < nown(a.lv[k]); lt += nth) x[lt] = czero<V>();
+        const int cnt = a.lv[k].rp * (a.lv[k].n1 + 2 * G);
+        for (int t = tid; t < cnt; t += nth) vec(off)[t] = czero<V>();
     };
     auto copy_vec = [&](int k, unsigned from, unsigned to) {
-        const V* s = vec(from);
-        V* d = vec(to);
-        for (int lt = tid; lt < nown(a.lv[k]); lt += nth) d[lt] = s[lt];
+        const int cnt = a.lv[k].rp * (a.lv[k].n1 + 2 * G);
+        for (int t = tid; t < cnt; t += nth) vec(to)[t] = vec(from)[t];
     };
 
     // ---- the cycle: an explicit walk over the recursion of Algorithm 1 ----
@@ -403,9 +426,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
         }
         if (op < 0) continue;
         switch (op) {
-        case kJacobi: jacobi(kk, u, v, zero); break;
+        case kJacobi:
+        case kResidual:
+            if (zero) jacobi_zero(kk, v);
+            else stencil_phase(kk, u, v, op == kResidual);
+            break;
         case kZero: zero_vec(kk, u); break;
-        case kResidual: residual(kk, u, v); break;
         case kRestrict: restrict_(kk, u); break;
         case kCoarse: coarse(); break;
         case kProlong: prolong(kk, u); break;
@@ -420,7 +446,11 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
         const int own = nown(L), g0 = p0(L);
         const size_t roff = (size_t)rr * L.n1 * L.n2 + g0;
         const V* x = vec(L.off_x);
-        for (int t = tid; t < own; t += nth) a.gx[z][roff + t] = x[t];
+        for (int t = tid; t < own; t += nth) {
+            int r, i;
+            own_rc(L, t, r, i);
+            ((V*)a.gx[z])[roff + t] = x[at(L, r, i)];
+        }
     }
     cluster_barrier();
 }
@@ -428,12 +458,14 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-static const void* smmg_fn(int rm) {
-    return rm <= 1 ? (const void*)k_cluster_mg<1> : (const void*)k_cluster_mg<2>;
+template <int MODE> static const void* smmg_fn(int rm) {
+    return rm <= 1 ? (const void*)k_cluster_mg<MODE, 1> : (const void*)k_cluster_mg<MODE, 2>;
 }
 
-size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs) {
-    size_t off = 0;
+size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs, int mode, int rm) {
+    const size_t vb = mode == BAH_MIXED ? sizeof(float2) : sizeof(double2);
+    const size_t cb = mode == BAH_MIXED ? sizeof(__nv_bfloat162) : sizeof(double2);
+    size_t off = 0, halo = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
         off += (bytes + 15) & ~size_t(15);
@@ -447,26 +479,29 @@ size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max
         L.rp = (n2[k] + cs - 1) / cs;
         L.inv_rp = 1.0f / (float)L.rp;
         L.inv_n1 = 1.0f / (float)L.n1;
-        const size_t cap = (size_t)L.rp * L.n1;
+        L.inv_p = 1.0f / (float)(L.n1 + 2 * rm);
+        const size_t cap = (size_t)L.rp * L.n1, padded = (size_t)L.rp * (L.n1 + 2 * rm);
         if (k < nlev - 1) {
-            L.off_c = take(cap * nslot_max[k] * 4);
-            L.off_t = take(cap * 8);
+            L.off_c = take(cap * nslot_max[k] * cb);
+            L.off_t = take(padded * vb);
+            halo = std::max(halo, (size_t)2 * rm * (L.n1 + 2 * rm) * vb);
         } else {
             L.off_c = 0;
             L.off_t = 0;
         }
-        L.off_x = take(cap * 8);
-        L.off_b = take(cap * 8);
+        L.off_x = take(padded * vb);
+        L.off_b = take(cap * vb);
     }
+    // the sweeps' halo rows and the coarsest solve's right-hand side are never in use together
     const SmLevel& Lc = a.lv[nlev - 1];
     const size_t npc = (size_t)Lc.n1 * Lc.n2;
-    a.off_g = take(npc * 16);
+    a.off_g = take(std::max(npc * 16, halo));
     a.off_r = take(32 * 4);
     return off;
 }
 
-int smmg_prepare(int rm, int cs, size_t smem) {
-    const void* fn = smmg_fn(rm);
+int smmg_prepare(int rm, int cs, size_t smem, int mode) {
+    const void* fn = mode == BAH_MIXED ? smmg_fn<BAH_MIXED>(rm) : smmg_fn<BAH_FP64>(rm);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         (cs > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         cudaGetLastError();
@@ -491,7 +526,7 @@ int smmg_prepare(int rm, int cs, size_t smem) {
     return n;
 }
 
-int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, cudaStream_t st) {
+int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, int mode, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs * a.nb * nrhs);
     cfg.blockDim = dim3(kSmThreads);
@@ -506,7 +541,9 @@ int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, cu
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = rm <= 1 ? cudaLaunchKernelEx(&cfg, k_cluster_mg<1>, a) : cudaLaunchKernelEx(&cfg, k_cluster_mg<2>, a);
+    auto fn = mode == BAH_MIXED ? (rm <= 1 ? k_cluster_mg<BAH_MIXED, 1> : k_cluster_mg<BAH_MIXED, 2>)
+                                : (rm <= 1 ? k_cluster_mg<BAH_FP64, 1> : k_cluster_mg<BAH_FP64, 2>);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a);
     return e == cudaSuccess ? 0 : (int)e;
 }
 

@@ -338,10 +338,10 @@ struct MG {
     }
 
     // levels sm_l0..L-1 held in one cluster's shared memory per block and
-    // right-hand side (mixed mode): right-hand sides in vB[sm_l0], results in
+    // right-hand side: right-hand sides in vB[sm_l0], results in
     // vX[sm_l0]; warm: start from the values in vX[sm_l0]
     static void smem_levels(Ctx& c, int b0, int nb, const Batch& bt, cudaStream_t st, bool warm = false) {
-        if constexpr (MODE == BAH_MIXED) {
+        {
             SmArgs a;
             std::memset(&a, 0, sizeof(a));
             const int l0 = c.sm_l0, nlev = c.L - l0;
@@ -352,27 +352,27 @@ struct MG {
                 for (int b = 0; b < 3; ++b)
                     ns[k] = std::max(ns[k], (2 * c.s64[l0 + k][b].rx + 1) * (2 * c.s64[l0 + k][b].rz + 1));
             }
-            smmg_layout(a, n1s, n2s, ns, nlev, c.sm_cs);
-            for (int k = 0; k < nlev; ++k) a.lv[k].w = (float)weight(c, l0 + k);
+            smmg_layout(a, n1s, n2s, ns, nlev, c.sm_cs, MODE, c.sm_rm);
+            for (int k = 0; k < nlev; ++k) a.lv[k].w = weight(c, l0 + k);
             a.b0 = b0; a.nb = nb; a.nu_pre = c.o.nu_pre; a.nu_post = c.o.nu_post; a.intergrid = c.o.intergrid;
             a.wcycle = c.o.cycle == BAH_CYCLE_W; a.warm = warm; a.active = bt.active;
             for (int z = 0; z < nb; ++z) {
                 const int b = b0 + z;
                 for (int k = 0; k < nlev - 1; ++k) {
-                    a.S[z][k] = (const __nv_bfloat162*)c.sst[l0 + k][b];
+                    a.S[z][k] = c.sst[l0 + k][b];
                     a.rx[z][k] = c.s64[l0 + k][b].rx; a.rz[z][k] = c.s64[l0 + k][b].rz;
                 }
-                a.gb[z] = (const float2*)c.vB[l0][b];
-                a.gx[z] = (float2*)c.vX[l0][b];
+                a.gb[z] = c.vB[l0][b];
+                a.gx[z] = c.vX[l0][b];
                 a.inv[z] = c.inv[b];
                 a.inve[z] = c.inve[b];
             }
             double bytes = 0;
             for (int k = 0; k < nlev - 1; ++k) bytes += coef_bytes(c, l0 + k, b0, nb) * bt.nr;
             const double npc = (double)c.ln1[c.L - 1] * c.ln2[c.L - 1];
-            bytes += nb * bt.nr * (npc * npc * 16.0 + (double)c.ln1[l0] * c.ln2[l0] * 8.0 * (warm ? 3 : 2));
+            bytes += nb * bt.nr * (npc * npc * 16.0 + (double)c.ln1[l0] * c.ln2[l0] * sizeof(V) * (warm ? 3 : 2));
             Prof pr(c, BAH_K_CLUSTER, st, bytes);
-            launch_cluster_mg(a, c.sm_rm, bt.nr, c.sm_cs, c.sm_bytes, st);
+            launch_cluster_mg(a, c.sm_rm, bt.nr, c.sm_cs, c.sm_bytes, MODE, st);
         }
     }
 
@@ -1037,9 +1037,9 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
             for (int cs = 16; cs >= 8 && c.sm_l0 == 0; cs /= 2) {
                 SmArgs a;
                 std::memset(&a, 0, sizeof(a));
-                const size_t bytes = smmg_layout(a, n1s, n2s, ns, nlev, cs);
+                const size_t bytes = smmg_layout(a, n1s, n2s, ns, nlev, cs, c.mode, rm);
                 if (bytes > (size_t)optin) continue;
-                if (smmg_prepare(rm, cs, bytes) >= 1) {
+                if (smmg_prepare(rm, cs, bytes, c.mode) >= 1) {
                     c.sm_l0 = l0; c.sm_cs = cs; c.sm_rm = rm; c.sm_bytes = bytes;
                 }
             }
