@@ -223,6 +223,7 @@ template <class C, class CC> struct Fine5 {
 template <class V, class CC> struct LvlBlk {
     int type;
     const CC* S;       // stencil [(2rz+1)(2rx+1)][n1*n2] (levels >= 1)
+    const CC* idg;     // inverse diagonal (FP64 mode)
     int rx, rz;
     const V* b;        // right-hand side
     const V* xin;      // current iterate
@@ -330,6 +331,17 @@ void launch_restrict(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::C
 template <int MODE>
 void launch_prolong_add(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fine,
                         const typename Prec<MODE>::V* const* coarse_x, cudaStream_t st, size_t coarse_stride = 0);
+// fused level-0 visits (k_fine.cu); in FP64 f5's diagonals are their inverses
+int fine_prepare();     // once per context, before the first launch
+template <int MODE>
+void launch_fine_down(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
+                      const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f5, double w,
+                      typename Prec<MODE>::V* const* coarse_b, int intergrid, size_t coarse_stride, cudaStream_t st);
+template <int MODE>
+void launch_fine_up(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
+                    const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f5, double w, int sweeps, bool from_b,
+                    const typename Prec<MODE>::V* const* coarse_x, size_t coarse_stride, cudaStream_t st);
+void launch_inverse_diag(const double2* x, double2* y, size_t n, cudaStream_t st);
 int coarse_prepare();   // once per context, before the first launch
 // x = A_c^{-1} b, the inverse as limbs and row exponents (launch_inverse_limbs)
 template <int MODE>

@@ -24,11 +24,15 @@ static inline int max_radius(const LS& s) {
     return r;
 }
 
+// threads per CTA: in FP64 one warp instruction takes 16 clocks of the SM's pipe,
+// so small CTAs spread a small level over more SMs
+template <int MODE> constexpr int kTpb = MODE == BAH_FP64 ? 64 : 256;
+
 // ---------------------------------------------------------------------------
 // damped Jacobi:  x_out = x_in + w D^{-1} (b - A x_in)   (zero_init: w D^{-1} b)
 // ---------------------------------------------------------------------------
 template <int MODE, bool L0, int RM>
-__global__ void __launch_bounds__(256) k_jacobi(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> s,
+__global__ void __launch_bounds__(kTpb<MODE>) k_jacobi(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> s,
                                                 Fine5<typename MGT<MODE>::C, typename MGT<MODE>::CC> f5,
                                                 typename MGT<MODE>::R w, int zero_init) {
     pdl_prologue();
@@ -43,6 +47,10 @@ __global__ void __launch_bounds__(256) k_jacobi(LvlSet<typename MGT<MODE>::V, ty
     if (!valid_pt(B.type, i, j)) { xout[t] = czero<V>(); return; }
     const V b = B.b[rr * B.sb + t];
     if (zero_init) {
+        if constexpr (MODE == BAH_FP64) {
+            xout[t] = cscale(cmul(B.idg[t], b), w);
+            return;
+        }
         const V dg = diag_only<MODE>(L0 ? &f5 : nullptr, B, np, t);
         xout[t] = cscale(cdiv(b, dg), w);
         return;
@@ -62,7 +70,7 @@ __global__ void __launch_bounds__(256) k_jacobi(LvlSet<typename MGT<MODE>::V, ty
 // residual:  r = b - A x
 // ---------------------------------------------------------------------------
 template <int MODE, bool L0, int RM>
-__global__ void __launch_bounds__(256) k_residual(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> s,
+__global__ void __launch_bounds__(kTpb<MODE>) k_residual(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> s,
                                                   Fine5<typename MGT<MODE>::C, typename MGT<MODE>::CC> f5) {
     pdl_prologue();
     using V = typename MGT<MODE>::V;
@@ -80,6 +88,73 @@ __global__ void __launch_bounds__(256) k_residual(LvlSet<typename MGT<MODE>::V, 
     if (L0) ax = apply_fine5_fn<MODE>(f5, B.type, i, j, t, X);
     else ax = apply_stencil_fn<MODE, RM>(B.S, B.rx, B.rz, n1, n2, i, j, t, X);
     xout[t] = csub(B.b[rr * B.sb + t], ax);
+}
+
+// ---------------------------------------------------------------------------
+// FP64 sweeps and residuals.  The FP64 pipe (2 operations per clock and SM)
+// bounds them, so the diagonal is inverted once at setup, the sweep is written
+// x_out = (1 - w) x + w D^{-1} (b - (A - D) x), radii are compile-time and a tap
+// outside the grid has its coefficient replaced by 0: 14 operations per point on
+// level 0 and 4 per tap + 8 above, where dividing and masking took 46 and
+// 6 per tap + 44 (with all 25 taps for the 15 of a displacement block).
+// 20 FP64 steps at 512 x 512: 27.8 -> 15.8 ms.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(64) k_sweep64_fine(LvlSet<double2, double2> s, Fine5<double, double2> f5, double w) {
+    pdl_prologue();
+    const auto& B = s.blk[blockIdx.y];
+    const int n1 = s.n1, n2 = s.n2;
+    const int t = blockIdx.x * 64 + threadIdx.x, rr = blockIdx.z;
+    if (t >= n1 * n2 || (s.active && !s.active[rr])) return;
+    double2* __restrict__ xout = B.xout + rr * B.sxo;
+    const int i = t % n1, j = t / n1;
+    if (!valid_pt(B.type, i, j)) { xout[t] = make_double2(0.0, 0.0); return; }
+    const double2* __restrict__ x = B.xin + rr * B.sxi;
+    const double2 r = csub_off_fine5(f5, B.type, i, j, t, B.b[rr * B.sb + t], [&](int g) { return x[g]; });
+    double2 v = cscale(x[t], 1.0 - w);
+    cfma(v, cscale(B.idg[t], w), r);
+    xout[t] = v;
+}
+
+template <int RX, int RZ, bool RES>
+__device__ __forceinline__ void galerkin64(const LvlSet<double2, double2>& s, const LvlBlk<double2, double2>& B, double w,
+                                           int t, int rr) {
+    const int n1 = s.n1, n2 = s.n2, np = n1 * n2;
+    const int i = t % n1, j = t / n1;
+    double2* __restrict__ xout = B.xout + rr * B.sxo;
+    if (!valid_pt(B.type, i, j)) { xout[t] = make_double2(0.0, 0.0); return; }
+    const double2* __restrict__ x = B.xin + rr * B.sxi;
+    // all loads first: at one to four points per SM the kernel is a chain of their latencies
+    constexpr int WX = 2 * RX + 1, NT = WX * (2 * RZ + 1);
+    double2 c[NT], xv[NT];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        const int dz = u / WX - RZ, dx = u % WX - RX;
+        const bool in = i + dx >= 0 && i + dx < n1 && j + dz >= 0 && j + dz < n2;
+        c[u] = B.S[(size_t)u * np + t];
+        xv[u] = x[in ? t + dz * n1 + dx : t];
+        if (!in) c[u] = make_double2(0.0, 0.0);
+    }
+    const double2 xc = xv[NT / 2];
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int u = 0; u < NT; ++u)
+        if (RES || u != NT / 2) cfma(acc, c[u], xv[u]);
+    const double2 r = csub(B.b[rr * B.sb + t], acc);
+    if (RES) { xout[t] = r; return; }
+    double2 v = cscale(xc, 1.0 - w);
+    cfma(v, cscale(B.idg[t], w), r);
+    xout[t] = v;
+}
+template <bool RES>
+__global__ void __launch_bounds__(64) k_galerkin64(LvlSet<double2, double2> s, double w) {
+    pdl_prologue();
+    const auto& B = s.blk[blockIdx.y];
+    const int t = blockIdx.x * 64 + threadIdx.x, rr = blockIdx.z;
+    if (t >= s.n1 * s.n2 || (s.active && !s.active[rr])) return;
+    if (B.rx == 2 && B.rz == 2) galerkin64<2, 2, RES>(s, B, w, t, rr);
+    else if (B.rx == 2) galerkin64<2, 1, RES>(s, B, w, t, rr);
+    else if (B.rz == 2) galerkin64<1, 2, RES>(s, B, w, t, rr);
+    else galerkin64<1, 1, RES>(s, B, w, t, rr);
 }
 
 // ---------------------------------------------------------------------------
@@ -171,32 +246,43 @@ template <int MODE>
 void launch_jacobi(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
                    const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>* f5, double w, int zero_init,
                    cudaStream_t st) {
-    const int np = s.n1 * s.n2;
-    dim3 g((np + 255) / 256, s.nb, s.nrhs);
+    const int np = s.n1 * s.n2, tpb = kTpb<MODE>;
+    dim3 g((np + tpb - 1) / tpb, s.nb, s.nrhs);
     using R = typename Prec<MODE>::R;
     const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC> nof{};
-    const int rm = f5 ? 1 : max_radius(s);
-    const size_t sm = (f5 || zero_init) ? 0 : staged_smem<MODE>(s, rm);
-    if (f5) launch_pdl(k_jacobi<MODE, true, 1>, dim3(g), dim3(256), 0, st, s, *f5, (R)w, zero_init);
-    else if (sm && rm <= 1) launch_pdl(k_stencil_staged<MODE, 1, false>, dim3(g), dim3(256), sm, st, s, (R)w);
-    else if (sm) launch_pdl(k_stencil_staged<MODE, 2, false>, dim3(g), dim3(256), sm, st, s, (R)w);
-    else if (rm <= 1) launch_pdl(k_jacobi<MODE, false, 1>, dim3(g), dim3(256), 0, st, s, nof, (R)w, zero_init);
-    else launch_pdl(k_jacobi<MODE, false, 2>, dim3(g), dim3(256), 0, st, s, nof, (R)w, zero_init);
+    if constexpr (MODE == BAH_FP64) {
+        if (zero_init) launch_pdl(k_jacobi<MODE, false, 1>, dim3(g), dim3(tpb), 0, st, s, nof, w, 1);
+        else if (f5) launch_pdl(k_sweep64_fine, dim3(g), dim3(tpb), 0, st, s, *f5, w);
+        else launch_pdl(k_galerkin64<false>, dim3(g), dim3(tpb), 0, st, s, w);
+    } else {
+        const int rm = f5 ? 1 : max_radius(s);
+        const size_t sm = (f5 || zero_init) ? 0 : staged_smem<MODE>(s, rm);
+        if (f5) launch_pdl(k_jacobi<MODE, true, 1>, dim3(g), dim3(tpb), 0, st, s, *f5, (R)w, zero_init);
+        else if (sm && rm <= 1) launch_pdl(k_stencil_staged<MODE, 1, false>, dim3(g), dim3(256), sm, st, s, (R)w);
+        else if (sm) launch_pdl(k_stencil_staged<MODE, 2, false>, dim3(g), dim3(256), sm, st, s, (R)w);
+        else if (rm <= 1) launch_pdl(k_jacobi<MODE, false, 1>, dim3(g), dim3(tpb), 0, st, s, nof, (R)w, zero_init);
+        else launch_pdl(k_jacobi<MODE, false, 2>, dim3(g), dim3(tpb), 0, st, s, nof, (R)w, zero_init);
+    }
 }
 template <int MODE>
 void launch_residual(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
                      const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>* f5, cudaStream_t st) {
-    const int np = s.n1 * s.n2;
-    dim3 g((np + 255) / 256, s.nb, s.nrhs);
+    const int np = s.n1 * s.n2, tpb = kTpb<MODE>;
+    dim3 g((np + tpb - 1) / tpb, s.nb, s.nrhs);
     const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC> nof{};
     using R = typename Prec<MODE>::R;
-    const int rm = f5 ? 1 : max_radius(s);
-    const size_t sm = f5 ? 0 : staged_smem<MODE>(s, rm);
-    if (f5) launch_pdl(k_residual<MODE, true, 1>, dim3(g), dim3(256), 0, st, s, *f5);
-    else if (sm && rm <= 1) launch_pdl(k_stencil_staged<MODE, 1, true>, dim3(g), dim3(256), sm, st, s, (R)0);
-    else if (sm) launch_pdl(k_stencil_staged<MODE, 2, true>, dim3(g), dim3(256), sm, st, s, (R)0);
-    else if (rm <= 1) launch_pdl(k_residual<MODE, false, 1>, dim3(g), dim3(256), 0, st, s, nof);
-    else launch_pdl(k_residual<MODE, false, 2>, dim3(g), dim3(256), 0, st, s, nof);
+    if constexpr (MODE == BAH_FP64) {
+        if (f5) launch_pdl(k_residual<MODE, true, 1>, dim3(g), dim3(tpb), 0, st, s, *f5);
+        else launch_pdl(k_galerkin64<true>, dim3(g), dim3(tpb), 0, st, s, 0.0);
+    } else {
+        const int rm = f5 ? 1 : max_radius(s);
+        const size_t sm = f5 ? 0 : staged_smem<MODE>(s, rm);
+        if (f5) launch_pdl(k_residual<MODE, true, 1>, dim3(g), dim3(tpb), 0, st, s, *f5);
+        else if (sm && rm <= 1) launch_pdl(k_stencil_staged<MODE, 1, true>, dim3(g), dim3(256), sm, st, s, (R)0);
+        else if (sm) launch_pdl(k_stencil_staged<MODE, 2, true>, dim3(g), dim3(256), sm, st, s, (R)0);
+        else if (rm <= 1) launch_pdl(k_residual<MODE, false, 1>, dim3(g), dim3(tpb), 0, st, s, nof);
+        else launch_pdl(k_residual<MODE, false, 2>, dim3(g), dim3(tpb), 0, st, s, nof);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -206,7 +292,7 @@ void launch_residual(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::C
 // support of a 1-D restriction row for coarse index c: first fine index
 
 template <int MODE>
-__global__ void __launch_bounds__(256) k_restrict(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> fine,
+__global__ void __launch_bounds__(kTpb<MODE>) k_restrict(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> fine,
                                                   PtrSet<typename MGT<MODE>::V> cb, int intergrid) {
     pdl_prologue();
     using V = typename MGT<MODE>::V;
@@ -255,15 +341,16 @@ void launch_restrict(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::C
     for (int z = 0; z < 3; ++z) cb.p[z] = z < fine.nb ? coarse_b[z] : nullptr;
     cb.s = coarse_stride;
     const int npc = (fine.n1 / 2) * (fine.n2 / 2);
-    dim3 g((npc + 255) / 256, fine.nb, fine.nrhs);
-    launch_pdl(k_restrict<MODE>, dim3(g), dim3(256), 0, st, fine, cb, intergrid);
+    const int tpb = kTpb<MODE>;
+    dim3 g((npc + tpb - 1) / tpb, fine.nb, fine.nrhs);
+    launch_pdl(k_restrict<MODE>, dim3(g), dim3(tpb), 0, st, fine, cb, intergrid);
 }
 
 // ---------------------------------------------------------------------------
 // prolongation and correction: x_f += P e_c  (x_f = blk.xout of the fine set)
 // ---------------------------------------------------------------------------
 template <int MODE>
-__global__ void __launch_bounds__(256) k_prolong_add(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> fine,
+__global__ void __launch_bounds__(kTpb<MODE>) k_prolong_add(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> fine,
                                                      PtrSet<typename MGT<MODE>::V> ce) {
     pdl_prologue();
     using V = typename MGT<MODE>::V;
@@ -278,28 +365,23 @@ __global__ void __launch_bounds__(256) k_prolong_add(LvlSet<typename MGT<MODE>::
     const bool nodx = B.type == 0, nodz = B.type == 1;
     const V* e = pick(ce, (int)blockIdx.y) + rr * ce.s;
     V* xo = B.xout + rr * B.sxo;
-    R px[3], pz[3];
+    int cx[2], cz[2];
+    R wx[2], wz[2];
+    pw_pair<R>(nodx, n1, i, cx, wx);
+    pw_pair<R>(nodz, n2, j, cz, wz);
+    V v[4];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        px[q] = pw_axis_t<R>(nodx, n1, i, (i >> 1) - 1 + q);
-        pz[q] = pw_axis_t<R>(nodz, n2, j, (j >> 1) - 1 + q);
-    }
-    V v[9];
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const bool ok = pz[a] != R(0) && px[q] != R(0);
-            v[a * 3 + q] = e[ok ? ((j >> 1) - 1 + a) * n1c + ((i >> 1) - 1 + q) : 0];
-        }
+        for (int q = 0; q < 2; ++q) v[a * 2 + q] = e[cz[a] * n1c + cx[q]];
     V acc = xo[t];
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const R wgt = pz[a] * px[q];
-            acc.x += wgt * v[a * 3 + q].x;
-            acc.y += wgt * v[a * 3 + q].y;
+        for (int q = 0; q < 2; ++q) {
+            const R wgt = wz[a] * wx[q];
+            acc.x += wgt * v[a * 2 + q].x;
+            acc.y += wgt * v[a * 2 + q].y;
         }
     xo[t] = acc;
 }
@@ -311,8 +393,9 @@ void launch_prolong_add(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>
     for (int z = 0; z < 3; ++z) ce.p[z] = z < fine.nb ? const_cast<typename Prec<MODE>::V*>(coarse_x[z]) : nullptr;
     ce.s = coarse_stride;
     const int np = fine.n1 * fine.n2;
-    dim3 g((np + 255) / 256, fine.nb, fine.nrhs);
-    launch_pdl(k_prolong_add<MODE>, dim3(g), dim3(256), 0, st, fine, ce);
+    const int tpb = kTpb<MODE>;
+    dim3 g((np + tpb - 1) / tpb, fine.nb, fine.nrhs);
+    launch_pdl(k_prolong_add<MODE>, dim3(g), dim3(tpb), 0, st, fine, ce);
 }
 
 // ---------------------------------------------------------------------------

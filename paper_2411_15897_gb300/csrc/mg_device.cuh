@@ -81,6 +81,29 @@ __device__ __forceinline__ typename MGT<MODE>::V apply_fine5_fn(const Fine5<type
     return apply_fine5_rel<MODE>(f, type, i, j, t, [&](int dx, int dz) { return X(t + dz * n1 + dx); });
 }
 
+// b + sum of k x_neighbour = b - (A - D) x of a level-0 block in FP64 (neighbours
+// that do not exist enter with k = 0)
+template <class XF>
+__device__ __forceinline__ double2 csub_off_fine5(const Fine5<double, double2>& f, int type, int i, int j, int t, double2 b,
+                                                  XF X) {
+    const int n1 = f.n1, n2 = f.n2;
+    const bool w = type == 0 ? i >= 2 : i >= 1, e = i + 1 < n1, s = type == 1 ? j >= 2 : j >= 1, n = j + 1 < n2;
+    const double* ax = type == 0 ? f.cx : (type == 1 ? f.nx : f.wx);
+    const double* az = type == 0 ? f.nz : (type == 1 ? f.cz : f.wz);
+    auto add = [&](bool ok, int ci, const double* a, int xi) {
+        const double k = a[ok ? ci : t];
+        const double2 v = X(ok ? xi : t);
+        const double kk = ok ? k : 0.0;
+        b.x = fma(kk, v.x, b.x);
+        b.y = fma(kk, v.y, b.y);
+    };
+    add(w, type == 1 ? t : t - 1, ax, t - 1);
+    add(e, type == 0 ? t : t + 1, ax, t + 1);
+    add(s, type == 0 ? t : t - n1, az, t - n1);
+    add(n, type == 1 ? t : t + n1, az, t + n1);
+    return b;
+}
+
 // Galerkin stencil product at point (i, j) of a level >= 1: coefficients
 // through an accessor S(slot), x through XR(dx, dz).  RM is the compile-time
 // maximum radius (1 or 2); rx, rz <= RM are the block's radii.  The loops

@@ -57,6 +57,7 @@ struct Ctx {
     // level-0 arrays in storage precision
     void *s_cx = nullptr, *s_cz = nullptr, *s_nx = nullptr, *s_nz = nullptr, *s_wx = nullptr, *s_wz = nullptr;
     void *s_dg[3] = {nullptr, nullptr, nullptr}, *s_dAp = nullptr;
+    std::vector<std::array<double2*, 3>> idg;        // FP64 mode: inverse diagonals per level
     // hierarchy
     std::vector<int> ln1, ln2;
     std::vector<std::array<StencilF64, 3>> s64;   // FP64 stencils per level (level 0: 3x3 fine operator)
@@ -314,6 +315,7 @@ struct MG {
             auto& B = s.blk[z];
             B.type = b;
             B.S = l > 0 ? (const CC*)c.sst[l][b] : nullptr;
+            if constexpr (MODE == BAH_FP64) B.idg = c.idg[l][b];
             B.rx = c.s64[l][b].rx; B.rz = c.s64[l][b].rz;
             B.b = (const V*)c.vB[l][b];
             B.sb = npl;
@@ -417,12 +419,41 @@ struct MG {
         V* cx[3];
         for (int z = 0; z < nb; ++z) { cb[z] = (V*)c.vB[l + 1][b0 + z]; cx[z] = (V*)c.vX[l + 1][b0 + z]; }
         const bool wcyc = c.o.cycle == BAH_CYCLE_W;
+        auto coarse_visits = [&]() {
+            if (c.sm_l0 == l + 1) {
+                smem_levels(c, b0, nb, bt, st);
+                if (wcyc && l + 1 < c.L - 1) smem_levels(c, b0, nb, bt, st, true);
+            } else {
+                cycle(c, l + 1, b0, nb, cx, nplc, bt, st);
+                if (wcyc && l + 1 < c.L - 1) cycle(c, l + 1, b0, nb, cx, nplc, bt, st, true);
+            }
+        };
+        // fused level-0 launches: prolongation with up to three post-sweeps, and with one
+        // pre-sweep (level 0 is always entered with a zero guess) the way down
+        // (in FP64 the halo's recomputation costs more than the launches it saves unless the
+        // CTAs fit the SMs in one wave: the FP64 pipe bounds both forms)
+        const bool one_wave = (c.n1 / 58 + 1) * (c.n2 / 26 + 1) * nb * bt.nr <= 152;
+        const bool fused_up = l == 0 && c.o.nu_post >= 1 && c.o.nu_post <= 3 && (MODE == BAH_MIXED || one_wave);
+        Fine5<C, CC> fi = f5;
+        if constexpr (MODE == BAH_FP64) { fi.dg0 = c.idg[0][0]; fi.dg1 = c.idg[0][1]; fi.dg2 = c.idg[0][2]; }
+        if (fused_up && c.o.nu_pre == 1) {
+            {
+                Prof pr(c, BAH_K_RESIDUAL, st, cb_ + nr * nb * npl * vs * 1.25);
+                launch_fine_down<MODE>(set(c, l, b0, nb, nullptr, 0, cur, cur_s, bt), fi, w, cb, c.o.intergrid, nplc, st);
+            }
+            coarse_visits();
+            {
+                Prof pr(c, BAH_K_JACOBI, st, cb_ + nr * nb * npl * vs * 2.25);
+                launch_fine_up<MODE>(set(c, l, b0, nb, nullptr, 0, cur, cur_s, bt), fi, w, c.o.nu_post, true, cx, nplc, st);
+            }
+            return;
+        }
         {
             // With a zero initial guess the caller's buffer holds nothing yet: if the
             // sweeps below swap the two buffers an odd number of times, start in the
             // other one, so that the last sweep lands in the caller's buffer and no
             // copy is needed.
-            if (!x0 && ((std::max(c.o.nu_pre - 1, 0) + c.o.nu_post) & 1)) swap_cur();
+            if (!x0 && ((std::max(c.o.nu_pre - 1, 0) + (fused_up ? 1 : c.o.nu_post)) & 1)) swap_cur();
             // pre-relaxation
             if (x0) {
                 for (int s = 0; s < c.o.nu_pre; ++s) {
@@ -456,22 +487,22 @@ struct MG {
                 launch_restrict<MODE>(rs, cb, c.o.intergrid, st, nplc);
             }
             // coarse-grid correction
-            if (c.sm_l0 == l + 1) {
-                smem_levels(c, b0, nb, bt, st);
-                if (wcyc && l + 1 < c.L - 1) smem_levels(c, b0, nb, bt, st, true);
-            } else {
-                cycle(c, l + 1, b0, nb, cx, nplc, bt, st);
-                if (wcyc && l + 1 < c.L - 1) cycle(c, l + 1, b0, nb, cx, nplc, bt, st, true);
-            }
-            {
-                Prof pr(c, BAH_K_PROLONG, st, nr * nb * npl * vs * 2.25);
-                launch_prolong_add<MODE>(set(c, l, b0, nb, nullptr, 0, cur, cur_s, bt), cx, st, nplc);
-            }
-            // post-relaxation
-            for (int s = 0; s < c.o.nu_post; ++s) {
-                Prof pr(c, BAH_K_JACOBI, st, sweep);
-                launch_jacobi<MODE>(set(c, l, b0, nb, cur, cur_s, oth, oth_s, bt), pf5, w, 0, st);
+            coarse_visits();
+            if (fused_up) {
+                Prof pr(c, BAH_K_JACOBI, st, sweep + nr * nb * npl * vs * 0.25);
+                launch_fine_up<MODE>(set(c, l, b0, nb, cur, cur_s, oth, oth_s, bt), fi, w, c.o.nu_post, false, cx, nplc, st);
                 swap_cur();
+            } else {
+                {
+                    Prof pr(c, BAH_K_PROLONG, st, nr * nb * npl * vs * 2.25);
+                    launch_prolong_add<MODE>(set(c, l, b0, nb, nullptr, 0, cur, cur_s, bt), cx, st, nplc);
+                }
+                // post-relaxation
+                for (int s = 0; s < c.o.nu_post; ++s) {
+                    Prof pr(c, BAH_K_JACOBI, st, sweep);
+                    launch_jacobi<MODE>(set(c, l, b0, nb, cur, cur_s, oth, oth_s, bt), pf5, w, 0, st);
+                    swap_cur();
+                }
             }
         }
         for (int z = 0; z < nb; ++z)
@@ -954,6 +985,14 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     TRY(c.alloc(&c.s_dAp, np * ccs));
     launch_round_cplx(c.dAp, c.s_dAp, np, c.mode, st);
 
+    TRY(fine_prepare());
+    c.idg.assign(c.L, {nullptr, nullptr, nullptr});
+    if (c.mode == BAH_FP64)
+        for (int b = 0; b < 3; ++b) {
+            TRY(c.alloc_t(&c.idg[0][b], np));
+            launch_inverse_diag(c.dg[b], c.idg[0][b], np, st);
+        }
+
     // hierarchy: level grids, FP64 stencils, Galerkin products, storage copies
     c.ln1.assign(c.L, 0); c.ln2.assign(c.L, 0);
     c.s64.assign(c.L, {}); c.sst.assign(c.L, {nullptr, nullptr, nullptr});
@@ -975,6 +1014,11 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
             if (l < c.L - 1) {
                 TRY(c.alloc(&c.sst[l][b], ns * ccs));
                 launch_round_cplx(s.S, c.sst[l][b], ns, c.mode, st);
+                if (c.mode == BAH_FP64) {
+                    const size_t npl = (size_t)s.n1 * s.n2;
+                    TRY(c.alloc_t(&c.idg[l][b], npl));
+                    launch_inverse_diag(s.S + (s.rz * (2 * s.rx + 1) + s.rx) * npl, c.idg[l][b], npl, st);
+                }
             }
         }
     }
