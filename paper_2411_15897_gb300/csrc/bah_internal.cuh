@@ -236,7 +236,7 @@ template <class V, class CC> struct LvlSet {
     LvlBlk<V, CC> blk[3];
     int nrhs;          // right-hand sides in the launch (blockIdx.z)
     const int* active; // per right-hand side, or nullptr
-    int staged;        // Galerkin-level sweeps may stage their inputs in shared memory
+    int staged;        // mixed mode: Galerkin levels by k_galerkin.cu (0: the plain kernels)
 };
 
 constexpr int kMaxLevels = 16;
@@ -331,6 +331,10 @@ void launch_restrict(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::C
 template <int MODE>
 void launch_prolong_add(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fine,
                         const typename Prec<MODE>::V* const* coarse_x, cudaStream_t st, size_t coarse_stride = 0);
+// sweep or residual on a Galerkin level (k_galerkin.cu)
+template <int MODE>
+void launch_galerkin_level(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s, double w, bool residual,
+                           cudaStream_t st);
 // fused level-0 visits (k_fine.cu); in FP64 f5's diagonals are their inverses
 int fine_prepare();     // once per context, before the first launch
 template <int MODE>
