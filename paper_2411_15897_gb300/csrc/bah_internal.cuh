@@ -475,11 +475,29 @@ void launch_urhs3(const Op3& op, const double2* r, const V* ep, V* const* su, cu
 // the level kernels run blocks type0 .. type0 + nq - 1 (nq <= 3) of one level in
 // one launch, block y on the y-th pointer of each array
 template <class V>
-// S: stencil entries, FP64 complex (V = double2) or bfloat16 complex (V = float2)
-void launch_jacobi3(int type0, int nq, const int* n, int ns, const void* const* S, const V* const* b,
-                    const V* const* xin, V* const* xout, double w, int zero, int res, cudaStream_t st);
+void launch_zero3(int type0, int nq, const int* n, const V* const* idg, const V* const* b, V* const* xout, double w,
+                  cudaStream_t st);
+// S: 27-point entries, FP64 complex (V = double2) or bfloat16 complex (V = float2); idg: inverse diagonals
 template <class V>
-void launch_restrict3(int type0, int nq, const int* nf, const V* const* r, V* const* bc, cudaStream_t st);
+void launch_level27(int type0, int nq, const int* n, const void* const* S, const V* const* idg, const V* const* b,
+                    const V* const* xin, V* const* xout, double w, bool res, cudaStream_t st);
+// the level-0 operators of the four blocks from per-point coefficients: cmu, cme as in Op3,
+// wv[a] = (lambda + 2 mu) / (lambda + mu) / h_a^2, the shifted diagonals and their inverses
+template <class C, class CC, class V> struct Fine3 {
+    int n[3];
+    const C *cmu[3], *cme[3][3], *wv[3];
+    const CC* dg[4];
+    const V* idg[4];
+};
+template <class V, class C, class SC>
+void launch_fine3(const Fine3<C, SC, V>& f, int type0, int nq, const V* const* b, const V* const* xin, V* const* xout, double w,
+                  bool res, bool from_b, cudaStream_t st);
+void launch_inverse3(const void* x, void* y, size_t n, int mode, cudaStream_t st);
+void launch_wp3(const double* mu, const double* cinv, double* w, size_t n, cudaStream_t st);
+// idg, x: with x[y] != nullptr also the coarse level's first sweep from zero
+template <class V>
+void launch_restrict3(int type0, int nq, const int* nf, const V* const* r, V* const* bc, const V* const* idg, V* const* x,
+                      double w, cudaStream_t st);
 template <class V>
 void launch_prolong3(int type0, int nq, const int* nf, const V* const* ec, V* const* x, cudaStream_t st);
 void launch_galerkin3(int type, const int* nf, int nsf, const double2* Sf, double2* Sc, int* err, cudaStream_t st);

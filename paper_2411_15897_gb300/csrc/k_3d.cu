@@ -350,94 +350,282 @@ template void launch_urhs3<float2>(const Op3&, const double2*, const float2*, fl
 // multigrid level kernels.  Stencils are stored entry-major: entry s of
 // point p at S[s * points + p].
 // ---------------------------------------------------------------------------
-// one damped Jacobi sweep x_out = x_in + w D^{-1} (b - A x_in) (zero: x_in = 0),
-// or the residual x_out = b - A x_in (res), for up to three blocks of one
-// level in one launch: blockIdx.y = y runs block type type0 + y on the y-th
-// pointers.  Stencil entries are stored as SC: FP64 complex, or bfloat16
-// complex in mixed mode, where every entry and neighbour of a point is loaded
-// before the first multiply-add.
-template <class V, class SC, int NS>
-__global__ void __launch_bounds__(256) k_jacobi3(int type0, int n1, int n2, int n3, Set3<const SC> Sset,
-                                                 Set3<const V> bset, Set3<const V> xiset, Set3<V> xoset,
-                                                 typename VecTraits<V>::R w, int zero, int res) {
-    pdl_prologue();
-    const int y = blockIdx.y, type = type0 + y;
-    const SC* __restrict__ S = pick(Sset, y);
-    const V* __restrict__ b = pick(bset, y);
-    const V* xin = pick(xiset, y);
-    V* xout = pick(xoset, y);
-    const int np = n1 * n2 * n3;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    int c[3];
-    coords3(p, n1, n2, c);
-    if (!valid3(type, c)) { xout[p] = czero<V>(); return; }
-    const int n[3] = {n1, n2, n3};
-    const int st[3] = {1, n1, n1 * n2};
-    V acc = b[p];
-    if (!zero) {
-        constexpr bool kBatch = sizeof(SC) <= 4;          // bf16 entries: all loads first
-        SC sv[kBatch ? NS : 1];
-        V xv[kBatch ? NS : 1];
-        bool inn[kBatch ? NS : 1];
-#pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            int o[3];
-            soff<NS>(s, o);
-            bool in = true;
-            int q = p;
-            for (int a = 0; a < 3; ++a) {
-                const int cc = c[a] + o[a];
-                if (cc < 0 || cc >= n[a]) in = false;
-                q += o[a] * st[a];
-            }
-            if constexpr (kBatch) {
-                inn[s] = in;
-                sv[s] = S[(size_t)s * np + p];
-                xv[s] = xin[in ? q : p];
-            } else {
-                if (in) acc = csub(acc, cmul(ldc(S[(size_t)s * np + p]), xin[q]));
-            }
-        }
-        if constexpr (kBatch) {
-#pragma unroll
-            for (int s = 0; s < NS; ++s)
-                if (inn[s]) acc = csub(acc, cmul(ldc(sv[s]), xv[s]));
-        }
-    }
-    if (res) { xout[p] = acc; return; }
-    const V upd = cscale(cdiv(acc, ldc(S[(size_t)scentre<NS>() * np + p])), w);
-    xout[p] = zero ? upd : cadd(xin[p], upd);
-}
-
+// A launch runs up to three blocks of one level: blockIdx.y = y runs block type
+// type0 + y on the y-th pointers.  Sweeps are written
+// x_out = (1 - w) x + w D^{-1} (b - (A - D) x) with D^{-1} formed at setup (a complex
+// reciprocal is some 40 instructions, in FP64 mode 10 of them on a pipe of two
+// operations per clock and SM).
 template <class T>
 static Set3<T> set3(T* const* v, int nq) {
     Set3<T> s;
     for (int y = 0; y < 3; ++y) s.p[y] = y < nq ? v[y] : nullptr;
     return s;
 }
+// loads issued here, wherever their results are used; stencil entries (constant) through the non-coherent path
+__device__ __forceinline__ double2 ld_now3(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ldv_now3(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ldv_now3(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned ld_now3(const __nv_bfloat162* p) {
+    unsigned v;
+    asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 entry3(double2 v) { return v; }
+__device__ __forceinline__ float2 entry3(unsigned v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
+// base[i] through a 32-bit byte offset (i < 2^28: a vector of one block is below 4 GB)
+template <class T> __device__ __forceinline__ T at3(const T* base, unsigned i) {
+    return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + (size_t)(i * (unsigned)sizeof(T)));
+}
+
+// first sweep from zero: x = w D^{-1} b (any level; below the first, k_restrict3 writes it)
+template <class V>
+__global__ void __launch_bounds__(128) k_zero3(int type0, int n1, int n2, int n3, Set3<const V> idgset, Set3<const V> bset,
+                                               Set3<V> xoset, typename VecTraits<V>::R w) {
+    pdl_prologue();
+    const int y = blockIdx.y, np = n1 * n2 * n3, p = blockIdx.x * 128 + threadIdx.x;
+    if (p >= np) return;
+    int c[3];
+    coords3(p, n1, n2, c);
+    pick(xoset, y)[p] = valid3(type0 + y, c) ? cmul(cscale(pick(idgset, y)[p], w), pick(bset, y)[p]) : czero<V>();
+}
+
+// Sweep or residual on a 27-point level.  The small levels of a W-cycle, visited most
+// often, are bound by the chain of memory latencies: every load is issued before the
+// first multiply-add, and CTAs are small, so that 16^3 points spread over 64 SMs
+// (16^3 points, mixed mode: 9.4 us with 256-thread CTAs and the loads left to the
+// compiler, 3.7 us).  Entries that would couple to a point outside the grid are zero
+// (the Galerkin product clamps at the ends), so such a neighbour's load is redirected
+// to the point itself and needs no test.
+constexpr int kT27 = 64;
+template <class V, class SC, bool RES>
+__global__ void __launch_bounds__(kT27) k_level27(int type0, int n1, int n2, int n3, Set3<const SC> Sset, Set3<const V> idgset,
+                                                  Set3<const V> bset, Set3<const V> xiset, Set3<V> xoset,
+                                                  typename VecTraits<V>::R w) {
+    pdl_prologue();
+    const int y = blockIdx.y, type = type0 + y;
+    const int np = n1 * n2 * n3;
+    const int p = blockIdx.x * kT27 + threadIdx.x;
+    if (p >= np) return;
+    const SC* S = pick(Sset, y) + p;
+    const V* xin = pick(xiset, y);
+    int c[3];
+    coords3(p, n1, n2, c);
+    if (!valid3(type, c)) { pick(xoset, y)[p] = czero<V>(); return; }
+    const int dx[3] = {c[0] >= 1 ? -1 : 0, 0, c[0] + 1 < n1 ? 1 : 0};
+    const int dy[3] = {c[1] >= 1 ? -n1 : 0, 0, c[1] + 1 < n2 ? n1 : 0};
+    const int dz[3] = {c[2] >= 1 ? -n1 * n2 : 0, 0, c[2] + 1 < n3 ? n1 * n2 : 0};
+    decltype(ld_now3(S)) raw[27];
+    V xv[27];
+#pragma unroll
+    for (int s = 0; s < 27; ++s) {
+        if (RES || s != 13) raw[s] = ld_now3(S);
+        S += np;
+        xv[s] = ldv_now3(reinterpret_cast<const V*>(reinterpret_cast<const char*>(xin) +
+                                                    (size_t)((unsigned)(p + dx[s % 3] + dy[s / 3 % 3] + dz[s / 9]) * (unsigned)sizeof(V))));
+    }
+    const V b = pick(bset, y)[p];
+    V g = b;
+    if (!RES) g = pick(idgset, y)[p];
+    V acc = czero<V>();
+#pragma unroll
+    for (int s = 0; s < 27; ++s)
+        if (RES || s != 13) cfma(acc, entry3(raw[s]), xv[s]);
+    V v = csub(b, acc);
+    if (!RES) {
+        const V d = v;
+        v = cscale(xv[13], 1 - w);
+        cfma(v, cscale(g, w), d);
+    }
+    pick(xoset, y)[p] = v;
+}
+
+// Level 0, the 7-point operators from per-point coefficients (mu at cells and edges
+// over h^2, (lambda + 2 mu) / (lambda + mu) over h^2): 6 to 10 bytes per point in
+// mixed mode where seven stored complex entries take 28, with the same values.
+// FROMB: the input iterate is the first sweep from zero, x = w D^{-1} b, formed here.
+// A thread takes kZ3 points of one column: the block type is a compile-time constant
+// of its loop, the column's tests and clamped offsets are formed once, and values and
+// coefficients along axis 2 pass from plane to plane in registers.  With a thread per
+// point of the flattened grid the kernel was bound by its 280 instructions per point
+// (three blocks of 128^3, mixed mode: 64 us a sweep, 100 us with FROMB; now 40 and 48,
+// against 79 us from the stored 7-point entries).
+constexpr int kZ3 = 4;
+template <class V, class C, class SC, bool RES, bool FROMB, int TYPE>
+__device__ __forceinline__ void fine3_column(const Fine3<C, SC, V>& f, const V* b, const V* xin, V* xout,
+                                             typename VecTraits<V>::R w, int cx, int cy, int z0) {
+    using R = typename VecTraits<V>::R;
+    const int n1 = f.n[0], n2 = f.n[1], n3 = f.n[2];
+    const unsigned pl = (unsigned)(n1 * n2);
+    unsigned p = (unsigned)((z0 * n2 + cy) * n1 + cx);
+    const int nz = min(kZ3, n3 - z0);
+    V out[kZ3];
+    if ((TYPE == 0 && cx == 0) || (TYPE == 1 && cy == 0)) {
+        for (int k = 0; k < nz; ++k) xout[p + k * pl] = czero<V>();
+        return;
+    }
+    const V* __restrict__ idg = f.idg[TYPE];
+    auto X = [&](unsigned q) {
+        if constexpr (FROMB) return cmul(cscale(at3(idg, q), w), at3(b, q));
+        else return at3(xin, q);
+    };
+    auto add = [](V& acc, R k, const V& v) {
+        acc.x = fma(k, v.x, acc.x);
+        acc.y = fma(k, v.y, acc.y);
+    };
+    const int cc[2] = {cx, cy};
+    const unsigned st[2] = {1u, (unsigned)n1};
+    bool lo[2], hi[2];
+    unsigned ql[2], qh[2];                       // offsets of the neighbours in the plane, zero where there is none
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        lo[a] = cc[a] >= (a == TYPE ? 2 : 1);
+        hi[a] = cc[a] + 1 < f.n[a];
+        ql[a] = lo[a] ? 0u - st[a] : 0u;
+        qh[a] = hi[a] ? st[a] : 0u;
+    }
+    constexpr int e2 = TYPE < 2 ? 1 - TYPE : 0;
+    const C* __restrict__ kz = TYPE == 3 ? f.wv[2] : (TYPE == 2 ? f.cmu[2] : f.cme[e2][2]);
+    // neighbours below and at the point along axis 2 and the couplings to the lower one and (TYPE 3) of the point
+    V xm = z0 >= (TYPE == 2 ? 2 : 1) ? X(p - pl) : czero<V>();
+    V xc = TYPE == 2 && z0 == 0 ? czero<V>() : X(p);
+    R kl = TYPE < 2 ? ldr(at3(kz, p)) : (z0 >= 1 ? ldr(at3(kz, p - pl)) : R(0));
+    R kc = TYPE == 3 ? ldr(at3(kz, p)) : R(0);
+#pragma unroll
+    for (int k = 0; k < kZ3; ++k) {
+        if (k >= nz) break;
+        const int z = z0 + k;
+        const bool up = z + 1 < n3;
+        const unsigned pu = up ? p + pl : p;
+        const V xu = up ? X(pu) : czero<V>();
+        const R kh = TYPE == 2 ? ldr(at3(kz, p)) : (up ? ldr(at3(kz, pu)) : R(0));
+        V acc = at3(b, p);
+        add(acc, kl, xm);
+        add(acc, kh, xu);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int e = TYPE == 3 || a == TYPE ? 0 : 3 - TYPE - a;
+            const C* __restrict__ ka = TYPE == 3 ? f.wv[a] : (a == TYPE ? f.cmu[a] : f.cme[e][a]);
+            const bool below = TYPE == 3 || a == TYPE;                   // the lower coupling is the lower point's coefficient
+            const R vl = ldr(at3(ka, below ? p + ql[a] : p)), vh = ldr(at3(ka, a == TYPE ? p : p + qh[a]));
+            add(acc, lo[a] ? vl : R(0), X(p + ql[a]));
+            add(acc, hi[a] ? vh : R(0), X(p + qh[a]));
+        }
+        // acc = b - (A - D) x
+        if constexpr (RES) {
+            out[k] = csub(acc, cmul(ldc(at3(f.dg[TYPE], p)), xc));
+        } else {
+            out[k] = cscale(xc, 1 - w);
+            cfma(out[k], cscale(at3(idg, p), w), acc);
+        }
+        if (TYPE == 2 && z == 0) out[k] = czero<V>();
+        xm = xc;
+        xc = xu;
+        kl = TYPE == 3 ? kc : kh;
+        kc = kh;
+        p += pl;
+    }
+    // stored after the last load: the loads of all planes can be in flight together
+    p = (unsigned)((z0 * n2 + cy) * n1 + cx);
+#pragma unroll
+    for (int k = 0; k < kZ3; ++k)
+        if (k < nz) xout[p + k * pl] = out[k];
+}
+template <class V, class C, class SC, bool RES, bool FROMB>
+__global__ void __launch_bounds__(256, sizeof(V) == 16 ? 3 : 5) k_fine3(int type0, int tx, Fine3<C, SC, V> f, Set3<const V> bset, Set3<const V> xiset,
+                                               Set3<V> xoset, typename VecTraits<V>::R w) {
+    pdl_prologue();
+    const int y = blockIdx.y;
+    const int ty = blockIdx.x / tx;
+    const int cx = (blockIdx.x - ty * tx) * blockDim.x + threadIdx.x, cy = ty * blockDim.y + threadIdx.y;
+    if (cx >= f.n[0] || cy >= f.n[1]) return;
+    const V *b = pick(bset, y), *xin = pick(xiset, y);
+    V* xout = pick(xoset, y);
+    const int z0 = blockIdx.z * kZ3;
+    switch (type0 + y) {
+        case 0: return fine3_column<V, C, SC, RES, FROMB, 0>(f, b, xin, xout, w, cx, cy, z0);
+        case 1: return fine3_column<V, C, SC, RES, FROMB, 1>(f, b, xin, xout, w, cx, cy, z0);
+        case 2: return fine3_column<V, C, SC, RES, FROMB, 2>(f, b, xin, xout, w, cx, cy, z0);
+        default: return fine3_column<V, C, SC, RES, FROMB, 3>(f, b, xin, xout, w, cx, cy, z0);
+    }
+}
 
 template <class V>
-void launch_jacobi3(int type0, int nq, const int* n, int ns, const void* const* S, const V* const* b,
-                    const V* const* xin, V* const* xout, double w, int zero, int res, cudaStream_t st) {
+void launch_zero3(int type0, int nq, const int* n, const V* const* idg, const V* const* b, V* const* xout, double w,
+                  cudaStream_t st) {
     const int np = n[0] * n[1] * n[2];
-    using R = typename VecTraits<V>::R;
+    launch_pdl(k_zero3<V>, dim3((np + 127) / 128, nq), dim3(128), 0, st, type0, n[0], n[1], n[2], set3<const V>(idg, nq),
+               set3<const V>(b, nq), set3<V>(xout, nq), (typename VecTraits<V>::R)w);
+}
+template <class V>
+void launch_level27(int type0, int nq, const int* n, const void* const* S, const V* const* idg, const V* const* b,
+                    const V* const* xin, V* const* xout, double w, bool res, cudaStream_t st) {
     using SC = typename std::conditional<std::is_same<V, double2>::value, double2, __nv_bfloat162>::type;
+    const int np = n[0] * n[1] * n[2];
     const SC* s[3];
     for (int y = 0; y < nq; ++y) s[y] = (const SC*)S[y];
-    const Set3<const SC> ss = set3<const SC>(s, nq);
-    const dim3 g((np + 255) / 256, nq);
-    if (ns == 7)
-        launch_pdl(k_jacobi3<V, SC, 7>, g, dim3(256), 0, st, type0, n[0], n[1], n[2], ss, set3<const V>(b, nq),
-                   set3<const V>(xin, nq), set3<V>(xout, nq), (R)w, zero, res);
-    else
-        launch_pdl(k_jacobi3<V, SC, 27>, g, dim3(256), 0, st, type0, n[0], n[1], n[2], ss, set3<const V>(b, nq),
-                   set3<const V>(xin, nq), set3<V>(xout, nq), (R)w, zero, res);
+    auto fn = res ? k_level27<V, SC, true> : k_level27<V, SC, false>;
+    launch_pdl(fn, dim3((np + kT27 - 1) / kT27, nq), dim3(kT27), 0, st, type0, n[0], n[1], n[2], set3<const SC>(s, nq),
+               set3<const V>(idg, nq), set3<const V>(b, nq), set3<const V>(xin, nq), set3<V>(xout, nq),
+               (typename VecTraits<V>::R)w);
 }
-template void launch_jacobi3<double2>(int, int, const int*, int, const void* const*, const double2* const*,
-                                      const double2* const*, double2* const*, double, int, int, cudaStream_t);
-template void launch_jacobi3<float2>(int, int, const int*, int, const void* const*, const float2* const*,
-                                     const float2* const*, float2* const*, double, int, int, cudaStream_t);
+template <class V, class C, class SC>
+void launch_fine3(const Fine3<C, SC, V>& f, int type0, int nq, const V* const* b, const V* const* xin, V* const* xout, double w,
+                  bool res, bool from_b, cudaStream_t st) {
+    auto fn = res ? k_fine3<V, C, SC, true, false> : k_fine3<V, C, SC, false, false>;
+    if constexpr (std::is_same<V, float2>::value)
+        if (from_b) fn = k_fine3<V, C, SC, false, true>;
+    // 32 x 8 columns, or 16 x 16 where that leaves fewer threads without a column
+    auto up = [](int n, int b) { return (n + b - 1) / b; };
+    const int bx = up(f.n[0], 16) * up(f.n[1], 16) < up(f.n[0], 32) * up(f.n[1], 8) ? 16 : 32, by = 256 / bx;
+    const int tx = up(f.n[0], bx);
+    launch_pdl(fn, dim3(tx * up(f.n[1], by), nq, up(f.n[2], kZ3)), dim3(bx, by), 0, st, type0, tx, f, set3<const V>(b, nq),
+               set3<const V>(xin, nq), set3<V>(xout, nq), (typename VecTraits<V>::R)w);
+}
+#define INST3(V, C, SC)                                                                                                   \
+    template void launch_zero3<V>(int, int, const int*, const V* const*, const V* const*, V* const*, double,              \
+                                  cudaStream_t);                                                                          \
+    template void launch_level27<V>(int, int, const int*, const void* const*, const V* const*, const V* const*,           \
+                                    const V* const*, V* const*, double, bool, cudaStream_t);                              \
+    template void launch_fine3<V, C, SC>(const Fine3<C, SC, V>&, int, int, const V* const*, const V* const*, V* const*,   \
+                                         double, bool, bool, cudaStream_t);
+INST3(double2, double, double2)
+INST3(float2, __nv_bfloat16, __nv_bfloat162)
+#undef INST3
+
+// 1 / x of the stored diagonals, in FP64, rounded to the cycle's type
+template <class V, class SC>
+__global__ void k_inverse3(const SC* __restrict__ x, V* __restrict__ y, size_t n) {
+    const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const auto d = ldc(x[e]);
+    y[e] = cconv<V>(cdiv(make_double2(1.0, 0.0), make_double2(d.x, d.y)));
+}
+void launch_inverse3(const void* x, void* y, size_t n, int mode, cudaStream_t st) {
+    const unsigned g = (unsigned)((n + 255) / 256);
+    if (mode == BAH_MIXED) k_inverse3<float2, __nv_bfloat162><<<g, 256, 0, st>>>((const __nv_bfloat162*)x, (float2*)y, n);
+    else k_inverse3<double2, double2><<<g, 256, 0, st>>>((const double2*)x, (double2*)y, n);
+}
+
+// (lambda + 2 mu) / (lambda + mu) at cells
+__global__ void k_wp3(const double* __restrict__ mu, const double* __restrict__ cinv, double* __restrict__ w, size_t n) {
+    const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (e < n) w[e] = 1.0 + mu[e] * cinv[e];
+}
+void launch_wp3(const double* mu, const double* cinv, double* w, size_t n, cudaStream_t st) {
+    k_wp3<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(mu, cinv, w, n);
+}
 
 // 1-D transfer weights.  Restriction (Eq. 4.1 / 4.4, mixed intergrid): along
 // the block's nodal axis 1/4 [1 2 1] around fine face 2K; along a cell-centred
@@ -474,139 +662,149 @@ __host__ __device__ __forceinline__ int plist3(bool nodal, int m, int nc, int* K
     return 2;
 }
 
-// the transfer weights of one axis as a fixed number of (index, weight)
-// pairs, unused pairs with weight 0 at an in-range index, so that the
-// kernels below keep them in registers: restriction, three fine indices;
-// prolongation, two coarse indices (the same weights as rlist3 / plist3)
-template <class R>
-__device__ __forceinline__ void raxis3(bool nodal, int J, int* f, R* w) {
-    if (nodal) {
-        f[0] = 2 * J - 1; w[0] = R(0.25);
-        f[1] = 2 * J;     w[1] = R(0.5);
-        f[2] = 2 * J + 1; w[2] = R(0.25);
-    } else {
-        f[0] = 2 * J;     w[0] = R(0.5);
-        f[1] = 2 * J + 1; w[1] = R(0.5);
-        f[2] = 2 * J;     w[2] = R(0);
-    }
+// The transfers run with the block type as a compile-time constant, so that every tap
+// is an unconditional load: 12 of a coarse point (8 on the pressure block), 12 of a
+// pair of fine points along axis 0.  With run-time lists of up to 27 and 8 predicated
+// taps, three blocks of 128^3 took 18.8 us down and 58 us up, now 12 and 27; the fine
+// array's bandwidth would allow 7 and 15.
+constexpr int kTr3 = 128;
+// b_c = R r on the coarse grid (fine grid f, coarse f / 2); with x, also the coarse
+// level's first sweep from zero, x = w D^{-1} b_c
+template <class V, int TYPE>
+__device__ __forceinline__ V restrict3_point(const V* r, int f1, int f2, const int* J) {
+    using R = typename VecTraits<V>::R;
+    V acc = czero<V>();
+#pragma unroll
+    for (int z = 0; z < (TYPE == 2 ? 3 : 2); ++z)
+#pragma unroll
+        for (int y = 0; y < (TYPE == 1 ? 3 : 2); ++y)
+#pragma unroll
+            for (int x = 0; x < (TYPE == 0 ? 3 : 2); ++x) {
+                // nodal axis: 1/4, 1/2, 1/4 at 2J - 1, 2J, 2J + 1; the others 1/2 at 2J, 2J + 1
+                const int tap = TYPE == 0 ? x : (TYPE == 1 ? y : z);
+                const R ww = TYPE == 3 ? R(0.125) : (tap == 1 ? R(0.125) : R(0.0625));
+                const int fx = 2 * J[0] + x - (TYPE == 0), fy = 2 * J[1] + y - (TYPE == 1), fz = 2 * J[2] + z - (TYPE == 2);
+                const V v = at3(r, (unsigned)((fz * f2 + fy) * f1 + fx));
+                acc.x = fma(ww, v.x, acc.x);
+                acc.y = fma(ww, v.y, acc.y);
+            }
+    return acc;
 }
-template <class R>
-__device__ __forceinline__ void paxis3(bool nodal, int m, int nc, int* K, R* w) {
-    if (nodal) {
-        if ((m & 1) == 0) {
-            K[0] = m >> 1; w[0] = (K[0] >= 1 && K[0] <= nc - 1) ? R(1) : R(0);
-            K[1] = K[0];   w[1] = R(0);
-        } else {
-            K[0] = (m - 1) >> 1; w[0] = K[0] >= 1 ? R(0.5) : R(0);
-            K[1] = (m + 1) >> 1; w[1] = K[1] <= nc - 1 ? R(0.5) : R(0);
-        }
-        K[0] = min(K[0], nc - 1);
-        K[1] = min(K[1], nc - 1);
-        return;
-    }
-    const int J = m >> 1;
-    int Jn = (m & 1) ? J + 1 : J - 1;
-    if (Jn < 0 || Jn > nc - 1) Jn = J;
-    K[0] = J;  w[0] = R(0.75);
-    K[1] = Jn; w[1] = R(0.25);
-}
-
-// b_c = R r on the coarse grid (fine grid n, coarse n/2), accumulated in the
-// cycle's arithmetic (FP32 in mixed mode; the weights 1/2 and 1/4 and their
-// products are exact there)
 template <class V>
-__global__ void __launch_bounds__(256) k_restrict3(int type0, int f1, int f2, int f3, Set3<const V> rset,
-                                                   Set3<V> bcset) {
+__global__ void __launch_bounds__(kTr3) k_restrict3(int type0, int f1, int f2, int f3, Set3<const V> rset, Set3<V> bcset,
+                                                    Set3<const V> idgset, Set3<V> xset, typename VecTraits<V>::R w) {
     pdl_prologue();
     const int type = type0 + (int)blockIdx.y;
-    const V* __restrict__ r = pick(rset, (int)blockIdx.y);
-    V* __restrict__ bc = pick(bcset, (int)blockIdx.y);
+    const V* r = pick(rset, (int)blockIdx.y);
+    V* x = pick(xset, (int)blockIdx.y);
     const int c1 = f1 / 2, c2 = f2 / 2, c3 = f3 / 2;
-    const int npc = c1 * c2 * c3;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= npc) return;
+    const int p = blockIdx.x * kTr3 + threadIdx.x;
+    if (p >= c1 * c2 * c3) return;
     int J[3];
     coords3(p, c1, c2, J);
-    if (!valid3(type, J)) { bc[p] = czero<V>(); return; }
-    using R = typename VecTraits<V>::R;
-    int fx[3], fy[3], fz[3];
-    R wx[3], wy[3], wz[3];
-    raxis3<R>(type == 0, J[0], fx, wx);
-    raxis3<R>(type == 1, J[1], fy, wy);
-    raxis3<R>(type == 2, J[2], fz, wz);
-    V acc = czero<V>();
-#pragma unroll
-    for (int z = 0; z < 3; ++z)
-#pragma unroll
-        for (int y = 0; y < 3; ++y) {
-            const R wzy = wz[z] * wy[y];
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                const R ww = wzy * wx[x];
-                if (ww != R(0)) {
-                    const V v = r[((size_t)fz[z] * f2 + fy[y]) * f1 + fx[x]];
-                    acc.x += ww * v.x;
-                    acc.y += ww * v.y;
-                }
-            }
+    V acc = czero<V>(), x1 = czero<V>();
+    if (valid3(type, J)) {
+        V g = acc;
+        if (x) g = pick(idgset, (int)blockIdx.y)[p];
+        switch (type) {
+            case 0: acc = restrict3_point<V, 0>(r, f1, f2, J); break;
+            case 1: acc = restrict3_point<V, 1>(r, f1, f2, J); break;
+            case 2: acc = restrict3_point<V, 2>(r, f1, f2, J); break;
+            default: acc = restrict3_point<V, 3>(r, f1, f2, J);
         }
-    bc[p] = acc;
+        x1 = cmul(cscale(g, w), acc);
+    }
+    pick(bcset, (int)blockIdx.y)[p] = acc;
+    if (x) x[p] = x1;
 }
 
-// x += P e_c on the fine grid
-template <class V>
-__global__ void __launch_bounds__(256) k_prolong3(int type0, int f1, int f2, int f3, Set3<const V> ecset,
-                                                  Set3<V> xset) {
-    pdl_prologue();
-    const int type = type0 + (int)blockIdx.y;
-    const V* __restrict__ ec = pick(ecset, (int)blockIdx.y);
-    V* __restrict__ x = pick(xset, (int)blockIdx.y);
-    const int c1 = f1 / 2, c2 = f2 / 2, c3 = f3 / 2;
-    const int np = f1 * f2 * f3;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    int F[3];
-    coords3(p, f1, f2, F);
-    if (!valid3(type, F)) return;
+// taps of fine index m along one axis: two coarse indices, an unused one with weight 0 at an in-range index
+template <class R, bool NODAL>
+__device__ __forceinline__ void paxis3(int m, int nc, int* K, R* w) {
+    const int J = m >> 1, odd = m & 1;
+    if (NODAL) {                                 // even: J; odd: the mean of J and J + 1 (coarse index 0 is no unknown)
+        K[0] = J;                  w[0] = J >= 1 ? (odd ? R(0.5) : R(1)) : R(0);
+        K[1] = min(J + odd, nc - 1); w[1] = odd && J + 1 < nc ? R(0.5) : R(0);
+    } else {                                     // 3/4 of the own cell, 1/4 of the nearer neighbour (constant beyond the ends)
+        K[0] = J;                                        w[0] = R(0.75);
+        K[1] = odd ? min(J + 1, nc - 1) : max(J - 1, 0); w[1] = R(0.25);
+    }
+}
+// x += P e_c at the fine points 2J, 2J + 1 of a row
+template <class V, int TYPE>
+__device__ __forceinline__ void prolong3_pair(const V* ec, V* x, int f1, int f2, int c1, int c2, int c3, int J, int fy, int fz) {
     using R = typename VecTraits<V>::R;
-    int kx[2], ky[2], kz[2];
-    R wx[2], wy[2], wz[2];
-    paxis3<R>(type == 0, F[0], c1, kx, wx);
-    paxis3<R>(type == 1, F[1], c2, ky, wy);
-    paxis3<R>(type == 2, F[2], c3, kz, wz);
-    V acc = czero<V>();
+    if ((TYPE == 1 && fy == 0) || (TYPE == 2 && fz == 0)) return;
+    int ky[2], kz[2];
+    R wy[2], wz[2];
+    paxis3<R, TYPE == 1>(fy, c2, ky, wy);
+    paxis3<R, TYPE == 2>(fz, c3, kz, wz);
+    constexpr int NX = TYPE == 0 ? 2 : 3;
+    const int kx[3] = {TYPE == 0 ? J : max(J - 1, 0), TYPE == 0 ? min(J + 1, c1 - 1) : J, min(J + 1, c1 - 1)};
+    V t[NX];
+#pragma unroll
+    for (int k = 0; k < NX; ++k) t[k] = czero<V>();
+    V* xr = x + (fz * f2 + fy) * f1 + 2 * J;
+    V x0 = xr[0], x1 = xr[1];
 #pragma unroll
     for (int z = 0; z < 2; ++z)
 #pragma unroll
         for (int y = 0; y < 2; ++y) {
-            const R wzy = wz[z] * wy[y];
+            const R ww = wz[z] * wy[y];
+            const unsigned row = (unsigned)((kz[z] * c2 + ky[y]) * c1);
 #pragma unroll
-            for (int xx = 0; xx < 2; ++xx) {
-                const R ww = wzy * wx[xx];
-                if (ww != R(0)) {
-                    const V v = ec[((size_t)kz[z] * c2 + ky[y]) * c1 + kx[xx]];
-                    acc.x += ww * v.x;
-                    acc.y += ww * v.y;
-                }
+            for (int k = 0; k < NX; ++k) {
+                const V v = at3(ec, row + kx[k]);
+                t[k].x = fma(ww, v.x, t[k].x);
+                t[k].y = fma(ww, v.y, t[k].y);
             }
         }
-    x[p] = cadd(x[p], acc);
+    if constexpr (TYPE == 0) {
+        const R we = J >= 1 ? R(1) : R(0), w0 = J >= 1 ? R(0.5) : R(0), w1 = J + 1 < c1 ? R(0.5) : R(0);
+        x0 = cmk<V>(fma(we, t[0].x, x0.x), fma(we, t[0].y, x0.y));
+        x1 = cmk<V>(x1.x + fma(w0, t[0].x, w1 * t[1].x), x1.y + fma(w0, t[0].y, w1 * t[1].y));
+    } else {
+        x0 = cmk<V>(x0.x + fma(R(0.75), t[1].x, R(0.25) * t[0].x), x0.y + fma(R(0.75), t[1].y, R(0.25) * t[0].y));
+        x1 = cmk<V>(x1.x + fma(R(0.75), t[1].x, R(0.25) * t[2].x), x1.y + fma(R(0.75), t[1].y, R(0.25) * t[2].y));
+    }
+    if (TYPE != 0 || J >= 1) xr[0] = x0;
+    xr[1] = x1;
+}
+template <class V>
+__global__ void __launch_bounds__(kTr3) k_prolong3(int type0, int f1, int f2, int f3, Set3<const V> ecset, Set3<V> xset) {
+    pdl_prologue();
+    const V* ec = pick(ecset, (int)blockIdx.y);
+    V* x = pick(xset, (int)blockIdx.y);
+    const int c1 = f1 / 2, c2 = f2 / 2, c3 = f3 / 2;
+    const int p = blockIdx.x * kTr3 + threadIdx.x;
+    if (p >= c1 * f2 * f3) return;
+    int F[3];
+    coords3(p, c1, f2, F);
+    switch (type0 + (int)blockIdx.y) {
+        case 0: return prolong3_pair<V, 0>(ec, x, f1, f2, c1, c2, c3, F[0], F[1], F[2]);
+        case 1: return prolong3_pair<V, 1>(ec, x, f1, f2, c1, c2, c3, F[0], F[1], F[2]);
+        case 2: return prolong3_pair<V, 2>(ec, x, f1, f2, c1, c2, c3, F[0], F[1], F[2]);
+        default: return prolong3_pair<V, 3>(ec, x, f1, f2, c1, c2, c3, F[0], F[1], F[2]);
+    }
 }
 
 template <class V>
-void launch_restrict3(int type0, int nq, const int* nf, const V* const* r, V* const* bc, cudaStream_t st) {
+void launch_restrict3(int type0, int nq, const int* nf, const V* const* r, V* const* bc, const V* const* idg, V* const* x,
+                      double w, cudaStream_t st) {
     const int npc = (nf[0] / 2) * (nf[1] / 2) * (nf[2] / 2);
-    launch_pdl(k_restrict3<V>, dim3((npc + 255) / 256, nq), dim3(256), 0, st, type0, nf[0], nf[1], nf[2],
-               set3<const V>(r, nq), set3<V>(bc, nq));
+    launch_pdl(k_restrict3<V>, dim3((npc + kTr3 - 1) / kTr3, nq), dim3(kTr3), 0, st, type0, nf[0], nf[1], nf[2],
+               set3<const V>(r, nq), set3<V>(bc, nq), set3<const V>(idg, nq), set3<V>(x, nq), (typename VecTraits<V>::R)w);
 }
 template <class V>
 void launch_prolong3(int type0, int nq, const int* nf, const V* const* ec, V* const* x, cudaStream_t st) {
-    const int np = nf[0] * nf[1] * nf[2];
-    launch_pdl(k_prolong3<V>, dim3((np + 255) / 256, nq), dim3(256), 0, st, type0, nf[0], nf[1], nf[2],
+    const int pairs = (nf[0] / 2) * nf[1] * nf[2];
+    launch_pdl(k_prolong3<V>, dim3((pairs + kTr3 - 1) / kTr3, nq), dim3(kTr3), 0, st, type0, nf[0], nf[1], nf[2],
                set3<const V>(ec, nq), set3<V>(x, nq));
 }
-template void launch_restrict3<double2>(int, int, const int*, const double2* const*, double2* const*, cudaStream_t);
-template void launch_restrict3<float2>(int, int, const int*, const float2* const*, float2* const*, cudaStream_t);
+template void launch_restrict3<double2>(int, int, const int*, const double2* const*, double2* const*, const double2* const*,
+                                       double2* const*, double, cudaStream_t);
+template void launch_restrict3<float2>(int, int, const int*, const float2* const*, float2* const*, const float2* const*,
+                                       float2* const*, double, cudaStream_t);
 template void launch_prolong3<double2>(int, int, const int*, const double2* const*, double2* const*, cudaStream_t);
 template void launch_prolong3<float2>(int, int, const int*, const float2* const*, float2* const*, cudaStream_t);
 

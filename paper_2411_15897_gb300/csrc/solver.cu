@@ -152,6 +152,9 @@ struct Ctx {
     std::vector<std::array<void*, 4>> v3B, v3X, v3T;
     int4* inv3[4] = {nullptr, nullptr, nullptr, nullptr};
     int* inv3e[4] = {nullptr, nullptr, nullptr, nullptr};
+    std::vector<std::array<void*, 4>> idg3;        // inverse diagonals per level, in the cycle's vector type
+    Fine3<double, double2, double2> f3d{};         // level-0 operators, FP64 / mixed mode
+    Fine3<__nv_bfloat16, __nv_bfloat162, float2> f3m{};
 
     static void clear_graph(IterGraph& G) {
         if (G.exec) cudaGraphExecDestroy(G.exec);
@@ -553,27 +556,37 @@ struct MG3 {
     using V = typename Prec<MODE>::V;
     static size_t pts(const Ctx& c, int l) { return (size_t)c.d3[l][0] * c.d3[l][1] * c.d3[l][2]; }
     static double jw(const Ctx& c, int l) { return c.o.jacobi_w[std::min(l, c.o.n_jacobi_w - 1)]; }
-    // for blocks q0 .. q0 + nq - 1 of level l in one launch: x_out = Jacobi sweep
-    // from x_in (zero: from x_in = 0), or x_out = b - A x_in (res)
-    static void sweep(Ctx& c, int l, int q0, int nq, V* const* xin, V* const* xout, int zero, int res,
-                      cudaStream_t st) {
-        const int ns = l == 0 ? 7 : 27;
-        const double vb = sizeof(V);
-        const double sb = MODE == BAH_MIXED ? 4.0 : 16.0;          // bytes per stored stencil entry
-        Prof pr(c, res ? BAH_K_RESIDUAL : BAH_K_JACOBI, st, (double)nq * pts(c, l) * (ns * sb + (zero ? 2.0 : 3.0) * vb));
+    // for blocks q0 .. q0 + nq - 1 of level l in one launch: x_out = Jacobi sweep from x_in
+    // (kZero: from zero; kTwo, level 0: two sweeps from zero), or x_out = b - A x_in (kRes)
+    enum { kSweep, kZero, kTwo, kRes };
+    static void sweep(Ctx& c, int l, int q0, int nq, V* const* xin, V* const* xout, int kind, cudaStream_t st) {
+        const double vb = sizeof(V), cb = sizeof(typename Prec<MODE>::C), db = sizeof(typename Prec<MODE>::CC);
+        // level 0: the inverse diagonal and one (p) or three (u) real coefficients per point
+        const double coef = kind == kZero ? vb : (l == 0 ? vb + (q0 == 3 ? 1 : 3) * cb : 27 * db);
+        Prof pr(c, kind == kRes ? BAH_K_RESIDUAL : BAH_K_JACOBI, st,
+                (double)nq * pts(c, l) * (coef + (kind == kZero || kind == kTwo ? 2.0 : 3.0) * vb));
         const void* S[3];
-        const V* b[3];
-        const V* xi[3];
+        const V *b[3], *xi[3], *id[3];
         for (int y = 0; y < nq; ++y) {
             S[y] = c.s3s[l][q0 + y];
+            id[y] = (const V*)c.idg3[l][q0 + y];
             b[y] = (const V*)c.v3B[l][q0 + y];
             xi[y] = xin[y];
         }
-        launch_jacobi3<V>(q0, nq, c.d3[l].data(), ns, S, b, xi, xout, jw(c, l), zero, res, st);
+        const double w = jw(c, l);
+        if (kind == kZero) return launch_zero3<V>(q0, nq, c.d3[l].data(), id, b, xout, w, st);
+        if (l > 0) return launch_level27<V>(q0, nq, c.d3[l].data(), S, id, b, xi, xout, w, kind == kRes, st);
+        if constexpr (MODE == BAH_MIXED) launch_fine3<V>(c.f3m, q0, nq, b, xi, xout, w, kind == kRes, kind == kTwo, st);
+        else launch_fine3<V>(c.f3d, q0, nq, b, xi, xout, w, kind == kRes, kind == kTwo, st);
     }
     // x_y = approximately A_{q0+y}^{-1} b_{q0+y} on level l for y < nq (b in v3B[l]),
-    // all blocks in the same launches; zero: zero initial guess, else start from x
-    static void cycle(Ctx& c, int l, int q0, int nq, V* const* x, bool zero, cudaStream_t st) {
+    // all blocks in the same launches; kFromX: start from x, kFromZero: from zero,
+    // kSwept: from zero with the first sweep done, by the restriction, in first_sweep()
+    enum { kFromX, kFromZero, kSwept };
+    static V* first_sweep(Ctx& c, int l, int q, V* x) {
+        return (c.o.nu_pre - 1 + c.o.nu_post) % 2 ? (V*)c.v3T[l][q] : x;
+    }
+    static void cycle(Ctx& c, int l, int q0, int nq, V* const* x, int start, cudaStream_t st) {
         const size_t np = pts(c, l);
         if (l == c.L - 1) {
             const double vb = sizeof(V);
@@ -600,39 +613,48 @@ struct MG3 {
         auto cur = [&]() { return inA ? A : B; };
         auto spare = [&]() { return inA ? B : A; };
         int s0 = 0;
-        if (zero) {
-            s0 = c.o.nu_pre >= 1 ? 1 : 0;
+        if (start == kSwept) {
+            s0 = 1;
+            inA = first_sweep(c, l, q0, A[0]) == A[0];
+        } else if (start == kFromZero) {
+            s0 = std::min(c.o.nu_pre, l == 0 && MODE == BAH_MIXED ? 2 : 1);    // sweeps of the first launch
             // start the ping-pong so that the last sweep writes x
             if (((c.o.nu_pre - s0) + c.o.nu_post) % 2) inA = false;
-            if (s0) sweep(c, l, q0, nq, cur(), cur(), 1, 0, st);
+            if (s0) sweep(c, l, q0, nq, cur(), cur(), s0 == 2 ? kTwo : kZero, st);
             else
                 for (int y = 0; y < nq; ++y) cudaMemsetAsync(cur()[y], 0, np * sizeof(V), st);
         }
         for (int s = s0; s < c.o.nu_pre; ++s) {
-            sweep(c, l, q0, nq, cur(), spare(), 0, 0, st);
+            sweep(c, l, q0, nq, cur(), spare(), kSweep, st);
             inA = !inA;
         }
-        sweep(c, l, q0, nq, cur(), spare(), 0, 1, st);
+        sweep(c, l, q0, nq, cur(), spare(), kRes, st);
         V* bc[3] = {nullptr, nullptr, nullptr};
         V* xc[3] = {nullptr, nullptr, nullptr};
+        V* xs[3] = {nullptr, nullptr, nullptr};          // the coarse level's first sweep
+        const V* id[3] = {nullptr, nullptr, nullptr};
+        const bool swept = l + 1 < c.L - 1 && c.o.nu_pre >= 1;
         for (int y = 0; y < nq; ++y) {
             bc[y] = (V*)c.v3B[l + 1][q0 + y];
             xc[y] = (V*)c.v3X[l + 1][q0 + y];
+            if (!swept) continue;
+            xs[y] = first_sweep(c, l + 1, q0 + y, xc[y]);
+            id[y] = (const V*)c.idg3[l + 1][q0 + y];
         }
         {
             Prof pr(c, BAH_K_RESTRICT, st, nq * (double)np * sizeof(V) * 1.125);
             const V* r[3] = {spare()[0], spare()[1], spare()[2]};
-            launch_restrict3<V>(q0, nq, c.d3[l].data(), r, bc, st);
+            launch_restrict3<V>(q0, nq, c.d3[l].data(), r, bc, id, xs, jw(c, l + 1), st);
         }
-        cycle(c, l + 1, q0, nq, xc, true, st);
-        if (c.o.cycle == BAH_CYCLE_W && l + 1 < c.L - 1) cycle(c, l + 1, q0, nq, xc, false, st);
+        cycle(c, l + 1, q0, nq, xc, swept ? kSwept : kFromZero, st);
+        if (c.o.cycle == BAH_CYCLE_W && l + 1 < c.L - 1) cycle(c, l + 1, q0, nq, xc, kFromX, st);
         {
             Prof pr(c, BAH_K_PROLONG, st, nq * (double)np * sizeof(V) * 2.125);
             const V* e[3] = {xc[0], xc[1], xc[2]};
             launch_prolong3<V>(q0, nq, c.d3[l].data(), e, cur(), st);
         }
         for (int s = 0; s < c.o.nu_post; ++s) {
-            sweep(c, l, q0, nq, cur(), spare(), 0, 0, st);
+            sweep(c, l, q0, nq, cur(), spare(), kSweep, st);
             inA = !inA;
         }
         if (!inA)
@@ -649,14 +671,14 @@ struct MG3 {
             launch_distrib3<V>(c.op3, r, (V*)c.v3B[0][3], st);
         }
         V* zp[1] = {z + 3 * np};
-        cycle(c, 0, 3, 1, zp, true, st);
+        cycle(c, 0, 3, 1, zp, kFromZero, st);
         {
             V* su[3] = {(V*)c.v3B[0][0], (V*)c.v3B[0][1], (V*)c.v3B[0][2]};
             Prof pr(c, BAH_K_URHS, st, (double)np * (48.0 + 4.0 * vb));
             launch_urhs3<V>(c.op3, r, z + 3 * np, su, st);
         }
         V* zu[3] = {z, z + np, z + 2 * np};
-        cycle(c, 0, 0, 3, zu, true, st);
+        cycle(c, 0, 0, 3, zu, kFromZero, st);
     }
 };
 
@@ -1194,9 +1216,11 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
             TRY(c.alloc_t(&c.s3[l][q], 27 * pts(l)));
             launch_galerkin3(q, c.d3[l - 1].data(), l == 1 ? 7 : 27, c.s3[l - 1][q], c.s3[l][q], err, st);
         }
+    c.idg3.assign(c.L, {nullptr, nullptr, nullptr, nullptr});
     for (int l = 0; l + 1 < c.L; ++l)
         for (int q = 0; q < 4; ++q) {
-            const size_t cnt = (l == 0 ? 7 : 27) * pts(l);
+            // level 0 keeps the diagonal only: its other entries are the real coefficients below
+            const size_t cnt = (l == 0 ? 1 : 27) * pts(l);
             if (c.mode == BAH_MIXED) {
                 // the mixed cycle's stencils in bfloat16 (entries rounded once from FP64)
                 TRY(c.alloc(&c.s3s[l][q], cnt * sizeof(__nv_bfloat162)));
@@ -1204,7 +1228,48 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
             } else {
                 c.s3s[l][q] = c.s3[l][q];
             }
+            TRY(c.alloc(&c.idg3[l][q], pts(l) * c.vsz));
+            const size_t centre = (l == 0 ? 0 : 13) * pts(l);
+            launch_inverse3((const char*)c.s3s[l][q] + centre * (c.mode == BAH_MIXED ? sizeof(__nv_bfloat162) : sizeof(double2)),
+                            c.idg3[l][q], pts(l), c.mode, st);
         }
+    // level-0 coefficients of the cycle: those of the operator, and the pressure block's
+    {
+        double* w = nullptr;
+        TRY(c.alloc_t(&w, np));
+        launch_wp3(mu, cinv, w, np, st);
+        const double* wv[3] = {nullptr, nullptr, nullptr};
+        for (int a = 0; a < 3; ++a) TRY(scaled(w, a, wv, &wv[a]));
+        auto real = [&](const double* src, const double* const* from, const __nv_bfloat16* const* to, int cnt,
+                        const __nv_bfloat16** dst) {
+            for (int k = 0; k < cnt; ++k)
+                if (from[k] == src && to[k]) { *dst = to[k]; return BAH_OK; }
+            void* d = nullptr;
+            TRY(c.alloc(&d, np * sizeof(__nv_bfloat16)));
+            launch_round_real(src, d, np, BAH_MIXED, st);
+            *dst = (const __nv_bfloat16*)d;
+            return BAH_OK;
+        };
+        for (int a = 0; a < 3; ++a) {
+            c.f3d.n[a] = c.f3m.n[a] = o.n[a];
+            c.f3d.cmu[a] = o.cmu[a];
+            c.f3d.wv[a] = wv[a];
+            for (int e = 0; e < 3; ++e) c.f3d.cme[e][a] = o.cme[e][a];
+        }
+        for (int q = 0; q < 4; ++q) {
+            c.f3d.dg[q] = (const double2*)c.s3s[0][q];
+            c.f3d.idg[q] = (const double2*)c.idg3[0][q];
+            c.f3m.dg[q] = (const __nv_bfloat162*)c.s3s[0][q];
+            c.f3m.idg[q] = (const float2*)c.idg3[0][q];
+        }
+        if (c.mode == BAH_MIXED)
+            for (int a = 0; a < 3; ++a) {
+                TRY(real(c.f3d.cmu[a], c.f3d.cmu, c.f3m.cmu, a, &c.f3m.cmu[a]));
+                TRY(real(c.f3d.wv[a], c.f3d.wv, c.f3m.wv, a, &c.f3m.wv[a]));
+                for (int e = 0; e < 3; ++e)
+                    if (e != a) TRY(real(c.f3d.cme[e][a], c.f3d.cme[e], c.f3m.cme[e], a, &c.f3m.cme[e][a]));
+            }
+    }
     BAH_CUDA_TRY(cudaGetLastError());
     int herr = 0;
     BAH_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -2094,12 +2159,12 @@ int bah_block_cycle(bah_ctx* h, int block, const void* b, void* x, void* stream)
         if (c.mode == BAH_MIXED) {
             launch_convert<double2, float2>((const double2*)b, (float2*)c.v3B[0][block], np, st);
             float2* xx[1] = {(float2*)c.ztmp};
-            MG3<BAH_MIXED>::cycle(c, 0, block, 1, xx, true, st);
+            MG3<BAH_MIXED>::cycle(c, 0, block, 1, xx, MG3<BAH_MIXED>::kFromZero, st);
             launch_convert<float2, double2>((const float2*)c.ztmp, (double2*)x, np, st);
         } else {
             BAH_CUDA_TRY(cudaMemcpyAsync(c.v3B[0][block], b, np * sizeof(double2), cudaMemcpyDeviceToDevice, st));
             double2* xx[1] = {(double2*)x};
-            MG3<BAH_FP64>::cycle(c, 0, block, 1, xx, true, st);
+            MG3<BAH_FP64>::cycle(c, 0, block, 1, xx, MG3<BAH_FP64>::kFromZero, st);
         }
         BAH_CUDA_TRY(cudaGetLastError());
         return BAH_OK;
