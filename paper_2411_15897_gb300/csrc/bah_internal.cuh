@@ -386,16 +386,27 @@ struct KS {                     // per-right-hand-side element strides and activ
 // The FP64 basis in block fixed point (k_gs.cu): vector i's limbs at
 // VL + i * tiles * 256, its tile exponents at VE + i * tiles.
 int gs_prepare();   // once per context, before the first launch
+// One Gram-Schmidt pass: launch_dot_norm, then launch_axpy_norm.  cnt: one counter per
+// right-hand side, zero between launches, with which a kernel's last CTA is found.
+// flag == nullptr in the launches of pass 1; pass 2 runs where the flag is set.
+struct GsNorm {
+    int* cnt;
+    int* flag;      // written by pass 1: 1 (second pass) when ||w'||^2 < eta2 ||w||^2 (DGKS; eta2 = 1/2 classically)
+    double* sc;     // scalars, 8 per right-hand side: [2] = ||w'||, [3] counts second passes
+    double eta2;
+};
 void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, size_t n, double2* partial, double2* out,
-                     const int* flag, int nrhs, const KS& ks, cudaStream_t st);
-// returns the number of partial sums of |w_new|^2 in npart
-int launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
-                     const int* flag, int nrhs, const KS& ks, cudaStream_t st);
+                     const int* flag, int* cnt, int nrhs, const KS& ks, cudaStream_t st);
+int dot_launches(size_t n, int nrhs);   // launches of launch_dot_norm
+// coef: the projections, followed by ||w||^2 (launch_dot_norm's out); npart: scratch, GS_CTAS per right-hand side
+void launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
+                      int pass, const GsNorm& nm, int nrhs, const KS& ks, cudaStream_t st);
 // v = w / sc[slot] as the preconditioner's input (vc, FP64 or rounded to FP32,
-// stride ks.sw) and as a basis vector (vl, ve)
+// stride ks.sw) and as a basis vector (vl, ve); with gv also the step's Givens update
+struct GivensArgs;
 template <class Vc>
 void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, size_t n,
-                        size_t sw, int nrhs, const KS& ks, cudaStream_t st);
+                        size_t sw, int nrhs, const KS& ks, cudaStream_t st, const GivensArgs* gv = nullptr);
 // flag = 1 (second pass) when ||w'||^2 < eta2 ||w||^2 (DGKS criterion; eta2 = 1/2 classically)
 void launch_dgks_decide(const double* npart, int np, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
                         const KS& ks, cudaStream_t st, double eta2 = 0.5);
@@ -409,9 +420,7 @@ void launch_update_x(const Vz* Z, const int* kk, const double2* y, double2* x, s
 void launch_sub(const double2* a, const double2* b, double2* c, size_t n, cudaStream_t st);
 void launch_scale_copy(const double2* w, const double* sc, int slot, double2* v, size_t n, size_t sw, size_t sv,
                        int nrhs, const KS& ks, cudaStream_t st);
-void launch_arnoldi_givens(double2* Hm, int ldh, const double2* h1, const double2* h2, const double* sc, int j,
-                           double2* cs, double2* sn, double2* g, double* status, int nrhs, const KS& ks,
-                           cudaStream_t st);
+void launch_arnoldi_givens(const GivensArgs& a, int nrhs, const KS& ks, cudaStream_t st);
 void launch_triangular_solve(const double2* Hm, int ldh, const double2* g, const int* kk, double2* y, int nrhs,
                              const KS& ks, cudaStream_t st);
 void launch_init_arnoldi(const double* sc, double2* g, int m, double* status, int nrhs, const KS& ks, cudaStream_t st);

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, co
                                                  size_t se, int k, int s, int rpc, const double2* __restrict__ W,
                                                  size_t n, double2* __restrict__ partial) {
     pdl_prologue();
-    extern __shared__ int4 g[];                                   // S x kTile
+    extern __shared__ __align__(128) int4 g[];                                   // S x kTile
     constexpr int CG = S < 8 ? S : 8, NV = 2 * CG;                // columns and values of one lane reduction
     __shared__ int ew[S];
     __shared__ double sum[kBlkRows][2 * S];
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL,
                                                     size_t se, int k, int s, const double2* __restrict__ C,
                                                     double2* __restrict__ W, size_t n) {
     pdl_prologue();
-    extern __shared__ int4 ring[];                                // kUpSlots x kUpG x kUpE
+    extern __shared__ __align__(128) int4 ring[];                                // kUpSlots x kUpG x kUpE
     __shared__ int4 csh[S][32];
     const size_t nt = tiles_of(n), npad = nt * kTile;
     const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
                                                    int4* __restrict__ vl, int* __restrict__ ve, size_t sv, size_t se,
                                                    size_t n) {
     pdl_prologue();
-    extern __shared__ int4 g[];                                   // S x kTile
+    extern __shared__ __align__(128) int4 g[];                                   // S x kTile
     __shared__ int ew[S];
     __shared__ int4 csh[S][16];
     const size_t nt = tiles_of(n);

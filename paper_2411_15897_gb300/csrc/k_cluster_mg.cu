@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
     const int tid = threadIdx.x, nth = blockDim.x;
     const int type = a.b0 + z;
     const bool nodx = type == 0, nodz = type == 1;
-    extern __shared__ __align__(16) unsigned char sm[];
+    extern __shared__ __align__(128) unsigned char sm[];
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sm);
     const int nlev = a.nlev, kc = nlev - 1;
 

@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtas<MODE>)
     const int rr = blockIdx.z;
     if (s.active && !s.active[rr]) return;
     const auto& B = s.blk[blockIdx.y];
-    extern __shared__ __align__(16) unsigned char fine_raw[];
+    extern __shared__ __align__(128) unsigned char fine_raw[];
     V* xs = reinterpret_cast<V*>(fine_raw);             // (kH + 2) x kP, then kH x kW
     const V* b = B.b + rr * B.sb;
     V* bc = pick(cb, (int)blockIdx.y) + rr * cb.s;
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtas<MODE>)
     const int rr = blockIdx.z;
     if (s.active && !s.active[rr]) return;
     const auto& B = s.blk[blockIdx.y];
-    extern __shared__ __align__(16) unsigned char fine_raw[];
+    extern __shared__ __align__(128) unsigned char fine_raw[];
     V* xs = reinterpret_cast<V*>(fine_raw);             // two buffers of (kH + 2) x kP
     const V* b = B.b + rr * B.sb;
     const V* e = pick(ce, (int)blockIdx.y) + rr * ce.s;

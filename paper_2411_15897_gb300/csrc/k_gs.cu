@@ -18,6 +18,7 @@
 // per-right-hand-side flag and return at once when it is clear.
 #include "bah_internal.cuh"
 #include "fix60.cuh"
+#include "givens.cuh"
 
 #include <algorithm>
 
@@ -28,6 +29,22 @@ __device__ __forceinline__ bool inactive_gs(const KS& ks, int r) { return ks.act
 constexpr int kGsThreads = 128;
 constexpr int kGsWarps = kGsThreads / 32;
 constexpr int kGsRows = 8;           // basis rows of one CTA
+constexpr int kGsFew = 64;           // up to so many partial sums a row are added by the dot kernel's last CTA
+
+// true in every thread of the last CTA (of `total`) to come here with this counter; what
+// the other CTAs wrote before is then visible.  The counter is zero again afterwards.
+__device__ __forceinline__ bool last_cta(int* cnt, int total) {
+    __shared__ int last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(cnt, 1) == total - 1;
+        if (last) *cnt = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
 
 // the tile's entries of w (zero beyond n) and its biased exponent
 __device__ __forceinline__ int load_tile(const double2* __restrict__ w, size_t e0, size_t n, double2 (&x)[kTileU]) {
@@ -56,19 +73,27 @@ __device__ __forceinline__ int load_tile(const double2* __restrict__ w, size_t e
 // converts w and adds up its lanes.
 // ---------------------------------------------------------------------------
 constexpr int kGsStages = 3;
+// The rings start on 128-byte boundaries: 16 or 48 bytes off, a warp's rows straddle lines and the
+// update of eight sources of 1024 x 512 took 636 us instead of 544.
 constexpr size_t kGsSmem = (size_t)kGsWarps * kGsStages * kTile * sizeof(int4);
 
 __device__ __forceinline__ void copy16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
-template <int R>
+template <int R, bool LAST>
 __global__ void __launch_bounds__(kGsThreads, 4) k_gs_dot(const int4* __restrict__ VL, const int* __restrict__ VE, int k,
                                                           int rows, const double2* __restrict__ w, size_t n,
-                                                          double2* __restrict__ partial, const int* flag, KS ks) {
+                                                          double2* __restrict__ partial, double2* __restrict__ out,
+                                                          const int* flag, int* cnt, KS ks) {
     pdl_prologue();
     const int r = blockIdx.z;
-    if (inactive_gs(ks, r) || (flag && flag[r] == 0)) return;
+    if (inactive_gs(ks, r)) return;
+    if (flag && flag[r] == 0) {
+        if (LAST && blockIdx.x == 0 && blockIdx.y == 0)
+            for (int i = threadIdx.x; i <= k; i += kGsThreads) out[r * ks.so + i] = make_double2(0.0, 0.0);
+        return;
+    }
     const size_t nt = tiles_of(n), npad = nt * kTile;
     VL += r * ks.sv;
     VE += r * ks.se;
@@ -80,7 +105,7 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_dot(const int4* __restrict
     // this CTA's rows [ya, yb), taken in groups of `rows`
     const int ya = blockIdx.y * rows, yb = gridDim.y > 1 ? min(k, ya + rows) : k;
     const size_t tstep = (size_t)gridDim.x * kGsWarps;
-    extern __shared__ int4 ring_all[];
+    extern __shared__ __align__(128) int4 ring_all[];
     const int4* ring = ring_all + (size_t)wp * kGsStages * kTile + lane;
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
     size_t pt = (size_t)blockIdx.x * kGsWarps + wp;             // next row to copy: tile, row, slot
@@ -186,6 +211,23 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_dot(const int4* __restrict
         for (int u = 0; u < kGsWarps; ++u) s += sum[u][2 * 64];
         partial[(size_t)k * gridDim.x + blockIdx.x] = make_double2(s, 0.0);
     }
+    if (!LAST || !last_cta(cnt + r, gridDim.x * gridDim.y)) return;
+    // few partial sums: added here, four lanes to a row
+    for (int y = threadIdx.x >> 2; y < ((k + 1 + 7) & ~7); y += kGsThreads / 4) {
+        double2 s = make_double2(0.0, 0.0);
+        if (y <= k)
+            for (int e = threadIdx.x & 3; e < gridDim.x; e += 4) {
+                const double2 a = __ldcg(partial + (size_t)y * gridDim.x + e);
+                s.x += a.x;
+                s.y += a.y;
+            }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+            s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+        }
+        if ((threadIdx.x & 3) == 0 && y <= k) out[r * ks.so + y] = s;
+    }
 }
 
 __global__ void __launch_bounds__(128) k_gs_reduce(const double2* __restrict__ partial, int np, double2* out,
@@ -225,19 +267,32 @@ static int gs_ctas(size_t n, int nrhs) {
     return (int)((nt + per * kGsWarps - 1) / (per * kGsWarps));
 }
 
+// Rows go to groups in different CTAs while the tiles alone fill less than half the chip;
+// then a group is as small as fills it (one or two rows: all its loads are in flight at
+// once).  Up to kGsFew partial sums a row, the last CTA adds them (one launch less): one
+// source at 64 x 64, k = 20, 7.3 us and 4 us for the sum -> 9.0 us with it.
 void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, size_t n, double2* partial, double2* out,
-                     const int* flag, int nrhs, const KS& ks, cudaStream_t st) {
-    const int groups = (k + kGsRows - 1) / kGsRows, rows = (k + groups - 1) / groups;
+                     const int* flag, int* cnt, int nrhs, const KS& ks, cudaStream_t st) {
     const int nc = gs_ctas(n, nrhs);
     const bool split = (size_t)nc * nrhs * 2 <= GS_CTAS;
-    const dim3 g(nc, split ? groups : 1, nrhs), b(kGsThreads);
+    int rows = split ? std::min(kGsRows, std::max(1, (k * nc * nrhs + GS_CTAS - 1) / GS_CTAS)) : kGsRows;
+    const int groups = (k + rows - 1) / rows;
+    rows = (k + groups - 1) / groups;
+    const bool last = nc <= kGsFew;
+    const dim3 g(nc, split ? (k + rows - 1) / rows : 1, nrhs), b(kGsThreads);
     switch (rows) {
-#define BAH_GS_DOT(R) case R: launch_pdl(k_gs_dot<R>, g, b, kGsSmem, st, VL, VE, k, rows, w, n, partial, flag, ks); break;
+#define BAH_GS_DOT(R)                                                                                                   \
+    case R:                                                                                                             \
+        launch_pdl(last ? k_gs_dot<R, true> : k_gs_dot<R, false>, g, b, kGsSmem, st, VL, VE, k, rows, w, n, partial, out, \
+                   flag, cnt, ks);                                                                                      \
+        break;
         BAH_GS_DOT(1) BAH_GS_DOT(2) BAH_GS_DOT(3) BAH_GS_DOT(4) BAH_GS_DOT(5) BAH_GS_DOT(6) BAH_GS_DOT(7) BAH_GS_DOT(8)
 #undef BAH_GS_DOT
     }
-    launch_pdl(k_gs_reduce, dim3(1, k + 1, nrhs), dim3(128), 0, st, (const double2*)partial, nc, out, flag, ks);
+    if (!last) launch_pdl(k_gs_reduce, dim3(1, k + 1, nrhs), dim3(128), 0, st, (const double2*)partial, nc, out, flag, ks);
 }
+
+int dot_launches(size_t n, int nrhs) { return gs_ctas(n, nrhs) <= kGsFew ? 1 : 2; }
 
 // ---------------------------------------------------------------------------
 // w -= sum_i coef_i V_i, and per-CTA partial sums of |w_new|^2.  One warp per
@@ -247,12 +302,111 @@ void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, siz
 // exact integer, rounded once and subtracted from w in FP64.  The rows, and w
 // as the last row of each tile, come through the same ring as in k_gs_dot.
 // ---------------------------------------------------------------------------
+// ||w'||^2 from the CTAs' sums (thread 0 holds this CTA's), by the last CTA: after pass 1
+// the DGKS decision too.  Separate kernels for this cost 4.7 and 4 us per step.
+__device__ __forceinline__ void gs_norm(double s, double* npart, const double2* coef, int k, int r, int pass,
+                                        const GsNorm& nm) {
+    if (threadIdx.x == 0) npart[blockIdx.x] = s;
+    if (!last_cta(nm.cnt + r, gridDim.x)) return;
+    __shared__ double sh[kGsWarps];
+    s = 0.0;
+    for (int e = threadIdx.x; e < gridDim.x; e += kGsThreads) s += __ldcg(npart + e);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    s = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+    double* sc = nm.sc + r * 8;
+    sc[2] = sqrt(s);
+    if (pass == 1) {
+        const int f = s < nm.eta2 * coef[k].x ? 1 : 0;           // coef[k]: ||w||^2 before pass 1
+        nm.flag[r] = f;
+        sc[3] += (double)f;
+    }
+}
+
+// the coefficients' share of the common exponent, for the rows lane and lane + 32
+struct GsCoef {
+    double2 c[2];
+    int ec[2];
+    bool bad;
+    __device__ __forceinline__ GsCoef(const double2* coef, int k, int lane) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = lane + 32 * q;
+            c[q] = i < k ? coef[i] : make_double2(0.0, 0.0);
+            ec[q] = max(abs_hi(c[q].x), abs_hi(c[q].y)) >> 20;   // biased exponent field (0: no contribution)
+        }
+        bad = __any_sync(0xffffffffu, ec[0] == 0x7ff || ec[1] == 0x7ff);
+    }
+    // limbs of every coefficient scaled to the tile's common exponent; returns the scale of the
+    // sums, whose units are 2^(60 - sb) of integers scaled by 2^(59 - Ev) 2^(59 - Ec)
+    __device__ __forceinline__ double limbs(const int (&ev)[2], int k, int lane, int head, int sb, int4* out) const {
+        int eo = 0;
+        bool b = bad;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            b |= ev[q] == kExpBad;
+            if (ec[q] > 0) eo = max(eo, ev[q] + ec[q] + 1 + head);
+        }
+        eo = (int)__reduce_max_sync(0xffffffffu, (unsigned)eo);  // biased twice
+        b = __any_sync(0xffffffffu, b);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = lane + 32 * q;
+            if (i < k) {
+                const int eb = eo - ev[q];                       // exponent the coefficient is scaled to
+                out[i] = ec[q] > 0 && eb >= kExpMin ? limbs2(c[q], eb) : make_int4(0, 0, 0, 0);
+            }
+        }
+        __syncwarp();
+        return b ? __longlong_as_double(0x7ff8000000000000ll) : pow2((eo - 2 * 1023) - 118 + 60 - sb);
+    }
+};
+// the coefficients keep 58 bits, so hh holds 2k products of 2^56: 32 rows fit 2^62, and
+// the shift sb uses the bits left
+__device__ __forceinline__ int gs_head(int k) { return k > 32 ? 3 : 2; }
+__device__ __forceinline__ int gs_shift(int k) {
+    return k > 16 ? 0 : (k > 8 ? 1 : (k > 4 ? 2 : (k > 2 ? 3 : (k > 1 ? 4 : 5))));
+}
+// hh and cross sums of c b, both parts, over one row's entries
+__device__ __forceinline__ void gs_row(const int4* row, const int4& cc, long long (&hr)[kTileU], long long (&cr)[kTileU],
+                                       long long (&hi)[kTileU], long long (&ci)[kTileU]) {
+    const int nz = -cc.z, nw = -cc.w;
+#pragma unroll
+    for (int u = 0; u < kTileU; ++u) {
+        const int4 b = row[32 * u];
+        // c b = (cx bx - cy by) + i (cx by + cy bx)
+        mad(hr[u], cc.x, b.x); mad(hr[u], nz, b.z);
+        mad(cr[u], cc.x, b.y); mad(cr[u], cc.y, b.x);
+        mad(cr[u], nz, b.w); mad(cr[u], nw, b.z);
+        mad(hi[u], cc.x, b.z); mad(hi[u], cc.z, b.x);
+        mad(ci[u], cc.x, b.w); mad(ci[u], cc.y, b.z);
+        mad(ci[u], cc.z, b.y); mad(ci[u], cc.w, b.x);
+    }
+}
+// the cross sums hold 8 rows: carry into hh
+__device__ __forceinline__ void gs_carry(long long (&hr)[kTileU], long long (&cr)[kTileU], long long (&hi)[kTileU],
+                                         long long (&ci)[kTileU]) {
+#pragma unroll
+    for (int u = 0; u < kTileU; ++u) {
+        hr[u] += cr[u] >> 30; cr[u] &= 0x3fffffff;
+        hi[u] += ci[u] >> 30; ci[u] &= 0x3fffffff;
+    }
+}
+// x - the sum, rounded once to 2^(60 - sb)
+__device__ __forceinline__ double gs_sub(double x, long long h, long long c, int sb, double sc) {
+    return fma(-(double)((h << sb) + ((c + (1ll << (29 - sb))) >> (30 - sb))), sc, x);
+}
+
 __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restrict__ VL, const int* __restrict__ VE, int k,
                                                            const double2* __restrict__ coef, double2* __restrict__ w,
-                                                           size_t n, double* __restrict__ npart, const int* flag, KS ks) {
+                                                           size_t n, double* __restrict__ npart, int pass, GsNorm nm, KS ks) {
     pdl_prologue();
     const int r = blockIdx.z;
-    if (inactive_gs(ks, r) || (flag && flag[r] == 0)) return;
+    if (inactive_gs(ks, r) || (pass == 2 && nm.flag[r] == 0)) return;
     const size_t nt = tiles_of(n), npad = nt * kTile;
     VL += r * ks.sv;
     VE += r * ks.se;
@@ -262,7 +416,7 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restric
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const size_t tstep = (size_t)gridDim.x * kGsWarps;
     size_t t = (size_t)blockIdx.x * kGsWarps + wp;
-    extern __shared__ int4 ring_all[];
+    extern __shared__ __align__(128) int4 ring_all[];
     const int4* ring = ring_all + (size_t)wp * kGsStages * kTile + lane;
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
     size_t pt = t;
@@ -297,84 +451,36 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restric
         return row;
     };
     __shared__ int4 csh[kGsWarps][64];
-    // rows lane and lane + 32
-    double2 c[2];
-    int ec[2], evn[2];
+    const GsCoef gc(coef, k, lane);
+    int evn[2];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int i = lane + 32 * q;
-        c[q] = i < k ? coef[i] : make_double2(0.0, 0.0);
-        ec[q] = max(abs_hi(c[q].x), abs_hi(c[q].y)) >> 20;       // biased exponent field (0: no contribution)
-        evn[q] = i < k && t < nt ? VE[(size_t)i * nt + t] : kExpMin;
-    }
-    const bool cbad = __any_sync(0xffffffffu, ec[0] == 0x7ff || ec[1] == 0x7ff);
-    // the coefficients keep 58 bits, so hh holds 2k products of 2^56: 32 rows fit 2^62, and
-    // the shift sb uses the bits left
-    const int head = k > 32 ? 3 : 2;
-    const int sb = k > 16 ? 0 : (k > 8 ? 1 : (k > 4 ? 2 : (k > 2 ? 3 : (k > 1 ? 4 : 5))));
+    for (int q = 0; q < 2; ++q) evn[q] = lane + 32 * q < k && t < nt ? VE[(size_t)(lane + 32 * q) * nt + t] : kExpMin;
+    const int head = gs_head(k), sb = gs_shift(k);
     double nn = 0.0;
     for (; t < nt; t += tstep) {
-        int ev[2], eo = 0;
-        bool bad = cbad;
+        int ev[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int i = lane + 32 * q;
             ev[q] = evn[q];
-            bad |= ev[q] == kExpBad;
-            if (ec[q] > 0) eo = max(eo, ev[q] + ec[q] + 1 + head);
             evn[q] = i < k && t + tstep < nt ? VE[(size_t)i * nt + t + tstep] : kExpMin;
         }
-        eo = (int)__reduce_max_sync(0xffffffffu, (unsigned)eo);  // biased twice
-        bad = __any_sync(0xffffffffu, bad);
-        __syncwarp();
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int i = lane + 32 * q;
-            if (i < k) {
-                const int eb = eo - ev[q];                       // exponent the coefficient is scaled to
-                csh[wp][i] = ec[q] > 0 && eb >= kExpMin ? limbs2(c[q], eb) : make_int4(0, 0, 0, 0);
-            }
-        }
-        __syncwarp();
-        // T units: 2^(60 - sb) of integers scaled by 2^(59 - Ev) 2^(59 - Ec)
-        double sc = pow2((eo - 2 * 1023) - 118 + 60 - sb);
-        if (bad) sc = __longlong_as_double(0x7ff8000000000000ll);
+        const double sc = gc.limbs(ev, k, lane, head, sb, csh[wp]);
         long long hr[kTileU], cr[kTileU], hi[kTileU], ci[kTileU];
 #pragma unroll
         for (int u = 0; u < kTileU; ++u) hr[u] = cr[u] = hi[u] = ci[u] = 0;
         for (int i = 0; i < k; ++i) {
-            const int4* row = next_row();
-            const int4 cc = csh[wp][i];
-            const int nz = -cc.z, nw = -cc.w;
-#pragma unroll
-            for (int u = 0; u < kTileU; ++u) {
-                const int4 b = row[32 * u];
-                // c b = (cx bx - cy by) + i (cx by + cy bx)
-                mad(hr[u], cc.x, b.x); mad(hr[u], nz, b.z);
-                mad(cr[u], cc.x, b.y); mad(cr[u], cc.y, b.x);
-                mad(cr[u], nz, b.w); mad(cr[u], nw, b.z);
-                mad(hi[u], cc.x, b.z); mad(hi[u], cc.z, b.x);
-                mad(ci[u], cc.x, b.w); mad(ci[u], cc.y, b.z);
-                mad(ci[u], cc.z, b.y); mad(ci[u], cc.w, b.x);
-            }
-            if ((i & 7) == 7) {                                  // the cross sums hold 8 rows: carry into hh
-#pragma unroll
-                for (int u = 0; u < kTileU; ++u) {
-                    hr[u] += cr[u] >> 30; cr[u] &= 0x3fffffff;
-                    hi[u] += ci[u] >> 30; ci[u] &= 0x3fffffff;
-                }
-            }
+            gs_row(next_row(), csh[wp][i], hr, cr, hi, ci);
+            if ((i & 7) == 7) gs_carry(hr, cr, hi, ci);
         }
         const double2* wrow = reinterpret_cast<const double2*>(next_row());
         const size_t e0 = t * kTile + lane;
 #pragma unroll
         for (int u = 0; u < kTileU; ++u) {
             if (e0 + 32 * u < n) {
-                const long long tr = (hr[u] << sb) + ((cr[u] + (1ll << (29 - sb))) >> (30 - sb));
-                const long long ti = (hi[u] << sb) + ((ci[u] + (1ll << (29 - sb))) >> (30 - sb));
                 double2 x = wrow[32 * u];
-                x.x = fma(-(double)tr, sc, x.x);
-                x.y = fma(-(double)ti, sc, x.y);
+                x.x = gs_sub(x.x, hr[u], cr[u], sb, sc);
+                x.y = gs_sub(x.y, hi[u], ci[u], sb, sc);
                 w[e0 + 32 * u] = x;
                 nn = fma(x.x, x.x, nn);
                 nn = fma(x.y, x.y, nn);
@@ -386,21 +492,136 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restric
     __shared__ double sh[kGsWarps];
     if (lane == 0) sh[wp] = nn;
     __syncthreads();
-    if (threadIdx.x == 0) npart[blockIdx.x] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+    gs_norm((sh[0] + sh[1]) + (sh[2] + sh[3]), npart, coef, k, r, pass, nm);
 }
-int launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
-                     const int* flag, int nrhs, const KS& ks, cudaStream_t st) {
-    const int nc = gs_ctas(n, nrhs);
-    launch_pdl(k_gs_axpy, dim3(nc, 1, nrhs), dim3(kGsThreads), kGsSmem, st, VL, VE, k, coef, w, n, npart, flag, ks);
-    return nc;
+
+// The same with one tile per CTA, its rows split over the four warps: on a small grid a
+// warp that takes 20 rows in turn is a chain of load latencies (one source at 64 x 64,
+// k = 20, 12 CTAs: 10.7 us; so 48 CTAs, 8.9 us with the norm, of which 4 to 5 was a launch
+// of its own).  The warps' sums are integers, so that their total does not
+// depend on the split.  ST: ring slots per warp.
+template <int ST>
+__global__ void __launch_bounds__(kGsThreads, ST > 3 ? 2 : 4) k_gs_axpy_split(const int4* __restrict__ VL, const int* __restrict__ VE,
+                                                                 int k, const double2* __restrict__ coef,
+                                                                 double2* __restrict__ w, size_t n,
+                                                                 double* __restrict__ npart, int pass, GsNorm nm, KS ks) {
+    pdl_prologue();
+    const int r = blockIdx.z;
+    if (inactive_gs(ks, r) || (pass == 2 && nm.flag[r] == 0)) return;
+    const size_t nt = tiles_of(n), npad = nt * kTile, t = blockIdx.x;
+    VL += r * ks.sv;
+    VE += r * ks.se;
+    w += r * ks.sw;
+    coef += r * ks.so;
+    npart += r * GS_CTAS;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int per = (k + kGsWarps - 1) / kGsWarps, i0 = min(k, wp * per), i1 = min(k, i0 + per);
+    extern __shared__ __align__(128) int4 ring_all[];
+    const int4* ring = ring_all + (size_t)wp * ST * kTile + lane;
+    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+    int py = i0, ps = 0, cs = 0;
+    auto prefetch = [&]() {
+        if (py < i1) {
+            const int4* src = VL + (size_t)py * npad + t * kTile + lane;
+#pragma unroll
+            for (int u = 0; u < kTileU; ++u) copy16(ring_s + (uint32_t)(ps * kTile) * 16u + 512u * u, src + 32 * u);
+            ++py;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ps = ps == ST - 1 ? 0 : ps + 1;
+    };
+#pragma unroll
+    for (int i = 0; i < ST - 1; ++i) prefetch();
+    // the two entries of w that this thread finishes
+    double2 x[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const size_t e = t * kTile + threadIdx.x + kGsThreads * q;
+        x[q] = e < n ? w[e] : make_double2(0.0, 0.0);
+    }
+    __shared__ int4 csh[kGsWarps][64];
+    int ev[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) ev[q] = lane + 32 * q < k ? VE[(size_t)(lane + 32 * q) * nt + t] : kExpMin;
+    const GsCoef gc(coef, k, lane);
+    const int head = gs_head(k), sb = gs_shift(k);
+    const double sc = gc.limbs(ev, k, lane, head, sb, csh[wp]);
+    long long hr[kTileU], cr[kTileU], hi[kTileU], ci[kTileU];
+#pragma unroll
+    for (int u = 0; u < kTileU; ++u) hr[u] = cr[u] = hi[u] = ci[u] = 0;
+    for (int i = i0; i < i1; ++i) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
+        prefetch();                              // into the slot of the row before this one
+        gs_row(ring + cs * kTile, csh[wp][i], hr, cr, hi, ci);
+        cs = cs == ST - 1 ? 0 : cs + 1;
+        if (((i - i0) & 7) == 7) gs_carry(hr, cr, hi, ci);
+    }
+    gs_carry(hr, cr, hi, ci);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    // the sums of all warps, over the warp's own ring: [sum][entry], 8 KB of its at least 12
+    long long* acc = reinterpret_cast<long long*>(ring_all + (size_t)wp * ST * kTile);
+#pragma unroll
+    for (int u = 0; u < kTileU; ++u) {
+        acc[lane + 32 * u] = hr[u];
+        acc[kTile + lane + 32 * u] = cr[u];
+        acc[2 * kTile + lane + 32 * u] = hi[u];
+        acc[3 * kTile + lane + 32 * u] = ci[u];
+    }
+    __syncthreads();
+    double nn = 0.0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int e = threadIdx.x + kGsThreads * q;
+        long long s[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int v = 0; v < kGsWarps; ++v) {
+            const long long* a = reinterpret_cast<const long long*>(ring_all + (size_t)v * ST * kTile);
+#pragma unroll
+            for (int z = 0; z < 4; ++z) s[z] += a[z * kTile + e];
+        }
+        if (t * kTile + e < n) {
+            x[q].x = gs_sub(x[q].x, s[0], s[1], sb, sc);
+            x[q].y = gs_sub(x[q].y, s[2], s[3], sb, sc);
+            w[t * kTile + e] = x[q];
+            nn = fma(x[q].x, x[q].x, nn);
+            nn = fma(x[q].y, x[q].y, nn);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
+    __shared__ double sh[kGsWarps];
+    if (lane == 0) sh[wp] = nn;
+    __syncthreads();
+    gs_norm((sh[0] + sh[1]) + (sh[2] + sh[3]), npart, coef, k, r, pass, nm);
+}
+constexpr int kGsDeep = 6;
+constexpr size_t kGsDeepSmem = (size_t)kGsWarps * kGsDeep * kTile * sizeof(int4);
+
+// one tile per CTA while all of them run at once (four CTAs to an SM; with a CTA or two to
+// an SM the deeper ring)
+void launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
+                      int pass, const GsNorm& nm, int nrhs, const KS& ks, cudaStream_t st) {
+    const size_t nt = tiles_of(n);
+    const dim3 b(kGsThreads);
+    if (nt * nrhs <= GS_CTAS / 2)
+        launch_pdl(k_gs_axpy_split<kGsDeep>, dim3((unsigned)nt, 1, nrhs), b, kGsDeepSmem, st, VL, VE, k, coef, w, n, npart, pass,
+                   nm, ks);
+    else if (nt * nrhs <= GS_CTAS)
+        launch_pdl(k_gs_axpy_split<kGsStages>, dim3((unsigned)nt, 1, nrhs), b, kGsSmem, st, VL, VE, k, coef, w, n, npart, pass,
+                   nm, ks);
+    else
+        launch_pdl(k_gs_axpy, dim3(gs_ctas(n, nrhs), 1, nrhs), b, kGsSmem, st, VL, VE, k, coef, w, n, npart, pass, nm, ks);
 }
 
 int gs_prepare() {
-    const void* fn[] = {(const void*)k_gs_dot<1>, (const void*)k_gs_dot<2>, (const void*)k_gs_dot<3>, (const void*)k_gs_dot<4>,
-                        (const void*)k_gs_dot<5>, (const void*)k_gs_dot<6>, (const void*)k_gs_dot<7>, (const void*)k_gs_dot<8>,
-                        (const void*)k_gs_axpy};
+    const void* fn[] = {
+#define BAH_GS_DOT(R) (const void*)k_gs_dot<R, true>, (const void*)k_gs_dot<R, false>,
+        BAH_GS_DOT(1) BAH_GS_DOT(2) BAH_GS_DOT(3) BAH_GS_DOT(4) BAH_GS_DOT(5) BAH_GS_DOT(6) BAH_GS_DOT(7) BAH_GS_DOT(8)
+#undef BAH_GS_DOT
+        (const void*)k_gs_axpy, (const void*)k_gs_axpy_split<kGsStages>};
     for (const void* f : fn)
         BAH_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGsSmem));
+    BAH_CUDA_TRY(cudaFuncSetAttribute(k_gs_axpy_split<kGsDeep>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGsDeepSmem));
     return BAH_OK;
 }
 
@@ -412,9 +633,12 @@ int gs_prepare() {
 template <class Vc>
 __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restrict__ w, const double* sc, int slot,
                                                          Vc* __restrict__ vc, int4* __restrict__ vl,
-                                                         int* __restrict__ ve, size_t n, size_t sw, KS ks) {
+                                                         int* __restrict__ ve, size_t n, size_t sw, KS ks, int givens,
+                                                         GivensArgs gv) {
     pdl_prologue();
     const int r = blockIdx.y;
+    // the first CTA runs the step's Givens update beside the copy (a launch of its own took 11 us)
+    if (givens && blockIdx.x == 0) return arnoldi_givens(gv, r, ks);
     if (inactive_gs(ks, r)) return;
     const size_t nt = tiles_of(n);
     w += r * sw;
@@ -423,7 +647,8 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
     ve += r * ks.se;
     const int lane = threadIdx.x & 31;
     const double s = 1.0 / sc[r * 8 + slot];
-    for (size_t t = (size_t)blockIdx.x * kGsWarps + (threadIdx.x >> 5); t < nt; t += (size_t)gridDim.x * kGsWarps) {
+    const size_t t = (size_t)(blockIdx.x - givens) * kGsWarps + (threadIdx.x >> 5);
+    if (t < nt) {
         const size_t e0 = t * kTile + lane;
         double2 x[kTileU];
         int mx = 0;
@@ -446,14 +671,15 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
 }
 template <class Vc>
 void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, size_t n,
-                        size_t sw, int nrhs, const KS& ks, cudaStream_t st) {
+                        size_t sw, int nrhs, const KS& ks, cudaStream_t st, const GivensArgs* gv) {
     const size_t nt = tiles_of(n);
-    launch_pdl(k_gs_store<Vc>, dim3((unsigned)((nt + kGsWarps - 1) / kGsWarps), nrhs), dim3(kGsThreads), 0, st, w, sc, slot, vc,
-               vl, ve, n, sw, ks);
+    const int givens = gv ? 1 : 0;
+    launch_pdl(k_gs_store<Vc>, dim3((unsigned)((nt + kGsWarps - 1) / kGsWarps) + givens, nrhs), dim3(kGsThreads), 0, st, w, sc,
+               slot, vc, vl, ve, n, sw, ks, givens, gv ? *gv : GivensArgs());
 }
 template void launch_basis_store<double2>(const double2*, const double*, int, double2*, int4*, int*, size_t, size_t, int,
-                                          const KS&, cudaStream_t);
+                                          const KS&, cudaStream_t, const GivensArgs*);
 template void launch_basis_store<float2>(const double2*, const double*, int, float2*, int4*, int*, size_t, size_t, int,
-                                         const KS&, cudaStream_t);
+                                         const KS&, cudaStream_t, const GivensArgs*);
 
 }  // namespace bah

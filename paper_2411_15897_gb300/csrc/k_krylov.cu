@@ -6,6 +6,7 @@
 // problem, the triangular solve and the solution update x += Z y.
 // A right-hand side whose active flag is 0 is skipped by every kernel.
 #include "bah_internal.cuh"
+#include "givens.cuh"
 #include "df.cuh"
 
 namespace bah {
@@ -44,7 +45,7 @@ __device__ __forceinline__ bool inactive(const KS& ks, int r) { return ks.active
 // ---------------------------------------------------------------------------
 // reduce the pass-1 norm, decide on the second pass, set ||w|| for the Givens
 // step: sc[2] = ||w_final||, sc[3] counts second passes; flag = 1 when
-// ||w'||^2 < ||w||^2 / 2
+// ||w'||^2 < ||w||^2 / 2 (with the FP64 basis the last CTA of k_gs_axpy does both)
 __global__ void __launch_bounds__(256) k_dgks_decide(const double* npart, int np, const double2* h1norm, int k,
                                                      int* flag, double* sc, double eta2, KS ks) {
     pdl_prologue();
@@ -223,92 +224,61 @@ void launch_scale_copy(const double2* w, const double* sc, int slot, double2* v,
 
 // ---------------------------------------------------------------------------
 // Hessenberg column j = h1 + h2 (two Gram-Schmidt passes) with subdiagonal
-// ||w||; apply the previous Givens rotations, form the new one, update g.
+// ||w||; apply the previous Givens rotations, form the new one, update g (givens.cuh;
+// with the FP64 basis k_gs_store runs it beside the copy of the new basis vector).
 // Rotation [c s; -conj(s) c] with c real.  status[0] = |g_{j+1}|,
 // status[1] = h_{j+1,j}, status[2] = 1 if a non-finite value appeared.
 // ---------------------------------------------------------------------------
-__global__ void k_arnoldi_givens(double2* Hm, int ldh, const double2* h1, const double2* h2, const double* sc, int j,
-                                 double2* cs, double2* sn, double2* g, double* status, KS ks) {
+__global__ void __launch_bounds__(32) k_arnoldi_givens(GivensArgs a, KS ks) {
     pdl_prologue();
-    const int r = blockIdx.x;
-    if (inactive(ks, r)) return;
-    double2* Hcol = Hm + r * ks.sh + (size_t)j * ldh;
-    h1 += r * ks.so;
-    h2 += r * ks.so;
-    cs += r * ks.so;
-    sn += r * ks.so;
-    g += r * ks.so;
-    status += r * 4;
-    __shared__ double2 h[66];
-    __shared__ double2 ssn[65];
-    __shared__ double scs[65];
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-        h[i] = cadd(h1[i], h2[i]);
-        if (i < j) { scs[i] = cs[i].x; ssn[i] = sn[i]; }
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    const double wn = sc[r * 8 + 2];
-    h[j + 1] = make_double2(wn, 0.0);
-    bool bad = !isfinite(wn);
-    for (int i = 0; i <= j; ++i) bad |= !isfinite(h[i].x) || !isfinite(h[i].y);
-    for (int i = 0; i < j; ++i) {
-        const double c = scs[i];
-        const double2 s = ssn[i];
-        const double2 a = h[i], b = h[i + 1];
-        h[i] = cadd(cscale(a, c), cmul(s, b));
-        h[i + 1] = csub(cscale(b, c), cmul(cconj(s), a));
-    }
-    const double2 a = h[j], b = h[j + 1];
-    const double na2 = a.x * a.x + a.y * a.y, nb2 = b.x * b.x + b.y * b.y;
-    double c;
-    double2 s;
-    if (nb2 == 0.0) {
-        c = 1.0; s = make_double2(0.0, 0.0);
-    } else if (na2 == 0.0) {
-        c = 0.0; s = cscale(cconj(b), 1.0 / sqrt(nb2));
-    } else {
-        const double na = sqrt(na2), rr = sqrt(na2 + nb2);
-        c = na / rr;
-        s = cscale(cmul(a, cconj(b)), 1.0 / (na * rr));
-    }
-    cs[j] = make_double2(c, 0.0);
-    sn[j] = s;
-    h[j] = cadd(cscale(a, c), cmul(s, b));
-    h[j + 1] = make_double2(0.0, 0.0);
-    for (int i = 0; i <= j + 1; ++i) Hcol[i] = h[i];
-    const double2 gj = g[j];
-    g[j] = cscale(gj, c);
-    const double2 gn = cscale(cmul(cconj(s), gj), -1.0);
-    g[j + 1] = gn;
-    status[0] = sqrt(gn.x * gn.x + gn.y * gn.y);
-    status[1] = wn;
-    status[2] = bad ? 1.0 : 0.0;
+    arnoldi_givens(a, blockIdx.x, ks);
 }
-void launch_arnoldi_givens(double2* Hm, int ldh, const double2* h1, const double2* h2, const double* sc, int j,
-                           double2* cs, double2* sn, double2* g, double* status, int nrhs, const KS& ks,
-                           cudaStream_t st) {
-    launch_pdl(k_arnoldi_givens, dim3(nrhs), dim3(32), 0, st, Hm, ldh, h1, h2, sc, j, cs, sn, g, status, ks);
+void launch_arnoldi_givens(const GivensArgs& a, int nrhs, const KS& ks, cudaStream_t st) {
+    launch_pdl(k_arnoldi_givens, dim3(nrhs), dim3(32), 0, st, a, ks);
 }
 
-// R y = g(0..k-1), R upper triangular stored column-major with leading dimension ldh
-__global__ void k_triangular_solve(const double2* Hm, int ldh, const double2* g, const int* kk, double2* y, KS ks) {
+// R y = g(0..k-1), R upper triangular stored column-major with leading dimension ldh,
+// k <= kMaxTri.  The triangle is copied to shared memory at once; then one warp takes the
+// columns from the last, a lane per row (two above 32).  By one thread, with each entry
+// loaded when its product was due, k = 20 took 79 us; now 17.
+constexpr int kMaxTri = 64;
+__global__ void __launch_bounds__(128) k_triangular_solve(const double2* Hm, int ldh, const double2* g, const int* kk,
+                                                          double2* y, KS ks) {
     pdl_prologue();
     const int r = blockIdx.x;
     const int k = kk[r];
-    if (threadIdx.x != 0 || k <= 0) return;
+    if (k <= 0) return;
     Hm += r * ks.sh;
     g += r * ks.so;
     y += r * ks.so;
-    for (int i = k - 1; i >= 0; --i) {
-        double2 acc = g[i];
-        for (int c = i + 1; c < k; ++c) acc = csub(acc, cmul(Hm[(size_t)c * ldh + i], y[c]));
-        y[i] = cdiv(acc, Hm[(size_t)i * ldh + i]);
+    __shared__ double2 R[kMaxTri * (kMaxTri + 1) / 2];            // column c at c (c + 1) / 2
+    const int lane = threadIdx.x & 31;
+    for (int c = threadIdx.x >> 5; c < k; c += 4)
+        for (int i = lane; i <= c; i += 32) R[c * (c + 1) / 2 + i] = Hm[(size_t)c * ldh + i];
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double2 acc[2], inv[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int i = lane + 32 * q;
+        acc[q] = i < k ? g[i] : make_double2(0.0, 0.0);
+        inv[q] = i < k ? cdiv(make_double2(1.0, 0.0), R[i * (i + 1) / 2 + i]) : make_double2(0.0, 0.0);
+    }
+    for (int c = k - 1; c >= 0; --c) {
+        const bool up = c >= 32;
+        const double2 v = cmul(up ? acc[1] : acc[0], up ? inv[1] : inv[0]);
+        const double2 yc = make_double2(__shfl_sync(0xffffffffu, v.x, c & 31), __shfl_sync(0xffffffffu, v.y, c & 31));
+        if (lane == (c & 31)) y[c] = yc;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = lane + 32 * q;
+            if (i < c) acc[q] = csub(acc[q], cmul(R[c * (c + 1) / 2 + i], yc));
+        }
     }
 }
 void launch_triangular_solve(const double2* Hm, int ldh, const double2* g, const int* kk, double2* y, int nrhs,
                              const KS& ks, cudaStream_t st) {
-    launch_pdl(k_triangular_solve, dim3(nrhs), dim3(32), 0, st, Hm, ldh, g, kk, y, ks);
+    launch_pdl(k_triangular_solve, dim3(nrhs), dim3(128), 0, st, Hm, ldh, g, kk, y, ks);
 }
 
 // g = beta e_1, status = (beta, 0, 0)

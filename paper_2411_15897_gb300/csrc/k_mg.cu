@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(256) k_coarse_apply(int npts, int rows, PtrSet
     const int rr = blockIdx.z;
     if (active && !active[rr]) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    extern __shared__ int4 g[];
+    extern __shared__ __align__(128) int4 g[];
     __shared__ int red[32];
     const V* bb = pick(b, z) + rr * b.s;
     const int eg = dense_load<V, typename VecTraits<V>::R>(g, npts, red, [&](int c) { return bb[c]; });

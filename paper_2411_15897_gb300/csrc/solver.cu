@@ -7,6 +7,7 @@
 // and FGMRES (right preconditioned, two-pass classical Gram-Schmidt, Givens
 // rotations on the device) wraps it with the FP64 operator H of Eq. 2.6.
 #include "bah_internal.cuh"
+#include "givens.cuh"
 #include "fix60.cuh"
 
 #include <algorithm>
@@ -100,6 +101,7 @@ struct Ctx {
 
     // Gram-Schmidt flag and per-step graphs
     int* gsflag = nullptr;
+    int* gscnt = nullptr;                // zero between launches: CTAs of a Gram-Schmidt kernel that are done
     struct IterGraph {
         cudaGraphExec_t exec = nullptr;
         unsigned mask = ~0u;
@@ -130,7 +132,7 @@ struct Ctx {
     double2 *ih1 = nullptr, *ih2 = nullptr, *ics = nullptr, *isn = nullptr, *igv = nullptr, *iy = nullptr;
     double2* ipart = nullptr;
     double *inrm = nullptr, *idpart = nullptr, *istatus = nullptr;
-    int *iflag = nullptr, *ijk = nullptr;
+    int *iflag = nullptr, *ijk = nullptr, *icnt = nullptr;
     double* histat = nullptr;           // pinned: 8 status / norm slots and one int
     double2 *ez = nullptr, *etp = nullptr, *esu = nullptr;
     long long block_iters = 0;
@@ -737,16 +739,14 @@ static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t
             }
             // w = M z_j, Gram-Schmidt with selective reorthogonalisation, Givens, v_{j+1}
             launch_block_apply64(c.f5x, b, zj, c.iW, nullptr, st);
-            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih1, nullptr, 1, ks, st);
-            const int npt = launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih1, c.iW, np, c.idpart, nullptr, 1, ks, st);
-            launch_dgks_decide(c.idpart, npt, c.ih1, j + 1, c.iflag, c.inrm, 1, ks, st);
-            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih2, c.iflag, 1, ks, st);
-            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih2, c.iW, np, c.idpart, c.iflag, 1, ks, st);
-            launch_pass2_norm(c.idpart, npt, c.iflag, c.inrm, 1, ks, st);
-            launch_arnoldi_givens(c.iH, m + 1, c.ih1, c.ih2, c.inrm, j, c.ics, c.isn, c.igv, c.istatus, 1, ks, st);
+            const GsNorm nm{c.icnt, c.iflag, c.inrm, 0.5};
+            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih1, nullptr, c.icnt, 1, ks, st);
+            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih1, c.iW, np, c.idpart, 1, nm, 1, ks, st);
+            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih2, c.iflag, c.icnt, 1, ks, st);
+            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih2, c.iW, np, c.idpart, 2, nm, 1, ks, st);
+            const GivensArgs gv{c.iH, m + 1, j, c.ih1, c.ih2, c.inrm, c.ics, c.isn, c.igv, c.istatus, c.histat};
             launch_basis_store(c.iW, c.inrm, 2, c.iVc, c.iVL + (j + 1) * tiles_of(np) * kTile,
-                               c.iVE + (j + 1) * tiles_of(np), np, 0, 1, ks, st);
-            BAH_CUDA_TRY(cudaMemcpyAsync(c.histat, c.istatus, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
+                               c.iVE + (j + 1) * tiles_of(np), np, 0, 1, ks, st, &gv);
             BAH_CUDA_TRY(cudaStreamSynchronize(st));
             ++total;
             jd = j + 1;
@@ -822,12 +822,12 @@ static void precond_newest(Ctx& c, void* z, const Batch& bt, cudaStream_t st) {
     else precond_any(c, (const double2*)c.Vc, c.ks.sw, z, c.ks.sz, bt, st);
 }
 // w / sc[slot] as basis vector i and as the newest vector
-static void store_basis(Ctx& c, const double2* w, int slot, int i, cudaStream_t st) {
+static void store_basis(Ctx& c, const double2* w, int slot, int i, cudaStream_t st, const GivensArgs* gv = nullptr) {
     const size_t n = c.vec_len(), nt = tiles_of(n);
     int4* vl = c.VL + i * nt * kTile;
     int* ve = c.VE + i * nt;
-    if (c.vc32) launch_basis_store(w, c.nrm, slot, (float2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st);
-    else launch_basis_store(w, c.nrm, slot, (double2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st);
+    if (c.vc32) launch_basis_store(w, c.nrm, slot, (float2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st, gv);
+    else launch_basis_store(w, c.nrm, slot, (double2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st, gv);
 }
 // algorithmic bytes of one operator apply: input (3 components), FP64
 // output, coefficients cx, nx (z-aliases when h1 == h2), d1, d2, 1/(lambda+mu)
@@ -900,7 +900,8 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     TRY(c.alloc(&c.ztmp, n * c.vsz));
     TRY(c.alloc_t(&c.Hm, (size_t)(m + 1) * m * nbt));
     TRY(c.alloc_t(&c.h1v, so * nbt)); TRY(c.alloc_t(&c.h2v, so * nbt));
-    TRY(c.alloc_t(&c.gsflag, nbt));
+    TRY(c.alloc_t(&c.gsflag, nbt)); TRY(c.alloc_t(&c.gscnt, nbt));
+    BAH_CUDA_TRY(cudaMemsetAsync(c.gscnt, 0, nbt * sizeof(int), st));
     TRY(c.alloc_t(&c.cs, so * nbt)); TRY(c.alloc_t(&c.sn, so * nbt)); TRY(c.alloc_t(&c.g, so * nbt));
     TRY(c.alloc_t(&c.y, so * nbt));
     TRY(c.alloc_t(&c.partial, so * GS_CTAS * nbt));
@@ -1149,7 +1150,9 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
         TRY(c.alloc_t(&c.ih1, so)); TRY(c.alloc_t(&c.ih2, so)); TRY(c.alloc_t(&c.ics, so)); TRY(c.alloc_t(&c.isn, so));
         TRY(c.alloc_t(&c.igv, so)); TRY(c.alloc_t(&c.iy, so));
         TRY(c.alloc_t(&c.ipart, so * GS_CTAS)); TRY(c.alloc_t(&c.idpart, (size_t)GS_CTAS));
-        TRY(c.alloc_t(&c.inrm, 8)); TRY(c.alloc_t(&c.istatus, 4)); TRY(c.alloc_t(&c.iflag, 1)); TRY(c.alloc_t(&c.ijk, 1));
+        TRY(c.alloc_t(&c.inrm, 8)); TRY(c.alloc_t(&c.istatus, 4)); TRY(c.alloc_t(&c.iflag, 1)); TRY(c.alloc_t(&c.icnt, 1));
+        BAH_CUDA_TRY(cudaMemsetAsync(c.icnt, 0, sizeof(int), st));
+        TRY(c.alloc_t(&c.ijk, 1));
         TRY(c.alloc_t(&c.ez, 3 * (size_t)np)); TRY(c.alloc_t(&c.etp, np)); TRY(c.alloc_t(&c.esu, 2 * (size_t)np));
         BAH_CUDA_TRY(cudaMemsetAsync(c.inrm, 0, 8 * sizeof(double), st));
         BAH_CUDA_TRY(cudaMallocHost((void**)&c.histat, 16 * sizeof(double)));
@@ -1353,39 +1356,45 @@ static void iter_body(Ctx& c, int j, cudaStream_t st) {
     else precond_newest(c, zj, bt, st);
     op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
     const double k1 = j + 1;
-    int npt = 0;                 // partial sums of ||w'||^2
+    int npt = 0;                 // partial sums of ||w'||^2 (double-float basis)
+    const GsNorm nm{c.gscnt, c.gsflag, c.nrm, c.dgks_eta2};
+    const GivensArgs gv{c.Hm, m + 1, j, c.h1v, c.h2v, c.nrm, c.cs, c.sn, c.g, c.status, status_slot(c, j)};
+    const int ndot = c.kdf ? 2 : dot_launches(n, nb);
     {
-        Prof pr(c, BAH_K_DOT, st, nb * (k1 + 1) * n * 16.0, 2);
+        Prof pr(c, BAH_K_DOT, st, nb * (k1 + 1) * n * 16.0, ndot);
         if (c.kdf) launch_dot_norm_df(Vd, j + 1, Wd, n, c.partial, c.h1v, nullptr, nb, ks, st);
-        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h1v, nullptr, nb, ks, st);
+        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h1v, nullptr, c.gscnt, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_AXPY, st, nb * (k1 + 2) * n * 16.0);
         if (c.kdf) npt = launch_axpy_norm_df(Vd, j + 1, c.h1v, Wd, n, c.dpart, nullptr, nb, ks, st);
-        else npt = launch_axpy_norm(c.VL, c.VE, j + 1, c.h1v, c.W, n, c.dpart, nullptr, nb, ks, st);
+        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h1v, c.W, n, c.dpart, 1, nm, nb, ks, st);
     }
-    {
+    if (c.kdf) {
         Prof pr(c, BAH_K_NORM, st, 0.0);
         launch_dgks_decide(c.dpart, npt, c.h1v, j + 1, c.gsflag, c.nrm, nb, ks, st, c.dgks_eta2);
     }
     {
-        Prof pr(c, BAH_K_DOT, st, 0.0, 2);      // runs only where the flag is set (bytes counted as zero)
+        Prof pr(c, BAH_K_DOT, st, 0.0, ndot);   // runs only where the flag is set (bytes counted as zero)
         if (c.kdf) launch_dot_norm_df(Vd, j + 1, Wd, n, c.partial, c.h2v, c.gsflag, nb, ks, st);
-        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h2v, c.gsflag, nb, ks, st);
+        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h2v, c.gsflag, c.gscnt, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_AXPY, st, 0.0);
         if (c.kdf) launch_axpy_norm_df(Vd, j + 1, c.h2v, Wd, n, c.dpart, c.gsflag, nb, ks, st);
-        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h2v, c.W, n, c.dpart, c.gsflag, nb, ks, st);
+        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h2v, c.W, n, c.dpart, 2, nm, nb, ks, st);
     }
     {
-        Prof pr(c, BAH_K_SMALL, st, nb * n * 32.0, 3);
-        launch_pass2_norm(c.dpart, npt, c.gsflag, c.nrm, nb, ks, st);
-        launch_arnoldi_givens(c.Hm, m + 1, c.h1v, c.h2v, c.nrm, j, c.cs, c.sn, c.g, c.status, nb, ks, st);
-        if (c.kdf) launch_scale_copy_df(c.W, false, c.nrm, 2, Vd + (size_t)(j + 1) * n, n, n, ks.sv, nb, ks, st);
-        else store_basis(c, c.W, 2, j + 1, st);
+        // the status goes to its pinned slot from the Givens update itself
+        Prof pr(c, BAH_K_SMALL, st, nb * n * 32.0, c.kdf ? 3 : 1);
+        if (c.kdf) {
+            launch_pass2_norm(c.dpart, npt, c.gsflag, c.nrm, nb, ks, st);
+            launch_arnoldi_givens(gv, nb, ks, st);
+            launch_scale_copy_df(c.W, false, c.nrm, 2, Vd + (size_t)(j + 1) * n, n, n, ks.sv, nb, ks, st);
+        } else {
+            store_basis(c, c.W, 2, j + 1, st, &gv);
+        }
     }
-    cudaMemcpyAsync(status_slot(c, j), c.status, 4 * (size_t)nb * sizeof(double), cudaMemcpyDeviceToHost, st);
 }
 
 static int ensure_graph(Ctx& c, int j) {
