@@ -240,6 +240,8 @@ template <class V, class CC> struct LvlSet {
 };
 
 constexpr int kMaxLevels = 16;
+constexpr int kClusterRhs = 3;       // most right-hand sides of a cluster multigrid launch
+constexpr int kClusterCoarse = 256;  // most points of its coarsest level
 // shared-memory-resident cluster multigrid: levels l0 .. L-1 of
 // one block set, one cluster per block and right-hand side; lv[k] is level
 // l0 + k, its rows split in slabs of rp rows per CTA, and off_* are byte
@@ -264,11 +266,11 @@ struct SmArgs {
 };
 // fills the shared-memory layout of a (n1, n2, slot counts per level from l0);
 // returns the bytes of dynamic shared memory per CTA
-size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs, int mode,
+size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs,
                    int rm);
 // sets the kernel attributes; returns how many clusters of cs CTAs fit (0: none)
-int smmg_prepare(int rm, int cs, size_t smem, int mode);
-int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, int mode, cudaStream_t st);
+int smmg_prepare(int rm, int cs, size_t smem);
+int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, cudaStream_t st);
 
 // right-hand-side batching: element strides between consecutive right-hand
 // sides for up to three pointers of a launch (blockIdx.y or .z is the

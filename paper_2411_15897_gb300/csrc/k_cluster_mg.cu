@@ -45,12 +45,9 @@ __device__ __forceinline__ uint32_t mapa_rank(uint32_t local_addr, unsigned rank
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
     return r;
 }
-template <class V> __device__ __forceinline__ V ld_cluster_at(uint32_t cluster_addr) {
-    V v;
-    if constexpr (sizeof(V) == 8)
-        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr));
-    else
-        asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(cluster_addr));
+__device__ __forceinline__ float2 ld_cluster_at(uint32_t cluster_addr) {
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr));
     return v;
 }
 template <int BYTES> __device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
@@ -59,8 +56,9 @@ template <int BYTES> __device__ __forceinline__ void cp_async(uint32_t dst, cons
 
 }  // namespace
 
-template <int MODE, int RM>
+template <int RM>
 __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
+    constexpr int MODE = BAH_MIXED;
     using V = typename Prec<MODE>::V;
     using CC = typename Prec<MODE>::CC;
     using R = typename Prec<MODE>::R;
@@ -165,7 +163,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
             const int h = (int)(((float)e + 0.5f) * L.inv_p), col = e - h * P - G;
             const int row = h < RZ ? r0 - RZ + h : r0 + rows + h - RZ;
             const bool in = row >= 0 && row < L.n2 && col >= 0 && col < L.n1;
-            halo[e] = in ? ld_cluster_at<V>(row_addr(L, xin, row) + (uint32_t)col * kV) : czero<V>();
+            halo[e] = in ? ld_cluster_at(row_addr(L, xin, row) + (uint32_t)col * kV) : czero<V>();
         }
         __syncthreads();
         const V* b = vec(L.off_b);
@@ -239,7 +237,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
 #pragma unroll
                     for (int f = 0; f < 4; ++f) {
                         const bool ok = rok && wxs[f] != R(0);
-                        v[e * 4 + f] = ld_cluster_at<V>(ra + (uint32_t)(ok ? bx + f : 0) * kV);
+                        v[e * 4 + f] = ld_cluster_at(ra + (uint32_t)(ok ? bx + f : 0) * kV);
                     }
                 }
 #pragma unroll
@@ -273,7 +271,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
             for (int e = 0; e < 2; ++e) {
                 const uint32_t ra = row_addr(Lc, Lc.off_x, cz[e]);
 #pragma unroll
-                for (int f = 0; f < 2; ++f) v[e * 2 + f] = ld_cluster_at<V>(ra + (uint32_t)cx[f] * kV);
+                for (int f = 0; f < 2; ++f) v[e * 2 + f] = ld_cluster_at(ra + (uint32_t)cx[f] * kV);
             }
             const int o = at(L, r, i);
             V acc = x[o];
@@ -293,7 +291,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
         const int npc = L.n1 * L.n2, own = nown(L), g0 = p0(L);
         int4* gath = reinterpret_cast<int4*>(sm + a.off_g);
         const int eg = dense_load<V, R>(gath, npc, reinterpret_cast<int*>(sm + a.off_r), [&](int g) {
-            return ld_cluster_at<V>(row_addr_b(L, g / L.n1) + (uint32_t)(g % L.n1) * kV);
+            return ld_cluster_at(row_addr_b(L, g / L.n1) + (uint32_t)(g % L.n1) * kV);
         });
         V* x = vec(L.off_x);
         const int lane = tid & 31;
@@ -458,13 +456,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_cluster_mg(SmArgs a) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-template <int MODE> static const void* smmg_fn(int rm) {
-    return rm <= 1 ? (const void*)k_cluster_mg<MODE, 1> : (const void*)k_cluster_mg<MODE, 2>;
-}
+static auto smmg_fn(int rm) { return rm <= 1 ? k_cluster_mg<1> : k_cluster_mg<2>; }
 
-size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs, int mode, int rm) {
-    const size_t vb = mode == BAH_MIXED ? sizeof(float2) : sizeof(double2);
-    const size_t cb = mode == BAH_MIXED ? sizeof(__nv_bfloat162) : sizeof(double2);
+size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max, int nlev, int cs, int rm) {
+    const size_t vb = sizeof(float2), cb = sizeof(__nv_bfloat162);
     size_t off = 0, halo = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -500,8 +495,8 @@ size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max
     return off;
 }
 
-int smmg_prepare(int rm, int cs, size_t smem, int mode) {
-    const void* fn = mode == BAH_MIXED ? smmg_fn<BAH_MIXED>(rm) : smmg_fn<BAH_FP64>(rm);
+int smmg_prepare(int rm, int cs, size_t smem) {
+    const void* fn = (const void*)smmg_fn(rm);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         (cs > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         cudaGetLastError();
@@ -526,7 +521,7 @@ int smmg_prepare(int rm, int cs, size_t smem, int mode) {
     return n;
 }
 
-int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, int mode, cudaStream_t st) {
+int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs * a.nb * nrhs);
     cfg.blockDim = dim3(kSmThreads);
@@ -541,9 +536,7 @@ int launch_cluster_mg(const SmArgs& a, int rm, int nrhs, int cs, size_t smem, in
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    auto fn = mode == BAH_MIXED ? (rm <= 1 ? k_cluster_mg<BAH_MIXED, 1> : k_cluster_mg<BAH_MIXED, 2>)
-                                : (rm <= 1 ? k_cluster_mg<BAH_FP64, 1> : k_cluster_mg<BAH_FP64, 2>);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, smmg_fn(rm), a);
     return e == cudaSuccess ? 0 : (int)e;
 }
 

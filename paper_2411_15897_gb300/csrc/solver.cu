@@ -359,7 +359,7 @@ struct MG {
                 for (int b = 0; b < 3; ++b)
                     ns[k] = std::max(ns[k], (2 * c.s64[l0 + k][b].rx + 1) * (2 * c.s64[l0 + k][b].rz + 1));
             }
-            smmg_layout(a, n1s, n2s, ns, nlev, c.sm_cs, MODE, c.sm_rm);
+            smmg_layout(a, n1s, n2s, ns, nlev, c.sm_cs, c.sm_rm);
             for (int k = 0; k < nlev; ++k) a.lv[k].w = weight(c, l0 + k);
             a.b0 = b0; a.nb = nb; a.nu_pre = c.o.nu_pre; a.nu_post = c.o.nu_post; a.intergrid = c.o.intergrid;
             a.wcycle = c.o.cycle == BAH_CYCLE_W; a.warm = warm; a.active = bt.active;
@@ -379,7 +379,7 @@ struct MG {
             const double npc = (double)c.ln1[c.L - 1] * c.ln2[c.L - 1];
             bytes += nb * bt.nr * (npc * npc * 16.0 + (double)c.ln1[l0] * c.ln2[l0] * sizeof(V) * (warm ? 3 : 2));
             Prof pr(c, BAH_K_CLUSTER, st, bytes);
-            launch_cluster_mg(a, c.sm_rm, bt.nr, c.sm_cs, c.sm_bytes, MODE, st);
+            launch_cluster_mg(a, c.sm_rm, bt.nr, c.sm_cs, c.sm_bytes, st);
         }
     }
 
@@ -425,7 +425,12 @@ struct MG {
         for (int z = 0; z < nb; ++z) { cb[z] = (V*)c.vB[l + 1][b0 + z]; cx[z] = (V*)c.vX[l + 1][b0 + z]; }
         const bool wcyc = c.o.cycle == BAH_CYCLE_W;
         auto coarse_visits = [&]() {
-            if (c.sm_l0 == l + 1) {
+            // the cluster kernel keeps 16 SMs per block and right-hand side, 152 SMs hold 8
+            // clusters, and from four right-hand sides on the level kernels, which read a
+            // stencil once for several of them, are faster (256 x 256, V(1,2), ten steps of
+            // 1, 2, 3, 4, 8 sources: 2.1, 2.3, 3.0, 4.8 ms from two on with clusters,
+            // 2.2, 2.5, 2.9, 4.1 ms without; 32 sources of 1024 x 512: 188.6 and 182.0 ms)
+            if (MODE == BAH_MIXED && c.sm_l0 == l + 1 && bt.nr <= kClusterRhs) {
                 smem_levels(c, b0, nb, bt, st);
                 if (wcyc && l + 1 < c.L - 1) smem_levels(c, b0, nb, bt, st, true);
             } else {
@@ -1082,8 +1087,13 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     }
     // shared-memory cluster multigrid (mixed mode; BAH_SMEM_MG=0 turns it off):
     // from the first level below the fine grid whose levels, down to the
-    // coarsest, fit in the shared memory of one cluster (16 CTAs, else 8)
-    if (c.mode == BAH_MIXED && c.L >= 3 && c.L <= kMaxLevels) {
+    // coarsest, fit in the shared memory of one cluster (16 CTAs, else 8).  The
+    // coarsest solve runs on those 16 SMs too: with more than kClusterCoarse unknowns the
+    // level kernels, whose dense solve spreads over the chip, are faster (one source,
+    // coarsest level 400, 576, 676, 800 points: 4.12, 4.68, 5.18, 5.60 ms with the cluster,
+    // 4.03, 4.45, 4.73, 4.66 ms without; 256 points: 5.53 and 5.71 ms, a W-cycle 9.2 and
+    // 10.4).  FP64 mode: 14.62 ms with its small levels in a cluster, 14.56 without.
+    if (c.mode == BAH_MIXED && c.L >= 3 && c.L <= kMaxLevels && c.ln1[c.L - 1] * c.ln2[c.L - 1] <= kClusterCoarse) {
         bool on = true;
         if (const char* e = getenv("BAH_SMEM_MG")) on = e[0] != '0';
         int dev = 0, optin = 0;
@@ -1104,9 +1114,9 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
             for (int cs = 16; cs >= 8 && c.sm_l0 == 0; cs /= 2) {
                 SmArgs a;
                 std::memset(&a, 0, sizeof(a));
-                const size_t bytes = smmg_layout(a, n1s, n2s, ns, nlev, cs, c.mode, rm);
+                const size_t bytes = smmg_layout(a, n1s, n2s, ns, nlev, cs, rm);
                 if (bytes > (size_t)optin) continue;
-                if (smmg_prepare(rm, cs, bytes, c.mode) >= 1) {
+                if (smmg_prepare(rm, cs, bytes) >= 1) {
                     c.sm_l0 = l0; c.sm_cs = cs; c.sm_rm = rm; c.sm_bytes = bytes;
                 }
             }
