@@ -239,6 +239,19 @@ template <class V, class CC> struct LvlSet {
     int staged;        // mixed mode: Galerkin levels by k_galerkin.cu (0: the plain kernels)
 };
 
+// the first sweep from zero of the level below, x = w D^{-1} b, written by the kernel that
+// forms b (x[y] == nullptr: not wanted); d: the diagonals (FP64 mode: their inverses)
+template <class V, class CC> struct FirstSweep {
+    V* x[3];
+    const CC* d[3];
+    size_t sx;         // element stride between right-hand sides
+    double w;
+};
+template <int MODE, class V, class CC> __device__ __forceinline__ V first_sweep(const CC* d, int t, V b, double w) {
+    if constexpr (MODE == BAH_FP64) return cscale(cmul(d[t], b), w);
+    else return cscale(cdiv(b, ldc(d[t])), (typename VecTraits<V>::R)w);
+}
+
 constexpr int kMaxLevels = 16;
 constexpr int kClusterRhs = 3;       // most right-hand sides of a cluster multigrid launch
 constexpr int kClusterCoarse = 256;  // most points of its coarsest level
@@ -329,7 +342,8 @@ void launch_residual(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::C
                      const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>* f5, cudaStream_t st);
 template <int MODE>
 void launch_restrict(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fine,
-                     typename Prec<MODE>::V* const* coarse_b, int intergrid, cudaStream_t st, size_t coarse_stride = 0);
+                     typename Prec<MODE>::V* const* coarse_b, int intergrid, cudaStream_t st, size_t coarse_stride,
+                     const FirstSweep<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fs);
 template <int MODE>
 void launch_prolong_add(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fine,
                         const typename Prec<MODE>::V* const* coarse_x, cudaStream_t st, size_t coarse_stride = 0);
@@ -342,7 +356,7 @@ int fine_prepare();     // once per context, before the first launch
 template <int MODE>
 void launch_fine_down(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
                       const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f5, double w,
-                      typename Prec<MODE>::V* const* coarse_b, int intergrid, size_t coarse_stride, cudaStream_t st);
+                      typename Prec<MODE>::V* const* coarse_b, int intergrid, size_t coarse_stride, const FirstSweep<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fs, cudaStream_t st);
 template <int MODE>
 void launch_fine_up(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
                     const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f5, double w, int sweeps, bool from_b,

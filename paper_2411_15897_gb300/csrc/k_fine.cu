@@ -103,6 +103,7 @@ template <int MODE, int TYPE>
 __device__ __forceinline__ void fine_down(const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f,
                                           const typename Prec<MODE>::V* __restrict__ b, typename Prec<MODE>::R w,
                                           typename Prec<MODE>::V* __restrict__ bc, int intergrid,
+                                          typename Prec<MODE>::V* __restrict__ x1, const typename Prec<MODE>::CC* d1, double w1c,
                                           typename Prec<MODE>::V* xs) {
     using V = typename Prec<MODE>::V;
     using R = typename Prec<MODE>::R;
@@ -155,6 +156,7 @@ __device__ __forceinline__ void fine_down(const Fine5<typename Prec<MODE>::C, ty
             }
         }
         bc[(size_t)J * n1c + I] = acc;
+        if (x1) x1[(size_t)J * n1c + I] = valid_pt(TYPE, I, J) ? first_sweep<MODE>(d1, J * n1c + I, acc, w1c) : czero<V>();
     }
 }
 
@@ -256,12 +258,13 @@ __device__ __forceinline__ void fine_up(const Fine5<typename Prec<MODE>::C, type
 
 }  // namespace
 
-// b_c = R (b - A x), x = w D^{-1} b
+// b_c = R (b - A x), x = w D^{-1} b, and (fs) the coarse level's first sweep
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, kMinCtas<MODE>)
     k_fine_down(LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC> s,
                 Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC> f, typename Prec<MODE>::R w,
-                PtrSet<typename Prec<MODE>::V> cb, int intergrid) {
+                PtrSet<typename Prec<MODE>::V> cb, int intergrid,
+                FirstSweep<typename Prec<MODE>::V, typename Prec<MODE>::CC> fs) {
     pdl_prologue();
     using V = typename Prec<MODE>::V;
     const int rr = blockIdx.z;
@@ -271,9 +274,13 @@ __global__ void __launch_bounds__(kThreads, kMinCtas<MODE>)
     V* xs = reinterpret_cast<V*>(fine_raw);             // (kH + 2) x kP, then kH x kW
     const V* b = B.b + rr * B.sb;
     V* bc = pick(cb, (int)blockIdx.y) + rr * cb.s;
-    if (B.type == 0) fine_down<MODE, 0>(f, b, w, bc, intergrid, xs);
-    else if (B.type == 1) fine_down<MODE, 1>(f, b, w, bc, intergrid, xs);
-    else fine_down<MODE, 2>(f, b, w, bc, intergrid, xs);
+    const int y = blockIdx.y;
+    V* x1 = y == 0 ? fs.x[0] : (y == 1 ? fs.x[1] : fs.x[2]);
+    const auto* d1 = y == 0 ? fs.d[0] : (y == 1 ? fs.d[1] : fs.d[2]);
+    if (x1) x1 += rr * fs.sx;
+    if (B.type == 0) fine_down<MODE, 0>(f, b, w, bc, intergrid, x1, d1, fs.w, xs);
+    else if (B.type == 1) fine_down<MODE, 1>(f, b, w, bc, intergrid, x1, d1, fs.w, xs);
+    else fine_down<MODE, 2>(f, b, w, bc, intergrid, x1, d1, fs.w, xs);
 }
 
 // x_out = NS Jacobi sweeps from x + P e_c; x is w D^{-1} b (FROMB: the state after
@@ -306,13 +313,14 @@ template <int MODE> static constexpr size_t fine_smem() {
 template <int MODE>
 void launch_fine_down(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
                       const Fine5<typename Prec<MODE>::C, typename Prec<MODE>::CC>& f5, double w,
-                      typename Prec<MODE>::V* const* coarse_b, int intergrid, size_t coarse_stride, cudaStream_t st) {
+                      typename Prec<MODE>::V* const* coarse_b, int intergrid, size_t coarse_stride,
+                      const FirstSweep<typename Prec<MODE>::V, typename Prec<MODE>::CC>& fs, cudaStream_t st) {
     PtrSet<typename Prec<MODE>::V> cb;
     for (int z = 0; z < 3; ++z) cb.p[z] = z < s.nb ? coarse_b[z] : nullptr;
     cb.s = coarse_stride;
     const int n1c = s.n1 / 2, n2c = s.n2 / 2;
     const dim3 g(((n1c + kCw - 1) / kCw) * ((n2c + kCh - 1) / kCh), s.nb, s.nrhs);
-    launch_pdl(k_fine_down<MODE>, g, dim3(kThreads), fine_smem<MODE>(), st, s, f5, (typename Prec<MODE>::R)w, cb, intergrid);
+    launch_pdl(k_fine_down<MODE>, g, dim3(kThreads), fine_smem<MODE>(), st, s, f5, (typename Prec<MODE>::R)w, cb, intergrid, fs);
 }
 template <int MODE>
 void launch_fine_up(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>::CC>& s,
@@ -358,7 +366,8 @@ int fine_prepare() {
 
 #define INST(M)                                                                                                     \
     template void launch_fine_down<M>(const LvlSet<Prec<M>::V, Prec<M>::CC>&, const Fine5<Prec<M>::C, Prec<M>::CC>&, \
-                                      double, Prec<M>::V* const*, int, size_t, cudaStream_t);                       \
+                                      double, Prec<M>::V* const*, int, size_t,                                        \
+                                      const FirstSweep<Prec<M>::V, Prec<M>::CC>&, cudaStream_t);                      \
     template void launch_fine_up<M>(const LvlSet<Prec<M>::V, Prec<M>::CC>&, const Fine5<Prec<M>::C, Prec<M>::CC>&,   \
                                     double, int, bool, const Prec<M>::V* const*, size_t, cudaStream_t);
 INST(BAH_FP64)

@@ -211,22 +211,24 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_dot(const int4* __restrict
         for (int u = 0; u < kGsWarps; ++u) s += sum[u][2 * 64];
         partial[(size_t)k * gridDim.x + blockIdx.x] = make_double2(s, 0.0);
     }
-    if (!LAST || !last_cta(cnt + r, gridDim.x * gridDim.y)) return;
-    // few partial sums: added here, four lanes to a row
-    for (int y = threadIdx.x >> 2; y < ((k + 1 + 7) & ~7); y += kGsThreads / 4) {
-        double2 s = make_double2(0.0, 0.0);
-        if (y <= k)
-            for (int e = threadIdx.x & 3; e < gridDim.x; e += 4) {
-                const double2 a = __ldcg(partial + (size_t)y * gridDim.x + e);
-                s.x += a.x;
-                s.y += a.y;
-            }
+    if constexpr (LAST) {
+        if (!last_cta(cnt + r, gridDim.x * gridDim.y)) return;
+        // few partial sums: added here, four lanes to a row
+        for (int y = threadIdx.x >> 2; y < ((k + 1 + 7) & ~7); y += kGsThreads / 4) {
+            double2 s = make_double2(0.0, 0.0);
+            if (y <= k)
+                for (int e = threadIdx.x & 3; e < gridDim.x; e += 4) {
+                    const double2 a = __ldcg(partial + (size_t)y * gridDim.x + e);
+                    s.x += a.x;
+                    s.y += a.y;
+                }
 #pragma unroll
-        for (int o = 1; o < 4; o <<= 1) {
-            s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-            s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+            for (int o = 1; o < 4; o <<= 1) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+                s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+            }
+            if ((threadIdx.x & 3) == 0 && y <= k) out[r * ks.so + y] = s;
         }
-        if ((threadIdx.x & 3) == 0 && y <= k) out[r * ks.so + y] = s;
     }
 }
 

@@ -389,8 +389,9 @@ struct MG {
     // values already in out[z].  A W-cycle visits the coarse problem twice: the
     // second visit starts from the first one's result (Sec. 2.2, two recursive
     // calls), except when the coarse level is the coarsest, solved exactly once.
+    // swept: from zero, with the first sweep done by the kernel that formed the right-hand side.
     static void cycle(Ctx& c, int l, int b0, int nb, V* const* out, size_t ostride, const Batch& bt,
-                      cudaStream_t st, bool x0 = false) {
+                      cudaStream_t st, bool x0 = false, bool swept = false) {
         const size_t npl = (size_t)c.ln1[l] * c.ln2[l];
         const double vs = sizeof(V), ccs = sizeof(CC);
         const double nr = bt.nr;
@@ -424,17 +425,28 @@ struct MG {
         V* cx[3];
         for (int z = 0; z < nb; ++z) { cb[z] = (V*)c.vB[l + 1][b0 + z]; cx[z] = (V*)c.vX[l + 1][b0 + z]; }
         const bool wcyc = c.o.cycle == BAH_CYCLE_W;
+        // the cluster kernel keeps 16 SMs per block and right-hand side, 152 SMs hold 8
+        // clusters, and from four right-hand sides on the level kernels, which read a
+        // stencil once for several of them, are faster (256 x 256, V(1,2), ten steps of
+        // 2, 3, 4, 8 sources: 2.1, 2.3, 3.0, 4.8 ms with clusters, 2.2, 2.5, 2.9, 4.1 ms
+        // without; 32 sources of 1024 x 512: 188.6 and 182.0 ms)
+        const bool to_cluster = MODE == BAH_MIXED && c.sm_l0 == l + 1 && bt.nr <= kClusterRhs;
+        // the level below starts from zero: its first sweep goes with the restriction, into the
+        // buffer its own visit starts in
+        FirstSweep<V, CC> fs{{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}, nplc, weight(c, std::min(l + 1, c.L - 1))};
+        const bool sweep_below = !to_cluster && l + 1 < c.L - 1 && c.o.nu_pre >= 1;
+        for (int z = 0; z < nb && sweep_below; ++z) {
+            fs.x[z] = (c.o.nu_pre - 1 + c.o.nu_post) & 1 ? (V*)c.vT[l + 1][b0 + z] : cx[z];
+            const StencilF64& S = c.s64[l + 1][b0 + z];
+            if constexpr (MODE == BAH_FP64) fs.d[z] = c.idg[l + 1][b0 + z];
+            else fs.d[z] = (const CC*)c.sst[l + 1][b0 + z] + (size_t)(S.rz * (2 * S.rx + 1) + S.rx) * nplc;
+        }
         auto coarse_visits = [&]() {
-            // the cluster kernel keeps 16 SMs per block and right-hand side, 152 SMs hold 8
-            // clusters, and from four right-hand sides on the level kernels, which read a
-            // stencil once for several of them, are faster (256 x 256, V(1,2), ten steps of
-            // 1, 2, 3, 4, 8 sources: 2.1, 2.3, 3.0, 4.8 ms from two on with clusters,
-            // 2.2, 2.5, 2.9, 4.1 ms without; 32 sources of 1024 x 512: 188.6 and 182.0 ms)
-            if (MODE == BAH_MIXED && c.sm_l0 == l + 1 && bt.nr <= kClusterRhs) {
+            if (to_cluster) {
                 smem_levels(c, b0, nb, bt, st);
                 if (wcyc && l + 1 < c.L - 1) smem_levels(c, b0, nb, bt, st, true);
             } else {
-                cycle(c, l + 1, b0, nb, cx, nplc, bt, st);
+                cycle(c, l + 1, b0, nb, cx, nplc, bt, st, false, sweep_below);
                 if (wcyc && l + 1 < c.L - 1) cycle(c, l + 1, b0, nb, cx, nplc, bt, st, true);
             }
         };
@@ -449,7 +461,7 @@ struct MG {
         if (fused_up && c.o.nu_pre == 1) {
             {
                 Prof pr(c, BAH_K_RESIDUAL, st, cb_ + nr * nb * npl * vs * 1.25);
-                launch_fine_down<MODE>(set(c, l, b0, nb, nullptr, 0, cur, cur_s, bt), fi, w, cb, c.o.intergrid, nplc, st);
+                launch_fine_down<MODE>(set(c, l, b0, nb, nullptr, 0, cur, cur_s, bt), fi, w, cb, c.o.intergrid, nplc, fs, st);
             }
             coarse_visits();
             {
@@ -472,7 +484,7 @@ struct MG {
                     swap_cur();
                 }
             } else if (c.o.nu_pre >= 1) {
-                {
+                if (!swept) {
                     Prof pr(c, BAH_K_JACOBI, st, nr * nb * npl * (2.0 * vs + ccs));
                     launch_jacobi<MODE>(set(c, l, b0, nb, nullptr, 0, cur, cur_s, bt), pf5, w, 1, st);
                 }
@@ -494,7 +506,7 @@ struct MG {
             }
             {
                 Prof pr(c, BAH_K_RESTRICT, st, nr * nb * npl * vs * 1.25);
-                launch_restrict<MODE>(rs, cb, c.o.intergrid, st, nplc);
+                launch_restrict<MODE>(rs, cb, c.o.intergrid, st, nplc, fs);
             }
             // coarse-grid correction
             coarse_visits();
