@@ -83,24 +83,27 @@ PRESETS = {
 WORKLOAD = WORKLOADS["c2"]
 L2_FLUSH_BYTES = 512 << 20
 FP64_PEAK_TFLOPS = 152 * 2.07e9 * 4 / 1e12   # 2 DFMA/clk/SM at the 2070 MHz maximum clock (1.26 TFLOP/s)
-KERNEL_NAMES = {0: "k_elastic_apply", 1: "k_distributor", 2: "k_u_rhs", 3: "k_jacobi", 4: "k_residual",
-                5: "k_restrict", 6: "k_prolong_add", 7: "k_coarse_apply", 8: "k_dot_norm_partial",
-                9: "k_axpy_norm", 10: "k_norm2_partial", 11: "k_update_x", 12: "small kernels",
-                14: "k_cluster_mg"}
-KERNEL_NAMES_3D = {0: "k_apply3", 1: "k_distrib3", 2: "k_urhs3", 3: "k_jacobi3", 4: "k_jacobi3 (residual)",
-                   5: "k_restrict3", 6: "k_prolong3", 7: "k_coarse_apply", 8: "k_dot_norm_partial",
-                   9: "k_axpy_norm", 10: "k_norm2_partial", 11: "k_update_x", 12: "small kernels"}
-# FP64 flops per algorithmic byte of the FP64 classes (2 flops per real FMA):
-#   dot/axpy: 8 flops per complex MAC on 16 streamed bytes; operator: ~84 flops per cell on ~200 bytes
-FP64_FLOP_PER_BYTE = {"dot": 0.5, "axpy": 0.5, "update": 8.0 / 8.0, "operator": 84.0 / 200.0}
+# the kernels of each class (the level-0 visits and the Galerkin levels share a class)
+KERNEL_NAMES = {0: "k_elastic_apply", 1: "k_distributor", 2: "k_u_rhs", 3: "k_fine_up / k_galerkin_level",
+                4: "k_fine_down / k_galerkin_level (residual)", 5: "k_restrict", 6: "k_prolong_add",
+                7: "k_coarse_apply", 8: "k_gs_dot", 9: "k_gs_axpy", 10: "k_norm2_partial", 11: "k_update_x",
+                12: "small kernels", 14: "k_cluster_mg"}
+KERNEL_NAMES_3D = {0: "k_apply3", 1: "k_distrib3", 2: "k_urhs3", 3: "k_fine3 / k_level27",
+                   4: "k_fine3 / k_level27 (residual)", 5: "k_restrict3", 6: "k_prolong3", 7: "k_coarse_apply",
+                   8: "k_gs_dot", 9: "k_gs_axpy", 10: "k_norm2_partial", 11: "k_update_x", 12: "small kernels"}
+# FP64 flops per algorithmic byte of the classes on the FP64 pipe (2 flops per real FMA): solution
+# update, 8 flops per complex MAC on 8 streamed bytes; operator, ~84 flops per cell on ~200 bytes.
+# (The Gram-Schmidt runs on the integer pipe, its basis in 60-bit block fixed point: HBM-bound.)
+FP64_FLOP_PER_BYTE = {"update": 8.0 / 8.0, "operator": 84.0 / 200.0}
 # DRAM bytes (read + write) per launch of a kernel class, averaged over the class's launches in one
 # FGMRES step as they occur in the solve, from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum) of the same build and workload; the summaries under profiles/ give the
 # command and the per-kernel figures.  (workload, class) -> bytes per launch.
 TRAFFIC_PER_LAUNCH = {
-    # 512x512 layered: k_jacobi (level 0) and k_stencil_staged sweeps (level 1), 161 launches over
-    # 10 FGMRES steps of the launch list in profiles/launches_c2_512x512_mixed.md
-    ("c2", "jacobi"): 7.289e6,
+    # 512x512 layered, 10 FGMRES steps of the launch list in profiles/launches_c2_512x512_mixed.md:
+    # k_cluster_mg (21 launches); k_fine_up and the k_galerkin_level sweeps (86 launches)
+    ("c2", "cluster"): 4.294e6,
+    ("c2", "jacobi"): 8.173e6,
 }
 
 
@@ -607,9 +610,9 @@ def run_bah(args):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": statistics.mean(step_ms), "setup_s": setup_s, "higher_is_better": True, "scaling": "strong" if nsrc_all > 1 else "weak", "vs_baseline": None,
         "dtype": (("mixed: bf16 stencils, f32 multigrid, " if prob.dim == 3 else "mixed: bf16 coefficients, f32 multigrid, ")
-                  + "f64 coarsest solve (f64 inverse applied in f64), "
+                  + "f64 coarsest solve (inverse in 60-bit block fixed point), "
                   + ("double-f32 (48-bit) Krylov basis and Gram-Schmidt" if args.krylov == "df"
-                     else "f64 Krylov basis and Gram-Schmidt")
+                     else "f64 Krylov basis and Gram-Schmidt (basis in 60-bit block fixed point)")
                   + (", operator w = H z on the f32 flexible basis in double-f32 arithmetic" if prob.dim == 2 else
                      ", f64 operator")
                   + ", f64 Hessenberg / Givens / true residual / solution"),

@@ -179,7 +179,8 @@ int bah_sizes(const bah_ctx* ctx, long long* vector_len, int* levels);
 /* What the context chose (after defaults were applied): level count, the
  * shift alpha of Eq. 2.8, the coarsest grid's point count, and the first
  * level held in a thread-block cluster's shared memory (0: none) with the
- * CTAs per cluster and the bytes of shared memory per CTA.  The paper has no
+ * CTAs per cluster and the bytes of shared memory per CTA (launches of up to
+ * three right-hand sides; larger batches run the level kernels).  The paper has no
  * counterpart; this is for reporting and tests. */
 typedef struct {
     int       levels;
@@ -303,8 +304,8 @@ int bah_level_stencil(const bah_ctx* ctx, int block, int level, double* out, int
 #define BAH_K_RESIDUAL  4   /* multigrid residual, all levels */
 #define BAH_K_RESTRICT  5   /* restriction (Eq. 4.1, 4.2, 4.4) */
 #define BAH_K_PROLONG   6   /* prolongation + correction */
-#define BAH_K_COARSE    7   /* coarsest-level FP64 inverse applied in FP64 */
-#define BAH_K_DOT       8   /* Gram-Schmidt block dot products (2 kernels) */
+#define BAH_K_COARSE    7   /* coarsest-level inverse (block fixed point, exact sums) */
+#define BAH_K_DOT       8   /* Gram-Schmidt block dot products (1 or 2 kernels) */
 #define BAH_K_AXPY      9   /* Gram-Schmidt update w -= V h */
 #define BAH_K_NORM     10   /* 2-norms (2 kernels) */
 #define BAH_K_UPDATE   11   /* x += Z y */

@@ -10,10 +10,11 @@
 // type 3 (p) at every point; the other points hold structural zeros, which
 // every kernel writes as zero and none reads as an unknown.
 //
-// Each kernel runs one thread per point and bounds-checks every neighbour
-// against the grid before it loads it.  The kernels of the solve's step begin
-// with pdl_prologue() and are launched with programmatic dependent launch; the
-// level kernels run the three displacement blocks of a level in one launch.
+// One thread per point, per column of four planes (level 0) or per pair of points
+// (prolongation); a neighbour outside the grid is loaded at a clamped index and does
+// not count.  The kernels of the solve's step begin with pdl_prologue() and are
+// launched with programmatic dependent launch; the level kernels run the three
+// displacement blocks of a level in one launch.
 #include "bah_internal.cuh"
 #include "op_rows.cuh"
 

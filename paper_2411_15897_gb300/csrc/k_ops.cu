@@ -16,8 +16,6 @@ __device__ __forceinline__ double2 ld64(const V* p, int idx) {
 }
 __device__ __forceinline__ double2 ld64(const float4* p, int idx) { return cdf_to_double2(p[idx]); }
 // preconditioner input in the preconditioner's real type R
-template <class R> __device__ __forceinline__ R ldr_in(const double2& v, int c) { return (R)(c ? v.y : v.x); }
-__device__ __forceinline__ float ldf_in(const double2& v, bool im) { return (float)(im ? v.y : v.x); }
 template <class R> struct InLoad;
 template <> struct InLoad<double> {
     __device__ static double2 get(const double2* p, size_t i) { return p[i]; }

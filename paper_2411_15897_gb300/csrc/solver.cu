@@ -546,7 +546,7 @@ struct MG {
         {
             RhsStride rs;
             rs.s0 = rstride; rs.s1 = np; rs.active = bt.active;
-            Prof pr(c, BAH_K_DISTRIB, st, (double)bt.nr * np * (48.0 + sizeof(C) + sizeof(CC) + vs));
+            Prof pr(c, BAH_K_DISTRIB, st, (double)bt.nr * np * (3.0 * sizeof(RIN) + sizeof(C) + sizeof(CC) + vs));
             launch_distributor<MODE, RIN>(c.n1, c.n2, 1.0 / c.h1, 1.0 / c.h2, f5, r, (V*)c.vB[0][2], st, bt.nr, rs);
         }
         V* outp[1] = {z + 2 * (size_t)np};
@@ -554,7 +554,7 @@ struct MG {
         {
             RhsStride rs;
             rs.s0 = rstride; rs.s1 = zstride; rs.s2 = np; rs.active = bt.active;
-            Prof pr(c, BAH_K_URHS, st, (double)bt.nr * np * (32.0 + 3.0 * vs));
+            Prof pr(c, BAH_K_URHS, st, (double)bt.nr * np * (2.0 * sizeof(RIN) + 3.0 * vs));
             launch_u_rhs<MODE, RIN>(c.n1, c.n2, 1.0 / c.h1, 1.0 / c.h2, r, z + 2 * (size_t)np, (V*)c.vB[0][0],
                                     (V*)c.vB[0][1], st, bt.nr, rs);
         }
