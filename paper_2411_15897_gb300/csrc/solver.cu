@@ -1764,6 +1764,12 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
     BAH_CUDA_TRY(cudaMemsetAsync(x, 0, (size_t)s * n * sizeof(double2), st));
     BAH_CUDA_TRY(cudaMemcpyAsync(c.R, b, (size_t)s * n * sizeof(double2), cudaMemcpyDeviceToDevice, st));
     beta = bn;
+    // a step is queued ahead of the one the host looks at: on every way out, an error's
+    // included, the call leaves nothing of its own running on the context's workspace
+    struct Drain {
+        cudaStream_t st;
+        ~Drain() { cudaStreamSynchronize(st); }
+    } drain{st};
     int total = 0, restarts = 0;
     std::vector<cdx> S0, R, Y;
     std::vector<double> res;
