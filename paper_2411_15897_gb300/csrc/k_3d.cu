@@ -201,8 +201,8 @@ __global__ void __launch_bounds__(256) k_apply3(Op3 op, const Vin* __restrict__ 
         acc.x = fma(-k, v.x, acc.x);
         acc.y = fma(-k, v.y, acc.y);
     };
-    // every neighbour is loaded (at a clamped index) and its coefficient replaced by 0
-    // outside the grid, so that the loads issue together
+    // every neighbour is loaded (at a clamped index) so that the loads issue together, and
+    // replaced by 0 where there is no unknown: what stands in a boundary-normal entry does not count
     const double2 pc = ld(3, p), zero = make_double2(0.0, 0.0);
     double2 out[4];
     double2 div = cscale(pc, -op.cinv[p]);
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(256) k_apply3(Op3 op, const Vin* __restrict__ 
         add(div, op.ih[a], csub(uc, ue));
         const double2 uw = ld(a, pm);
         const double kw = op.cmu[a][pm], ke = op.cmu[a][p];
-        double2 acc = cscale(uw, c[a] >= 2 ? kw : 0.0);
+        double2 acc = cscale(c[a] >= 2 ? uw : zero, kw);
         add(acc, ke, ue);
 #pragma unroll
         for (int bb = 0; bb < 3; ++bb) {
@@ -224,8 +224,8 @@ __global__ void __launch_bounds__(256) k_apply3(Op3 op, const Vin* __restrict__ 
             const int qm = bl ? p - st[bb] : p, qe = bh ? p + st[bb] : p;
             const double km = me[p], kp = me[qe];
             const double2 um = ld(a, qm), up = ld(a, qe);
-            add(acc, bl ? km : 0.0, um);
-            add(acc, bh ? kp : 0.0, up);
+            add(acc, km, bl ? um : zero);
+            add(acc, kp, bh ? up : zero);
         }
         sub(acc, op.ih[a], csub(pc, ld(3, pm)));
         out[a] = lo ? diag_minus(op.dg[a][p], uc, conj, acc) : zero;
@@ -300,8 +300,8 @@ __global__ void __launch_bounds__(256) k_distrib3(Op3 op, const double2* __restr
         const double2 gl = ra[p], gh = ra[qe], rl = rp[qm], rh = rp[qe];
         const double kl = op.cmu[a][qm], kh = op.cmu[a][qe], kp = op.cmu[a][p];
         const double2 zero = make_double2(0.0, 0.0);
-        add(lo ? kl : 0.0, rl);
-        add(hi ? kh : 0.0, rh);
+        add(kl, lo ? rl : zero);
+        add(kh, hi ? rh : zero);
         add(op.ih[a], csub(lo ? gl : zero, hi ? gh : zero));
         k0 += lo && hi ? 2.0 * kp : (lo || hi ? kp : 0.0);
     }
