@@ -497,7 +497,14 @@ size_t smmg_layout(SmArgs& a, const int* n1, const int* n2, const int* nslot_max
 
 int smmg_prepare(int rm, int cs, size_t smem) {
     const void* fn = (const void*)smmg_fn(rm);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    // The attribute is the kernel's, shared by all contexts: it is always set to the most the device
+    // gives a CTA, because a context that set it to its own size would take it from one created before.
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, fn) != cudaSuccess || smem + fa.sharedSizeBytes > (size_t)most ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes) != cudaSuccess ||
         (cs > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         cudaGetLastError();
         return 0;
