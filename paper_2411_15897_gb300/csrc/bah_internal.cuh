@@ -401,6 +401,7 @@ struct KS {                     // per-right-hand-side element strides and activ
 };
 // The FP64 basis in block fixed point (k_gs.cu): vector i's limbs at
 // VL + i * tiles * 256, its tile exponents at VE + i * tiles.
+struct Tiles;       // fix60.cuh
 int gs_prepare();   // once per context, before the first launch
 // One Gram-Schmidt pass: launch_dot_norm, then launch_axpy_norm.  cnt: one counter per
 // right-hand side, zero between launches, with which a kernel's last CTA is found.
@@ -411,17 +412,17 @@ struct GsNorm {
     double* sc;     // scalars, 8 per right-hand side: [2] = ||w'||, [3] counts second passes
     double eta2;
 };
-void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, size_t n, double2* partial, double2* out,
+void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, const Tiles& tl, double2* partial, double2* out,
                      const int* flag, int* cnt, int nrhs, const KS& ks, cudaStream_t st);
-int dot_launches(size_t n, int nrhs);   // launches of launch_dot_norm
+int dot_launches(const Tiles& tl, int nrhs);   // launches of launch_dot_norm
 // coef: the projections, followed by ||w||^2 (launch_dot_norm's out); npart: scratch, GS_CTAS per right-hand side
-void launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
+void launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, const Tiles& tl, double* npart,
                       int pass, const GsNorm& nm, int nrhs, const KS& ks, cudaStream_t st);
 // v = w / sc[slot] as the preconditioner's input (vc, FP64 or rounded to FP32,
 // stride ks.sw) and as a basis vector (vl, ve); with gv also the step's Givens update
 struct GivensArgs;
 template <class Vc>
-void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, size_t n,
+void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, const Tiles& tl,
                         size_t sw, int nrhs, const KS& ks, cudaStream_t st, const GivensArgs* gv = nullptr);
 // flag = 1 (second pass) when ||w'||^2 < eta2 ||w||^2 (DGKS criterion; eta2 = 1/2 classically)
 void launch_dgks_decide(const double* npart, int np, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
@@ -452,16 +453,16 @@ void launch_scale_copy_df(const void* w, bool from64, const double* sc, int slot
 // block FGMRES kernels (k_block.cu); s <= 16 columns; the basis in block fixed
 // point: block i, column a at VL + a * sv + i * tiles * 256 and VE + a * se + i * tiles
 int block_prepare();   // once per context, before the first launch
-void launch_block_dot(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
+void launch_block_dot(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, const Tiles& tl,
                       double2* partial, double2* C, cudaStream_t st);
-void launch_block_gram(int s, const double2* W, size_t n, double2* partial, double2* C, cudaStream_t st);
+void launch_block_gram(int s, const double2* W, const Tiles& tl, double2* partial, double2* C, cudaStream_t st);
 void launch_block_update(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* C, double2* W,
-                         size_t n, cudaStream_t st);
+                         const Tiles& tl, cudaStream_t st);
 void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStream_t st);
 // dst: FP64, or (with vl) rounded to FP32
 template <class Vd>
 void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, int4* vl, int* ve, size_t sv, size_t se,
-                        size_t n, cudaStream_t st);
+                        const Tiles& tl, cudaStream_t st);
 template <class Vz>
 void launch_block_xupdate(const Vz* Z, size_t sz, int k, int s, const double2* Y, double2* X, size_t n,
                           cudaStream_t st);

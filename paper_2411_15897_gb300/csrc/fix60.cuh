@@ -27,7 +27,25 @@ constexpr int kTile = 32 * kTileU;        // entries of a tile: entry u * 32 + l
 constexpr int kExpBad = 0x800;            // exponent of a tile that holds a non-finite entry
 constexpr int kExpMin = 64;
 
-inline __host__ __device__ size_t tiles_of(size_t n) { return (n + kTile - 1) / kTile; }
+// A vector of n entries in components of nc as tiles: a tile belongs to one component (the
+// displacements' and the pressure's entries have unrelated units: in one tile, entries 2^-33 of
+// its largest would keep 27 bits), the last tile of a component is partial.  Tile t's limbs
+// stand at t * kTile.
+struct Tiles {
+    size_t n, nc;
+    unsigned per, count;     // tiles per component and in all
+    Tiles() = default;
+    Tiles(size_t n_, size_t nc_) : n(n_), nc(nc_), per((unsigned)((nc_ + kTile - 1) / kTile)), count(per * (unsigned)(n_ / nc_)) {}
+    size_t padded() const { return (size_t)count * kTile; }
+#ifdef __CUDACC__
+    // first entry of tile t, and the end of its component
+    __device__ __forceinline__ size_t first(unsigned t, size_t& end) const {
+        const unsigned c = (t >= per) + (t >= 2 * per) + (t >= 3 * per);      // at most four components
+        end = (c + 1) * nc;
+        return c * nc + (size_t)(t - c * per) * kTile;
+    }
+#endif
+};
 
 // the exponent field (with the bits below it) of |x|, for the maximum over a tile
 __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }

@@ -33,13 +33,14 @@ __device__ __forceinline__ void bmac(double2& acc, const double2& a, const doubl
     acc.y = fma(a.y, b.x, acc.y);
 }
 
-// one warp: column b's entries of tile t as limbs in g[0 .. kTile); the exponent
-__device__ __forceinline__ int stage_tile(const double2* __restrict__ w, size_t t, size_t n, int4* g, int lane) {
-    const size_t e0 = t * kTile + lane;
+// one warp: a column's entries of tile t as limbs in g[0 .. kTile); the exponent
+__device__ __forceinline__ int stage_tile(const double2* __restrict__ w, size_t t, const Tiles& tl, int4* g, int lane) {
+    size_t end;
+    const size_t e0 = tl.first((unsigned)t, end) + lane;
     double2 x[kTileU];
     int mx = 0;
 #pragma unroll
-    for (int u = 0; u < kTileU; ++u) x[u] = e0 + 32 * u < n ? w[e0 + 32 * u] : make_double2(0.0, 0.0);
+    for (int u = 0; u < kTileU; ++u) x[u] = e0 + 32 * u < end ? w[e0 + 32 * u] : make_double2(0.0, 0.0);
 #pragma unroll
     for (int u = 0; u < kTileU; ++u) mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
     const int eb = tile_exp((int)__reduce_max_sync(0xffffffffu, (unsigned)mx));
@@ -59,13 +60,13 @@ __device__ __forceinline__ int stage_tile(const double2* __restrict__ w, size_t 
 template <int S, bool SELF>
 __global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, const int* __restrict__ VE, size_t sv,
                                                  size_t se, int k, int s, int rpc, const double2* __restrict__ W,
-                                                 size_t n, double2* __restrict__ partial) {
+                                                 Tiles tl, double2* __restrict__ partial) {
     pdl_prologue();
     extern __shared__ __align__(128) int4 g[];                                   // S x kTile
     constexpr int CG = S < 8 ? S : 8, NV = 2 * CG;                // columns and values of one lane reduction
     __shared__ int ew[S];
     __shared__ double sum[kBlkRows][2 * S];
-    const size_t nt = tiles_of(n), npad = nt * kTile;
+    const size_t n = tl.n, nt = tl.count, npad = nt * kTile;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int nrow = SELF ? s : k * s, row0 = blockIdx.y * rpc;
     for (int q = threadIdx.x; q < kBlkRows * 2 * S; q += 256) (&sum[0][0])[q] = 0.0;
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(256, 2) k_bdot(const int4* __restrict__ VL, co
     for (size_t t = blockIdx.x; t < nt; t += gridDim.x) {
         __syncthreads();
         for (int b = wp; b < s; b += 8) {
-            const int e = stage_tile(W + (size_t)b * n, t, n, g + b * kTile, lane);
+            const int e = stage_tile(W + (size_t)b * n, t, tl, g + b * kTile, lane);
             if (lane == 0) ew[b] = e;
         }
         __syncthreads();
@@ -158,27 +159,27 @@ __global__ void __launch_bounds__(128) k_bdot_reduce(const double2* __restrict__
     if (lane == 0) C[q] = t;
 }
 template <int S, bool SELF>
-static void bdot_t(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
+static void bdot_t(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, const Tiles& tl,
                    double2* partial, double2* C, cudaStream_t st) {
     const int rows = SELF ? s : k * s, chunks = (rows + kBlkRows - 1) / kBlkRows;
     const int rpc = ((rows + chunks - 1) / chunks + 7) / 8 * 8;      // equal chunks, whole rounds of the eight warps
     // two CTAs per SM in all, whole rounds of tiles
-    const size_t nt = tiles_of(n), most = std::max(1, RED_CTAS / chunks), per = (nt + most - 1) / most;
+    const size_t nt = tl.count, most = std::max(1, RED_CTAS / chunks), per = (nt + most - 1) / most;
     const int nc = (int)((nt + per - 1) / per);
     launch_pdl(k_bdot<S, SELF>, dim3(nc, chunks), dim3(256), (size_t)s * kTile * sizeof(int4), st, VL, VE, sv, se, k, s, rpc,
-               W, n, partial);
+               W, tl, partial);
     launch_pdl(k_bdot_reduce, dim3((rows * s + 3) / 4), dim3(128), 0, st, (const double2*)partial, nc, rows * s, C);
 }
-void launch_block_dot(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, size_t n,
+void launch_block_dot(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* W, const Tiles& tl,
                       double2* partial, double2* C, cudaStream_t st) {
-    if (s <= 4) bdot_t<4, false>(VL, VE, sv, se, k, s, W, n, partial, C, st);
-    else if (s <= 8) bdot_t<8, false>(VL, VE, sv, se, k, s, W, n, partial, C, st);
-    else bdot_t<16, false>(VL, VE, sv, se, k, s, W, n, partial, C, st);
+    if (s <= 4) bdot_t<4, false>(VL, VE, sv, se, k, s, W, tl, partial, C, st);
+    else if (s <= 8) bdot_t<8, false>(VL, VE, sv, se, k, s, W, tl, partial, C, st);
+    else bdot_t<16, false>(VL, VE, sv, se, k, s, W, tl, partial, C, st);
 }
-void launch_block_gram(int s, const double2* W, size_t n, double2* partial, double2* C, cudaStream_t st) {
-    if (s <= 4) bdot_t<4, true>(nullptr, nullptr, 0, 0, 1, s, W, n, partial, C, st);
-    else if (s <= 8) bdot_t<8, true>(nullptr, nullptr, 0, 0, 1, s, W, n, partial, C, st);
-    else bdot_t<16, true>(nullptr, nullptr, 0, 0, 1, s, W, n, partial, C, st);
+void launch_block_gram(int s, const double2* W, const Tiles& tl, double2* partial, double2* C, cudaStream_t st) {
+    if (s <= 4) bdot_t<4, true>(nullptr, nullptr, 0, 0, 1, s, W, tl, partial, C, st);
+    else if (s <= 8) bdot_t<8, true>(nullptr, nullptr, 0, 0, 1, s, W, tl, partial, C, st);
+    else bdot_t<16, true>(nullptr, nullptr, 0, 0, 1, s, W, tl, partial, C, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -235,16 +236,16 @@ constexpr int kUpG = 8, kUpSlots = 3, kUpU = kTileU / 2, kUpE = 32 * kUpU;
 template <int S>
 __global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL, const int* __restrict__ VE, size_t sv,
                                                     size_t se, int k, int s, const double2* __restrict__ C,
-                                                    double2* __restrict__ W, size_t n) {
+                                                    double2* __restrict__ W, Tiles tl) {
     pdl_prologue();
     extern __shared__ __align__(128) int4 ring[];                                // kUpSlots x kUpG x kUpE
     __shared__ int4 csh[S][32];
-    const size_t nt = tiles_of(n), npad = nt * kTile;
+    const size_t nt = tl.count, npad = nt * kTile;
     const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
     const int rows = k * s, head = rows_head(rows), ngrp = (rows + kUpG - 1) / kUpG;
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
     for (size_t h = blockIdx.x; h < 2 * nt; h += gridDim.x) {
-        const size_t t = h >> 1, eb0 = h * kUpE;                  // tile and first entry
+        const size_t t = h >> 1, eb0 = h * kUpE;                  // tile and its first entry among the padded ones
         auto fetch = [&](int gq) {                                // group gq's rows into its slot
             if (gq < ngrp)
                 for (int e = threadIdx.x; e < kUpG * kUpE; e += 32 * S) {
@@ -303,21 +304,22 @@ __global__ void __launch_bounds__(32 * S) k_bupdate(const int4* __restrict__ VL,
             const int p = (eo - 2 * 1023) - 118;
             double s1 = pow2(p + 60), s2 = pow2(p + 30);
             if (bad) s1 = __longlong_as_double(0x7ff8000000000000ll);
-            double2* w = W + (size_t)b * n;
-            const size_t e0 = eb0 + lane;
+            double2* w = W + (size_t)b * tl.n;
+            size_t end;
+            const size_t e0 = tl.first((unsigned)t, end) + (h & 1) * kUpE + lane;
 #pragma unroll
             for (int u = 0; u < kUpU; ++u)
-                if (e0 + 32 * u < n) w[e0 + 32 * u] = acc.minus(w[e0 + 32 * u], u, s1, s2);
+                if (e0 + 32 * u < end) w[e0 + 32 * u] = acc.minus(w[e0 + 32 * u], u, s1, s2);
         }
     }
 }
 void launch_block_update(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* C, double2* W,
-                         size_t n, cudaStream_t st) {
+                         const Tiles& tl, cudaStream_t st) {
     const size_t smem = (size_t)kUpSlots * kUpG * kUpE * sizeof(int4);
-    const unsigned nt = 2 * (unsigned)tiles_of(n);
-    if (s <= 4) launch_pdl(k_bupdate<4>, dim3(std::min(nt, 1216u)), dim3(128), smem, st, VL, VE, sv, se, k, s, C, W, n);
-    else if (s <= 8) launch_pdl(k_bupdate<8>, dim3(std::min(nt, 608u)), dim3(256), smem, st, VL, VE, sv, se, k, s, C, W, n);
-    else launch_pdl(k_bupdate<16>, dim3(std::min(nt, 304u)), dim3(512), smem, st, VL, VE, sv, se, k, s, C, W, n);
+    const unsigned nt = 2 * tl.count;
+    if (s <= 4) launch_pdl(k_bupdate<4>, dim3(std::min(nt, 1216u)), dim3(128), smem, st, VL, VE, sv, se, k, s, C, W, tl);
+    else if (s <= 8) launch_pdl(k_bupdate<8>, dim3(std::min(nt, 608u)), dim3(256), smem, st, VL, VE, sv, se, k, s, C, W, tl);
+    else launch_pdl(k_bupdate<16>, dim3(std::min(nt, 304u)), dim3(512), smem, st, VL, VE, sv, se, k, s, C, W, tl);
 }
 
 // ---------------------------------------------------------------------------
@@ -375,19 +377,19 @@ void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStre
 template <int S, class Vd>
 __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, const double2* __restrict__ T, Vd* dst,
                                                    int4* __restrict__ vl, int* __restrict__ ve, size_t sv, size_t se,
-                                                   size_t n) {
+                                                   Tiles tl) {
     pdl_prologue();
     extern __shared__ __align__(128) int4 g[];                                   // S x kTile
     __shared__ int ew[S];
     __shared__ int4 csh[S][16];
-    const size_t nt = tiles_of(n);
+    const size_t n = tl.n, nt = tl.count;
     const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
     const double2 c = lane <= b && b < s ? T[lane * s + b] : make_double2(0.0, 0.0);
     const int ec = coef_exp(c), head = 2;
     for (size_t t = blockIdx.x; t < nt; t += gridDim.x) {
         __syncthreads();
         if (b < s) {
-            const int e = stage_tile(W + (size_t)b * n, t, n, g + b * kTile, lane);
+            const int e = stage_tile(W + (size_t)b * n, t, tl, g + b * kTile, lane);
             if (lane == 0) ew[b] = e;
         }
         __syncthreads();                                          // all of the tile is in shared memory: dst may be W
@@ -411,13 +413,14 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
         double s1 = -pow2(p + 60);
         const double s2 = -pow2(p + 30);
         if (bad) s1 = __longlong_as_double(0x7ff8000000000000ll);
-        const size_t e0 = t * kTile + lane;
+        size_t end;
+        const size_t e0 = tl.first((unsigned)t, end) + lane;
         double2 x[kTileU];
         int mx = 0;
 #pragma unroll
         for (int u = 0; u < kTileU; ++u) {
             x[u] = make_double2(0.0, 0.0);
-            if (e0 + 32 * u < n) {
+            if (e0 + 32 * u < end) {
                 x[u] = acc.minus(x[u], u, s1, s2);
                 dst[(size_t)b * n + e0 + 32 * u] = cconv<Vd>(x[u]);
             }
@@ -427,18 +430,18 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
             const int eb = tile_exp((int)__reduce_max_sync(0xffffffffu, (unsigned)mx));
             if (lane == 0) ve[(size_t)b * se + t] = eb;
 #pragma unroll
-            for (int u = 0; u < kTileU; ++u) vl[(size_t)b * sv + e0 + 32 * u] = limbs2(x[u], eb);
+            for (int u = 0; u < kTileU; ++u) vl[(size_t)b * sv + t * kTile + lane + 32 * u] = limbs2(x[u], eb);
         }
     }
 }
 template <class Vd>
 void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, int4* vl, int* ve, size_t sv, size_t se,
-                        size_t n, cudaStream_t st) {
+                        const Tiles& tl, cudaStream_t st) {
     const size_t smem = (size_t)s * kTile * sizeof(int4);
-    const unsigned nt = (unsigned)tiles_of(n);
-    if (s <= 4) launch_pdl(k_bscale<4, Vd>, dim3(std::min(nt, 608u)), dim3(128), smem, st, W, s, T, dst, vl, ve, sv, se, n);
-    else if (s <= 8) launch_pdl(k_bscale<8, Vd>, dim3(std::min(nt, 304u)), dim3(256), smem, st, W, s, T, dst, vl, ve, sv, se, n);
-    else launch_pdl(k_bscale<16, Vd>, dim3(std::min(nt, 152u)), dim3(512), smem, st, W, s, T, dst, vl, ve, sv, se, n);
+    const unsigned nt = tl.count;
+    if (s <= 4) launch_pdl(k_bscale<4, Vd>, dim3(std::min(nt, 608u)), dim3(128), smem, st, W, s, T, dst, vl, ve, sv, se, tl);
+    else if (s <= 8) launch_pdl(k_bscale<8, Vd>, dim3(std::min(nt, 304u)), dim3(256), smem, st, W, s, T, dst, vl, ve, sv, se, tl);
+    else launch_pdl(k_bscale<16, Vd>, dim3(std::min(nt, 152u)), dim3(512), smem, st, W, s, T, dst, vl, ve, sv, se, tl);
 }
 
 // X[b][e] += sum over rows (i, a) < k s of Z_i[a][e] Y[row, b]  (Z FP32 or FP64 complex)
@@ -491,9 +494,9 @@ int block_prepare() {
     return BAH_OK;
 }
 template void launch_block_scale<double2>(const double2*, int, const double2*, double2*, int4*, int*, size_t, size_t,
-                                          size_t, cudaStream_t);
+                                          const Tiles&, cudaStream_t);
 template void launch_block_scale<float2>(const double2*, int, const double2*, float2*, int4*, int*, size_t, size_t,
-                                         size_t, cudaStream_t);
+                                         const Tiles&, cudaStream_t);
 template void launch_block_xupdate<float2>(const float2*, size_t, int, int, const double2*, double2*, size_t,
                                            cudaStream_t);
 template void launch_block_xupdate<double2>(const double2*, size_t, int, int, const double2*, double2*, size_t,

@@ -46,11 +46,11 @@ __device__ __forceinline__ bool last_cta(int* cnt, int total) {
     return last;
 }
 
-// the tile's entries of w (zero beyond n) and its biased exponent
-__device__ __forceinline__ int load_tile(const double2* __restrict__ w, size_t e0, size_t n, double2 (&x)[kTileU]) {
+// the tile's entries of w from this lane's first one, e0 (zero from `end` on), and its biased exponent
+__device__ __forceinline__ int load_tile(const double2* __restrict__ w, size_t e0, size_t end, double2 (&x)[kTileU]) {
     int mx = 0;
 #pragma unroll
-    for (int u = 0; u < kTileU; ++u) x[u] = e0 + 32 * u < n ? w[e0 + 32 * u] : make_double2(0.0, 0.0);
+    for (int u = 0; u < kTileU; ++u) x[u] = e0 + 32 * u < end ? w[e0 + 32 * u] : make_double2(0.0, 0.0);
 #pragma unroll
     for (int u = 0; u < kTileU; ++u) mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
     return tile_exp((int)__reduce_max_sync(0xffffffffu, (unsigned)mx));
@@ -83,7 +83,7 @@ __device__ __forceinline__ void copy16(uint32_t dst, const void* src) {
 
 template <int R, bool LAST>
 __global__ void __launch_bounds__(kGsThreads, 4) k_gs_dot(const int4* __restrict__ VL, const int* __restrict__ VE, int k,
-                                                          int rows, const double2* __restrict__ w, size_t n,
+                                                          int rows, const double2* __restrict__ w, Tiles tl,
                                                           double2* __restrict__ partial, double2* __restrict__ out,
                                                           const int* flag, int* cnt, KS ks) {
     pdl_prologue();
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_dot(const int4* __restrict
             for (int i = threadIdx.x; i <= k; i += kGsThreads) out[r * ks.so + i] = make_double2(0.0, 0.0);
         return;
     }
-    const size_t nt = tiles_of(n), npad = nt * kTile;
+    const size_t nt = tl.count, npad = nt * kTile;
     VL += r * ks.sv;
     VE += r * ks.se;
     w += r * ks.sw;
@@ -127,9 +127,10 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_dot(const int4* __restrict
     __syncwarp();
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     for (size_t t = (size_t)blockIdx.x * kGsWarps + wp; t < nt; t += tstep) {
-        const size_t e0 = t * kTile + lane;
+        size_t end;
+        const size_t e0 = tl.first((unsigned)t, end) + lane;
         double2 x[kTileU];
-        const int ew = load_tile(w, e0, n, x);
+        const int ew = load_tile(w, e0, end, x);
         int4 a[kTileU];
 #pragma unroll
         for (int u = 0; u < kTileU; ++u) a[u] = limbs2(x[u], ew);
@@ -262,8 +263,8 @@ __global__ void __launch_bounds__(128) k_gs_reduce(const double2* __restrict__ p
 
 // CTAs along the tiles: whole rounds of tiles per warp; at most GS_CTAS, and for
 // a batch about two waves in all (a CTA's fixed cost then falls on many tiles)
-static int gs_ctas(size_t n, int nrhs) {
-    const size_t nt = tiles_of(n);
+static int gs_ctas(const Tiles& tl, int nrhs) {
+    const size_t nt = tl.count;
     const size_t most = (size_t)std::max(16, std::min(GS_CTAS, 2 * GS_CTAS / nrhs)) * kGsWarps;
     const size_t per = (nt + most - 1) / most;
     return (int)((nt + per * kGsWarps - 1) / (per * kGsWarps));
@@ -273,9 +274,9 @@ static int gs_ctas(size_t n, int nrhs) {
 // then a group is as small as fills it (one or two rows: all its loads are in flight at
 // once).  Up to kGsFew partial sums a row, the last CTA adds them (one launch less): one
 // source at 64 x 64, k = 20, 7.3 us and 4 us for the sum -> 9.0 us with it.
-void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, size_t n, double2* partial, double2* out,
+void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, const Tiles& tl, double2* partial, double2* out,
                      const int* flag, int* cnt, int nrhs, const KS& ks, cudaStream_t st) {
-    const int nc = gs_ctas(n, nrhs);
+    const int nc = gs_ctas(tl, nrhs);
     const bool split = (size_t)nc * nrhs * 2 <= GS_CTAS;
     int rows = split ? std::min(kGsRows, std::max(1, (k * nc * nrhs + GS_CTAS - 1) / GS_CTAS)) : kGsRows;
     const int groups = (k + rows - 1) / rows;
@@ -285,7 +286,7 @@ void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, siz
     switch (rows) {
 #define BAH_GS_DOT(R)                                                                                                   \
     case R:                                                                                                             \
-        launch_pdl(last ? k_gs_dot<R, true> : k_gs_dot<R, false>, g, b, kGsSmem, st, VL, VE, k, rows, w, n, partial, out, \
+        launch_pdl(last ? k_gs_dot<R, true> : k_gs_dot<R, false>, g, b, kGsSmem, st, VL, VE, k, rows, w, tl, partial, out, \
                    flag, cnt, ks);                                                                                      \
         break;
         BAH_GS_DOT(1) BAH_GS_DOT(2) BAH_GS_DOT(3) BAH_GS_DOT(4) BAH_GS_DOT(5) BAH_GS_DOT(6) BAH_GS_DOT(7) BAH_GS_DOT(8)
@@ -294,7 +295,7 @@ void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, siz
     if (!last) launch_pdl(k_gs_reduce, dim3(1, k + 1, nrhs), dim3(128), 0, st, (const double2*)partial, nc, out, flag, ks);
 }
 
-int dot_launches(size_t n, int nrhs) { return gs_ctas(n, nrhs) <= kGsFew ? 1 : 2; }
+int dot_launches(const Tiles& tl, int nrhs) { return gs_ctas(tl, nrhs) <= kGsFew ? 1 : 2; }
 
 // ---------------------------------------------------------------------------
 // w -= sum_i coef_i V_i, and per-CTA partial sums of |w_new|^2.  One warp per
@@ -405,11 +406,11 @@ __device__ __forceinline__ double gs_sub(double x, long long h, long long c, int
 
 __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restrict__ VL, const int* __restrict__ VE, int k,
                                                            const double2* __restrict__ coef, double2* __restrict__ w,
-                                                           size_t n, double* __restrict__ npart, int pass, GsNorm nm, KS ks) {
+                                                           Tiles tl, double* __restrict__ npart, int pass, GsNorm nm, KS ks) {
     pdl_prologue();
     const int r = blockIdx.z;
     if (inactive_gs(ks, r) || (pass == 2 && nm.flag[r] == 0)) return;
-    const size_t nt = tiles_of(n), npad = nt * kTile;
+    const size_t nt = tl.count, npad = nt * kTile;
     VL += r * ks.sv;
     VE += r * ks.se;
     w += r * ks.sw;
@@ -432,10 +433,11 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restric
                 for (int u = 0; u < kTileU; ++u) copy16(dst + 512u * u, src + 32 * u);
                 ++py;
             } else {
-                const size_t e0 = pt * kTile + lane;
+                size_t end;
+                const size_t e0 = tl.first((unsigned)pt, end) + lane;
 #pragma unroll
                 for (int u = 0; u < kTileU; ++u)
-                    if (e0 + 32 * u < n) copy16(dst + 512u * u, w + e0 + 32 * u);
+                    if (e0 + 32 * u < end) copy16(dst + 512u * u, w + e0 + 32 * u);
                 py = 0;
                 pt += tstep;
             }
@@ -476,10 +478,11 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restric
             if ((i & 7) == 7) gs_carry(hr, cr, hi, ci);
         }
         const double2* wrow = reinterpret_cast<const double2*>(next_row());
-        const size_t e0 = t * kTile + lane;
+        size_t end;
+        const size_t e0 = tl.first((unsigned)t, end) + lane;
 #pragma unroll
         for (int u = 0; u < kTileU; ++u) {
-            if (e0 + 32 * u < n) {
+            if (e0 + 32 * u < end) {
                 double2 x = wrow[32 * u];
                 x.x = gs_sub(x.x, hr[u], cr[u], sb, sc);
                 x.y = gs_sub(x.y, hi[u], ci[u], sb, sc);
@@ -505,12 +508,14 @@ __global__ void __launch_bounds__(kGsThreads, 4) k_gs_axpy(const int4* __restric
 template <int ST>
 __global__ void __launch_bounds__(kGsThreads, ST > 3 ? 2 : 4) k_gs_axpy_split(const int4* __restrict__ VL, const int* __restrict__ VE,
                                                                  int k, const double2* __restrict__ coef,
-                                                                 double2* __restrict__ w, size_t n,
+                                                                 double2* __restrict__ w, Tiles tl,
                                                                  double* __restrict__ npart, int pass, GsNorm nm, KS ks) {
     pdl_prologue();
     const int r = blockIdx.z;
     if (inactive_gs(ks, r) || (pass == 2 && nm.flag[r] == 0)) return;
-    const size_t nt = tiles_of(n), npad = nt * kTile, t = blockIdx.x;
+    const size_t nt = tl.count, npad = nt * kTile, t = blockIdx.x;
+    size_t end;
+    const size_t e0 = tl.first((unsigned)t, end);
     VL += r * ks.sv;
     VE += r * ks.se;
     w += r * ks.sw;
@@ -538,8 +543,8 @@ __global__ void __launch_bounds__(kGsThreads, ST > 3 ? 2 : 4) k_gs_axpy_split(co
     double2 x[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        const size_t e = t * kTile + threadIdx.x + kGsThreads * q;
-        x[q] = e < n ? w[e] : make_double2(0.0, 0.0);
+        const size_t e = e0 + threadIdx.x + kGsThreads * q;
+        x[q] = e < end ? w[e] : make_double2(0.0, 0.0);
     }
     __shared__ int4 csh[kGsWarps][64];
     int ev[2];
@@ -582,10 +587,10 @@ __global__ void __launch_bounds__(kGsThreads, ST > 3 ? 2 : 4) k_gs_axpy_split(co
 #pragma unroll
             for (int z = 0; z < 4; ++z) s[z] += a[z * kTile + e];
         }
-        if (t * kTile + e < n) {
+        if (e0 + e < end) {
             x[q].x = gs_sub(x[q].x, s[0], s[1], sb, sc);
             x[q].y = gs_sub(x[q].y, s[2], s[3], sb, sc);
-            w[t * kTile + e] = x[q];
+            w[e0 + e] = x[q];
             nn = fma(x[q].x, x[q].x, nn);
             nn = fma(x[q].y, x[q].y, nn);
         }
@@ -601,18 +606,18 @@ constexpr size_t kGsDeepSmem = (size_t)kGsWarps * kGsDeep * kTile * sizeof(int4)
 
 // one tile per CTA while all of them run at once (four CTAs to an SM; with a CTA or two to
 // an SM the deeper ring)
-void launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, size_t n, double* npart,
+void launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, const Tiles& tl, double* npart,
                       int pass, const GsNorm& nm, int nrhs, const KS& ks, cudaStream_t st) {
-    const size_t nt = tiles_of(n);
+    const size_t nt = tl.count;
     const dim3 b(kGsThreads);
     if (nt * nrhs <= GS_CTAS / 2)
-        launch_pdl(k_gs_axpy_split<kGsDeep>, dim3((unsigned)nt, 1, nrhs), b, kGsDeepSmem, st, VL, VE, k, coef, w, n, npart, pass,
+        launch_pdl(k_gs_axpy_split<kGsDeep>, dim3((unsigned)nt, 1, nrhs), b, kGsDeepSmem, st, VL, VE, k, coef, w, tl, npart, pass,
                    nm, ks);
     else if (nt * nrhs <= GS_CTAS)
-        launch_pdl(k_gs_axpy_split<kGsStages>, dim3((unsigned)nt, 1, nrhs), b, kGsSmem, st, VL, VE, k, coef, w, n, npart, pass,
+        launch_pdl(k_gs_axpy_split<kGsStages>, dim3((unsigned)nt, 1, nrhs), b, kGsSmem, st, VL, VE, k, coef, w, tl, npart, pass,
                    nm, ks);
     else
-        launch_pdl(k_gs_axpy, dim3(gs_ctas(n, nrhs), 1, nrhs), b, kGsSmem, st, VL, VE, k, coef, w, n, npart, pass, nm, ks);
+        launch_pdl(k_gs_axpy, dim3(gs_ctas(tl, nrhs), 1, nrhs), b, kGsSmem, st, VL, VE, k, coef, w, tl, npart, pass, nm, ks);
 }
 
 int gs_prepare() {
@@ -635,14 +640,14 @@ int gs_prepare() {
 template <class Vc>
 __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restrict__ w, const double* sc, int slot,
                                                          Vc* __restrict__ vc, int4* __restrict__ vl,
-                                                         int* __restrict__ ve, size_t n, size_t sw, KS ks, int givens,
+                                                         int* __restrict__ ve, Tiles tl, size_t sw, KS ks, int givens,
                                                          GivensArgs gv) {
     pdl_prologue();
     const int r = blockIdx.y;
     // the first CTA runs the step's Givens update beside the copy (a launch of its own took 11 us)
     if (givens && blockIdx.x == 0) return arnoldi_givens(gv, r, ks);
     if (inactive_gs(ks, r)) return;
-    const size_t nt = tiles_of(n);
+    const size_t nt = tl.count;
     w += r * sw;
     vc += r * ks.sw;
     vl += r * ks.sv;
@@ -651,14 +656,15 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
     const double s = 1.0 / sc[r * 8 + slot];
     const size_t t = (size_t)(blockIdx.x - givens) * kGsWarps + (threadIdx.x >> 5);
     if (t < nt) {
-        const size_t e0 = t * kTile + lane;
+        size_t end;
+        const size_t e0 = tl.first((unsigned)t, end) + lane;
         double2 x[kTileU];
         int mx = 0;
 #pragma unroll
-        for (int u = 0; u < kTileU; ++u) x[u] = e0 + 32 * u < n ? w[e0 + 32 * u] : make_double2(0.0, 0.0);
+        for (int u = 0; u < kTileU; ++u) x[u] = e0 + 32 * u < end ? w[e0 + 32 * u] : make_double2(0.0, 0.0);
 #pragma unroll
         for (int u = 0; u < kTileU; ++u) {
-            if (e0 + 32 * u < n) {
+            if (e0 + 32 * u < end) {
                 x[u].x *= s;
                 x[u].y *= s;
                 vc[e0 + 32 * u] = cconv<Vc>(x[u]);
@@ -668,20 +674,20 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
         const int eb = tile_exp((int)__reduce_max_sync(0xffffffffu, (unsigned)mx));
         if (lane == 0) ve[t] = eb;
 #pragma unroll
-        for (int u = 0; u < kTileU; ++u) vl[e0 + 32 * u] = limbs2(x[u], eb);
+        for (int u = 0; u < kTileU; ++u) vl[t * kTile + lane + 32 * u] = limbs2(x[u], eb);
     }
 }
 template <class Vc>
-void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, size_t n,
+void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, const Tiles& tl,
                         size_t sw, int nrhs, const KS& ks, cudaStream_t st, const GivensArgs* gv) {
-    const size_t nt = tiles_of(n);
+    const size_t nt = tl.count;
     const int givens = gv ? 1 : 0;
     launch_pdl(k_gs_store<Vc>, dim3((unsigned)((nt + kGsWarps - 1) / kGsWarps) + givens, nrhs), dim3(kGsThreads), 0, st, w, sc,
-               slot, vc, vl, ve, n, sw, ks, givens, gv ? *gv : GivensArgs());
+               slot, vc, vl, ve, tl, sw, ks, givens, gv ? *gv : GivensArgs());
 }
-template void launch_basis_store<double2>(const double2*, const double*, int, double2*, int4*, int*, size_t, size_t, int,
+template void launch_basis_store<double2>(const double2*, const double*, int, double2*, int4*, int*, const Tiles&, size_t, int,
                                           const KS&, cudaStream_t, const GivensArgs*);
-template void launch_basis_store<float2>(const double2*, const double*, int, float2*, int4*, int*, size_t, size_t, int,
+template void launch_basis_store<float2>(const double2*, const double*, int, float2*, int4*, int*, const Tiles&, size_t, int,
                                          const KS&, cudaStream_t, const GivensArgs*);
 
 }  // namespace bah

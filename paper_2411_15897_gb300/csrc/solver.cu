@@ -194,6 +194,7 @@ struct Ctx {
         return s;
     }
     size_t vec_len() const { return (size_t)(dim + 1) * np; }
+    Tiles tiles() const { return Tiles(vec_len(), np); }      // of a Krylov vector
 };
 
 // ---------------------------------------------------------------------------
@@ -721,6 +722,7 @@ template <int MODE>
 static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t st) {
     using V = typename Prec<MODE>::V;
     const size_t np = c.np;
+    const Tiles tl(np, np);
     const int m = c.mi;
     const double rtol = c.o.block_rtol;
     KS ks;                                  // one right-hand side: no strides, no flags
@@ -737,7 +739,7 @@ static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t
     int total = 0;
     while (beta > rtol * bn) {
         if (total >= c.o.block_maxit) { ++c.block_failures; break; }
-        launch_basis_store(c.iR, c.inrm, 0, c.iVc, c.iVL, c.iVE, np, 0, 1, ks, st);
+        launch_basis_store(c.iR, c.inrm, 0, c.iVc, c.iVL, c.iVE, tl, 0, 1, ks, st);
         launch_init_arnoldi(c.inrm, c.igv, m, c.istatus, 1, ks, st);
         int jd = 0;
         for (int j = 0; j < m && total < c.o.block_maxit; ++j) {
@@ -757,13 +759,13 @@ static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t
             // w = M z_j, Gram-Schmidt with selective reorthogonalisation, Givens, v_{j+1}
             launch_block_apply64(c.f5x, b, zj, c.iW, nullptr, st);
             const GsNorm nm{c.icnt, c.iflag, c.inrm, 0.5};
-            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih1, nullptr, c.icnt, 1, ks, st);
-            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih1, c.iW, np, c.idpart, 1, nm, 1, ks, st);
-            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, np, c.ipart, c.ih2, c.iflag, c.icnt, 1, ks, st);
-            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih2, c.iW, np, c.idpart, 2, nm, 1, ks, st);
+            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, tl, c.ipart, c.ih1, nullptr, c.icnt, 1, ks, st);
+            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih1, c.iW, tl, c.idpart, 1, nm, 1, ks, st);
+            launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, tl, c.ipart, c.ih2, c.iflag, c.icnt, 1, ks, st);
+            launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih2, c.iW, tl, c.idpart, 2, nm, 1, ks, st);
             const GivensArgs gv{c.iH, m + 1, j, c.ih1, c.ih2, c.inrm, c.ics, c.isn, c.igv, c.istatus, c.histat};
-            launch_basis_store(c.iW, c.inrm, 2, c.iVc, c.iVL + (j + 1) * tiles_of(np) * kTile,
-                               c.iVE + (j + 1) * tiles_of(np), np, 0, 1, ks, st, &gv);
+            launch_basis_store(c.iW, c.inrm, 2, c.iVc, c.iVL + (j + 1) * tl.padded(),
+                               c.iVE + (size_t)(j + 1) * tl.count, tl, 0, 1, ks, st, &gv);
             BAH_CUDA_TRY(cudaStreamSynchronize(st));
             ++total;
             jd = j + 1;
@@ -840,11 +842,12 @@ static void precond_newest(Ctx& c, void* z, const Batch& bt, cudaStream_t st) {
 }
 // w / sc[slot] as basis vector i and as the newest vector
 static void store_basis(Ctx& c, const double2* w, int slot, int i, cudaStream_t st, const GivensArgs* gv = nullptr) {
-    const size_t n = c.vec_len(), nt = tiles_of(n);
-    int4* vl = c.VL + i * nt * kTile;
-    int* ve = c.VE + i * nt;
-    if (c.vc32) launch_basis_store(w, c.nrm, slot, (float2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st, gv);
-    else launch_basis_store(w, c.nrm, slot, (double2*)c.Vc, vl, ve, n, n, c.nbatch, c.ks, st, gv);
+    const size_t n = c.vec_len();
+    const Tiles tl = c.tiles();
+    int4* vl = c.VL + i * tl.padded();
+    int* ve = c.VE + (size_t)i * tl.count;
+    if (c.vc32) launch_basis_store(w, c.nrm, slot, (float2*)c.Vc, vl, ve, tl, n, c.nbatch, c.ks, st, gv);
+    else launch_basis_store(w, c.nrm, slot, (double2*)c.Vc, vl, ve, tl, n, c.nbatch, c.ks, st, gv);
 }
 // algorithmic bytes of one operator apply: input (3 components), FP64
 // output, coefficients cx, nx (z-aliases when h1 == h2), d1, d2, 1/(lambda+mu)
@@ -900,12 +903,13 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     const int m = c.m;
     const size_t nbt = c.nbatch;
     const size_t so = m + 2;
-    const size_t nt = tiles_of(n);
+    const Tiles tl = c.tiles();
+    const size_t nt = tl.count;
     if (c.kdf) {
         TRY(c.alloc_t(&c.V, n * (m + 1) * nbt));
     } else {
         TRY(gs_prepare());
-        TRY(c.alloc_t(&c.VL, nt * kTile * (m + 1) * nbt));
+        TRY(c.alloc_t(&c.VL, tl.padded() * (m + 1) * nbt));
         TRY(c.alloc_t(&c.VE, nt * (m + 1) * nbt));
         // the 2-D FP32 cycles read the newest vector in FP32 only
         c.vc32 = c.mode == BAH_MIXED && c.dim == 2 && !c.exact;
@@ -930,7 +934,7 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     BAH_CUDA_TRY(cudaMemsetAsync(c.nrm, 0, 8 * nbt * sizeof(double), st));
     BAH_CUDA_TRY(cudaMallocHost((void**)&c.hstatus, (4 * (size_t)(m + 1) * nbt + 8 * nbt) * sizeof(double)));
     BAH_CUDA_TRY(cudaMallocHost((void**)&c.hint, kIntSlots * nbt * sizeof(int)));
-    c.ks.sv = (size_t)(m + 1) * (c.VL ? nt * kTile : n); c.ks.se = (size_t)(m + 1) * nt;
+    c.ks.sv = (size_t)(m + 1) * (c.VL ? tl.padded() : n); c.ks.se = (size_t)(m + 1) * nt;
     c.ks.sw = n; c.ks.sp = so * GS_CTAS; c.ks.so = so;
     c.ks.sh = (size_t)(m + 1) * m; c.ks.sz = (size_t)m * n; c.ks.sx = n; c.ks.active = c.active;
     BAH_CUDA_TRY(cudaStreamCreateWithFlags(&c.cap_stream, cudaStreamNonBlocking));
@@ -1165,7 +1169,8 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
         c.f5x = Fine5<double, double2>{c.n1, c.n2, c.cx, c.cz, c.nx, c.nz, c.wx, c.wz, dgb[0], dgb[1], dgb[2], c.dAp};
         const size_t so = c.mi + 2;
         TRY(gs_prepare());
-        TRY(c.alloc_t(&c.iVL, (c.mi + 1) * tiles_of(np) * kTile)); TRY(c.alloc_t(&c.iVE, (c.mi + 1) * tiles_of(np)));
+        const Tiles tl(np, np);
+        TRY(c.alloc_t(&c.iVL, (c.mi + 1) * tl.padded())); TRY(c.alloc_t(&c.iVE, (size_t)(c.mi + 1) * tl.count));
         TRY(c.alloc_t(&c.iVc, np)); TRY(c.alloc_t(&c.iZ, (size_t)c.mi * np));
         TRY(c.alloc_t(&c.iW, np)); TRY(c.alloc_t(&c.iR, np));
         TRY(c.alloc_t(&c.iH, (size_t)(c.mi + 1) * c.mi));
@@ -1381,16 +1386,16 @@ static void iter_body(Ctx& c, int j, cudaStream_t st) {
     int npt = 0;                 // partial sums of ||w'||^2 (double-float basis)
     const GsNorm nm{c.gscnt, c.gsflag, c.nrm, c.dgks_eta2};
     const GivensArgs gv{c.Hm, m + 1, j, c.h1v, c.h2v, c.nrm, c.cs, c.sn, c.g, c.status, status_slot(c, j)};
-    const int ndot = c.kdf ? 2 : dot_launches(n, nb);
+    const int ndot = c.kdf ? 2 : dot_launches(c.tiles(), nb);
     {
         Prof pr(c, BAH_K_DOT, st, nb * (k1 + 1) * n * 16.0, ndot);
         if (c.kdf) launch_dot_norm_df(Vd, j + 1, Wd, n, c.partial, c.h1v, nullptr, nb, ks, st);
-        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h1v, nullptr, c.gscnt, nb, ks, st);
+        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, c.tiles(), c.partial, c.h1v, nullptr, c.gscnt, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_AXPY, st, nb * (k1 + 2) * n * 16.0);
         if (c.kdf) npt = launch_axpy_norm_df(Vd, j + 1, c.h1v, Wd, n, c.dpart, nullptr, nb, ks, st);
-        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h1v, c.W, n, c.dpart, 1, nm, nb, ks, st);
+        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h1v, c.W, c.tiles(), c.dpart, 1, nm, nb, ks, st);
     }
     if (c.kdf) {
         Prof pr(c, BAH_K_NORM, st, 0.0);
@@ -1399,12 +1404,12 @@ static void iter_body(Ctx& c, int j, cudaStream_t st) {
     {
         Prof pr(c, BAH_K_DOT, st, 0.0, ndot);   // runs only where the flag is set (bytes counted as zero)
         if (c.kdf) launch_dot_norm_df(Vd, j + 1, Wd, n, c.partial, c.h2v, c.gsflag, nb, ks, st);
-        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, n, c.partial, c.h2v, c.gsflag, c.gscnt, nb, ks, st);
+        else launch_dot_norm(c.VL, c.VE, j + 1, c.W, c.tiles(), c.partial, c.h2v, c.gsflag, c.gscnt, nb, ks, st);
     }
     {
         Prof pr(c, BAH_K_AXPY, st, 0.0);
         if (c.kdf) launch_axpy_norm_df(Vd, j + 1, c.h2v, Wd, n, c.dpart, c.gsflag, nb, ks, st);
-        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h2v, c.W, n, c.dpart, 2, nm, nb, ks, st);
+        else launch_axpy_norm(c.VL, c.VE, j + 1, c.h2v, c.W, c.tiles(), c.dpart, 2, nm, nb, ks, st);
     }
     {
         // the status goes to its pinned slot from the Givens update itself
@@ -1614,16 +1619,17 @@ using cdx = std::complex<double>;
 // CholQR2 of the s columns of W, enqueued: basis block i and the newest block
 // = Q with W = Q R, R = R_2 R_1, both written to R12 (2 s x s, row-major; NaN
 // where a Gram matrix is not positive definite).  W is overwritten.
-static void enqueue_cholqr2(Ctx& c, int s, double2* W, size_t n, int i, double2* R12, cudaStream_t st) {
-    int4* vl = c.VL + i * tiles_of(n) * kTile;
-    int* ve = c.VE + i * tiles_of(n);
-    launch_block_gram(s, W, n, c.bpart, c.bG, st);
+static void enqueue_cholqr2(Ctx& c, int s, double2* W, int i, double2* R12, cudaStream_t st) {
+    const Tiles tl = c.tiles();
+    int4* vl = c.VL + i * tl.padded();
+    int* ve = c.VE + (size_t)i * tl.count;
+    launch_block_gram(s, W, tl, c.bpart, c.bG, st);
     launch_block_chol(c.bG, s, R12, c.bT, st);
-    launch_block_scale(W, s, c.bT, W, nullptr, nullptr, 0, 0, n, st);
-    launch_block_gram(s, W, n, c.bpart, c.bG, st);
+    launch_block_scale(W, s, c.bT, W, nullptr, nullptr, 0, 0, tl, st);
+    launch_block_gram(s, W, tl, c.bpart, c.bG, st);
     launch_block_chol(c.bG, s, R12 + s * s, c.bT, st);
-    if (c.vc32) launch_block_scale(W, s, c.bT, (float2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, n, st);
-    else launch_block_scale(W, s, c.bT, (double2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, n, st);
+    if (c.vc32) launch_block_scale(W, s, c.bT, (float2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, tl, st);
+    else launch_block_scale(W, s, c.bT, (double2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, tl, st);
 }
 // R = R_2 R_1 from the host copy of R12
 static int host_r(int s, const double2* R12, std::vector<cdx>& R) {
@@ -1731,6 +1737,7 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
     bt.nr = s;
     bt.active = nullptr;
     const size_t s2 = (size_t)s * s;
+    const Tiles tl = c.tiles();
     // step j up to and including its copy to host slot j & 1: [R_1 | R_2 | C_1 | C_2]
     auto enqueue = [&](int j) {
         NvtxRange nvs("block fgmres step");
@@ -1740,10 +1747,10 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
         const size_t cnt = (size_t)(j + 1) * s2;
         for (int pass = 0; pass < 2; ++pass) {            // block CGS2
             double2* C = c.bC + 2 * s2 + pass * cnt;
-            launch_block_dot(c.VL, c.VE, ks.sv, ks.se, j + 1, s, c.W, n, c.bpart, C, st);
-            launch_block_update(c.VL, c.VE, ks.sv, ks.se, j + 1, s, C, c.W, n, st);
+            launch_block_dot(c.VL, c.VE, ks.sv, ks.se, j + 1, s, c.W, tl, c.bpart, C, st);
+            launch_block_update(c.VL, c.VE, ks.sv, ks.se, j + 1, s, C, c.W, tl, st);
         }
-        enqueue_cholqr2(c, s, c.W, n, j + 1, c.bC, st);
+        enqueue_cholqr2(c, s, c.W, j + 1, c.bC, st);
         BAH_CUDA_TRY(cudaMemcpyAsync(c.bhost + (j & 1) * c.bslot, c.bC, (2 * s2 + 2 * cnt) * sizeof(double2),
                                      cudaMemcpyDeviceToHost, st));
         BAH_CUDA_TRY(cudaEventRecord(c.itev[j], st));
@@ -1780,7 +1787,7 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
     while (!done() && total < c.o.maxit) {
         NvtxRange nvc("block fgmres restart cycle");
         // R_0 = V_0 S_0
-        enqueue_cholqr2(c, s, c.R, n, 0, c.bC, st);
+        enqueue_cholqr2(c, s, c.R, 0, c.bC, st);
         BAH_CUDA_TRY(cudaMemcpyAsync(c.bhost, c.bC, 2 * s2 * sizeof(double2), cudaMemcpyDeviceToHost, st));
         BAH_CUDA_TRY(cudaStreamSynchronize(st));
         TRY(host_r(s, c.bhost, S0));
