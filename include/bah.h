@@ -154,6 +154,7 @@ void bah_default_opts(bah_opts* opts);
  * Galerkin hierarchies R A P (Eq. 4.3) and the FP64 inverse of every coarsest
  * block, and allocates all solve workspace.  Synchronous.  *out receives the
  * context; on failure *out is NULL and nothing is leaked.
+ * 3-D grids have fewer than 2^29 cells, in FP64 at most 2^28 (else BAH_ERR_ARG).
  * block_rtol > 0 needs a 2-D grid and rhs_block = 1 (else BAH_ERR_UNSUPPORTED).
  * 3-D grids (dim 3) follow the paper's 3-D multigrid (Sec. 4.5): they need
  * intergrid = BAH_INTERGRID_MIXED (Eq. 4.4; with it every Galerkin level is a

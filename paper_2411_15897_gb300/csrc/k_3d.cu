@@ -385,7 +385,8 @@ __device__ __forceinline__ unsigned ld_now3(const __nv_bfloat162* p) {
 }
 __device__ __forceinline__ double2 entry3(double2 v) { return v; }
 __device__ __forceinline__ float2 entry3(unsigned v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
-// base[i] through a 32-bit byte offset (i < 2^28: a vector of one block is below 4 GB)
+// base[i] through a 32-bit byte offset: a vector of one block is at most 4 GB (bah_create refuses
+// more than 2^28 cells in FP64 and 2^29 in mixed mode)
 template <class T> __device__ __forceinline__ T at3(const T* base, unsigned i) {
     return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + (size_t)(i * (unsigned)sizeof(T)));
 }

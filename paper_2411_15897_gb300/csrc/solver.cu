@@ -1939,6 +1939,11 @@ int bah_create(const bah_grid* grid, const bah_medium* med, const bah_opts* opts
     bah_opts o;
     if (opts) o = *opts; else bah_default_opts(&o);
     if (o.precision != BAH_FP64 && o.precision != BAH_MIXED) { set_error("bad precision"); return BAH_ERR_ARG; }
+    // the level kernels address a block's vector through 32-bit byte offsets (at3 in k_3d.cu)
+    if (dim == 3 && o.precision == BAH_FP64 && (long long)grid->n[0] * grid->n[1] * grid->n[2] > 1LL << 28) {
+        set_error("3-D grid too large (2^28 cells in FP64)");
+        return BAH_ERR_ARG;
+    }
     if (o.restart < 1 || o.restart > 64) { set_error("restart must be in 1..64"); return BAH_ERR_ARG; }
     if (o.maxit < 1) { set_error("maxit must be >= 1"); return BAH_ERR_ARG; }
     if (o.rhs_block < 1 || o.rhs_block > 256) { set_error("rhs_block must be in 1..256"); return BAH_ERR_ARG; }
