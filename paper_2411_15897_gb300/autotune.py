@@ -12,8 +12,11 @@ candidate runs a fixed number of FGMRES iterations on its batch (tolerance
 below reach, so no source stops early) and the cost per source and iteration
 is compared.  The variants are the library's per-context launch switches
 (environment variables read when a context is created): the shared-memory
-cluster multigrid of the small levels (``BAH_SMEM_MG``) and the
-shared-memory staging of the Galerkin-level sweeps (``BAH_STAGED``).
+cluster multigrid of the small levels (``BAH_SMEM_MG``; mixed mode, 2-D, a
+coarsest level of at most 256 points, batches of up to three right-hand
+sides) and the register-stencil sweeps of the Galerkin levels
+(``BAH_STAGED``; mixed mode, 2-D).  Where a switch changes no launch the
+variant is the default program, and is not timed a second time.
 
 Results are cached in a JSON file keyed by grid, sources, precision and
 device, so a job tunes once.  ``tune`` takes the timing function as an
@@ -37,6 +40,7 @@ VARIANTS = {
     "no-cluster-mg": {"BAH_SMEM_MG": "0"},
     "no-staging": {"BAH_STAGED": "0"},
 }
+CLUSTER_RHS = 3                       # most right-hand sides of a cluster multigrid launch (kClusterRhs)
 
 
 @dataclass
@@ -101,12 +105,35 @@ def candidates(nsrc, limit=256):
     return out
 
 
+def program(env, rhs_block, info, ndim=2, mixed=True):
+    """What a batch of ``rhs_block`` sources launches under the settings ``env``: equal values,
+    equal launches.  ``info``: the default context's (``Solver.info``)."""
+    rest = tuple(sorted((k, v) for k, v in env.items() if k not in ("BAH_SMEM_MG", "BAH_STAGED")))
+    if ndim != 2 or not mixed:
+        return False, False, rest
+    cluster = env.get("BAH_SMEM_MG", "1")[0] != "0" and info["cluster_level"] > 0 and rhs_block <= CLUSTER_RHS
+    # levels 1 .. last run Galerkin sweeps outside the cluster
+    last = info["cluster_level"] - 1 if cluster else info["levels"] - 2
+    return cluster, last >= 1 and env.get("BAH_STAGED", "1")[0] != "0", rest
+
+
+def _default_info(problem, opts):
+    from . import Solver
+
+    s = Solver.from_problem(problem, **dict(opts, rhs_block=1))
+    info = dict(s.info)
+    s.close()
+    return info
+
+
 def tune(problem, nsrc=None, opts=None, iters=20, variants=None, measure=time_batch, cache_path=None,
          device=None) -> Choice:
     """Cheapest (rhs_block, variant) per source and iteration for ``nsrc``
     sources of ``problem``.  ``measure(problem, rhs_block, env, opts, iters)``
     returns seconds per source per iteration; ``cache_path`` (JSON) stores
-    the choice under the problem's key and is read back on the next call."""
+    the choice under the problem's key and is read back on the next call.
+    With the default ``measure``, variants that launch the same program are
+    timed once (the first of them) and share its cost."""
     opts = dict(opts or {})
     nsrc = int(nsrc or len(problem.sources) or 1)
     variants = variants or VARIANTS
@@ -126,9 +153,14 @@ def tune(problem, nsrc=None, opts=None, iters=20, variants=None, measure=time_ba
             return Choice(c["rhs_block"], c["variant"], c["cost"], c.get("table", {}))
     table = {}
     best = None
+    info = _default_info(problem, opts) if measure is time_batch and len(variants) > 1 else None
     for rb in candidates(nsrc):
+        timed = {}
         for name, env in variants.items():
-            cost = float(measure(problem, rb, env, opts, iters))
+            prog = program(env, rb, info, len(problem.n), opts.get("precision", 1) == 1) if info else name
+            if prog not in timed:
+                timed[prog] = float(measure(problem, rb, env, opts, iters))
+            cost = timed[prog]
             table[f"{rb}/{name}"] = cost
             if best is None or cost < best.cost:
                 best = Choice(rb, name, cost)
