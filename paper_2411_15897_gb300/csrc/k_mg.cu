@@ -29,7 +29,8 @@ static inline int max_radius(const LS& s) {
 template <int MODE> constexpr int kTpb = MODE == BAH_FP64 ? 64 : 256;
 
 // ---------------------------------------------------------------------------
-// damped Jacobi:  x_out = x_in + w D^{-1} (b - A x_in)   (zero_init: w D^{-1} b)
+// damped Jacobi:  x_out = x_in + w D^{-1} (b - A x_in)   (zero_init: w D^{-1} b, on level 0;
+// below it the restriction writes the first sweep).  FP64: the first sweep only.
 // ---------------------------------------------------------------------------
 template <int MODE, bool L0, int RM>
 __global__ void __launch_bounds__(kTpb<MODE>) k_jacobi(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> s,
@@ -46,13 +47,12 @@ __global__ void __launch_bounds__(kTpb<MODE>) k_jacobi(LvlSet<typename MGT<MODE>
     const int i = t % n1, j = t / n1;
     if (!valid_pt(B.type, i, j)) { xout[t] = czero<V>(); return; }
     const V b = B.b[rr * B.sb + t];
-    if (zero_init) {
-        if constexpr (MODE == BAH_FP64) {
-            xout[t] = cscale(cmul(B.idg[t], b), w);
-            return;
-        }
-        const V dg = diag_only<MODE>(L0 ? &f5 : nullptr, B, np, t);
-        xout[t] = cscale(cdiv(b, dg), w);
+    if constexpr (MODE == BAH_FP64) {
+        xout[t] = cscale(cmul(B.idg[t], b), w);
+        return;
+    }
+    if (L0 && zero_init) {
+        xout[t] = cscale(cdiv(b, diag_only<MODE>(&f5, B, np, t)), w);
         return;
     }
     const V* __restrict__ xin = B.xin + rr * B.sxi;

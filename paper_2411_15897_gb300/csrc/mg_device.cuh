@@ -149,13 +149,6 @@ __device__ __forceinline__ typename MGT<MODE>::V apply_stencil_fn(const typename
                                        [&](int dx, int dz) { return X(t + dz * n1 + dx); });
 }
 
-// the stencil through an accessor S(slot) (e.g. shared memory), x by flat index
-template <int MODE, int RM, class SF, class XF>
-__device__ __forceinline__ typename MGT<MODE>::V apply_stencil_acc(SF S, int rx, int rz, int n1, int n2, int i, int j,
-                                                                  int t, XF X) {
-    return apply_stencil_rel<MODE, RM>(S, rx, rz, n1, n2, i, j, [&](int dx, int dz) { return X(t + dz * n1 + dx); });
-}
-
 template <int MODE>
 __device__ __forceinline__ typename MGT<MODE>::V diag_only(const Fine5<typename MGT<MODE>::C, typename MGT<MODE>::CC>* f5,
                                                           const LvlBlk<typename MGT<MODE>::V, typename MGT<MODE>::CC>& B,

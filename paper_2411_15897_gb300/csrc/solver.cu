@@ -119,7 +119,6 @@ struct Ctx {
     int sm_l0 = 0;                       // first level of the shared-memory cluster multigrid (0: off)
     int sm_cs = 0, sm_rm = 2;            // its CTAs per cluster and stencil radius bound
     size_t sm_bytes = 0;                 // its dynamic shared memory per CTA
-    int nsm = 0;
 
     // exact-block preconditioner (block_rtol > 0): each acoustic block solved
     // by an inner FGMRES(mi) in FP64, preconditioned by its multigrid cycle
@@ -1096,11 +1095,6 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
             BAH_CUDA_TRY(cudaMemsetAsync(c.vB[l][b], 0, bytes, st));
             BAH_CUDA_TRY(cudaMemsetAsync(c.vT[l][b], 0, bytes, st));
         }
-    {
-        int dev = 0;
-        BAH_CUDA_TRY(cudaGetDevice(&dev));
-        BAH_CUDA_TRY(cudaDeviceGetAttribute(&c.nsm, cudaDevAttrMultiProcessorCount, dev));
-    }
     // shared-memory cluster multigrid (mixed mode; BAH_SMEM_MG=0 turns it off):
     // from the first level below the fine grid whose levels, down to the
     // coarsest, fit in the shared memory of one cluster (16 CTAs, else 8).  The
