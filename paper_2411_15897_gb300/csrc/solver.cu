@@ -1151,8 +1151,8 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
         {
             void* scratch = nullptr;
             BAH_CUDA_TRY(cudaMalloc(&scratch, (size_t)np * (7 * sizeof(double) + 3 * sizeof(double2))));
-            double* sd = (double*)scratch;
-            double2* sc2 = (double2*)(sd + 7 * (size_t)np);
+            double2* sc2 = (double2*)scratch;              // first: 16-byte alignment for any number of points
+            double* sd = (double*)(sc2 + 3 * (size_t)np);
             launch_medium_prep(c.n1, c.n2, c.h1, c.h2, c.omega, c.o.block_alpha, lam, mu, rho, gam, sd, sd + np,
                                sd + 2 * (size_t)np, sd + 3 * (size_t)np, sd + 4 * (size_t)np, sd + 5 * (size_t)np,
                                sc2, sc2 + np, sd + 6 * (size_t)np, dgb[0], dgb[1], dgb[2], sc2 + 2 * (size_t)np, st);
