@@ -414,15 +414,16 @@ struct GsNorm {
 };
 void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, const Tiles& tl, double2* partial, double2* out,
                      const int* flag, int* cnt, int nrhs, const KS& ks, cudaStream_t st);
+int dot_ctas(const Tiles& tl, int nrhs);       // partial sums of a row (size of `partial`: (k + 1) times as many)
 int dot_launches(const Tiles& tl, int nrhs);   // launches of launch_dot_norm
 // coef: the projections, followed by ||w||^2 (launch_dot_norm's out); npart: scratch, GS_CTAS per right-hand side
 void launch_axpy_norm(const int4* VL, const int* VE, int k, const double2* coef, double2* w, const Tiles& tl, double* npart,
                       int pass, const GsNorm& nm, int nrhs, const KS& ks, cudaStream_t st);
-// v = w / sc[slot] as the preconditioner's input (vc, FP64 or rounded to FP32,
-// stride ks.sw) and as a basis vector (vl, ve); with gv also the step's Givens update
+// v = w / sc[slot] as the preconditioner's input (vc, FP64 or rounded to FP32, stride svc;
+// may be w itself, or null) and as a basis vector (vl, ve); with gv also the step's Givens update
 struct GivensArgs;
 template <class Vc>
-void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, const Tiles& tl,
+void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, size_t svc, int4* vl, int* ve, const Tiles& tl,
                         size_t sw, int nrhs, const KS& ks, cudaStream_t st, const GivensArgs* gv = nullptr);
 // flag = 1 (second pass) when ||w'||^2 < eta2 ||w||^2 (DGKS criterion; eta2 = 1/2 classically)
 void launch_dgks_decide(const double* npart, int np, const double2* h1norm, int k, int* flag, double* sc, int nrhs,
@@ -459,9 +460,9 @@ void launch_block_gram(int s, const double2* W, const Tiles& tl, double2* partia
 void launch_block_update(const int4* VL, const int* VE, size_t sv, size_t se, int k, int s, const double2* C, double2* W,
                          const Tiles& tl, cudaStream_t st);
 void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStream_t st);
-// dst: FP64, or (with vl) rounded to FP32
+// dst (column b at b * sd; may be W itself, or null): FP64, or (with vl) rounded to FP32
 template <class Vd>
-void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, int4* vl, int* ve, size_t sv, size_t se,
+void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, size_t sd, int4* vl, int* ve, size_t sv, size_t se,
                         const Tiles& tl, cudaStream_t st);
 template <class Vz>
 void launch_block_xupdate(const Vz* Z, size_t sz, int k, int s, const double2* Y, double2* X, size_t n,

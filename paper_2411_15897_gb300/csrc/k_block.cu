@@ -2,8 +2,8 @@
 // (the batched form of the outer solve; FGMRES of Sec. 2.2 and Sec. 4 applied
 // to a block).  The basis is stored in block fixed point (fix60.cuh): column a
 // of basis block i has its limbs at VL + a * sv + i * tiles * 256 and its tile
-// exponents at VE + a * se + i * tiles; the newest block is also kept in FP64
-// (Vc, column b at b * n).  W and X hold column b at b * n.
+// exponents at VE + a * se + i * tiles; the newest block also stands as the preconditioner's
+// input, in W in FP64 or in its slot of Z in FP32.  W and X hold column b at b * n.
 //
 //   block dot    C[(i, a), b] = sum_e conj(V_i[a][e]) W[b][e]      ((k s) x s, k blocks)
 //   block Gram   C[a, b] = sum_e conj(W[a][e]) W[b][e]
@@ -371,11 +371,11 @@ void launch_block_chol(const double2* G, int s, double2* R, double2* T, cudaStre
 }
 
 // V[b] = sum_(b' <= b) W[b'] T[b', b] (T upper triangular, s x s, row-major),
-// written to dst (column b at b * n; may be W itself) and, with vl, as basis
+// written to dst (column b at b * sd; may be W itself, or null) and, with vl, as basis
 // columns.  One CTA of S warps per tile: warp b converts column b to limbs in
 // shared memory, then sums column b of the product.
 template <int S, class Vd>
-__global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, const double2* __restrict__ T, Vd* dst,
+__global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, const double2* __restrict__ T, Vd* dst, size_t sd,
                                                    int4* __restrict__ vl, int* __restrict__ ve, size_t sv, size_t se,
                                                    Tiles tl) {
     pdl_prologue();
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
             x[u] = make_double2(0.0, 0.0);
             if (e0 + 32 * u < end) {
                 x[u] = acc.minus(x[u], u, s1, s2);
-                dst[(size_t)b * n + e0 + 32 * u] = cconv<Vd>(x[u]);
+                if (dst) dst[b * sd + e0 + 32 * u] = cconv<Vd>(x[u]);
             }
             mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
         }
@@ -435,13 +435,13 @@ __global__ void __launch_bounds__(32 * S) k_bscale(const double2* W, int s, cons
     }
 }
 template <class Vd>
-void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, int4* vl, int* ve, size_t sv, size_t se,
+void launch_block_scale(const double2* W, int s, const double2* T, Vd* dst, size_t sd, int4* vl, int* ve, size_t sv, size_t se,
                         const Tiles& tl, cudaStream_t st) {
     const size_t smem = (size_t)s * kTile * sizeof(int4);
     const unsigned nt = tl.count;
-    if (s <= 4) launch_pdl(k_bscale<4, Vd>, dim3(std::min(nt, 608u)), dim3(128), smem, st, W, s, T, dst, vl, ve, sv, se, tl);
-    else if (s <= 8) launch_pdl(k_bscale<8, Vd>, dim3(std::min(nt, 304u)), dim3(256), smem, st, W, s, T, dst, vl, ve, sv, se, tl);
-    else launch_pdl(k_bscale<16, Vd>, dim3(std::min(nt, 152u)), dim3(512), smem, st, W, s, T, dst, vl, ve, sv, se, tl);
+    if (s <= 4) launch_pdl(k_bscale<4, Vd>, dim3(std::min(nt, 608u)), dim3(128), smem, st, W, s, T, dst, sd, vl, ve, sv, se, tl);
+    else if (s <= 8) launch_pdl(k_bscale<8, Vd>, dim3(std::min(nt, 304u)), dim3(256), smem, st, W, s, T, dst, sd, vl, ve, sv, se, tl);
+    else launch_pdl(k_bscale<16, Vd>, dim3(std::min(nt, 152u)), dim3(512), smem, st, W, s, T, dst, sd, vl, ve, sv, se, tl);
 }
 
 // X[b][e] += sum over rows (i, a) < k s of Z_i[a][e] Y[row, b]  (Z FP32 or FP64 complex)
@@ -493,9 +493,9 @@ int block_prepare() {
     for (const auto& q : fns) BAH_CUDA_TRY(cudaFuncSetAttribute(q.f, cudaFuncAttributeMaxDynamicSharedMemorySize, q.b));
     return BAH_OK;
 }
-template void launch_block_scale<double2>(const double2*, int, const double2*, double2*, int4*, int*, size_t, size_t,
+template void launch_block_scale<double2>(const double2*, int, const double2*, double2*, size_t, int4*, int*, size_t, size_t,
                                           const Tiles&, cudaStream_t);
-template void launch_block_scale<float2>(const double2*, int, const double2*, float2*, int4*, int*, size_t, size_t,
+template void launch_block_scale<float2>(const double2*, int, const double2*, float2*, size_t, int4*, int*, size_t, size_t,
                                          const Tiles&, cudaStream_t);
 template void launch_block_xupdate<float2>(const float2*, size_t, int, int, const double2*, double2*, size_t,
                                            cudaStream_t);

@@ -295,6 +295,7 @@ void launch_dot_norm(const int4* VL, const int* VE, int k, const double2* w, con
     if (!last) launch_pdl(k_gs_reduce, dim3(1, k + 1, nrhs), dim3(128), 0, st, (const double2*)partial, nc, out, flag, ks);
 }
 
+int dot_ctas(const Tiles& tl, int nrhs) { return gs_ctas(tl, nrhs); }
 int dot_launches(const Tiles& tl, int nrhs) { return gs_ctas(tl, nrhs) <= kGsFew ? 1 : 2; }
 
 // ---------------------------------------------------------------------------
@@ -638,8 +639,8 @@ int gs_prepare() {
 // nothing: the distributor of 32 sources of 1024 x 512 493 -> 116 us) and its limbs and tile exponents in the basis
 // ---------------------------------------------------------------------------
 template <class Vc>
-__global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restrict__ w, const double* sc, int slot,
-                                                         Vc* __restrict__ vc, int4* __restrict__ vl,
+__global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* w, const double* sc, int slot,
+                                                         Vc* vc, size_t svc, int4* __restrict__ vl,
                                                          int* __restrict__ ve, Tiles tl, size_t sw, KS ks, int givens,
                                                          GivensArgs gv) {
     pdl_prologue();
@@ -649,7 +650,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
     if (inactive_gs(ks, r)) return;
     const size_t nt = tl.count;
     w += r * sw;
-    vc += r * ks.sw;
+    if (vc) vc += r * svc;
     vl += r * ks.sv;
     ve += r * ks.se;
     const int lane = threadIdx.x & 31;
@@ -667,7 +668,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
             if (e0 + 32 * u < end) {
                 x[u].x *= s;
                 x[u].y *= s;
-                vc[e0 + 32 * u] = cconv<Vc>(x[u]);
+                if (vc) vc[e0 + 32 * u] = cconv<Vc>(x[u]);
             }
             mx = max(mx, max(abs_hi(x[u].x), abs_hi(x[u].y)));
         }
@@ -678,16 +679,16 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_store(const double2* __restri
     }
 }
 template <class Vc>
-void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, int4* vl, int* ve, const Tiles& tl,
+void launch_basis_store(const double2* w, const double* sc, int slot, Vc* vc, size_t svc, int4* vl, int* ve, const Tiles& tl,
                         size_t sw, int nrhs, const KS& ks, cudaStream_t st, const GivensArgs* gv) {
     const size_t nt = tl.count;
     const int givens = gv ? 1 : 0;
     launch_pdl(k_gs_store<Vc>, dim3((unsigned)((nt + kGsWarps - 1) / kGsWarps) + givens, nrhs), dim3(kGsThreads), 0, st, w, sc,
-               slot, vc, vl, ve, tl, sw, ks, givens, gv ? *gv : GivensArgs());
+               slot, vc, svc, vl, ve, tl, sw, ks, givens, gv ? *gv : GivensArgs());
 }
-template void launch_basis_store<double2>(const double2*, const double*, int, double2*, int4*, int*, const Tiles&, size_t, int,
+template void launch_basis_store<double2>(const double2*, const double*, int, double2*, size_t, int4*, int*, const Tiles&, size_t, int,
                                           const KS&, cudaStream_t, const GivensArgs*);
-template void launch_basis_store<float2>(const double2*, const double*, int, float2*, int4*, int*, const Tiles&, size_t, int,
+template void launch_basis_store<float2>(const double2*, const double*, int, float2*, size_t, int4*, int*, const Tiles&, size_t, int,
                                          const KS&, cudaStream_t, const GivensArgs*);
 
 }  // namespace bah

@@ -50,7 +50,7 @@ struct Ctx {
 
     // FP64 coefficient arrays (cells)
     double *cx = nullptr, *cz = nullptr, *nx = nullptr, *nz = nullptr, *wx = nullptr, *wz = nullptr, *cinv = nullptr;
-    double2 *d1 = nullptr, *d2 = nullptr, *dg[3] = {nullptr, nullptr, nullptr}, *dAp = nullptr;
+    double2 *d1 = nullptr, *d2 = nullptr, *dAp = nullptr;
     double* gam = nullptr;               // attenuation at cells (device), for the gradient
     OpCoef op{};
     OpCoefDF opdf{};                     // double-float copies (mixed mode with the double-float basis)
@@ -69,11 +69,11 @@ struct Ctx {
     // Krylov workspace
     int m = 20;
     double2 *V = nullptr, *W = nullptr, *R = nullptr, *Bs = nullptr, *X = nullptr;
-    // the FP64 basis: limbs and tile exponents (fix60.cuh), and the newest vector as the
-    // preconditioner's input, FP64 or (vc32) rounded to FP32; V is the double-float basis
+    // the FP64 basis: limbs and tile exponents (fix60.cuh).  The newest vector, as the
+    // preconditioner's input, stands in W in FP64, or (vc32) rounded to FP32 in its own slot
+    // of Z, where the preconditioner works in place.  V is the double-float basis
     int4* VL = nullptr;
     int* VE = nullptr;
-    void* Vc = nullptr;
     bool vc32 = false;
     double2 *Hm = nullptr, *h1v = nullptr, *h2v = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr;
     double2* partial = nullptr;
@@ -127,7 +127,7 @@ struct Ctx {
     int mi = 60;                        // inner restart length
     int4* iVL = nullptr;
     int* iVE = nullptr;
-    double2 *iVc = nullptr, *iZ = nullptr, *iW = nullptr, *iR = nullptr, *iH = nullptr;
+    double2 *iZ = nullptr, *iW = nullptr, *iR = nullptr, *iH = nullptr;
     double2 *ih1 = nullptr, *ih2 = nullptr, *ics = nullptr, *isn = nullptr, *igv = nullptr, *iy = nullptr;
     double2* ipart = nullptr;
     double *inrm = nullptr, *idpart = nullptr, *istatus = nullptr;
@@ -185,6 +185,13 @@ struct Ctx {
         }
         allocs.push_back(*p);
         return BAH_OK;
+    }
+    // give back a buffer of alloc() before the context ends
+    void release(void* p) {
+        const auto it = std::find(allocs.begin(), allocs.end(), p);
+        if (it == allocs.end()) return;
+        allocs.erase(it);
+        cudaFree(p);
     }
     template <class T> int alloc_t(T** p, size_t count) {
         void* q;
@@ -738,11 +745,11 @@ static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t
     int total = 0;
     while (beta > rtol * bn) {
         if (total >= c.o.block_maxit) { ++c.block_failures; break; }
-        launch_basis_store(c.iR, c.inrm, 0, c.iVc, c.iVL, c.iVE, tl, 0, 1, ks, st);
+        launch_basis_store(c.iR, c.inrm, 0, c.iW, np, c.iVL, c.iVE, tl, 0, 1, ks, st);
         launch_init_arnoldi(c.inrm, c.igv, m, c.istatus, 1, ks, st);
         int jd = 0;
         for (int j = 0; j < m && total < c.o.block_maxit; ++j) {
-            const double2* vj = c.iVc;
+            const double2* vj = c.iW;                // the newest basis vector
             double2* zj = c.iZ + (size_t)j * np;
             // z_j = (one multigrid cycle of the block) v_j
             if constexpr (MODE == BAH_MIXED) {
@@ -763,7 +770,7 @@ static int block_solve(Ctx& c, int b, const double2* s, double2* e, cudaStream_t
             launch_dot_norm(c.iVL, c.iVE, j + 1, c.iW, tl, c.ipart, c.ih2, c.iflag, c.icnt, 1, ks, st);
             launch_axpy_norm(c.iVL, c.iVE, j + 1, c.ih2, c.iW, tl, c.idpart, 2, nm, 1, ks, st);
             const GivensArgs gv{c.iH, m + 1, j, c.ih1, c.ih2, c.inrm, c.ics, c.isn, c.igv, c.istatus, c.histat};
-            launch_basis_store(c.iW, c.inrm, 2, c.iVc, c.iVL + (j + 1) * tl.padded(),
+            launch_basis_store(c.iW, c.inrm, 2, c.iW, np, c.iVL + (j + 1) * tl.padded(),
                                c.iVE + (size_t)(j + 1) * tl.count, tl, 0, 1, ks, st, &gv);
             BAH_CUDA_TRY(cudaStreamSynchronize(st));
             ++total;
@@ -834,10 +841,17 @@ static void precond_any(Ctx& c, const RIN* r, size_t rstride, void* z, size_t zs
     if (c.mode == BAH_MIXED) MG<BAH_MIXED>::template precond<RIN>(c, r, rstride, (float2*)z, zstride, bt, st);
     else MG<BAH_FP64>::template precond<RIN>(c, r, rstride, (double2*)z, zstride, bt, st);
 }
-// z = P^{-1} D v for the newest basis vector(s)
-static void precond_newest(Ctx& c, void* z, const Batch& bt, cudaStream_t st) {
-    if (c.vc32) MG<BAH_MIXED>::template precond<float2>(c, (const float2*)c.Vc, c.ks.sw, (float2*)z, c.ks.sz, bt, st);
-    else precond_any(c, (const double2*)c.Vc, c.ks.sw, z, c.ks.sz, bt, st);
+// slot j of the flexible basis
+static void* z_slot(Ctx& c, int j) { return (char*)c.Z + (size_t)j * c.vec_len() * c.vsz; }
+// where vector i stands as the preconditioner's input in FP32 (the last one is no input)
+static float2* vc32_slot(Ctx& c, int i) { return i < c.m ? (float2*)z_slot(c, i) : nullptr; }
+// z_j = P^{-1} D v_j for the newest basis vector(s).  In place (vc32): the distributor has read
+// all of v before the pressure cycle writes, and the displacements' right-hand sides read v's
+// displacements before their cycles write
+static void precond_newest(Ctx& c, int j, const Batch& bt, cudaStream_t st) {
+    void* z = z_slot(c, j);
+    if (c.vc32) MG<BAH_MIXED>::template precond<float2>(c, (const float2*)z, c.ks.sz, (float2*)z, c.ks.sz, bt, st);
+    else precond_any(c, c.W, c.ks.sw, z, c.ks.sz, bt, st);
 }
 // w / sc[slot] as basis vector i and as the newest vector
 static void store_basis(Ctx& c, const double2* w, int slot, int i, cudaStream_t st, const GivensArgs* gv = nullptr) {
@@ -845,8 +859,8 @@ static void store_basis(Ctx& c, const double2* w, int slot, int i, cudaStream_t 
     const Tiles tl = c.tiles();
     int4* vl = c.VL + i * tl.padded();
     int* ve = c.VE + (size_t)i * tl.count;
-    if (c.vc32) launch_basis_store(w, c.nrm, slot, (float2*)c.Vc, vl, ve, tl, n, c.nbatch, c.ks, st, gv);
-    else launch_basis_store(w, c.nrm, slot, (double2*)c.Vc, vl, ve, tl, n, c.nbatch, c.ks, st, gv);
+    if (c.vc32) launch_basis_store(w, c.nrm, slot, vc32_slot(c, i), c.ks.sz, vl, ve, tl, n, c.nbatch, c.ks, st, gv);
+    else launch_basis_store(w, c.nrm, slot, c.W, n, vl, ve, tl, n, c.nbatch, c.ks, st, gv);
 }
 // algorithmic bytes of one operator apply: input (3 components), FP64
 // output, coefficients cx, nx (z-aliases when h1 == h2), d1, d2, 1/(lambda+mu)
@@ -894,6 +908,15 @@ static void op_apply_z(Ctx& c, const void* z, size_t zstride, void* y, size_t ys
     }
 }
 
+// The solve's x and b buffers, allocated first: until the first solve they hold what only the
+// setup needs (the medium and what is formed from it), so that it takes no memory of its own.
+static int alloc_setup(Ctx& c) {
+    const size_t n = c.vec_len() * c.nbatch;
+    TRY(c.alloc_t(&c.X, n));
+    TRY(c.alloc_t(&c.Bs, n));
+    return BAH_OK;
+}
+
 // FGMRES workspace for nbatch right-hand sides: bases V (FP64 or
 // double-float) and Z (the preconditioner's precision), Hessenberg matrices,
 // rotations, reduction partials, status slots and the per-step graphs
@@ -912,11 +935,9 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
         TRY(c.alloc_t(&c.VE, nt * (m + 1) * nbt));
         // the 2-D FP32 cycles read the newest vector in FP32 only
         c.vc32 = c.mode == BAH_MIXED && c.dim == 2 && !c.exact;
-        TRY(c.alloc(&c.Vc, n * nbt * (c.vc32 ? sizeof(float2) : sizeof(double2))));
     }
     TRY(c.alloc(&c.Z, n * m * c.vsz * nbt));
-    TRY(c.alloc_t(&c.W, n * nbt)); TRY(c.alloc_t(&c.R, n * nbt)); TRY(c.alloc_t(&c.Bs, n * nbt));
-    TRY(c.alloc_t(&c.X, n * nbt));
+    TRY(c.alloc_t(&c.W, n * nbt)); TRY(c.alloc_t(&c.R, n * nbt));
     TRY(c.alloc(&c.ztmp, n * c.vsz));
     TRY(c.alloc_t(&c.Hm, (size_t)(m + 1) * m * nbt));
     TRY(c.alloc_t(&c.h1v, so * nbt)); TRY(c.alloc_t(&c.h2v, so * nbt));
@@ -924,7 +945,8 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     BAH_CUDA_TRY(cudaMemsetAsync(c.gscnt, 0, nbt * sizeof(int), st));
     TRY(c.alloc_t(&c.cs, so * nbt)); TRY(c.alloc_t(&c.sn, so * nbt)); TRY(c.alloc_t(&c.g, so * nbt));
     TRY(c.alloc_t(&c.y, so * nbt));
-    TRY(c.alloc_t(&c.partial, so * GS_CTAS * nbt));
+    const size_t np = c.kdf ? RED_CTAS : dot_ctas(tl, c.nbatch);      // partial sums of a row
+    TRY(c.alloc_t(&c.partial, so * np * nbt));
     TRY(c.alloc_t(&c.dpart, (size_t)GS_CTAS * nbt));
     TRY(c.alloc_t(&c.nrm, 8 * nbt));
     TRY(c.alloc_t(&c.status, 4 * nbt));
@@ -934,7 +956,7 @@ static int alloc_krylov(Ctx& c, cudaStream_t st) {
     BAH_CUDA_TRY(cudaMallocHost((void**)&c.hstatus, (4 * (size_t)(m + 1) * nbt + 8 * nbt) * sizeof(double)));
     BAH_CUDA_TRY(cudaMallocHost((void**)&c.hint, kIntSlots * nbt * sizeof(int)));
     c.ks.sv = (size_t)(m + 1) * (c.VL ? tl.padded() : n); c.ks.se = (size_t)(m + 1) * nt;
-    c.ks.sw = n; c.ks.sp = so * GS_CTAS; c.ks.so = so;
+    c.ks.sw = n; c.ks.sp = so * np; c.ks.so = so;
     c.ks.sh = (size_t)(m + 1) * m; c.ks.sz = (size_t)m * n; c.ks.sx = n; c.ks.active = c.active;
     BAH_CUDA_TRY(cudaStreamCreateWithFlags(&c.cap_stream, cudaStreamNonBlocking));
     c.ig.assign(m, Ctx::IterGraph());
@@ -952,8 +974,9 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     const int np = c.np;
     const size_t cs = c.mode == BAH_MIXED ? 2 : 8, ccs = c.mode == BAH_MIXED ? 4 : 16;
     // medium upload
-    double *lam, *mu, *rho, *gam;
-    TRY(c.alloc_t(&lam, np)); TRY(c.alloc_t(&mu, np)); TRY(c.alloc_t(&rho, np)); TRY(c.alloc_t(&gam, np));
+    TRY(alloc_setup(c));
+    double *lam = (double*)c.X, *mu = lam + np, *rho = mu + np, *gam;
+    TRY(c.alloc_t(&gam, np));
     BAH_CUDA_TRY(cudaMemcpyAsync(lam, med->lambda, np * sizeof(double), cudaMemcpyHostToDevice, st));
     BAH_CUDA_TRY(cudaMemcpyAsync(mu, med->mu, np * sizeof(double), cudaMemcpyHostToDevice, st));
     BAH_CUDA_TRY(cudaMemcpyAsync(rho, med->rho, np * sizeof(double), cudaMemcpyHostToDevice, st));
@@ -961,10 +984,10 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     TRY(c.alloc_t(&c.cx, np)); TRY(c.alloc_t(&c.cz, np)); TRY(c.alloc_t(&c.nx, np)); TRY(c.alloc_t(&c.nz, np));
     TRY(c.alloc_t(&c.wx, np)); TRY(c.alloc_t(&c.wz, np)); TRY(c.alloc_t(&c.cinv, np));
     TRY(c.alloc_t(&c.d1, np)); TRY(c.alloc_t(&c.d2, np)); TRY(c.alloc_t(&c.dAp, np));
-    for (int b = 0; b < 3; ++b) TRY(c.alloc_t(&c.dg[b], np));
+    double2* const dg[3] = {c.Bs, c.Bs + np, c.Bs + 2 * (size_t)np};
     c.gam = gam;
     launch_medium_prep(c.n1, c.n2, c.h1, c.h2, c.omega, c.alpha, lam, mu, rho, gam, c.cx, c.cz, c.nx, c.nz, c.wx,
-                       c.wz, c.d1, c.d2, c.cinv, c.dg[0], c.dg[1], c.dg[2], c.dAp, st);
+                       c.wz, c.d1, c.d2, c.cinv, dg[0], dg[1], dg[2], c.dAp, st);
     BAH_CUDA_TRY(cudaGetLastError());
     c.op = OpCoef{c.n1, c.n2, c.cx, c.cz, c.nx, c.nz, c.d1, c.d2, c.cinv, 1.0 / c.h1, 1.0 / c.h2};
     // double-float copies of the operator coefficients for w = H z on the FP32
@@ -1023,7 +1046,7 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     }
     for (int b = 0; b < 3; ++b) {
         TRY(c.alloc(&c.s_dg[b], np * ccs));
-        launch_round_cplx(c.dg[b], c.s_dg[b], np, c.mode, st);
+        launch_round_cplx(dg[b], c.s_dg[b], np, c.mode, st);
     }
     TRY(c.alloc(&c.s_dAp, np * ccs));
     launch_round_cplx(c.dAp, c.s_dAp, np, c.mode, st);
@@ -1033,7 +1056,7 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     if (c.mode == BAH_FP64)
         for (int b = 0; b < 3; ++b) {
             TRY(c.alloc_t(&c.idg[0][b], np));
-            launch_inverse_diag(c.dg[b], c.idg[0][b], np, st);
+            launch_inverse_diag(dg[b], c.idg[0][b], np, st);
         }
 
     // hierarchy: level grids, FP64 stencils, Galerkin products, storage copies
@@ -1044,7 +1067,7 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
         StencilF64& s0 = c.s64[0][b];
         s0.rx = 1; s0.rz = 1; s0.n1 = c.n1; s0.n2 = c.n2;
         TRY(c.alloc_t(&s0.S, (size_t)9 * np));
-        launch_fine_stencil(b, c.n1, c.n2, c.cx, c.cz, c.nx, c.nz, c.wx, c.wz, c.dg[b], s0.S, st);
+        launch_fine_stencil(b, c.n1, c.n2, c.cx, c.cz, c.nx, c.nz, c.wx, c.wz, dg[b], s0.S, st);
         for (int l = 1; l < c.L; ++l) {
             StencilF64& s = c.s64[l][b];
             const bool bil = c.o.intergrid == BAH_INTERGRID_BILINEAR;
@@ -1055,9 +1078,12 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
             TRY(c.alloc_t(&s.S, ns));
             launch_galerkin(b, c.o.intergrid, c.s64[l - 1][b], s, st);
             if (l < c.L - 1) {
-                TRY(c.alloc(&c.sst[l][b], ns * ccs));
-                launch_round_cplx(s.S, c.sst[l][b], ns, c.mode, st);
-                if (c.mode == BAH_FP64) {
+                if (c.mode == BAH_MIXED) {
+                    TRY(c.alloc(&c.sst[l][b], ns * ccs));
+                    launch_round_cplx(s.S, c.sst[l][b], ns, c.mode, st);
+                } else {
+                    TRY(c.alloc(&c.sst[l][b], ns * ccs));
+                    launch_round_cplx(s.S, c.sst[l][b], ns, c.mode, st);
                     const size_t npl = (size_t)s.n1 * s.n2;
                     TRY(c.alloc_t(&c.idg[l][b], npl));
                     launch_inverse_diag(s.S + (s.rz * (2 * s.rx + 1) + s.rx) * npl, c.idg[l][b], npl, st);
@@ -1165,12 +1191,12 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
         TRY(gs_prepare());
         const Tiles tl(np, np);
         TRY(c.alloc_t(&c.iVL, (c.mi + 1) * tl.padded())); TRY(c.alloc_t(&c.iVE, (size_t)(c.mi + 1) * tl.count));
-        TRY(c.alloc_t(&c.iVc, np)); TRY(c.alloc_t(&c.iZ, (size_t)c.mi * np));
+        TRY(c.alloc_t(&c.iZ, (size_t)c.mi * np));
         TRY(c.alloc_t(&c.iW, np)); TRY(c.alloc_t(&c.iR, np));
         TRY(c.alloc_t(&c.iH, (size_t)(c.mi + 1) * c.mi));
         TRY(c.alloc_t(&c.ih1, so)); TRY(c.alloc_t(&c.ih2, so)); TRY(c.alloc_t(&c.ics, so)); TRY(c.alloc_t(&c.isn, so));
         TRY(c.alloc_t(&c.igv, so)); TRY(c.alloc_t(&c.iy, so));
-        TRY(c.alloc_t(&c.ipart, so * GS_CTAS)); TRY(c.alloc_t(&c.idpart, (size_t)GS_CTAS));
+        TRY(c.alloc_t(&c.ipart, so * dot_ctas(tl, 1))); TRY(c.alloc_t(&c.idpart, (size_t)GS_CTAS));
         TRY(c.alloc_t(&c.inrm, 8)); TRY(c.alloc_t(&c.istatus, 4)); TRY(c.alloc_t(&c.iflag, 1)); TRY(c.alloc_t(&c.icnt, 1));
         BAH_CUDA_TRY(cudaMemsetAsync(c.icnt, 0, sizeof(int), st));
         TRY(c.alloc_t(&c.ijk, 1));
@@ -1182,7 +1208,6 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
     if (const char* e = getenv("BAH_STAGED")) c.staged = (e[0] != '0');
     if (const char* e = getenv("BAH_DGKS_ETA2")) c.dgks_eta2 = atof(e);
     BAH_CUDA_TRY(cudaStreamSynchronize(st));
-    // the raw medium is no longer needed
     return BAH_OK;
 }
 
@@ -1193,15 +1218,17 @@ static int build(Ctx& c, const bah_medium* med, cudaStream_t st) {
 static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
     NvtxRange nv("bah setup (3-D)");
     const size_t np = c.np;
-    double *lam, *mu, *rho, *gam, *cinv, *mue[3];
+    TRY(alloc_setup(c));
+    double *lam = (double*)c.X, *mu = lam + np, *rho = mu + np, *w = rho + np, *gam, *cinv;
+    double* const mue[3] = {w + np, w + 2 * np, w + 3 * np};         // seven arrays of the eight that X has room for
     double2 *mrt, *dg[3];
-    TRY(c.alloc_t(&lam, np)); TRY(c.alloc_t(&mu, np)); TRY(c.alloc_t(&rho, np)); TRY(c.alloc_t(&gam, np));
+    TRY(c.alloc_t(&gam, np));
     BAH_CUDA_TRY(cudaMemcpyAsync(lam, med->lambda, np * sizeof(double), cudaMemcpyHostToDevice, st));
     BAH_CUDA_TRY(cudaMemcpyAsync(mu, med->mu, np * sizeof(double), cudaMemcpyHostToDevice, st));
     BAH_CUDA_TRY(cudaMemcpyAsync(rho, med->rho, np * sizeof(double), cudaMemcpyHostToDevice, st));
     BAH_CUDA_TRY(cudaMemcpyAsync(gam, med->gamma, np * sizeof(double), cudaMemcpyHostToDevice, st));
     TRY(c.alloc_t(&cinv, np)); TRY(c.alloc_t(&mrt, np));
-    for (int e = 0; e < 3; ++e) { TRY(c.alloc_t(&mue[e], np)); TRY(c.alloc_t(&dg[e], np)); }
+    for (int e = 0; e < 3; ++e) TRY(c.alloc_t(&dg[e], np));
     c.gam = gam;
     Op3& o = c.op3;
     o.n[0] = c.n1; o.n[1] = c.n2; o.n[2] = c.n3;
@@ -1249,6 +1276,9 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
                 // the mixed cycle's stencils in bfloat16 (entries rounded once from FP64)
                 TRY(c.alloc(&c.s3s[l][q], cnt * sizeof(__nv_bfloat162)));
                 launch_round_cplx(c.s3[l][q], c.s3s[l][q], cnt, BAH_MIXED, st);
+            } else if (l == 0) {
+                TRY(c.alloc(&c.s3s[l][q], cnt * sizeof(double2)));
+                BAH_CUDA_TRY(cudaMemcpyAsync(c.s3s[l][q], c.s3[l][q], cnt * sizeof(double2), cudaMemcpyDeviceToDevice, st));
             } else {
                 c.s3s[l][q] = c.s3[l][q];
             }
@@ -1259,8 +1289,6 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
         }
     // level-0 coefficients of the cycle: those of the operator, and the pressure block's
     {
-        double* w = nullptr;
-        TRY(c.alloc_t(&w, np));
         launch_wp3(mu, cinv, w, np, st);
         const double* wv[3] = {nullptr, nullptr, nullptr};
         for (int a = 0; a < 3; ++a) TRY(scaled(w, a, wv, &wv[a]));
@@ -1301,6 +1329,11 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
     if (herr) {
         set_error("3-D Galerkin product produced a coupling beyond one coarse point");
         return BAH_ERR_CUDA;
+    }
+    // the seven-point level-0 stencils have served the Galerkin product
+    for (int q = 0; q < 4; ++q) {
+        c.release(c.s3[0][q]);
+        c.s3[0][q] = nullptr;
     }
     // coarsest inverses
     TRY(coarse_prepare());
@@ -1370,11 +1403,11 @@ static void iter_body(Ctx& c, int j, cudaStream_t st) {
     Batch bt;
     bt.nr = nb;
     bt.active = c.active;
-    void* zj = (char*)c.Z + (size_t)j * n * c.vsz;
+    void* zj = z_slot(c, j);
     float4* Vd = (float4*)c.V;
     float4* Wd = (float4*)c.W;
     if (c.kdf) precond_any(c, Vd + (size_t)j * n, ks.sv, zj, ks.sz, bt, st);
-    else precond_newest(c, zj, bt, st);
+    else precond_newest(c, j, bt, st);
     op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
     const double k1 = j + 1;
     int npt = 0;                 // partial sums of ||w'||^2 (double-float basis)
@@ -1619,11 +1652,11 @@ static void enqueue_cholqr2(Ctx& c, int s, double2* W, int i, double2* R12, cuda
     int* ve = c.VE + (size_t)i * tl.count;
     launch_block_gram(s, W, tl, c.bpart, c.bG, st);
     launch_block_chol(c.bG, s, R12, c.bT, st);
-    launch_block_scale(W, s, c.bT, W, nullptr, nullptr, 0, 0, tl, st);
+    launch_block_scale(W, s, c.bT, W, tl.n, nullptr, nullptr, 0, 0, tl, st);
     launch_block_gram(s, W, tl, c.bpart, c.bG, st);
     launch_block_chol(c.bG, s, R12 + s * s, c.bT, st);
-    if (c.vc32) launch_block_scale(W, s, c.bT, (float2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, tl, st);
-    else launch_block_scale(W, s, c.bT, (double2*)c.Vc, vl, ve, c.ks.sv, c.ks.se, tl, st);
+    if (c.vc32) launch_block_scale(W, s, c.bT, vc32_slot(c, i), c.ks.sz, vl, ve, c.ks.sv, c.ks.se, tl, st);
+    else launch_block_scale(W, s, c.bT, c.W, tl.n, vl, ve, c.ks.sv, c.ks.se, tl, st);
 }
 // R = R_2 R_1 from the host copy of R12
 static int host_r(int s, const double2* R12, std::vector<cdx>& R) {
@@ -1735,9 +1768,8 @@ static int fgmres_block(Ctx& c, const double2* b, double2* x, int s, double rtol
     // step j up to and including its copy to host slot j & 1: [R_1 | R_2 | C_1 | C_2]
     auto enqueue = [&](int j) {
         NvtxRange nvs("block fgmres step");
-        void* zj = (char*)c.Z + (size_t)j * n * c.vsz;
-        precond_newest(c, zj, bt, st);
-        op_apply_z(c, zj, ks.sz, c.W, n, bt, st);
+        precond_newest(c, j, bt, st);
+        op_apply_z(c, z_slot(c, j), ks.sz, c.W, n, bt, st);
         const size_t cnt = (size_t)(j + 1) * s2;
         for (int pass = 0; pass < 2; ++pass) {            // block CGS2
             double2* C = c.bC + 2 * s2 + pass * cnt;

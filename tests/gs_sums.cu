@@ -26,7 +26,7 @@ struct Basis {                      // vectors of V (n entries each) as basis ve
     }
     bool ok() const { return vl.p && ve.p && vc.p && sc.p; }
     void store(const double2* v, int row) {
-        launch_basis_store(v, sc.as<double>(), 0, vc.as<double2>(), vl.as<int4>() + row * tl.padded(),
+        launch_basis_store(v, sc.as<double>(), 0, vc.as<double2>(), tl.n, vl.as<int4>() + row * tl.padded(),
                            ve.as<int>() + (size_t)row * tl.count, tl, 0, 1, KS(), 0);
     }
 };
@@ -67,7 +67,7 @@ int block_products(const double2* V, int k, int s, double2* W, long long n, long
     const int* ve = b.ve.as<int>();
     launch_block_dot(vl, ve, sv, se, k, s, W, b.tl, part.as<double2>(), C, 0);
     launch_block_gram(s, W, b.tl, part.as<double2>(), G, 0);
-    launch_block_scale(W, s, T, W2, nullptr, nullptr, 0, 0, b.tl, 0);
+    launch_block_scale(W, s, T, W2, b.tl.n, nullptr, nullptr, 0, 0, b.tl, 0);
     launch_block_update(vl, ve, sv, se, k, s, Y, W, b.tl, 0);
     return finish();
 }
