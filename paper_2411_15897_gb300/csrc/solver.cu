@@ -1242,7 +1242,8 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
     auto pts = [&](int l) { return (size_t)c.d3[l][0] * c.d3[l][1] * c.d3[l][2]; };
     c.s3.assign(c.L, {nullptr, nullptr, nullptr, nullptr});
     c.s3s.assign(c.L, {nullptr, nullptr, nullptr, nullptr});
-    for (int q = 0; q < 4; ++q) TRY(c.alloc_t(&c.s3[0][q], 7 * np));
+    TRY(c.alloc_t(&c.s3[0][0], 4 * 7 * np));
+    for (int q = 1; q < 4; ++q) c.s3[0][q] = c.s3[0][0] + q * 7 * np;
     launch_prep3(o, c.omega, c.alpha, lam, mu, rho, gam, cinv, mrt, mue, dg, c.s3[0].data(), st);
     // mu and its edge means divided by the squared spacings
     auto scaled = [&](const double* src, int a, const double* const* earlier, const double** dst) {
@@ -1331,10 +1332,8 @@ static int build3(Ctx& c, const bah_medium* med, cudaStream_t st) {
         return BAH_ERR_CUDA;
     }
     // the seven-point level-0 stencils have served the Galerkin product
-    for (int q = 0; q < 4; ++q) {
-        c.release(c.s3[0][q]);
-        c.s3[0][q] = nullptr;
-    }
+    c.release(c.s3[0][0]);
+    c.s3[0] = {nullptr, nullptr, nullptr, nullptr};
     // coarsest inverses
     TRY(coarse_prepare());
     {
