@@ -468,7 +468,7 @@ def run_bah(args):
                 "ms_per_step": statistics.mean(ms64), "relres_true": stt["relres_true"]}
         s64.close()
 
-    # the same mixed solve with the Krylov basis in double-FP32 (48-bit) instead of IEEE FP64
+    # the same mixed solve with the Krylov basis in double-FP32 (48-bit) instead of 60-bit block fixed point
     kdf = None
     if args.krylov == "fp64" and args.krylov_df_steps > 0 and prob.dim == 2:
         sk = bah.Solver.from_problem(prob, **dict(opts, krylov_arith=bah.BAH_KRYLOV_DF))

@@ -1,21 +1,30 @@
-// FP64-accurate sums of products on the integer pipe.
+// Sums of products on the integer pipe, with FP64's rounding in the norm.
 //
 // GB300 issues 2 FP64 multiply-adds per clock and SM, but 28 integer ones of
 // 32 x 32 + 64 bits (both measured; a complex product takes 4 of the first or
-// 12 of the second).  A vector that meets many others is therefore held as block fixed point: the entries of a tile (kTile entries)
+// 12 of the second).  A vector that meets many others is therefore held as block
+// fixed point: the entries of a tile (kTile entries of one component)
 // share one exponent E, |x| < 2^E for every real of the tile, and each real is
 // the 60-bit integer X = round(x 2^(59 - E)), split into two signed limbs,
 // X = h 2^30 + l with |h| <= 2^29, -2^29 <= l < 2^29.  A product of two such
 // integers takes three multiply-adds (h h, and h l + l h into a second
 // accumulator); l l lies below 2^-60 of the largest product and its mean is
 // zero unless both factors are the same number.  Sums of the products are
-// exact integers.  So the error is that of rounding the inputs to 2^-60 of
-// the tile's largest entry, where an FP64 sum rounds every partial sum to
-// 2^-53 of itself: a tile's largest entry is at most 22 times its r.m.s.
+// exact integers, rounded to FP64 once.
+//
+// Error: every factor is rounded to 2^-59 of its tile's largest real.  Where one
+// factor is a coefficient, it gives up head bits so that all rows' products fit
+// (rounding and l l terms: 2^-56 of the largest product with up to 32 rows, 2^-51
+// with 1024); a dense row of np points gives up dense_head(np).  An FP64 sum
+// rounds every partial sum to 2^-53 of itself.  So the bound is one in the norm
+// (a tile's largest real is at most sqrt(512) = 22.6 times its r.m.s.), and none
+// per entry: a real 2^-q below its tile's largest keeps 60 - q bits, where FP64
+// keeps 53, and from q = 60 on it counts as 0.  Entries of unrelated size (the
+// components of a vector, in their own units) therefore never share a tile.
 //
 // Exponents are stored biased as in an FP64 number (E + 1023), at least
 // kExpMin; a tile with an infinity or NaN stores kExpBad, and every sum it
-// enters becomes NaN.  Entries below 2^-60 of the tile's largest count as 0.
+// enters becomes NaN.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -136,11 +145,10 @@ __device__ __forceinline__ T warp_sum_values(T* v, int lane) {
 // row) and g converted once per CTA: the coarsest solve with the FP64 inverse.
 // dense_head(np): bits that g gives up so that a lane's np / 32 products of
 // 2 x 2^58 fit 2^62 (none up to 256 points, 4 at 4096).
-// Bound: reading the inverse from L2.  With FP64 multiply-adds the solve was
-// bound by the FP64 pipe, on 16 SMs inside the cluster kernel: W(1,2) on
-// 400 x 128 (800 points, 4 or 8 solves per launch) 215 -> 89 us per launch,
-// 64 x 64 (256 points) 27.6 -> 21.5 us, 48 x 40 x 28 (840 points, three blocks,
-// all SMs) 32 -> 14 us per launch.
+// Bound: the chain of conversion, barriers and L2 reads.  With FP64 multiply-adds the
+// solve was bound by the FP64 pipe: 48 x 40 x 28 (840 points, three blocks, all SMs)
+// 32 -> 14 us per launch; inside the cluster kernel, on 16 SMs, 64 x 64 (256 points)
+// 27.6 -> 21.5 us.
 // ---------------------------------------------------------------------------
 __host__ __device__ inline int dense_head(int np) {
     int h = 0;

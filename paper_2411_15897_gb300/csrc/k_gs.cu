@@ -9,8 +9,10 @@
 //   7.1 -> 3.1 ms (6.6 and 6.4 TB/s); one source at 1024 x 1024: 450 -> 136 us
 //   and 262 -> 128 us; 128^3: 1.28 -> 0.32 ms and 0.74 -> 0.33 ms.
 // Accuracy against 113-bit sums on the Arnoldi vectors of a point source
-// (320 x 200, k = 1 .. 20): update error 0.7e-16 .. 1.2e-16 of |w'| (FP64 sums:
-// 0.7e-16 .. 3.9e-16, growing with k), projections within 9e-17 |w| (7e-17).
+// (320 x 200), in the norm: update error 0.2e-16 of |w'| at k = 1 and 1.2e-16 at
+// k = 2 (FP64 sums: 0 and 0.7e-16; v_0 has one nonzero entry), 0.7e-16 .. 1.0e-16
+// for k = 3 .. 20 (1.1e-16 .. 3.9e-16, growing with k); projections within
+// 9e-17 |w| (7e-17).  Per entry there is no such bound (fix60.cuh).
 //
 // Batched over right-hand sides (blockIdx.z) with the flags and strides of
 // k_krylov.cu: pass 1 forms h1 = V^H w together with ||w||^2 and then

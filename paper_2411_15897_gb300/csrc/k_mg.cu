@@ -269,8 +269,9 @@ void launch_prolong_add(const LvlSet<typename Prec<MODE>::V, typename Prec<MODE>
 // ---------------------------------------------------------------------------
 // coarsest level: x = A_c^{-1} b with the stored FP64 inverse (one warp per
 // row).  The inverse and the right-hand side are in block fixed point and the
-// products are exact integers (fix60.cuh): no less accurate than FP64 sums, at
-// the integer pipe's rate instead of 2 FP64 multiply-adds per clock and SM.
+// products are exact integers (fix60.cuh; rounding relative to the largest entry of
+// a row and of the right-hand side, each block's own), at the integer pipe's rate
+// instead of 2 FP64 multiply-adds per clock and SM.
 // Each CTA converts the right-hand side once; the result is rounded once to
 // the cycle's precision.
 // ---------------------------------------------------------------------------
