@@ -30,7 +30,9 @@ template <int MODE> constexpr int kTpb = MODE == BAH_FP64 ? 64 : 256;
 
 // ---------------------------------------------------------------------------
 // damped Jacobi:  x_out = x_in + w D^{-1} (b - A x_in)   (zero_init: w D^{-1} b, on level 0;
-// below it the restriction writes the first sweep).  FP64: the first sweep only.
+// below it the restriction writes the first sweep).  FP64 launches it for the first sweep only;
+// compiled for that alone (24 registers instead of 42), 20 steps of 512 x 512 took 14.54 ms
+// instead of 14.48, so the general path stays beside it.
 // ---------------------------------------------------------------------------
 template <int MODE, bool L0, int RM>
 __global__ void __launch_bounds__(kTpb<MODE>) k_jacobi(LvlSet<typename MGT<MODE>::V, typename MGT<MODE>::CC> s,
@@ -47,13 +49,14 @@ __global__ void __launch_bounds__(kTpb<MODE>) k_jacobi(LvlSet<typename MGT<MODE>
     const int i = t % n1, j = t / n1;
     if (!valid_pt(B.type, i, j)) { xout[t] = czero<V>(); return; }
     const V b = B.b[rr * B.sb + t];
-    if constexpr (MODE == BAH_FP64) {
-        xout[t] = cscale(cmul(B.idg[t], b), w);
-        return;
-    }
-    if (L0 && zero_init) {
-        xout[t] = cscale(cdiv(b, diag_only<MODE>(&f5, B, np, t)), w);
-        return;
+    if (zero_init) {
+        if constexpr (MODE == BAH_FP64) {
+            xout[t] = cscale(cmul(B.idg[t], b), w);
+            return;
+        } else if constexpr (L0) {
+            xout[t] = cscale(cdiv(b, diag_only<MODE>(&f5, B, np, t)), w);
+            return;
+        }
     }
     const V* __restrict__ xin = B.xin + rr * B.sxi;
     auto X = [&](int g) { return xin[g]; };
